@@ -734,9 +734,8 @@ int32_t sfs_generate_begin(sfs_session *s, const int32_t *d_prompt, int32_t B, i
         if (rc != SFS_OK) return rc;
         // Long bf16 rows: the LM head takes the first pass of the row statistics in its epilogue (one record per row,
         // column tile and epilogue-warp parity), so the selection step never streams the logits back from memory.
-        // (tiles of at least 128 columns: then both epilogue-warp parities own columns of every 256-row block)
-        if (row_stats_two_pass_applies(s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab) && s->lm_plan.args.splits == 1 && s->lm_plan.args.bn >= 128) {
-            const int parts = 2 * s->lm_plan.args.n_col_tiles;
+        const int parts = s->lm_plan.args.stats_parts;
+        if (row_stats_two_pass_applies(s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab) && s->lm_plan.args.splits == 1 && parts > 0) {
             const size_t need = (size_t)B * gen_len * parts;
             if (s->lm_stats_cap < need) {
                 SFS_CUDA(cudaStreamSynchronize(st));

@@ -23,17 +23,19 @@ struct GemmArgs {
     int n_per_map;           // rows of each B matrix
     int bn, stages;          // tile width (multiple of 16, <= 256) and depth of the shared-memory ring
     int mb;                  // 256-row blocks per tile (1 or 2)
-    int one_cta;             // 1: tiles of 128 rows computed by single CTAs (few rows: the weights stream through every SM)
-    int tile_rows;           // output rows per tile: mb * 256, or 128
+    int few;                 // 1: at most 128 rows, tiles of 128 x (nb x bn) (the weights stream through every SM)
+    int nb;                  // N-blocks of bn weight rows per few-row tile (1 or 2; SwiGLU: gate and up)
+    int tile_rows, tile_cols;        // output rows (mb * 256, or 128) and columns per tile
     int n_col_tiles;         // column tiles over all B matrices
     int splits, kb_per_split;        // split-K: the k-blocks are cut into `splits` ranges, range s writes slab s of C
     long long split_stride;          // elements between slabs
     int acc_bufs;            // accumulator buffers in tensor memory (2 when they fit: epilogue overlaps the next tile)
     // Optional (GEMM_STORE, bf16 output, no split): row statistics of the stored values, taken in the epilogue.  Per output
-    // row, column tile and epilogue-warp parity one record (maximum, reference, sum of 2^((x - reference) log2 e), first
-    // position of the maximum as int bits) at stats[row * stats_ld + 2 * column_tile + parity]: the first pass of the
-    // selection step's row statistics, fused into the LM head (the logits are not read back for it).
+    // row, column tile (few rows: N-block and column half of it) and epilogue-warp parity one record (maximum, reference, sum
+    // of 2^((x - reference) log2 e), first position of the maximum as int bits) at stats[row * stats_ld + record]: the first
+    // pass of the selection step's row statistics, fused into the LM head (the logits are not read back for it).
     float4 *stats; int stats_ld;
+    int stats_parts;         // records per row (0: this tile shape leaves none)
     int32_t *err;            // device status word, set to SFS_ERR_TIMEOUT if a bounded wait gives up
     const int32_t *d_active; // optional: the kernel does nothing when *d_active == 0
 };
@@ -46,7 +48,7 @@ struct GemmPlan {
 };
 
 // Optional overrides of the tile shape the planner would pick (0 = keep the planner's choice); for measurements.
-struct GemmTune { int mb, bn, stages, splits; };
+struct GemmTune { int mb, bn, stages, splits, nb; };
 
 // Bs: n_maps weight matrices [n_per_map, K] (ldb elements between rows) whose outputs are concatenated along
 // the columns of C (QKV), or gate / up for GEMM_SWIGLU (then C has n_per_map columns).

@@ -60,7 +60,8 @@ constexpr int BM = 128, BK = 64;         // rows per CTA of one 256-row MMA bloc
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
 constexpr int A_BYTES = BM * BK * 2;
-constexpr int kMaxStages = 8;
+constexpr int FM = 64;                   // few-row tiles: rows per CTA of the pair's 128-row MMA
+constexpr int kMaxStages = 12;
 constexpr int kSmemBudget = 227 * 1024 - 64;      // the opt-in maximum minus the kernel's static shared memory
 // barriers: full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2]; then the TMEM base slot
 constexpr int kBarBytes = (2 * kMaxStages + 4) * 8 + 16;
@@ -93,13 +94,12 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int
     const int n_tile = rest / g.splits;
     t.split = rest - n_tile * g.splits;
     if (g.mode == GEMM_SWIGLU) {
-        const int half = g.bn >> 1;
-        t.map_idx = 0; t.n_local = n_tile * half; t.ncol0 = t.n_local; t.ncols = min(half, g.N - t.ncol0);
+        t.map_idx = 0; t.n_local = n_tile * g.tile_cols; t.ncol0 = t.n_local; t.ncols = min(g.tile_cols, g.N - t.ncol0);
     } else {
         t.map_idx = n_tile / g.tiles_per_map;
-        t.n_local = (n_tile - t.map_idx * g.tiles_per_map) * g.bn;
+        t.n_local = (n_tile - t.map_idx * g.tiles_per_map) * g.tile_cols;
         t.ncol0 = t.map_idx * g.n_per_map + t.n_local;
-        t.ncols = min(g.bn, g.n_per_map - t.n_local);
+        t.ncols = min(g.tile_cols, g.n_per_map - t.n_local);
     }
     return t;
 }
@@ -156,44 +156,52 @@ __device__ __forceinline__ void flush_unit(const GemmArgs &g, long long slab, ui
     }
 }
 
-// One warp's share of a tile's epilogue: TMEM lane quarter q (32 rows) of every 256-row block, the units of parity `par`.
-// A unit may reach past the tile's valid columns: those accumulator columns exist (inside the 256-column buffer) and
+// Where one warp's share of a tile's accumulators lies: `blocks` blocks of `seg` output columns each (the pair kernel: 256-row
+// blocks under one another; the few-row kernel: N-blocks beside one another).
+struct EpiShare {
+    uint32_t tmem, tmem_block;   // tensor-memory address of block 0 (with the warp's lane quarter), columns between blocks
+    uint32_t up;                 // SwiGLU: columns from a gate accumulator to its up accumulator
+    int row0, row_block;         // output row of lane 0 in block 0, rows between blocks
+    int col0, col_block;         // output column of the first accumulator column in block 0, columns between blocks
+    int blocks, seg;             // number of blocks, accumulator columns of each that may be valid
+    int col_end;                 // columns at or beyond this belong to another tile or matrix
+    int rec, rec_block;          // fused row statistics: record of block 0, records between blocks
+    __device__ __forceinline__ int lim(int b) const { return min(col_end, col0 + b * col_block + seg); }
+};
+
+// One warp's share of a tile's epilogue: 32 rows of every block, the 64-column (fp32: 32-column) units of parity `par`.
+// A unit may reach past the block's valid columns: those accumulator columns exist (inside the 256-column buffer) and
 // are never stored.  The tensor-memory loads of the next piece are issued as soon as the current piece has been
 // converted, so their latency hides behind the parking and the stores of the current one.
 template <bool STATS>
-__device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord &t, uint32_t tmem_acc, uint32_t bn_pad, uint32_t stage,
-                                              int q, int par, int lane, int rank, int M)
+__device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare &e, int split, uint32_t stage, int par, int lane, int M)
 {
-    const int HALF = g.bn >> 1;
-    const int lim = min(t.ncol0 + t.ncols, g.N);         // first output column this tile must not touch
-    const uint32_t tq = tmem_acc + ((uint32_t)(q * 32) << 16);
-    const int grow_q = t.m0 + rank * BM + q * 32;        // first row of block 0 handled by this warp
-    if (g.mode == GEMM_SWIGLU || (g.mode == GEMM_STORE && !g.out_f32 && !(g.vt != nullptr && t.ncol0 >= g.vt_col0))) {
+    if (g.mode == GEMM_SWIGLU || (g.mode == GEMM_STORE && !g.out_f32 && !(g.vt != nullptr && e.col0 >= g.vt_col0))) {
         // ---- bf16 output (plain or SwiGLU): units of 64 output columns, handled as two pieces of 32
         const bool swiglu = (g.mode == GEMM_SWIGLU);
-        // the units of all 256-row blocks, numbered block by block, alternate between the two warps of a lane quarter
-        const int upb = (t.ncols + 63) / 64;                              // units per 256-row block
-        const int n_pieces = 2 * ((g.mb * upb - par + 1) / 2);
+        // the units of all blocks, numbered block by block, alternate between the two warps of a lane quarter
+        const int upb = (e.seg + 63) / 64;                                // units per block
+        const int n_pieces = 2 * ((e.blocks * upb - par + 1) / 2);
         auto piece_addr = [&](int pc) {                                   // tensor-memory column of piece pc
             const int u = par + 2 * (pc >> 1), b = u / upb, c = 64 * (u - b * upb);
-            return tq + (uint32_t)(b * bn_pad + c + 32 * (pc & 1));
+            return e.tmem + (uint32_t)b * e.tmem_block + (uint32_t)(c + 32 * (pc & 1));
         };
         uint32_t x0[32], x1[32];
         if (n_pieces > 0) {
             tc::tmem_ld32(piece_addr(0), x0);
-            if (swiglu) tc::tmem_ld32(piece_addr(0) + HALF, x1);
+            if (swiglu) tc::tmem_ld32(piece_addr(0) + e.up, x1);
         }
-        // fused row statistics (LM head): this lane's row of the current 256-row block
+        // fused row statistics (LM head): this lane's row of the current block
         const bool stats_on = STATS && (g.stats != nullptr) && !swiglu;
         float st_mx = -INFINITY, st_ref = 0.f, st_nref = 0.f, st_sum = 0.f;
         int st_arg = 0x7FFFFFFF, st_b = -1;
-        const int n_tile = (t.ncol0 / g.bn);                             // one weight matrix: column tile index
         auto stats_flush = [&]() {
             if (st_b < 0) return;
-            const int grow = grow_q + st_b * 2 * BM + lane;
-            if (grow < M) g.stats[(long long)grow * g.stats_ld + 2 * n_tile + par] = make_float4(st_mx, st_ref, st_sum, __int_as_float(st_arg));
+            const int grow = e.row0 + st_b * e.row_block + lane;
+            if (grow < M) g.stats[(long long)grow * g.stats_ld + e.rec + st_b * e.rec_block + par] = make_float4(st_mx, st_ref, st_sum, __int_as_float(st_arg));
         };
         for (int pc = 0; pc < n_pieces; ++pc) {
+            const int u = par + 2 * (pc >> 1), b = u / upb, col0 = e.col0 + b * e.col_block + 64 * (u - b * upb);
             uint32_t o[16];
             tc::tmem_ld_wait32(x0);
             if (swiglu) tc::tmem_ld_wait32(x1);
@@ -208,13 +216,13 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
             }
             if (pc + 1 < n_pieces) {
                 tc::tmem_ld32(piece_addr(pc + 1), x0);
-                if (swiglu) tc::tmem_ld32(piece_addr(pc + 1) + HALF, x1);
+                if (swiglu) tc::tmem_ld32(piece_addr(pc + 1) + e.up, x1);
             }
             if (stats_on) {
                 // statistics of the ROUNDED values, as a reader of the stored logits would see them
-                const int u = par + 2 * (pc >> 1), b = u / upb, col0 = t.ncol0 + 64 * (u - b * upb) + 32 * (pc & 1);
+                const int c0 = col0 + 32 * (pc & 1);
                 if (b != st_b) { stats_flush(); st_b = b; st_mx = -INFINITY; st_sum = 0.f; st_arg = 0x7FFFFFFF; st_ref = 0.f; st_nref = 0.f; }
-                const int nvalid = min(32, lim - col0);                  // columns of this piece inside the matrix (warp-uniform)
+                const int nvalid = min(32, e.lim(b) - c0);               // columns of this piece inside the matrix (warp-uniform)
                 float pm = -INFINITY;
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -231,8 +239,8 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
 #pragma unroll
                     for (int j = 15; j >= 0; --j) {
                         const float lo = __uint_as_float(o[j] << 16), hi = __uint_as_float(o[j] & 0xFFFF0000u);
-                        if (2 * j + 1 < nvalid && hi == pm) st_arg = col0 + 2 * j + 1;
-                        if (2 * j < nvalid && lo == pm) st_arg = col0 + 2 * j;
+                        if (2 * j + 1 < nvalid && hi == pm) st_arg = c0 + 2 * j + 1;
+                        if (2 * j < nvalid && lo == pm) st_arg = c0 + 2 * j;
                     }
                 }
                 float s0 = 0.f, s1 = 0.f;
@@ -248,21 +256,20 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
             }
             park16(stage, lane, 4 * (pc & 1), o);
             if (pc & 1) {
-                const int u = par + 2 * (pc >> 1), b = u / upb, c = 64 * (u - b * upb);
                 __syncwarp();
-                flush_unit<2, false>(g, 0, stage, lane, grow_q + b * 2 * BM, M, t.ncol0 + c, lim);
+                flush_unit<2, false>(g, 0, stage, lane, e.row0 + b * e.row_block, M, col0, e.lim(b));
                 __syncwarp();
             }
         }
         if (stats_on) stats_flush();
-    } else if (g.vt != nullptr && t.ncol0 >= g.vt_col0) {
+    } else if (g.vt != nullptr && e.col0 >= g.vt_col0) {
         // ---- V columns of the QKV projection go out transposed: the 32 lanes hold 32 consecutive tokens of a feature
-        const int upb = (t.ncols + 31) / 32;
-        const int n_pieces = (g.mb * upb - par + 1) / 2;
+        const int upb = (e.seg + 31) / 32;
+        const int n_pieces = (e.blocks * upb - par + 1) / 2;
         auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u / upb; return 32 * (u - *b * upb); };
         uint32_t v[32];
         int b0;
-        if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(tq + (uint32_t)(b0 * bn_pad + c), v); }
+        if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(e.tmem + (uint32_t)b0 * e.tmem_block + (uint32_t)c, v); }
         for (int pc = 0; pc < n_pieces; ++pc) {
             int b;
             const int c = piece_col(pc, &b);
@@ -270,11 +277,11 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
             tc::tmem_ld_wait32(v);
 #pragma unroll
             for (int j = 0; j < 32; ++j) { __nv_bfloat16 r = __float2bfloat16_rn(__uint_as_float(v[j]) * g.scale); h[j] = *reinterpret_cast<uint16_t *>(&r); }
-            if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(tq + (uint32_t)(bn2 * bn_pad + c2), v); }
-            const int grow = grow_q + b * 2 * BM + lane;
+            if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(e.tmem + (uint32_t)bn2 * e.tmem_block + (uint32_t)c2, v); }
+            const int grow = e.row0 + b * e.row_block + lane, col0 = e.col0 + b * e.col_block + c;
             if (grow < M) {
-                uint16_t *dst = reinterpret_cast<uint16_t *>(g.vt) + (long long)(t.ncol0 + c - g.vt_col0) * g.ldvt + grow;
-                const int nv = lim - (t.ncol0 + c);                        // valid features of this piece
+                uint16_t *dst = reinterpret_cast<uint16_t *>(g.vt) + (long long)(col0 - g.vt_col0) * g.ldvt + grow;
+                const int nv = e.lim(b) - col0;                            // valid features of this piece
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (j < nv) dst[(long long)j * g.ldvt] = h[j];
@@ -282,13 +289,13 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
         }
     } else {
         // ---- fp32 output (residual add, split-K slab, or fp32 logits): units of 32 columns
-        const int upb = (t.ncols + 31) / 32;
-        const int n_pieces = (g.mb * upb - par + 1) / 2;
+        const int upb = (e.seg + 31) / 32;
+        const int n_pieces = (e.blocks * upb - par + 1) / 2;
         auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u / upb; return 32 * (u - *b * upb); };
         const bool scale = (g.mode != GEMM_RESIDUAL_F32 && g.scale != 1.0f);
         uint32_t v[32];
         int b0;
-        if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(tq + (uint32_t)(b0 * bn_pad + c), v); }
+        if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(e.tmem + (uint32_t)b0 * e.tmem_block + (uint32_t)c, v); }
         for (int pc = 0; pc < n_pieces; ++pc) {
             int b;
             const int c = piece_col(pc, &b);
@@ -296,12 +303,13 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const TileCoord
             tc::tmem_ld_wait32(v);
 #pragma unroll
             for (int j = 0; j < 32; ++j) o[j] = scale ? __float_as_uint(__uint_as_float(v[j]) * g.scale) : v[j];
-            if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(tq + (uint32_t)(bn2 * bn_pad + c2), v); }
+            if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(e.tmem + (uint32_t)bn2 * e.tmem_block + (uint32_t)c2, v); }
             park16(stage, lane, 0, o);
             park16(stage, lane, 4, o + 16);
             __syncwarp();
-            if (g.mode == GEMM_RESIDUAL_F32 && g.splits == 1) flush_unit<4, true>(g, 0, stage, lane, grow_q + b * 2 * BM, M, t.ncol0 + c, lim);
-            else flush_unit<4, false>(g, (long long)t.split * g.split_stride, stage, lane, grow_q + b * 2 * BM, M, t.ncol0 + c, lim);
+            const int row = e.row0 + b * e.row_block, col0 = e.col0 + b * e.col_block + c;
+            if (g.mode == GEMM_RESIDUAL_F32 && g.splits == 1) flush_unit<4, true>(g, 0, stage, lane, row, M, col0, e.lim(b));
+            else flush_unit<4, false>(g, (long long)split * g.split_stride, stage, lane, row, M, col0, e.lim(b));
             __syncwarp();
         }
     }
@@ -454,7 +462,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
-            epilogue_tile<STATS>(g, t, tmem_base + buf * buf_stride, bn_pad, stage, q, par, lane, (int)rank, M);
+            EpiShare e;
+            e.tmem = tmem_base + buf * buf_stride + ((uint32_t)(q * 32) << 16); e.tmem_block = bn_pad; e.up = (uint32_t)HALF;
+            e.row0 = t.m0 + (int)rank * BM + q * 32; e.row_block = 2 * BM;
+            e.col0 = t.ncol0; e.col_block = 0; e.blocks = MB; e.seg = STATS ? BN : t.ncols;      // (every record is written)
+            e.col_end = min(t.ncol0 + t.ncols, g.N);
+            e.rec = 2 * (t.ncol0 / BN); e.rec_block = 0;
+            epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
@@ -469,22 +483,29 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (threadIdx.x == 0 && s_abort && g.err) atomicExch(g.err, SFS_ERR_TIMEOUT);
 }
 
-// ---- few rows (M <= 128): one CTA per tile ------------------------------------------------------------------
-// With at most 128 rows half of a pair's 256-row MMA would multiply padding, and what bounds the projection is streaming the
-// weights: every SM should pull its own slab of weight rows at full rate.  A CTA computes a 128 x BN tile with
-// tcgen05.mma.cta_group::1 (M = 128, N = BN), loading the 128 activation rows and BN weight rows of every k-block itself (the
-// weight rows as two boxes of BN / 2, SwiGLU: gate rows then up rows, so the accumulator layout and the epilogue are those
-// of the pair kernel); BN is chosen so that the tiles fill the SMs in whole waves.  Same warp roles, ring and bounded waits.
+// ---- few rows (M <= 128): weights stream through all SMs ---------------------------------------------------------
+// With at most 128 rows the projection is bound by streaming its weights: from HBM once, and from L2 into the SMs together
+// with the activation rows that every tile needs again.  A pair of CTAs computes a 128 x (NB x BN) tile with
+// tcgen05.mma.cta_group::2, M = 128: each CTA stages 64 activation rows and half of the weight rows of every N-block, so per
+// k-block an SM pulls 64 + NB * BN / 2 rows and the ring holds up to nine k-blocks of wide tiles.  Measured at 128 rows, 8B
+// widths, weights from HBM, QKV / O / gate-up / down in us: 24.8 / 12.0 / 40.2 / 24.0 (the HBM floor at 6458 GB/s: 15.6 / 5.2 /
+// 31.2 / 15.6); single-CTA 128 x BN tiles, which pull 128 + BN rows for BN weight rows, took 29.1 / 12.0 / 42.3 / 24.7.
+// SwiGLU: N-block 0
+// holds gate rows, N-block 1 the up rows of the same features.  Of an N-block's accumulators every CTA holds its 64 rows:
+// tensor-memory lanes 0-63 the columns [0, BN/2), lanes 64-127 the columns [BN/2, BN), in BN/2 tensor-memory columns.
+// Warp roles, ring, hand-over and bounded waits are those of the pair kernel above.
 template <bool STATS>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_kernel_1cta(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
-                 const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, GemmArgs g)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
+gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
+                const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, GemmArgs g)
 {
     pdl_trigger();
-    if ((int)blockIdx.x >= ((g.M + BM - 1) / BM) * g.n_col_tiles * g.splits) return;     // beyond the tiles of even the largest row count
+    const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
+    if (pair >= ((g.M + 2 * FM - 1) / (2 * FM)) * g.n_col_tiles * g.splits) return;      // beyond the tiles of even the largest row count
 
-    const int BN = g.bn, STAGES = g.stages, HALF = BN >> 1;
-    const int STAGE_BYTES = A_BYTES + BN * BK * 2;
+    const int BN = g.bn, NB = g.nb, STAGES = g.stages, HALF = BN >> 1;
+    const int B_BYTES = HALF * BK * 2, STAGE_BYTES = FM * BK * 2 + NB * B_BYTES;
+    const uint32_t rank = tc::cluster_ctarank();
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
@@ -496,117 +517,133 @@ gemm_kernel_1cta(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     const uint32_t smem_base = tc::smem_u32(smem);
     const uint32_t bar_full = tc::smem_u32(bars), bar_empty = bar_full + 8 * kMaxStages;
     const uint32_t bar_acc_full = bar_full + 16 * kMaxStages, bar_acc_empty = bar_acc_full + 16;
+    const uint32_t lead_full = tc::mapa(bar_full, 0), lead_acc_empty = tc::mapa(bar_acc_empty, 0);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { tc::mbar_init(bar_full + 8 * s, 1); tc::mbar_init(bar_empty + 8 * s, 1); }
-        for (int b = 0; b < 2; ++b) { tc::mbar_init(bar_acc_full + 8 * b, 1); tc::mbar_init(bar_acc_empty + 8 * b, kEpiWarps); }
+        for (int b = 0; b < 2; ++b) { tc::mbar_init(bar_acc_full + 8 * b, 1); tc::mbar_init(bar_acc_empty + 8 * b, 2 * kEpiWarps); }
         s_abort = 0;
         tc::mbar_init_fence();
     }
     __syncwarp();
-    if (warp == 1) { tc::tmem_alloc(tc::smem_u32(tmem_slot), kTmemCols); tc::tmem_relinquish(); }
+    if (warp == 1) { tc::tmem_alloc_2cta(tc::smem_u32(tmem_slot), kTmemCols); tc::tmem_relinquish_2cta(); }
     tc::tc_fence_before();
-    __syncthreads();
+    tc::cluster_sync();
     tc::tc_fence_after();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
-    const uint32_t bn_pad = (uint32_t)((BN + 31) & ~31);
-    const uint32_t n_bufs = (uint32_t)g.acc_bufs, buf_stride = 256;
     const bool swiglu = (g.mode == GEMM_SWIGLU);
-    const int num_ctas = (int)gridDim.x;
 
     pdl_wait();                                             // the kernel before this one has completed: global memory from here on
     const bool live = !(g.d_active && *g.d_active == 0);    // nothing left to decode: the loops below find no tile
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
-    const int m_groups = (M + BM - 1) / BM;
+    const int m_groups = (M + 2 * FM - 1) / (2 * FM);
     const int num_tiles = live ? m_groups * g.n_col_tiles * g.splits : 0;
 
     if (warp == 0) {
-        // ---------------- TMA producer
+        // ---------------- TMA producer (both CTAs; completion bytes are counted on the leader's barrier)
         if (lane == 0) { tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB0); }
-        uint32_t it = 0;
+        uint32_t it = 0, s = 0, ph = 0;
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += num_ctas) {
+        for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
             const TileCoord t = tile_coord(g, tile, m_groups);
             const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
             const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
-            const int brow1 = swiglu ? t.n_local : t.n_local + HALF;
+            const int brow0 = t.n_local + (int)rank * HALF, brow1 = swiglu ? brow0 : brow0 + BN;
+            const int arow = t.m0 + (int)rank * FM;
             const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
                 if (!ready) ready = tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, &s_abort);
                 ok = __all_sync(0xffffffffu, ready);
                 if (!ok) break;
-                const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
+                const uint32_t ns = s + 1u == (uint32_t)STAGES ? 0u : s + 1u, nph = ns == 0u ? ph ^ 1u : ph;
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
-                tc::mbar_expect_tx_elect(bar_full + 8 * s, (uint32_t)STAGE_BYTES);
-                tc::tma_load_2d_elect(sa, &tmA, kb * BK, t.m0, bar_full + 8 * s);
-                tc::tma_load_2d_elect(sa + A_BYTES, m0, kb * BK, t.n_local, bar_full + 8 * s);
-                tc::tma_load_2d_elect(sa + A_BYTES + HALF * BK * 2, m1, kb * BK, brow1, bar_full + 8 * s);
+                if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
+                tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, kb * BK, brow0, lead_full + 8 * s);
+                if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, kb * BK, brow1, lead_full + 8 * s);
+                tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
+                s = ns; ph = nph;
             }
         }
-        if (s_abort && lane == 0) {
-            // give copies already in flight a bounded chance to land before the CTA retires
+        if (s_abort && rank == 0 && lane == 0) {
+            // give copies already in flight (both CTAs') a bounded chance to land before the pair retires
             const uint32_t first = it > (uint32_t)STAGES ? it - (uint32_t)STAGES : 0u;
             for (uint32_t j = first; j < it; ++j) {
-                const uint32_t bar = bar_full + 8 * (j % (uint32_t)STAGES), ph = (j / (uint32_t)STAGES) & 1u;
-                for (int i = 0; i < (1 << 16) && !tc::mbar_try(bar, ph); ++i) {}
+                const uint32_t bar = bar_full + 8 * (j % (uint32_t)STAGES), pj = (j / (uint32_t)STAGES) & 1u;
+                for (int i = 0; i < (1 << 16) && !tc::mbar_try(bar, pj); ++i) {}
             }
         }
     } else if (warp == 1) {
-        // ---------------- MMA issuer
-        const uint32_t idesc = tc::idesc_bf16_f32(BM, BN);
-        uint32_t it = 0, lt = 0;
-        bool ok = true;
-        bool ready = tc::mbar_test(bar_full, 0u);
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += num_ctas, ++lt) {
-            const uint32_t buf = lt % n_bufs, use = lt / n_bufs;
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(bar_acc_empty + 8 * buf, (use & 1u) ^ 1u, &s_abort));
-            if (!ok) break;
-            tc::tc_fence_after();
-            const uint32_t d_tmem = tmem_base + buf * buf_stride;
-            const int kb0 = tile_coord(g, tile, m_groups).split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
-            for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
-                if (!ready) ready = tc::mbar_wait(bar_full + 8 * s, ph, &s_abort);
-                ok = __all_sync(0xffffffffu, ready);
+        if (rank == 0) {
+            // ---------------- MMA issuer (leader CTA only)
+            const uint32_t idesc = tc::idesc_bf16_f32(2 * FM, BN);
+            uint32_t lt = 0, s = 0, ph = 0;
+            bool ok = true;
+            bool ready = tc::mbar_test(bar_full, 0u);
+            for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {
+                const uint32_t buf = lt & 1u, use = lt >> 1;
+                // both CTAs' epilogues have drained this accumulator buffer
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(bar_acc_empty + 8 * buf, (use & 1u) ^ 1u, &s_abort));
                 if (!ok) break;
                 tc::tc_fence_after();
-                const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
-                ready = tc::mbar_test(bar_full + 8 * ns, nph);
-                const uint32_t sa = smem_base + s * STAGE_BYTES;
-                const uint64_t da = tc::smem_desc_sw128(sa), db = tc::smem_desc_sw128(sa + A_BYTES);
-                tc::mma_bf16_elect(d_tmem, da, db, idesc, kb != kb0 ? 1u : 0u);
+                const uint32_t d_tmem = tmem_base + buf * 256u;
+                const int kb0 = tile_coord(g, tile, m_groups).split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
+                for (int kb = kb0; kb < kb1; ++kb) {
+                    if (!ready) ready = tc::mbar_wait(bar_full + 8 * s, ph, &s_abort);
+                    ok = __all_sync(0xffffffffu, ready);
+                    if (!ok) break;
+                    tc::tc_fence_after();
+                    const uint32_t ns = s + 1u == (uint32_t)STAGES ? 0u : s + 1u, nph = ns == 0u ? ph ^ 1u : ph;
+                    ready = tc::mbar_test(bar_full + 8 * ns, nph);
+                    const uint32_t sa = smem_base + s * STAGE_BYTES;
+                    const uint64_t da = tc::smem_desc_sw128(sa), db = tc::smem_desc_sw128(sa + FM * BK * 2);
+                    const uint32_t acc = kb != kb0 ? 1u : 0u;
+                    tc::mma_bf16_2cta_elect(d_tmem, da, db, idesc, acc);
 #pragma unroll
-                for (int kk = 1; kk < BK / 16; ++kk) tc::mma_bf16_elect(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, 1u);
-                tc::mma_commit_elect(bar_empty + 8 * s);          // frees the stage once these MMAs have read it
+                    for (int kk = 1; kk < BK / 16; ++kk) tc::mma_bf16_2cta_elect(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, 1u);
+                    if (NB == 2) {
+                        const uint64_t db1 = tc::smem_desc_sw128(sa + FM * BK * 2 + B_BYTES);
+                        tc::mma_bf16_2cta_elect(d_tmem + (uint32_t)HALF, da, db1, idesc, acc);
+#pragma unroll
+                        for (int kk = 1; kk < BK / 16; ++kk) tc::mma_bf16_2cta_elect(d_tmem + (uint32_t)HALF, da + (uint64_t)(kk * 2), db1 + (uint64_t)(kk * 2), idesc, 1u);
+                    }
+                    tc::mma_commit_2cta_elect(bar_empty + 8 * s);     // frees the stage in both CTAs once these MMAs have read it
+                    s = ns; ph = nph;
+                }
+                tc::mma_commit_2cta_elect(bar_acc_full + 8 * buf);    // accumulator complete (or abandoned), both CTAs
             }
-            tc::mma_commit_elect(bar_acc_full + 8 * buf);         // accumulator complete (or abandoned)
         }
     } else {
-        // ---------------- epilogue: 8 warps; warp w reads TMEM lanes 32*(w%4).., the column units of parity (w-2)/4
-        const int q = warp & 3, par = (warp - 2) >> 2;
+        // ---------------- epilogue: 8 warps; warp w reads TMEM lanes 32*(w%4).. (rows 32*(w%2).. of this CTA, column half (w%4)/2)
+        const int q = warp & 3, par = (warp - 2) >> 2, hq = q >> 1;
         const uint32_t stage = smem_base + STAGES * STAGE_BYTES + kBarBytes + (uint32_t)(warp - 2) * (32 * 128);
         uint32_t lt = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; tile < num_tiles && ok; tile += num_ctas, ++lt) {
+        for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {
             const TileCoord t = tile_coord(g, tile, m_groups);
-            const uint32_t buf = lt % n_bufs, use = lt / n_bufs;
+            const uint32_t buf = lt & 1u, use = lt >> 1;
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
-            epilogue_tile<STATS>(g, t, tmem_base + buf * buf_stride, bn_pad, stage, q, par, lane, 0, M);
+            EpiShare e;
+            e.tmem = tmem_base + buf * 256u + ((uint32_t)(q * 32) << 16); e.tmem_block = (uint32_t)HALF; e.up = (uint32_t)HALF;
+            e.row0 = t.m0 + (int)rank * FM + (q & 1) * 32; e.row_block = 0;
+            e.col0 = t.ncol0 + hq * HALF; e.col_block = BN; e.blocks = swiglu ? 1 : NB; e.seg = HALF;
+            e.col_end = min(t.ncol0 + t.ncols, g.N);
+            e.rec = 4 * NB * (t.ncol0 / (NB * BN)) + 2 * hq; e.rec_block = 4;
+            epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(bar_acc_empty + 8 * buf);
+            if (lane == 0) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
         }
     }
 
+    // ---------------- teardown: no CTA of the pair leaves while the other may still signal its barriers
     __syncwarp();
     tc::tc_fence_before();
-    __syncthreads();
-    if (warp == 1) { tc::tc_fence_after(); tc::tmem_dealloc(tmem_base, kTmemCols); }
+    tc::cluster_sync();
+    if (warp == 1) { tc::tc_fence_after(); tc::tmem_dealloc_2cta(tmem_base, kTmemCols); }
     if (threadIdx.x == 0 && s_abort && g.err) atomicExch(g.err, SFS_ERR_TIMEOUT);
 }
 
@@ -621,11 +658,11 @@ int num_sms()
     return n;
 }
 
-// column tiles of a problem at tile width bn
-int col_tiles(int mode, int n_maps, int n_per_map, int bn)
+// column tiles of a problem at `tile_cols` output columns per tile
+int col_tiles(int mode, int n_maps, int n_per_map, int tile_cols)
 {
-    if (mode == GEMM_SWIGLU) return (n_per_map + bn / 2 - 1) / (bn / 2);
-    return n_maps * ((n_per_map + bn - 1) / bn);
+    const int per_map = (n_per_map + tile_cols - 1) / tile_cols;
+    return mode == GEMM_SWIGLU ? per_map : n_maps * per_map;
 }
 
 int stages_for(int mb, int bn)
@@ -645,7 +682,7 @@ long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int pa
 {
     const long long num_kb = (K + BK - 1) / BK, kbps = (num_kb + splits - 1) / splits;
     const int m_groups = (M + mb * 2 * BM - 1) / (mb * 2 * BM);
-    const long long tiles = (long long)m_groups * col_tiles(mode, n_maps, n_per_map, bn) * ((num_kb + kbps - 1) / kbps);
+    const long long tiles = (long long)m_groups * col_tiles(mode, n_maps, n_per_map, mode == GEMM_SWIGLU ? bn / 2 : bn) * ((num_kb + kbps - 1) / kbps);
     const long long waves = (tiles + pairs - 1) / pairs;
     const long long mma = (long long)mb * bn * 2, load = (long long)(mb * BM + bn / 2) * 128 / 40;
     long long kb_clk = mma > load ? mma : load;
@@ -672,36 +709,41 @@ void pick_tile(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int
             }
 }
 
-// Few rows: tiles of 128 x bn on single CTAs.  Per k-block a CTA streams (128 + bn) rows x 128 B at the ~40 B/clk an SM gets
-// from L2 when all SMs stream, against 2 * bn clocks of tensor-core work; 600 clocks is where the k-block time stops shrinking.
-long long model_clocks_1cta(int M, int K, int mode, int n_maps, int n_per_map, int sms, int bn, int splits)
+// Few rows: 128 x (nb x bn) tiles of CTA pairs.  Measured: a k-block costs the issuing warp 255 + 165 nb clocks, an SM's L2
+// port ~40 B/clk for its 64 + nb * bn / 2 rows of 128 B, and HBM 3370 B/clk over all pairs; the largest sets the pace.  A slab
+// of a split K costs its reader ~600 clocks and 1.2e-3 per element.  At 128 rows, 8B widths this picks QKV 192 x 1 (24.8 us; the
+// next best 224: 25.4, nb = 2: 28.1), O 192 x 1 in 3 ranges of K (12.0; 2 ranges of 128: 13.0), gate / up 192 (40.2; 224: 40.8),
+// down 256 x 1 in 4 ranges (24.0; 192 in 3: 24.8).
+long long model_clocks_few(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int bn, int nb, int splits)
 {
     const long long num_kb = (K + BK - 1) / BK, kbps = (num_kb + splits - 1) / splits;
-    const long long tiles = (long long)col_tiles(mode, n_maps, n_per_map, bn) * ((num_kb + kbps - 1) / kbps);
-    const long long waves = (tiles + sms - 1) / sms;
-    const long long mma = 2LL * bn, load = (long long)(BM + bn) * 128 / 40;
-    long long kb_clk = mma > load ? mma : load;
-    if (kb_clk < 600) kb_clk = 600;
-    const long long epi = (long long)bn * 16 + 3000;
+    const int tile_cols = mode == GEMM_SWIGLU ? bn : nb * bn;
+    const long long tiles = (long long)col_tiles(mode, n_maps, n_per_map, tile_cols) * ((num_kb + kbps - 1) / kbps);
+    const long long waves = (tiles + pairs - 1) / pairs;
+    const long long issue = 255 + 165 * nb, port = (long long)(FM + nb * bn / 2) * 128 / 40;
+    const long long hbm = (tiles < pairs ? tiles : pairs) * (long long)nb * bn * 128 / 3370;
+    long long kb_clk = issue > port ? issue : port;
+    if (kb_clk < hbm) kb_clk = hbm;
+    const long long epi = (long long)nb * bn * 8 + 3000;
     const long long n_out = (mode == GEMM_SWIGLU) ? n_per_map : (long long)n_maps * n_per_map;
-    const long long slab = 1500 + (long long)((double)M * (double)n_out * 1.2e-3);
+    const long long slab = 600 + (long long)((double)M * (double)n_out * 1.2e-3);
     return waves * kbps * kb_clk + epi + (splits > 1 ? slab * splits : 0);
 }
 
-void pick_tile_1cta(int M, int K, int mode, int n_maps, int n_per_map, int sms, int max_splits, int *bn_out, int *splits_out)
+void pick_tile_few(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int max_splits, int *bn_out, int *nb_out, int *splits_out)
 {
-    const int step = (mode == GEMM_SWIGLU) ? 32 : 16;
     long long best_cost = -1;
-    for (int bn = 256; bn >= 32; bn -= step)
-        for (int sp = 1; sp <= max_splits; ++sp) {
-            const long long cost = model_clocks_1cta(M, K, mode, n_maps, n_per_map, sms, bn, sp);
-            if (best_cost < 0 || cost < best_cost) { best_cost = cost; *bn_out = bn; *splits_out = sp; }
-        }
+    for (int nb = (mode == GEMM_SWIGLU ? 2 : 1); nb <= 2; ++nb)
+        for (int bn = 256; bn >= 32; bn -= 32)
+            for (int sp = 1; sp <= max_splits; ++sp) {
+                const long long cost = model_clocks_few(M, K, mode, n_maps, n_per_map, pairs, bn, nb, sp);
+                if (best_cost < 0 || cost < best_cost) { best_cost = cost; *bn_out = bn; *nb_out = nb; *splits_out = sp; }
+            }
 }
 
-int stages_for_1cta(int bn)
+int stages_for_few(int bn, int nb)
 {
-    const int stage_bytes = A_BYTES + bn * BK * 2;
+    const int stage_bytes = FM * BK * 2 + nb * (bn / 2) * BK * 2;
     const int s = (kSmemBudget - 1024 - kBarBytes - kEpiStageBytes) / stage_bytes;
     return s > kMaxStages ? kMaxStages : s;
 }
@@ -719,18 +761,20 @@ int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int
     memset(p, 0, sizeof(*p));
     const int N = (mode == GEMM_SWIGLU) ? n_per_map : n_per_map * n_maps;
     SFS_REQUIRE(aligned_to(C, 16) && (ldc % 8) == 0, SFS_ERR_INVALID_ARG, "gemm: C must be 16-byte aligned, ldc a multiple of 8");
-    int mb = 1, bn = 256;
+    int mb = 1, bn = 256, nb = 1;
     int sp_unused = 1;
-    // at most 128 rows: single-CTA tiles (a pair's 256-row MMA would be half padding); tune->mb = 1 or 2 forces the pair kernel
-    const bool one_cta = (M <= BM) && !(tune && (tune->mb == 1 || tune->mb == 2));
-    if (one_cta) pick_tile_1cta(M, K, mode, n_maps, n_per_map, num_sms(), 1, &bn, &sp_unused);
+    // at most 128 rows: few-row tiles (a pair's 256-row MMA would be half padding); tune->mb = 1 or 2 forces the pair kernel
+    const bool few = (M <= 2 * FM) && !(tune && (tune->mb == 1 || tune->mb == 2));
+    const int step = few ? 32 : ((mode == GEMM_SWIGLU) ? 32 : 16);
+    if (few) pick_tile_few(M, K, mode, n_maps, n_per_map, num_sms() / 2, 1, &bn, &nb, &sp_unused);
     else pick_tile(M, K, mode, n_maps, n_per_map, num_sms() / 2, 1, &mb, &bn, &sp_unused);
     if (tune) {                                              // measurement overrides; invalid values are ignored
         if (tune->mb == 1 || tune->mb == 2) mb = tune->mb;
-        if (tune->bn >= 32 && tune->bn <= 256 && (tune->bn % ((mode == GEMM_SWIGLU) ? 32 : 16)) == 0) bn = tune->bn;
+        if (tune->bn >= 32 && tune->bn <= 256 && (tune->bn % step) == 0) bn = tune->bn;
+        if (few && (tune->nb == 1 || tune->nb == 2) && mode != GEMM_SWIGLU) nb = tune->nb;
     }
     p->bn = bn; p->n_maps = n_maps; p->n_per_map = n_per_map;
-    int32_t rc = make_tmap_bf16(&p->tmA, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, BM);
+    int32_t rc = make_tmap_bf16(&p->tmA, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, few ? FM : BM);
     if (rc != SFS_OK) return rc;
     for (int i = 0; i < 3; ++i) {
         const void *b = Bs[i < n_maps ? i : 0];
@@ -740,13 +784,16 @@ int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int
     GemmArgs &g = p->args;
     g.M = M; g.N = N; g.K = K; g.mode = mode; g.out_f32 = out_f32; g.scale = scale;
     g.C = C; g.ldc = ldc; g.vt = vt; g.ldvt = ldvt; g.vt_col0 = vt_col0;
-    g.bn = bn; g.mb = one_cta ? 1 : mb; g.n_per_map = n_per_map;
-    g.one_cta = one_cta ? 1 : 0; g.tile_rows = one_cta ? BM : mb * 2 * BM;
-    g.tiles_per_map = (mode == GEMM_SWIGLU) ? 0x3FFFFFFF : (n_per_map + bn - 1) / bn;
-    g.n_col_tiles = col_tiles(mode, n_maps, n_per_map, bn);
-    g.stages = one_cta ? stages_for_1cta(bn) : stages_for(mb, bn);
+    g.bn = bn; g.mb = few ? 1 : mb; g.nb = few ? nb : 1; g.n_per_map = n_per_map;
+    g.few = few ? 1 : 0; g.tile_rows = few ? 2 * FM : mb * 2 * BM;
+    g.tile_cols = (mode == GEMM_SWIGLU) ? (few ? bn : bn / 2) : (few ? nb * bn : bn);
+    g.tiles_per_map = (mode == GEMM_SWIGLU) ? 0x3FFFFFFF : (n_per_map + g.tile_cols - 1) / g.tile_cols;
+    g.n_col_tiles = col_tiles(mode, n_maps, n_per_map, g.tile_cols);
+    g.stages = few ? stages_for_few(bn, nb) : stages_for(mb, bn);
     if (tune && tune->stages >= 1 && tune->stages <= g.stages) g.stages = tune->stages;
-    g.acc_bufs = (g.mb * ((bn + 31) & ~31) <= 256) ? 2 : 1;
+    g.acc_bufs = few || (g.mb * ((bn + 31) & ~31) <= 256) ? 2 : 1;
+    // records of the fused row statistics per row; both epilogue-warp parities must own columns of every block
+    g.stats_parts = few ? (bn / 2 > 64 ? 4 * nb * g.n_col_tiles : 0) : (bn > 64 ? 2 * g.n_col_tiles : 0);
     g.splits = 1; g.kb_per_split = (K + BK - 1) / BK; g.split_stride = 0;
     p->A = A; p->lda = lda; p->ldb = ldb;
     for (int i = 0; i < 3; ++i) p->Bs[i] = Bs[i < n_maps ? i : 0];
@@ -758,19 +805,20 @@ int32_t gemm_plan_enable_split(GemmPlan *p, float *ws, int32_t max_splits, const
     GemmArgs &g = p->args;
     const bool f32_out = g.mode == GEMM_RESIDUAL_F32 || (g.mode == GEMM_STORE && g.out_f32 && g.vt == nullptr);
     if (!f32_out || ws == nullptr || max_splits < 2) return SFS_OK;
-    int mb = g.mb, bn = g.bn, sp = 1;
-    const bool one_cta = g.one_cta != 0;
-    if (one_cta) pick_tile_1cta(g.M, g.K, g.mode, p->n_maps, p->n_per_map, num_sms(), max_splits, &bn, &sp);
+    int mb = g.mb, bn = g.bn, nb = g.nb, sp = 1;
+    const bool few = g.few != 0;
+    if (few) pick_tile_few(g.M, g.K, g.mode, p->n_maps, p->n_per_map, num_sms() / 2, max_splits, &bn, &nb, &sp);
     else pick_tile(g.M, g.K, g.mode, p->n_maps, p->n_per_map, num_sms() / 2, max_splits, &mb, &bn, &sp);
     if (tune) {
         if (tune->mb == 1 || tune->mb == 2) mb = tune->mb;
         if (tune->bn >= 32 && tune->bn <= 256 && (tune->bn % 16) == 0) bn = tune->bn;
+        if (tune->nb == 1 || tune->nb == 2) nb = tune->nb;
         if (tune->splits >= 1 && tune->splits <= max_splits) sp = tune->splits;
     }
     if (sp <= 1 && !tune) return SFS_OK;
     // rebuild the plan at the new tile shape, then cut K
     GemmPlan q;
-    GemmTune t2 = {one_cta ? 0 : mb, bn, tune ? tune->stages : 0, 0};
+    GemmTune t2 = {few ? 0 : mb, bn, tune ? tune->stages : 0, 0, nb};
     int32_t rc = gemm_plan_create(&q, p->A, p->lda, g.M, g.K, p->Bs, p->n_maps, p->n_per_map, p->ldb, g.mode, g.C, g.ldc, g.out_f32,
                                   g.scale, g.vt, g.ldvt, g.vt_col0, &t2);
     if (rc != SFS_OK) return rc;
@@ -800,21 +848,21 @@ int32_t gemm_launch(const GemmPlan &p, const int32_t *d_m, const int32_t *d_acti
     }
     GemmArgs g = p.args;
     g.d_m = d_m; g.err = err; g.d_active = d_active;
-    if (g.one_cta) {
+    if (g.few) {
         static bool configured1[kMaxDevices] = {};
         bool &done1 = configured1[current_device_slot()];
         if (!done1) {
-            SFS_CUDA(cudaFuncSetAttribute(gemm_kernel_1cta<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-            SFS_CUDA(cudaFuncSetAttribute(gemm_kernel_1cta<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+            SFS_CUDA(cudaFuncSetAttribute(gemm_few_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+            SFS_CUDA(cudaFuncSetAttribute(gemm_few_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
             done1 = true;
         }
-        size_t smem1 = (size_t)g.stages * (A_BYTES + g.bn * BK * 2) + kBarBytes + kEpiStageBytes + 1024;
+        size_t smem1 = (size_t)g.stages * (FM * BK * 2 + g.nb * (g.bn / 2) * BK * 2) + kBarBytes + kEpiStageBytes + 1024;
         if (smem1 < 120 * 1024) smem1 = 120 * 1024;            // one CTA per SM: all 512 tensor-memory columns are its own
-        const long long tiles1 = (long long)((g.M + BM - 1) / BM) * g.n_col_tiles * g.splits;
-        const int sms = num_sms();
-        const unsigned grid1 = (unsigned)(tiles1 < sms ? tiles1 : sms);
-        if (g.stats) SFS_CUDA(launch_pdl(gemm_kernel_1cta<true>, dim3(grid1), dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
-        else SFS_CUDA(launch_pdl(gemm_kernel_1cta<false>, dim3(grid1), dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
+        const long long tiles1 = (long long)((g.M + 2 * FM - 1) / (2 * FM)) * g.n_col_tiles * g.splits;
+        const int pairs1 = num_sms() / 2;
+        const dim3 grid1((unsigned)(2 * (tiles1 < pairs1 ? tiles1 : pairs1)));
+        if (g.stats) SFS_CUDA(launch_pdl(gemm_few_kernel<true>, grid1, dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
+        else SFS_CUDA(launch_pdl(gemm_few_kernel<false>, grid1, dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
         return SFS_OK;
     }
     size_t smem = (size_t)g.stages * (g.mb * A_BYTES + (g.bn / 2) * BK * 2) + kBarBytes + kEpiStageBytes + 1024;

@@ -1,0 +1,65 @@
+"""Projections of at most 128 rows (CTA pairs, tensor-memory tiles of 64 rows per CTA): edges of the row, column and K tiles, and the
+row statistics the LM head leaves when a generation has that few response rows."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import rowstats as RS
+from oracle.scheduler import SlowFastState, rows_needed, slowfast_step
+from paper_2506_10848_b200 import binding as sfs
+from paper_2506_10848_b200 import workloads as W
+
+from helpers import params_pair
+from test_gpu_linear import run
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+# rows on both sides of a CTA's 64; one tile, a ragged last tile and one that ends inside an N-block; K of one k-block, a tail of 8
+@pytest.mark.parametrize("M", [1, 63, 64, 65, 127, 128])
+@pytest.mark.parametrize("N,K", [(8, 64), (3000, 136), (9480, 520), (40008, 72)])
+def test_linear_edges(M, N, K):
+    for out_dtype in (0, 1):
+        got, ref = run(M, N, K, out_dtype, seed=M + N)
+        err = np.abs(got - ref)
+        # fp32 sums of K exact products (at most K roundings of 2^-24 of the running sum, |terms| < 4); bf16 output: half an ulp more
+        assert np.all(err <= 4.0 * K * K * 2.0 ** -24 + (2.0 ** -8 * np.abs(ref) if out_dtype == 0 else 0.0)), float(err.max())
+
+
+@pytest.mark.parametrize("B,L,vocab", [(1, 24, 70008), (2, 61, 65536), (1, 128, 99992)])
+def test_generation_with_few_long_rows_is_reproduced_by_the_oracle(B, L, vocab):
+    """Long vocabulary rows, at most 128 of them (ragged last column tile): the decisions come from the LM head's own records."""
+    P = 8 - L % 8
+    S = P + L
+    shape = W.Shape(n_layers=1, d_model=256, n_heads=2, head_dim=128, d_ff=512, vocab=vocab, mask_id=vocab - 1, rms_eps=1e-5,
+                    rope_theta=10000.0, logit_scale=60.0)
+    w = W.model_weights(shape, seed=9, device=DEV)
+    model = sfs.Model(shape, w)
+    session = sfs.sfs_session_create(model, B, S)
+    po, pg = params_pair()
+    try:
+        trace = torch.zeros((L, B, sfs.TRACE_INTS), dtype=torch.int32, device=DEV)
+        dump = torch.zeros((B * L, vocab), dtype=torch.bfloat16, device=DEV)
+        rows_d = torch.zeros(B * L, dtype=torch.int32, device=DEV)
+        n_d = torch.zeros(1, dtype=torch.int32, device=DEV)
+        sfs.sfs_generate_begin(session, W.prompt_ids(B, P, vocab - 2, seed=1).to(DEV), B, P, L, pg)
+        ost = [SlowFastState.fresh(L, po) for _ in range(B)]
+        for step in range(6):
+            if all(s.done for s in ost):
+                break
+            sfs.sfs_generate_steps(session, 1, trace, L, dump, rows_d, n_d)
+            torch.cuda.synchronize()
+            need = [(b, i) for b in range(B) for i in rows_needed(ost[b])]
+            assert rows_d[:int(n_d.item())].tolist() == [b * S + P + i for (b, i) in need]
+            st = RS.row_stats(W.bf16_bits(dump[:len(need)].cpu()))
+            for b in range(B):
+                if ost[b].done:
+                    continue
+                idx = {i: j for j, (bb, i) in enumerate(need) if bb == b}
+                rec = slowfast_step(ost[b], {i: int(st["argmax"][j]) for i, j in idx.items()}, {i: int(st["sq"][j]) for i, j in idx.items()}, po)
+                assert trace[step, b].tolist()[:6] == [rec.phase, rec.s, rec.hi, rec.e_cand, rec.stable, len(rec.positions)], (step, b)
+        sfs.sfs_check_device_status()
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
