@@ -1,15 +1,13 @@
 // Row statistics of the sampling epilogue (paper Section 3.1): per logits row the greedy token
 // r_hat = argmax_v x_v and the canonical fixed-point softmax denominator S_q (c = 2^28 / S_q).
 //
-// Fast paths (bf16 logits): a thread-block cluster owns one row and HBM is read exactly once.  Pass 1 finds the exact row
-// maximum, the CTAs push their slice maxima to each other through distributed shared memory (one cluster barrier), pass 2
-// evaluates the fixed-point exponentials with packed f32x2 arithmetic and sums them as integers; sums and first-maximum
-// candidates reach rank 0 by remote shared-memory atomics.  Integer sums make the result independent of how the row is
-// split over threads, warps and CTAs.  Rows of 128 KB and more are staged: each of 8 CTAs brings its contiguous slice into
-// shared memory with one bulk asynchronous copy (no registers tied up in flight, seven CTAs per SM); shorter rows stay in
-// registers (every thread keeps its 16-byte chunks between the passes).
-//
-// Generic path (bf16 or fp32, any vocabulary size or stride): one CTA per row, two sweeps over global memory.
+// A thread-block cluster owns one row and HBM is read once.  Pass 1 finds the exact row maximum, the CTAs push their slice
+// maxima to each other through distributed shared memory (one cluster barrier), pass 2 evaluates the fixed-point
+// exponentials with packed f32x2 arithmetic and sums them as integers; sums and first-maximum candidates reach rank 0 by
+// remote shared-memory atomics.  Integer sums make the result independent of how the row is split over threads, warps and
+// CTAs.  Rows stay in registers between the passes (any element type, length and alignment); many long aligned bf16 rows are
+// staged: each of 8 CTAs brings its contiguous slice into shared memory with one bulk asynchronous copy (no registers tied up
+// in flight, seven CTAs per SM).
 #include "sfs_common.cuh"
 
 #include <cooperative_groups.h>
@@ -34,19 +32,6 @@ __device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t s) {
     return r;
 }
 
-// one term e_v = trunc(2^28 * exp(x - m)), scalar form (generic kernel)
-__device__ __forceinline__ uint32_t canon_term(float x, float m) {
-    const float d = __fsub_rn(x, m);
-    const float r = __fmaf_rn(d, kLog2e, kMagic);
-    const float n = __fsub_rn(r, kMagic);
-    const float f = __fmaf_rn(n, -kLn2, d);
-    float q = __fmaf_rn(f, kC4, kC3);
-    q = __fmaf_rn(f, q, kC2);
-    q = __fmaf_rn(f, q, kC1);
-    const float P = __fmaf_rn(f, q, 3.0f);
-    return shr_clamp(__float_as_uint(P) << 9, kShiftBase - __float_as_uint(r));
-}
-
 // ---- packed f32x2 arithmetic (two lanes per instruction) ----------------------------------------------
 typedef unsigned long long f32x2;
 __device__ __forceinline__ f32x2 pack2(float lo, float hi) {
@@ -64,9 +49,8 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
 
 struct Consts2 { f32x2 negm, l2e, magic, negmagic, negln2, c1, c2, c3, c4, three; };
 
-// two terms from one 32-bit word holding two bf16 logits; returns e_lo + e_hi (each < 1.42 * 2^28)
-__device__ __forceinline__ uint32_t canon_pair(uint32_t w, const Consts2 &k) {
-    const f32x2 x = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u));
+// the terms of two packed logits; returns e_lo + e_hi (each < 1.42 * 2^28)
+__device__ __forceinline__ uint32_t canon2(f32x2 x, const Consts2 &k) {
     const f32x2 d = add2(x, k.negm);
     const f32x2 r = fma2(d, k.l2e, k.magic);
     const f32x2 n = add2(r, k.negmagic);
@@ -79,6 +63,21 @@ __device__ __forceinline__ uint32_t canon_pair(uint32_t w, const Consts2 &k) {
     unpack2(r, r0, r1);
     unpack2(P, p0, p1);
     return shr_clamp(p0 << 9, kShiftBase - r0) + shr_clamp(p1 << 9, kShiftBase - r1);
+}
+
+// the same from one 32-bit word holding two bf16 logits
+__device__ __forceinline__ uint32_t canon_pair(uint32_t w, const Consts2 &k) {
+    return canon2(pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)), k);
+}
+
+__device__ __forceinline__ Consts2 canon_consts(float m) {
+    Consts2 k;
+    k.negm = pack2(-m, -m);           k.l2e = pack2(kLog2e, kLog2e);
+    k.magic = pack2(kMagic, kMagic);  k.negmagic = pack2(-kMagic, -kMagic);
+    k.negln2 = pack2(-kLn2, -kLn2);
+    k.c1 = pack2(kC1, kC1); k.c2 = pack2(kC2, kC2); k.c3 = pack2(kC3, kC3); k.c4 = pack2(kC4, kC4);
+    k.three = pack2(3.0f, 3.0f);
+    return k;
 }
 
 // orders this thread's shared-memory traffic inside the cluster (cheaper than a device-wide fence)
@@ -122,16 +121,91 @@ __device__ __forceinline__ void write_row(const RowOut &o, int row, int arg, uns
 constexpr int kThreads = 256;
 constexpr uint32_t kNegInf2 = 0xFF80FF80u;
 
-// One cluster (1, 2, 4 or 8 CTAs) per logits row; NV 16-byte chunks per thread.
-template <int NV>
-__global__ void __launch_bounds__(kThreads, 4)
-rowstats_cluster_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nchunks, int vocab,
-                      const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
+// ---- a logits row as 16-byte chunks -----------------------------------------------------------------------------
+// A row may start anywhere (its stride need not be a multiple of 16 bytes): chunk c holds the elements c * PER - off ..
+// c * PER - off + PER - 1 of the row, off = elements between the 16-byte boundary at or before the row's start and the start.
+// Chunks that lie inside the row are one vector load; the first and last one are put together from the row's own elements,
+// with -inf in the places outside it (adds nothing, never is the maximum's first position).
+template <typename T> struct RowChunks {
+    static constexpr int PER = 16 / (int)sizeof(T);
+    const T *row;
+    const uint4 *base;
+    int off, vocab, n, in0, in1;                            // n chunks; [in0, in1) lie inside the row
+    __device__ __forceinline__ RowChunks(const T *logits, long long ld, int r, int V) {
+        row = logits + (long long)r * ld;
+        const unsigned long long a = (unsigned long long)row;
+        off = (int)(a & 15u) / (int)sizeof(T);
+        base = reinterpret_cast<const uint4 *>(a & ~15ull);
+        vocab = V;
+        n = (off + V + PER - 1) / PER; in0 = off ? 1 : 0; in1 = (off + V) / PER;
+    }
+    static __device__ __forceinline__ uint4 nothing();      // PER times -inf
+    __device__ __forceinline__ uint4 load(int c) const {
+        if (c >= in0 && c < in1) return ld_stream(base + c);
+        return c < n ? edge(c) : nothing();
+    }
+    __device__ __noinline__ uint4 edge(int c) const;
+    __device__ __forceinline__ int index(int c, int e) const { return c * PER + e - off; }
+};
+template <> __device__ __forceinline__ uint4 RowChunks<__nv_bfloat16>::nothing() { return make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2); }
+template <> __device__ __forceinline__ uint4 RowChunks<float>::nothing() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
+template <> __device__ __noinline__ uint4 RowChunks<__nv_bfloat16>::edge(int c) const {
+    uint32_t w[4];
+    for (int k = 0; k < 4; ++k) {
+        uint32_t h[2];
+        for (int e = 0; e < 2; ++e) {
+            const int i = index(c, 2 * k + e);
+            h[e] = (i >= 0 && i < vocab) ? reinterpret_cast<const unsigned short *>(row)[i] : 0xFF80u;
+        }
+        w[k] = h[0] | (h[1] << 16);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+template <> __device__ __noinline__ uint4 RowChunks<float>::edge(int c) const {
+    uint32_t w[4];
+    for (int e = 0; e < 4; ++e) {
+        const int i = index(c, e);
+        w[e] = (i >= 0 && i < vocab) ? __float_as_uint(row[i]) : 0xFF800000u;
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+// element e of a chunk, its maximum, and the sum of its terms (8 terms < 8 * 1.42 * 2^28 < 2^32)
+template <typename T> __device__ __forceinline__ float chunk_elem(const uint4 &v, int e);
+template <> __device__ __forceinline__ float chunk_elem<__nv_bfloat16>(const uint4 &v, int e) {
+    const uint32_t w = (e >> 1) == 0 ? v.x : ((e >> 1) == 1 ? v.y : ((e >> 1) == 2 ? v.z : v.w));
+    return (e & 1) ? __uint_as_float(w & 0xFFFF0000u) : __uint_as_float(w << 16);
+}
+template <> __device__ __forceinline__ float chunk_elem<float>(const uint4 &v, int e) {
+    return __uint_as_float(e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)));
+}
+template <typename T> __device__ __forceinline__ float chunk_max(const uint4 &v);
+template <> __device__ __forceinline__ float chunk_max<__nv_bfloat16>(const uint4 &v) {
+    __nv_bfloat162 m = __hmax2(__hmax2(as_bf162(v.x), as_bf162(v.y)), __hmax2(as_bf162(v.z), as_bf162(v.w)));
+    return bf162_max(*reinterpret_cast<uint32_t *>(&m));
+}
+template <> __device__ __forceinline__ float chunk_max<float>(const uint4 &v) {
+    return fmaxf(fmaxf(__uint_as_float(v.x), __uint_as_float(v.y)), fmaxf(__uint_as_float(v.z), __uint_as_float(v.w)));
+}
+template <typename T> __device__ __forceinline__ uint32_t chunk_terms(const uint4 &v, const Consts2 &k);
+template <> __device__ __forceinline__ uint32_t chunk_terms<__nv_bfloat16>(const uint4 &v, const Consts2 &k) {
+    return canon_pair(v.x, k) + canon_pair(v.y, k) + canon_pair(v.z, k) + canon_pair(v.w, k);
+}
+template <> __device__ __forceinline__ uint32_t chunk_terms<float>(const uint4 &v, const Consts2 &k) {
+    return canon2(pack2(__uint_as_float(v.x), __uint_as_float(v.y)), k) + canon2(pack2(__uint_as_float(v.z), __uint_as_float(v.w)), k);
+}
+
+// One cluster (1, 2, 4 or 8 CTAs) per logits row, any element type, length and alignment; a thread keeps NV 16-byte chunks of
+// the row in registers between the two passes (rows of more than C * 256 * NV chunks read the rest a second time, from L2).
+template <typename T, int NV>
+__global__ void __launch_bounds__(kThreads, NV > 8 ? 2 : 4)
+rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
 {
     cg::cluster_group cluster = cg::this_cluster();
     const int C    = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int row  = blockIdx.x / C;
+    pdl_wait();
+    pdl_trigger();
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
     if (row >= n_rows) return;                              // uniform over the cluster
 
@@ -143,26 +217,22 @@ rowstats_cluster_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int
     __shared__ int s_cta_arg;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint4 *rp = logits + (long long)row * ld_chunks;
+    const RowChunks<T> rc(logits, ld, row, vocab);
+    const int stride = C * kThreads, c0 = rank * kThreads + tid;
 
     // ---- the only pass over HBM: this thread's chunks of the row, kept in registers
     uint4 v[NV];
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const int chunk = (j * C + rank) * kThreads + tid;
-        v[j] = (chunk < nchunks) ? ld_stream(rp + chunk) : make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2);
-    }
+    for (int j = 0; j < NV; ++j) v[j] = rc.load(c0 + j * stride);
     if (tid == 0) { s_cta_arg = 0x7FFFFFFF; s_row_sum = 0; s_row_arg = 0x7FFFFFFF; s_arrived = 0; }
     // every CTA of the cluster announces that it runs (its shared memory exists) before anybody writes into a peer
     if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 
     // ---- pass 1: exact maximum
-    __nv_bfloat162 mx = as_bf162(kNegInf2);
+    float lmax = -INFINITY;
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        mx = __hmax2(mx, __hmax2(__hmax2(as_bf162(v[j].x), as_bf162(v[j].y)), __hmax2(as_bf162(v[j].z), as_bf162(v[j].w))));
-    }
-    const float lmax = bf162_max(*reinterpret_cast<uint32_t *>(&mx));
+    for (int j = 0; j < NV; ++j) lmax = fmaxf(lmax, chunk_max<T>(v[j]));
+    for (int c = c0 + NV * stride; c < rc.n; c += stride) lmax = fmaxf(lmax, chunk_max<T>(rc.load(c)));
     float m = warp_max(lmax);
     if (lane == 0) s_wmax[warp] = m;
     __syncthreads();
@@ -190,31 +260,28 @@ rowstats_cluster_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int
         int best = 0x7FFFFFFF;
 #pragma unroll
         for (int j = NV - 1; j >= 0; --j) {
-            const int chunk = (j * C + rank) * kThreads + tid;
-            const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
 #pragma unroll
-            for (int e = 7; e >= 0; --e) {
-                const float x = (e & 1) ? __uint_as_float(w[e >> 1] & 0xFFFF0000u) : __uint_as_float(w[e >> 1] << 16);
-                const int idx = chunk * 8 + e;
-                if (x == m && idx < vocab) best = idx;
+            for (int e = RowChunks<T>::PER - 1; e >= 0; --e) {
+                const int idx = rc.index(c0 + j * stride, e);
+                if (chunk_elem<T>(v[j], e) == m && idx >= 0 && idx < vocab) best = idx;
+            }
+        }
+        for (int c = c0 + NV * stride; c < rc.n && best == 0x7FFFFFFF; c += stride) {
+            const uint4 q = rc.load(c);
+            for (int e = RowChunks<T>::PER - 1; e >= 0; --e) {
+                const int idx = rc.index(c, e);
+                if (chunk_elem<T>(q, e) == m && idx >= 0 && idx < vocab) best = idx;
             }
         }
         if (best != 0x7FFFFFFF) atomicMin(&s_cta_arg, best);
     }
 
     // ---- pass 2: fixed-point exponentials, integer sum
-    Consts2 k;
-    k.negm = pack2(-m, -m);           k.l2e = pack2(kLog2e, kLog2e);
-    k.magic = pack2(kMagic, kMagic);  k.negmagic = pack2(-kMagic, -kMagic);
-    k.negln2 = pack2(-kLn2, -kLn2);
-    k.c1 = pack2(kC1, kC1); k.c2 = pack2(kC2, kC2); k.c3 = pack2(kC3, kC3); k.c4 = pack2(kC4, kC4);
-    k.three = pack2(3.0f, 3.0f);
+    const Consts2 k = canon_consts(m);
     unsigned long long acc = 0;
 #pragma unroll
-    for (int j = 0; j < NV; ++j) {
-        const uint32_t a = canon_pair(v[j].x, k) + canon_pair(v[j].y, k) + canon_pair(v[j].z, k) + canon_pair(v[j].w, k);
-        acc += a;                                           // 8 terms < 8 * 1.42 * 2^28 < 2^32
-    }
+    for (int j = 0; j < NV; ++j) acc += chunk_terms<T>(v[j], k);
+    for (int c = c0 + NV * stride; c < rc.n; c += stride) acc += chunk_terms<T>(rc.load(c), k);
     acc = warp_sum_u64(acc);
     if (lane == 0) s_wsum[warp] = acc;
     __syncthreads();
@@ -323,6 +390,8 @@ rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
     const int C    = (int)cluster.num_blocks();
     const int rank = (int)cluster.block_rank();
     const int row  = blockIdx.x / C;
+    pdl_wait();
+    pdl_trigger();
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
     if (row >= n_rows) return;                              // uniform over the cluster
 
@@ -398,12 +467,7 @@ rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
         }
         if (best != 0x7FFFFFFF) atomicMin(&s_cta_arg, best);
     }
-    Consts2 k;
-    k.negm = pack2(-m, -m);           k.l2e = pack2(kLog2e, kLog2e);
-    k.magic = pack2(kMagic, kMagic);  k.negmagic = pack2(-kMagic, -kMagic);
-    k.negln2 = pack2(-kLn2, -kLn2);
-    k.c1 = pack2(kC1, kC1); k.c2 = pack2(kC2, kC2); k.c3 = pack2(kC3, kC3); k.c4 = pack2(kC4, kC4);
-    k.three = pack2(3.0f, 3.0f);
+    const Consts2 k = canon_consts(m);
     unsigned long long acc = 0;
 #pragma unroll 4
     for (int c = tid; c < n; c += kStagedThreads) {
@@ -707,12 +771,7 @@ rowstats_list_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nc
         const int p = rows[row];
         if ((unsigned)p >= (unsigned)n_positions) continue;           // uniform over the CTA
         const float m = pos_max[p];
-        Consts2 k;
-        k.negm = pack2(-m, -m);           k.l2e = pack2(kLog2e, kLog2e);
-        k.magic = pack2(kMagic, kMagic);  k.negmagic = pack2(-kMagic, -kMagic);
-        k.negln2 = pack2(-kLn2, -kLn2);
-        k.c1 = pack2(kC1, kC1); k.c2 = pack2(kC2, kC2); k.c3 = pack2(kC3, kC3); k.c4 = pack2(kC4, kC4);
-        k.three = pack2(3.0f, 3.0f);
+        const Consts2 k = canon_consts(m);
         const uint4 *rp = logits + (long long)row * ld_chunks;
         const int c0 = part * per, c1 = min(nchunks, c0 + per);
         unsigned long long acc = 0;
@@ -742,24 +801,26 @@ rowstats_list_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nc
     }
 }
 
+int num_sms_rowstats()
+{
+    static int n[kMaxDevices] = {};
+    int &v = n[current_device_slot()];
+    if (v == 0) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 148;
+    }
+    return v;
+}
+
 int32_t launch_staged(const uint4 *logits, long long ld_chunks, int nchunks, int vocab, const int32_t *d_n_rows,
                       int max_rows, const RowOut &out, cudaStream_t stream)
 {
     const int per_cta = (nchunks + kStagedCluster - 1) / kStagedCluster;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(max_rows * kStagedCluster), 1, 1);
-    cfg.blockDim = dim3(kStagedThreads, 1, 1);
-    cfg.dynamicSmemBytes = (size_t)per_cta * 16;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)kStagedCluster; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    SFS_CUDA(cudaLaunchKernelEx(&cfg, rowstats_staged_bf16, logits, ld_chunks, nchunks, per_cta, vocab, d_n_rows, max_rows, out, out.err));
+    SFS_CUDA(launch_pdl_cluster(rowstats_staged_bf16, kStagedCluster, dim3((unsigned)(max_rows * kStagedCluster)), dim3(kStagedThreads),
+                                (size_t)per_cta * 16, stream, logits, ld_chunks, nchunks, per_cta, vocab, d_n_rows, max_rows, out, out.err));
     return SFS_OK;
 }
 
-int num_sms_rowstats();
 int32_t launch_bounds(const uint4 *logits, long long ld_chunks, int nchunks, int vocab, const int32_t *d_n_rows, int max_rows,
                       const BoundsOut &out, cudaStream_t stream)
 {
@@ -779,74 +840,34 @@ int32_t launch_bounds(const uint4 *logits, long long ld_chunks, int nchunks, int
     return SFS_OK;
 }
 
-// ---- generic path ------------------------------------------------------------------------------------
-template <typename T> __device__ __forceinline__ float load_as_f32(const T *p, long long i);
-template <> __device__ __forceinline__ float load_as_f32<float>(const float *p, long long i) { return p[i]; }
-template <> __device__ __forceinline__ float load_as_f32<__nv_bfloat16>(const __nv_bfloat16 *p, long long i) {
-    return bf16_bits_to_f32(reinterpret_cast<const unsigned short *>(p)[i]);
+template <typename T, int NV>
+int32_t launch_cluster(const void *logits, long long ld, int vocab, const int32_t *d_n_rows, int max_rows, int C, const RowOut &out, cudaStream_t stream)
+{
+    SFS_CUDA(launch_pdl_cluster(rowstats_cluster<T, NV>, C, dim3((unsigned)(max_rows * C)), dim3(kThreads), 0, stream,
+                                reinterpret_cast<const T *>(logits), ld, vocab, d_n_rows, max_rows, out, out.err));
+    return SFS_OK;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads)
-rowstats_generic(const T *__restrict__ logits, long long ld, int vocab,
-                 const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out)
+int32_t launch_rows(const void *logits, long long ld, int vocab, const int32_t *d_n_rows, int max_rows, const RowOut &out, cudaStream_t stream)
 {
-    const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
-    __shared__ float s_wmax[kThreads / 32];
-    __shared__ unsigned long long s_wsum[kThreads / 32];
-    __shared__ float s_max;
-    __shared__ int s_arg;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int row = blockIdx.x; row < n_rows; row += gridDim.x) {
-        const T *rp = logits + (long long)row * ld;
-        float lm = -INFINITY;
-        for (int v = tid; v < vocab; v += kThreads) lm = fmaxf(lm, load_as_f32(rp, v));
-        lm = warp_max(lm);
-        if (lane == 0) s_wmax[warp] = lm;
-        if (tid == 0) s_arg = 0x7FFFFFFF;
-        __syncthreads();
-        if (tid == 0) {
-            float t = s_wmax[0];
-            for (int w = 1; w < kThreads / 32; ++w) t = fmaxf(t, s_wmax[w]);
-            s_max = t;
-        }
-        __syncthreads();
-        const float m = s_max;
-        unsigned long long acc = 0;
-        int best = 0x7FFFFFFF;
-        for (int v = tid; v < vocab; v += kThreads) {
-            const float x = load_as_f32(rp, v);
-            acc += canon_term(x, m);
-            if (x == m && v < best) best = v;
-        }
-        if (best != 0x7FFFFFFF) atomicMin(&s_arg, best);
-        acc = warp_sum_u64(acc);
-        if (lane == 0) s_wsum[warp] = acc;
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long S = 0;
-            for (int w = 0; w < kThreads / 32; ++w) S += s_wsum[w];
-            write_row(out, row, s_arg == 0x7FFFFFFF ? 0 : s_arg, S);
-        }
-        __syncthreads();
-    }
-}
-
-template <int NV>
-int32_t launch_cluster(const uint4 *logits, long long ld_chunks, int nchunks, int vocab, const int32_t *d_n_rows,
-                       int max_rows, int C, const RowOut &out, cudaStream_t stream)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(max_rows * C), 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    SFS_CUDA(cudaLaunchKernelEx(&cfg, rowstats_cluster_bf16<NV>, logits, ld_chunks, nchunks, vocab, d_n_rows, max_rows, out, out.err));
-    return SFS_OK;
+    // Cluster size and chunks kept per thread.  A CTA costs ~2 us besides its chunks, so the fewest CTAs that keep at least 65 %
+    // of the row in registers (8 chunks a thread; 16 for rows beyond 256 KB) are best while they fill the machine, and
+    // more of them, down to 4 chunks a thread, when the rows are few.  Measured, us at 4 / 64 / 512 rows, three buffers in turn:
+    // bf16 50257: C = 2 8.6 / 9.4 / 28.3, C = 4 5.6 / 7.2 / 30.9, C = 8 4.9 / 7.5 / 45.1; fp32 50257: C = 4 7.3 / 9.5 / 41.2,
+    // C = 8 4.5 / 7.5 / 43.5; bf16 32000: C = 2 4.6 / 4.8 / 16.0, C = 4 4.0 / 5.1 / 20.8; bf16 8000: C = 1 2.6 / 2.9 / 5.2,
+    // C = 2 3.7 / 4.0 / 10.8 (the one-CTA-per-row two-sweep kernel before: bf16 50257 14.4 / 14.4 / 41.0, fp32 12.3 / 14.4 / 55.2).
+    const bool aligned = (reinterpret_cast<uintptr_t>(logits) % 16) == 0 && (ld * (long long)sizeof(T)) % 16 == 0;
+    const int nchunks = (int)((vocab * (long long)sizeof(T) + 15) / 16) + (aligned ? 0 : 1);      // an unaligned row touches one more
+    int C = 1;
+    while (C < 8 && (long long)C * 8 * kThreads * 20 < 13LL * nchunks) C *= 2;
+    while (C < 8 && (long long)max_rows * C < 2 * num_sms_rowstats() && nchunks > C * 4 * kThreads) C *= 2;
+    const int per_thread = (nchunks + C * kThreads - 1) / (C * kThreads);
+    if (per_thread <= 1) return launch_cluster<T, 1>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
+    if (per_thread <= 2) return launch_cluster<T, 2>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
+    if (per_thread <= 4) return launch_cluster<T, 4>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
+    if (C < 8 || per_thread <= 8) return launch_cluster<T, 8>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
+    return launch_cluster<T, 16>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
 }
 
 }  // namespace
@@ -862,53 +883,15 @@ int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t voc
     const bool fast = logits_dtype == SFS_LOGITS_BF16 && (vocab % 8) == 0 && (ld % 8) == 0 && aligned_to(d_logits, 16);
     if (fast) {
         const int nchunks = vocab / 8;
-        // long rows (128 KB and more, slices of at most 40 KB): staged through shared memory
-        if (nchunks >= 8192 && (nchunks + kStagedCluster - 1) / kStagedCluster <= 2560)
+        // Long rows (128 KB and more, slices of at most 40 KB): staged through shared memory, seven CTAs to an SM, unless the rows
+        // are so few that the register form's four to an SM are resident at once: 126464 bf16 logits, 64 rows 10.1 us against
+        // 12.3, 122 rows 16.3 against 15.7, 512 rows 51.8 against 46.1.
+        if (nchunks >= 8192 && (nchunks + kStagedCluster - 1) / kStagedCluster <= 2560 && max_rows * kStagedCluster > 4 * num_sms_rowstats())
             return launch_staged(reinterpret_cast<const uint4 *>(d_logits), ld / 8, nchunks, vocab, d_n_rows, max_rows, out, stream);
-        // smallest (cluster size, chunks per thread) that covers the row; at most 8 CTAs x 256 threads x 8 chunks
-        const int per_cta1 = kThreads;                      // chunks covered by one CTA with NV = 1
-        int C = 1, NV = 1;
-        auto covers = [&](int c, int nv) { return (long long)c * nv * per_cta1 >= nchunks; };
-        if (covers(1, 1)) { C = 1; NV = 1; }
-        else if (covers(1, 2)) { C = 1; NV = 2; }
-        else if (covers(1, 4)) { C = 1; NV = 4; }
-        else if (covers(2, 4)) { C = 2; NV = 4; }
-        else if (covers(4, 4)) { C = 4; NV = 4; }
-        else if (covers(8, 4)) { C = 8; NV = 4; }
-        else if (covers(8, 8)) { C = 8; NV = 8; }
-        else C = 0;
-        if (C) {
-            const uint4 *lp = reinterpret_cast<const uint4 *>(d_logits);
-            switch (NV) {
-                case 1: return launch_cluster<1>(lp, ld / 8, nchunks, vocab, d_n_rows, max_rows, C, out, stream);
-                case 2: return launch_cluster<2>(lp, ld / 8, nchunks, vocab, d_n_rows, max_rows, C, out, stream);
-                case 4: return launch_cluster<4>(lp, ld / 8, nchunks, vocab, d_n_rows, max_rows, C, out, stream);
-                default: return launch_cluster<8>(lp, ld / 8, nchunks, vocab, d_n_rows, max_rows, C, out, stream);
-            }
-        }
     }
-    const int grid = max_rows < 4096 ? max_rows : 4096;
-    if (logits_dtype == SFS_LOGITS_BF16) {
-        rowstats_generic<__nv_bfloat16><<<grid, kThreads, 0, stream>>>(
-            reinterpret_cast<const __nv_bfloat16 *>(d_logits), ld, vocab, d_n_rows, max_rows, out);
-    } else {
-        rowstats_generic<float><<<grid, kThreads, 0, stream>>>(
-            reinterpret_cast<const float *>(d_logits), ld, vocab, d_n_rows, max_rows, out);
-    }
-    SFS_LAUNCH_CHECK();
-    return SFS_OK;
+    return logits_dtype == SFS_LOGITS_BF16 ? launch_rows<__nv_bfloat16>(d_logits, ld, vocab, d_n_rows, max_rows, out, stream)
+                                           : launch_rows<float>(d_logits, ld, vocab, d_n_rows, max_rows, out, stream);
 }
-
-namespace { int num_sms_rowstats()
-{
-    static int n[kMaxDevices] = {};
-    int &v = n[current_device_slot()];
-    if (v == 0) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) v = 148;
-    }
-    return v;
-} }
 
 static bool staged_shape(int32_t logits_dtype, int32_t vocab, int64_t ld, const void *d_logits)
 {

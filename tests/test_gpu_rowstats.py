@@ -154,3 +154,26 @@ def test_enclosures_of_the_cheap_pass_contain_the_canonical_denominator(V, ld):
     mid = (lo.astype(np.float64) + hi.astype(np.float64)) / 2
     rows = [r for r in range(R) if r not in open_rows]
     assert np.max(np.abs(mid[rows] - sq[rows].astype(np.float64)) / sq[rows].astype(np.float64)) <= 2e-5 + V / float(1 << 28)
+
+
+@pytest.mark.parametrize("dtype", [sfs.LOGITS_BF16, sfs.LOGITS_F32])
+@pytest.mark.parametrize("R,V,ld", [(9, 2049, 2051), (9, 8197, 8199), (300, 8197, 8197), (9, 16391, 16391), (300, 33001, 33003), (9, 50257, 50257),
+                                    (80, 50257, 50258), (3, 66003, 66005), (5, 140001, 140003), (300, 4099, 4100)])
+def test_rows_at_every_alignment(R, V, ld, dtype):
+    """Odd lengths and strides: every row starts at another offset inside a 16-byte chunk; the cases cover one to eight CTAs per
+    row, a few to sixteen chunks per thread and rows longer than the registers hold.  The maximum sits in the first column, in
+    the last, twice, and inside; the padding between rows is larger than any logit."""
+    g = torch.Generator().manual_seed(V + R)
+    x = torch.randn((R, ld), generator=g) * 4
+    x[:, V:] = 1e30
+    x[0, 0] = 40.0
+    x[1, V - 1] = 40.0
+    x[2, V // 3] = 30.0; x[2, V - 2] = 30.0
+    if dtype == sfs.LOGITS_BF16:
+        x = x.to(torch.bfloat16)
+        ref = RS.row_stats(np.ascontiguousarray(W.bf16_bits(x)[:, :V]))
+    else:
+        ref = RS.row_stats(np.ascontiguousarray(x[:, :V].numpy()))
+    arg, sq, _ = gpu_stats(x.to(DEV), V, ld, dtype)
+    assert np.array_equal(arg, ref["argmax"]) and np.array_equal(sq, ref["sq"])
+    sfs.sfs_check_device_status()
