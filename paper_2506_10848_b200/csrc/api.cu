@@ -70,27 +70,22 @@ static int32_t dev_alloc(sfs_session *s, T **out, size_t count, bool zero)
     return SFS_OK;
 }
 
-// Row statistics of one selection step into the session's scratch: the two-pass (filter + exact) form for long bf16 rows,
-// the all-canonical kernels otherwise.  Either way the selection kernel finds, for every supplied row the rule reads, a
-// value in pos_sq that gives the decisions of the canonical S_q.
+// Row statistics of one selection step into the session's scratch: the first of two passes (filter + exact) for long bf16 rows,
+// whose second pass the selection kernel takes; the all-canonical kernels otherwise.  `a` learns which.
 static int32_t step_row_stats(sfs_session *s, const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
-                              const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const uint8_t *d_mask,
-                              int32_t B, int32_t S, int32_t P, const sfs_state *d_state, const sfs_params &params, bool *two_pass,
+                              const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, int32_t B, int32_t S, SelectArgs *a,
                               cudaStream_t st, const float4 *lm_stats = nullptr, int32_t lm_stats_ld = 0)
 {
     int32_t *err = device_status_word();
-    *two_pass = row_stats_two_pass_applies(d_logits, logits_dtype, vocab, ld);
-    if (!*two_pass)
+    if (max_rows <= 0 || !row_stats_two_pass_applies(d_logits, logits_dtype, vocab, ld))
         return launch_row_stats(d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, nullptr, nullptr, nullptr,
                                 s->pos_sq, s->pos_arg, B * S, err, st);
-    RefineArgs rf{};
-    rf.mask = d_mask; rf.B = B; rf.S = S; rf.P = P; rf.L = S - P; rf.state = d_state; rf.params = params;
-    rf.pos_lo = s->pos_lo; rf.pos_hi = s->pos_hi; rf.pos_sq = s->pos_sq; rf.pos_arg = s->pos_arg;
-    rf.slice_partials = s->slice_partials; rf.row_tickets = s->row_tickets;
-    rf.pos_row = s->pos_row; rf.pos_max = s->pos_max; rf.refine_list = s->refine_list; rf.refine_count = s->refine_count;
-    if (lm_stats != nullptr)       // the LM head's epilogue has taken the first pass: the logits are read only for the listed rows
-        return launch_row_stats_from_partials(lm_stats, lm_stats_ld, lm_stats_ld, d_logits, vocab, ld, d_n_rows, max_rows, d_rows, rf, err, st);
-    return launch_row_stats_two_pass(d_logits, vocab, ld, d_n_rows, max_rows, d_rows, rf, err, st);
+    a->pos_lo = s->pos_lo; a->pos_hi = s->pos_hi; a->pos_row = s->pos_row; a->pos_max = s->pos_max; a->seq_ticket = s->seq_ticket;
+    a->lrows = {reinterpret_cast<const uint4 *>(d_logits), (long long)(ld / 8), vocab / 8};
+    const BoundsScratch bs = {s->pos_lo, s->pos_hi, s->pos_arg, s->slice_partials, s->row_tickets, s->pos_row, s->pos_max, B * S};
+    if (lm_stats != nullptr)       // the LM head's epilogue has taken the first pass: the logits are read only for the open rows
+        return launch_row_stats_from_partials(lm_stats, lm_stats_ld, lm_stats_ld, vocab, d_n_rows, max_rows, d_rows, bs, err, st);
+    return launch_row_stats_two_pass(d_logits, vocab, ld, d_n_rows, max_rows, d_rows, bs, err, st);
 }
 
 static int32_t session_alloc_select(sfs_session *s)
@@ -105,8 +100,7 @@ static int32_t session_alloc_select(sfs_session *s)
     if ((rc = dev_alloc(s, &s->row_tickets, n, true)) != SFS_OK) return rc;
     if ((rc = dev_alloc(s, &s->pos_row, n, true)) != SFS_OK) return rc;
     if ((rc = dev_alloc(s, &s->pos_max, n, true)) != SFS_OK) return rc;
-    if ((rc = dev_alloc(s, &s->refine_list, n, true)) != SFS_OK) return rc;
-    if ((rc = dev_alloc(s, &s->refine_count, 4, true)) != SFS_OK) return rc;
+    if ((rc = dev_alloc(s, &s->seq_ticket, (size_t)s->max_batch, true)) != SFS_OK) return rc;
     if ((rc = dev_alloc(s, &s->seq_rows, n, true)) != SFS_OK) return rc;
     if ((rc = dev_alloc(s, &s->seq_row_count, (size_t)s->max_batch, true)) != SFS_OK) return rc;
     if ((rc = dev_alloc(s, &s->ticket, 4, true)) != SFS_OK) return rc;
@@ -393,16 +387,6 @@ __global__ void generate_init_kernel(const int32_t *prompt, int32_t *tokens, uin
     }
 }
 
-// host_active[0]: sequences still decoding; host_active[1]: denoising steps the device has finished in this generation
-__global__ void mirror_active_kernel(const int32_t *ctrl_active, int32_t *host_active, int32_t steps_done)
-{
-    pdl_wait();
-    pdl_trigger();
-    host_active[1] = steps_done;
-    __threadfence_system();
-    host_active[0] = *ctrl_active;
-}
-
 }  // namespace sfs
 
 using namespace sfs;
@@ -628,11 +612,9 @@ int32_t sfs_select(sfs_session *s, const void *d_logits, int32_t logits_dtype, i
     int32_t rc = check_params(params, S - P);
     if (rc != SFS_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    bool two_pass = false;
-    rc = step_row_stats(s, d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, d_mask, B, S, P, d_state, *params, &two_pass, st);
-    if (rc != SFS_OK) return rc;
     SelectArgs a{};
-    a.pos_lo = two_pass ? s->pos_lo : nullptr;
+    rc = step_row_stats(s, d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, B, S, &a, st);
+    if (rc != SFS_OK) return rc;
     a.tokens = d_tokens; a.mask = d_mask; a.B = B; a.S = S; a.P = P; a.L = S - P;
     a.state = d_state; a.params = *params;
     a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;
@@ -788,12 +770,10 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
             if (d_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_rows_dump, rows, (size_t)B * L * 4, cudaMemcpyDeviceToDevice, st));
             if (d_n_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_n_rows_dump, n_rows, 4, cudaMemcpyDeviceToDevice, st));
         }
-        bool two_pass = false;
-        if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
-                 return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, s->mask, B, S, P, s->state,
-                                       s->gen_params, &two_pass, st, s->lm_plan.args.stats, s->lm_plan.args.stats_ld); })) != SFS_OK) return rc;
         SelectArgs a{};
-        a.pos_lo = two_pass ? s->pos_lo : nullptr;
+        if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
+                 return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, s->lm_plan.args.stats,
+                                       s->lm_plan.args.stats_ld); })) != SFS_OK) return rc;
         a.tokens = s->tokens; a.mask = s->mask; a.B = B; a.S = S; a.P = P; a.L = L;
         a.state = s->state; a.params = s->gen_params;
         a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;
@@ -801,9 +781,8 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
         a.next_rows = s->rows[nxt]; a.next_n_rows = s->ctrl + nxt; a.n_active = s->ctrl + 2;
         a.ticket = s->ticket;
         a.trace = (d_trace && s->gen_steps < max_trace_steps) ? d_trace + (size_t)s->gen_steps * B * SFS_TRACE_INTS : nullptr;
+        a.host_active = s->host_active_dev; a.host_step = s->gen_steps + 1;
         if ((rc = timed_launch(s, SFS_K_SELECT, st, [&] { return launch_select(a, st); })) != SFS_OK) return rc;
-        SFS_CUDA(launch_pdl(mirror_active_kernel, dim3((unsigned)(1)), dim3((unsigned)(1)), (size_t)(0), st, s->ctrl + 2, s->host_active_dev, s->gen_steps + 1));
-        s->launches++;
         s->gen_cur = nxt;
         s->gen_steps++;
     }

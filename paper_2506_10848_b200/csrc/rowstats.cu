@@ -9,6 +9,7 @@
 // staged: each of 8 CTAs brings its contiguous slice into shared memory with one bulk asynchronous copy (no registers tied up
 // in flight, seven CTAs per SM).
 #include "sfs_common.cuh"
+#include "canonical.cuh"
 
 #include <cooperative_groups.h>
 #include <math_constants.h>
@@ -16,69 +17,6 @@ namespace cg = cooperative_groups;
 
 namespace sfs {
 namespace {
-
-constexpr float kLog2e = 0x1.715476p+0f;
-constexpr float kLn2   = 0x1.62e430p-1f;
-constexpr float kMagic = 12582912.0f;           // 1.5 * 2^23
-constexpr float kC1 = 0x1.fffa48p-1f;
-constexpr float kC2 = 0x1.fff8fcp-2f;
-constexpr float kC3 = 0x1.57f67cp-3f;
-constexpr float kC4 = 0x1.57de66p-5f;
-constexpr uint32_t kShiftBase = 0x4B400003u;    // bits(kMagic) + 3
-
-__device__ __forceinline__ uint32_t shr_clamp(uint32_t x, uint32_t s) {
-    uint32_t r;
-    asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));   // PTX semantics: shift >= 32 gives 0
-    return r;
-}
-
-// ---- packed f32x2 arithmetic (two lanes per instruction) ----------------------------------------------
-typedef unsigned long long f32x2;
-__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
-    f32x2 r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r;
-}
-__device__ __forceinline__ void unpack2(f32x2 v, uint32_t &lo, uint32_t &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v));
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-    f32x2 r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r;
-}
-
-struct Consts2 { f32x2 negm, l2e, magic, negmagic, negln2, c1, c2, c3, c4, three; };
-
-// the terms of two packed logits; returns e_lo + e_hi (each < 1.42 * 2^28)
-__device__ __forceinline__ uint32_t canon2(f32x2 x, const Consts2 &k) {
-    const f32x2 d = add2(x, k.negm);
-    const f32x2 r = fma2(d, k.l2e, k.magic);
-    const f32x2 n = add2(r, k.negmagic);
-    const f32x2 f = fma2(n, k.negln2, d);
-    f32x2 q = fma2(f, k.c4, k.c3);
-    q = fma2(f, q, k.c2);
-    q = fma2(f, q, k.c1);
-    const f32x2 P = fma2(f, q, k.three);
-    uint32_t r0, r1, p0, p1;
-    unpack2(r, r0, r1);
-    unpack2(P, p0, p1);
-    return shr_clamp(p0 << 9, kShiftBase - r0) + shr_clamp(p1 << 9, kShiftBase - r1);
-}
-
-// the same from one 32-bit word holding two bf16 logits
-__device__ __forceinline__ uint32_t canon_pair(uint32_t w, const Consts2 &k) {
-    return canon2(pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)), k);
-}
-
-__device__ __forceinline__ Consts2 canon_consts(float m) {
-    Consts2 k;
-    k.negm = pack2(-m, -m);           k.l2e = pack2(kLog2e, kLog2e);
-    k.magic = pack2(kMagic, kMagic);  k.negmagic = pack2(-kMagic, -kMagic);
-    k.negln2 = pack2(-kLn2, -kLn2);
-    k.c1 = pack2(kC1, kC1); k.c2 = pack2(kC2, kC2); k.c3 = pack2(kC3, kC3); k.c4 = pack2(kC4, kC4);
-    k.three = pack2(3.0f, 3.0f);
-    return k;
-}
 
 // orders this thread's shared-memory traffic inside the cluster (cheaper than a device-wide fence)
 __device__ __forceinline__ void cluster_fence() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
@@ -321,67 +259,6 @@ constexpr int kStagedCluster = 8;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Pass 2 of the two-pass form, first half: one CTA per sequence looks at what the step's rule will ask of its candidate rows
-// and sorts them into "the enclosure [lo, hi] of pass 1 answers it" (the lower bound is handed to the selection kernel) and
-// "must be recomputed canonically" (the logits row goes on a list that the staged kernel then works through).
-//   * a threshold is open when lo and hi fall on different sides of it;
-//   * the ranking (k most confident candidates, smallest S_q first) is open for every candidate whose lo does not exceed
-//     U = the k-th smallest hi among the candidates: the k rows with the smallest hi all have S_q <= U, so a row with
-//     lo > U is not among the k most confident, and its lower bound (still > U) orders it behind them.  Only k = 1 is
-//     evaluated this way (U = the smallest hi); for k > 1 every candidate is recomputed.
-constexpr int kDecideThreads = 256;
-__global__ void __launch_bounds__(kDecideThreads) refine_decide_kernel(RefineArgs rf)
-{
-    pdl_wait();
-    pdl_trigger();
-    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = rf.L;
-    const sfs_state &st = rf.state[b];
-    if (st.done || st.status != SFS_OK) return;
-    const StepAsk ask = step_ask(rf.params, st, L);
-    const long long base = (long long)b * rf.S + rf.P;
-    const uint8_t *msk = rf.mask + base;
-    const unsigned long long *plo = rf.pos_lo + base, *phi = rf.pos_hi + base;
-    __shared__ int s_cnt[kDecideThreads / 32];
-    __shared__ unsigned long long s_min[kDecideThreads / 32];
-    int cnt = 0;
-    unsigned long long umin = ~0ull;
-    for (int j = ask.lo + tid; j < ask.hi; j += kDecideThreads) {
-        if (!msk[j]) continue;
-        cnt++;
-        if (plo[j] != 0) umin = min(umin, phi[j]);
-    }
-    cnt = warp_sum_i32(cnt);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) umin = min(umin, __shfl_xor_sync(0xffffffffu, umin, o));
-    if (lane == 0) { s_cnt[warp] = cnt; s_min[warp] = umin; }
-    __syncthreads();
-    int n_cand = 0;
-    unsigned long long U = ~0ull;
-    for (int w = 0; w < kDecideThreads / 32; ++w) { n_cand += s_cnt[w]; U = min(U, s_min[w]); }
-    int k_top = 0;
-    if (ask.rank_needed) {
-        if (rf.params.sampler == SFS_SAMPLER_LOW_CONFIDENCE) {
-            const BlockStep blk = block_step(rf.params, L, st.steps_done);
-            const long long Lb = ask.hi - ask.lo, Nb = blk.steps_per_block;
-            k_top = (int)max(0ll, (Lb * (Nb - blk.k_b + 1)) / Nb - (Lb - n_cand));
-        } else {
-            k_top = (st.phase == SFS_PHASE_SLOW) ? rf.params.k_slow : rf.params.k_fast;
-        }
-        if (k_top >= n_cand) k_top = 0;                     // everything is chosen: no ranking
-    }
-    for (int j = ask.lo + tid; j < ask.hi; j += kDecideThreads) {
-        if (!msk[j]) continue;
-        const unsigned long long lo = plo[j], hi = phi[j];
-        if (lo == 0) continue;                              // no row supplied for this candidate
-        bool need = false;
-        if (ask.tau > 0.f) need = conf_exceeds(lo, ask.tau) && !conf_exceeds(hi, ask.tau);
-        if (k_top > 1) need = true;
-        else if (k_top == 1) need = need || lo <= U;
-        if (need) rf.refine_list[atomicAdd(rf.refine_count, 1)] = rf.pos_row[base + j];
-        else rf.pos_sq[base + j] = lo;
-    }
-}
-
 __global__ void __launch_bounds__(kStagedThreads)
 rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nchunks, int per_cta, int vocab,
                      const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
@@ -532,7 +409,6 @@ struct BoundsOut {
     unsigned long long *pos_lo, *pos_hi; int32_t *pos_arg;  // scattered by flat token index (optional)
     int32_t *pos_row;                                       // with them: the logits row a position's statistics came from
     float *pos_max;                                         //            and the exact row maximum
-    int32_t *list_count;                                    // optional: counter of the recompute list, cleared by this launch
     int32_t n_positions; int32_t *err;
     float4 *partial;                                        // scratch [max_rows * kSlices]: (slice max, reference, sum, argmax bits)
     int32_t *tickets;                                       // scratch [max_rows], zero between launches
@@ -573,7 +449,6 @@ combine_partials_kernel(const float4 *__restrict__ stats, int stats_ld, int n_pa
     pdl_trigger();
     const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && out.list_count) *out.list_count = 0;
     if (row >= n_rows) return;
     const float4 *ps = stats + (long long)row * stats_ld;
     float m = -INFINITY;
@@ -609,8 +484,9 @@ rowstats_bounds_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
                      const int32_t *__restrict__ n_rows_ptr, int max_rows, int slices, BoundsOut out)
 {
     const int row = blockIdx.x / slices, sl = blockIdx.x - row * slices;
+    pdl_wait();
+    pdl_trigger();
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && out.list_count) *out.list_count = 0;
     if (row >= n_rows) return;
     const int per = (nchunks + slices - 1) / slices;
     const int c0 = sl * per, c1 = min(nchunks, c0 + per);
@@ -748,59 +624,6 @@ rowstats_bounds_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
     write_enclosure(out, row, tot, arg, m, open, vocab);
 }
 
-// Pass 2 of the two-pass form, second half: the canonical S_q of the listed rows.  Pass 1 has left the exact row maximum, so one
-// sweep is enough; a listed row is cut into kListParts parts, a CTA takes (row, part) items in turn, reads its part (from L2:
-// pass 1 has just streamed the logits) and adds its integer partial sum to pos_sq with one atomic — integer addition commutes, so
-// the result does not depend on the order of arrival.  pos_sq of a listed row is zero on entry (the selection kernel clears what
-// it has consumed, and the deciding kernel writes only the rows it does not list).
-constexpr int kListParts = 8;
-constexpr int kListThreads = 256;
-__global__ void __launch_bounds__(kListThreads)
-rowstats_list_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nchunks, const int32_t *__restrict__ rows,
-                   const int32_t *__restrict__ list, const int32_t *__restrict__ list_count, const float *__restrict__ pos_max,
-                   unsigned long long *__restrict__ pos_sq, int n_positions)
-{
-    pdl_wait();
-    pdl_trigger();
-    const int n_items = *list_count * kListParts;
-    const int per = (nchunks + kListParts - 1) / kListParts;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    __shared__ unsigned long long s_w[kListThreads / 32];
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const int row = list[item / kListParts], part = item % kListParts;
-        const int p = rows[row];
-        if ((unsigned)p >= (unsigned)n_positions) continue;           // uniform over the CTA
-        const float m = pos_max[p];
-        const Consts2 k = canon_consts(m);
-        const uint4 *rp = logits + (long long)row * ld_chunks;
-        const int c0 = part * per, c1 = min(nchunks, c0 + per);
-        unsigned long long acc = 0;
-        int c = c0 + tid;
-        for (; c + 3 * kListThreads < c1; c += 4 * kListThreads) {    // four loads in flight
-            uint4 v[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) v[u] = rp[c + u * kListThreads];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                acc += (unsigned long long)(canon_pair(v[u].x, k) + canon_pair(v[u].y, k)) + (unsigned long long)(canon_pair(v[u].z, k) + canon_pair(v[u].w, k));
-        }
-        for (; c < c1; c += kListThreads) {
-            const uint4 v = rp[c];
-            acc += (unsigned long long)(canon_pair(v.x, k) + canon_pair(v.y, k)) + (unsigned long long)(canon_pair(v.z, k) + canon_pair(v.w, k));
-        }
-        acc = warp_sum_u64(acc);
-        if (lane == 0) s_w[warp] = acc;
-        __syncthreads();
-        if (tid == 0) {
-            unsigned long long t = 0;
-#pragma unroll
-            for (int w = 0; w < kListThreads / 32; ++w) t += s_w[w];
-            atomicAdd(&pos_sq[p], t);
-        }
-        __syncthreads();
-    }
-}
-
 int num_sms_rowstats()
 {
     static int n[kMaxDevices] = {};
@@ -834,9 +657,8 @@ int32_t launch_bounds(const uint4 *logits, long long ld_chunks, int nchunks, int
         const double fill = (double)ctas / (double)(waves * per_wave);
         if (fill > best + 0.02) { best = fill; slices = sl; }
     }
-    rowstats_bounds_bf16<4, false, false><<<(unsigned)(max_rows * slices), kBoundsThreads, 0, stream>>>(logits, ld_chunks, nchunks, vocab, d_n_rows,
-                                                                                                          max_rows, slices, out);
-    SFS_LAUNCH_CHECK();
+    SFS_CUDA(launch_pdl(rowstats_bounds_bf16<4, false, false>, dim3((unsigned)(max_rows * slices)), dim3(kBoundsThreads), 0, stream, logits, ld_chunks,
+                        nchunks, vocab, d_n_rows, max_rows, slices, out));
     return SFS_OK;
 }
 
@@ -924,39 +746,29 @@ int32_t launch_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld,
         SFS_CUDA(cudaMemset(s_tickets[dev], 0, (size_t)max_rows * sizeof(int32_t)));
         s_rows[dev] = max_rows;
     }
-    BoundsOut out{nullptr, d_lo, d_hi, d_argmax, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, d_err, s_partial[dev], s_tickets[dev]};
+    BoundsOut out{nullptr, d_lo, d_hi, d_argmax, nullptr, nullptr, nullptr, nullptr, nullptr, 0, d_err, s_partial[dev], s_tickets[dev]};
     return launch_bounds(reinterpret_cast<const uint4 *>(d_logits), ld / 8, vocab / 8, vocab, d_n_rows, max_rows, out, stream);
 }
 
 int32_t launch_row_stats_two_pass(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,
-                                  const int32_t *d_rows, const RefineArgs &rf, int32_t *d_err, cudaStream_t stream)
+                                  const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err, cudaStream_t stream)
 {
     if (max_rows <= 0) return SFS_OK;
     const uint4 *lp = reinterpret_cast<const uint4 *>(d_logits);
-    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.refine_count, rf.B * rf.S, d_err,
+    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.n_positions, d_err,
                  reinterpret_cast<float4 *>(rf.slice_partials), rf.row_tickets};
     int32_t rc = launch_bounds(lp, ld / 8, vocab / 8, vocab, d_n_rows, max_rows, bo, stream);
     if (rc != SFS_OK) return rc;
-    SFS_CUDA(launch_pdl(refine_decide_kernel, dim3((unsigned)(rf.B)), dim3((unsigned)(kDecideThreads)), (size_t)(0), stream, rf));
-    const int items = max_rows * kListParts, cap = 2 * num_sms_rowstats();
-    SFS_CUDA(launch_pdl(rowstats_list_bf16, dim3((unsigned)(items < cap ? items : cap)), dim3((unsigned)(kListThreads)), (size_t)(0), stream, lp, ld / 8, vocab / 8, d_rows, rf.refine_list, rf.refine_count,
-                                                                              rf.pos_max, rf.pos_sq, rf.B * rf.S));
     return SFS_OK;
 }
 
-int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, const void *d_logits, int32_t vocab, int64_t ld,
-                                       const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const RefineArgs &rf, int32_t *d_err,
+int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err,
                                        cudaStream_t stream)
 {
     if (max_rows <= 0) return SFS_OK;
-    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.refine_count, rf.B * rf.S, d_err,
+    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.n_positions, d_err,
                  nullptr, nullptr};
     SFS_CUDA(launch_pdl(combine_partials_kernel, dim3((unsigned)((max_rows + 3) / 4)), dim3((unsigned)(128)), (size_t)(0), stream, reinterpret_cast<const float4 *>(stats), stats_ld, n_parts, d_n_rows, max_rows, vocab, bo));
-    SFS_CUDA(launch_pdl(refine_decide_kernel, dim3((unsigned)(rf.B)), dim3((unsigned)(kDecideThreads)), (size_t)(0), stream, rf));
-    const uint4 *lp = reinterpret_cast<const uint4 *>(d_logits);
-    const int items = max_rows * kListParts, cap = 2 * num_sms_rowstats();
-    SFS_CUDA(launch_pdl(rowstats_list_bf16, dim3((unsigned)(items < cap ? items : cap)), dim3((unsigned)(kListThreads)), (size_t)(0), stream, lp, ld / 8, vocab / 8, d_rows, rf.refine_list, rf.refine_count,
-                                                                              rf.pos_max, rf.pos_sq, rf.B * rf.S));
     return SFS_OK;
 }
 

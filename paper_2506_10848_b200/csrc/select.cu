@@ -6,6 +6,7 @@
 // to finish concatenates the per-sequence row lists (sequence-major, positions ascending) so that the
 // next forward pass gets one deterministic row list without a host round trip.
 #include "sfs_common.cuh"
+#include "canonical.cuh"
 
 namespace sfs {
 namespace {
@@ -13,11 +14,6 @@ namespace {
 constexpr int kSelThreads = 256;
 constexpr unsigned long long kNoKey = ~0ull;
 constexpr int kPosBits = 17;                 // key = S_q << 17 | position  (S_q < 2^47, position < 2^17)
-
-__device__ __forceinline__ bool exceeds(unsigned long long sq, float tau) {
-    // c > tau  <=>  S_q * tau < 2^28, one IEEE double multiply
-    return __dmul_rn((double)sq, (double)tau) < (double)(1u << SFS_CONF_QBITS);
-}
 
 struct BlockRed {
     int n_cand, n_high, max_above, min_cand, n_masked, missing;
@@ -72,30 +68,149 @@ __device__ __forceinline__ uint32_t philox_first_word(uint32_t c0, uint32_t c1, 
     return c0;
 }
 
-// dynamic shared memory: keys u64[L] | flags u8[L] (selected) | flags u8[L] (above tau_high)
+// what the whole step leaves: the size of the next row list, the number of sequences still decoding and, in a generation, the
+// host's mirror of it (host_active[0]: sequences still decoding; host_active[1]: denoising steps finished)
+__device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int n_active)
+{
+    if (a.next_n_rows) *a.next_n_rows = n_next;
+    if (a.n_active) *a.n_active = n_active;
+    if (a.host_active) {
+        a.host_active[1] = a.host_step;
+        __threadfence_system();
+        a.host_active[0] = n_active;
+    }
+}
+
+__device__ unsigned long long block_min_u64(unsigned long long v, unsigned long long *s_tmp /* [8] */) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) s_tmp[threadIdx.x >> 5] = v;
+    __syncthreads();
+    unsigned long long r = s_tmp[0];
+#pragma unroll
+    for (int w = 1; w < kSelThreads / 32; ++w) r = min(r, s_tmp[w]);
+    return r;
+}
+
+// flags of a response position
+enum { F_MASKED = 1, F_HIGH = 2, F_SEL = 4, F_OPEN = 8 };
+
+// Which candidate rows of a step must be recomputed canonically (two-pass statistics): flags them F_OPEN and lists their logits
+// rows, in position order, in s_list; returns how many.  Every other candidate row's enclosure [lo, hi] answers what the step's
+// rule asks, and its lower bound stands for it:
+//   * a threshold is open when lo and hi fall on different sides of it;
+//   * the ranking (k most confident candidates, smallest S_q first) is open for every candidate whose lo does not exceed
+//     U = the k-th smallest hi among the candidates: the k rows with the smallest hi all have S_q <= U, so a row with
+//     lo > U is not among the k most confident, and its lower bound (still > U) orders it behind them.  Only k = 1 is
+//     evaluated this way (U = the smallest hi); for k > 1 every candidate is recomputed.
+__device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, uint8_t *s_fl, int32_t *s_list, int *s_tmp, unsigned long long *s_min)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
+    const StepAsk ask = step_ask(a.params, st, L);
+    const long long base = (long long)b * a.S + a.P;
+    const uint8_t *msk = a.mask + base;
+    const unsigned long long *plo = a.pos_lo + base, *phi = a.pos_hi + base;
+    int k_top = 0;
+    unsigned long long U = ~0ull;
+    if (ask.rank_needed) {
+        int cnt = 0;
+        for (int j = ask.lo + tid; j < ask.hi; j += kSelThreads) {
+            if (!msk[j]) continue;
+            cnt++;
+            if (plo[j] != 0) U = min(U, phi[j]);
+        }
+        const int n_cand = block_sum(cnt, s_tmp);
+        U = block_min_u64(U, s_min);
+        if (a.params.sampler == SFS_SAMPLER_LOW_CONFIDENCE) {
+            const BlockStep blk = block_step(a.params, L, st.steps_done);
+            const long long Lb = ask.hi - ask.lo, Nb = blk.steps_per_block;
+            k_top = (int)max(0ll, (Lb * (Nb - blk.k_b + 1)) / Nb - (Lb - n_cand));
+        } else {
+            k_top = (st.phase == SFS_PHASE_SLOW) ? a.params.k_slow : a.params.k_fast;
+        }
+        if (k_top >= n_cand) k_top = 0;                     // everything is chosen: no ranking
+    }
+    int n_open = 0;
+    for (int i0 = 0; i0 < L; i0 += kSelThreads) {
+        const int i = i0 + tid;
+        bool open = false;
+        if (i >= ask.lo && i < ask.hi && i < L && msk[i]) {
+            const unsigned long long lo = plo[i], hi = phi[i];
+            if (lo != 0) {                                  // 0: no row supplied for this candidate
+                if (ask.tau > 0.f) open = conf_exceeds(lo, ask.tau) && !conf_exceeds(hi, ask.tau);
+                if (k_top > 1) open = true;
+                else if (k_top == 1) open = open || lo <= U;
+            }
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, open);
+        __syncthreads();
+        if (lane == 0) s_tmp[warp] = __popc(bal);
+        __syncthreads();
+        int before = n_open, total = 0;
+#pragma unroll
+        for (int w = 0; w < kSelThreads / 32; ++w) { const int c = s_tmp[w]; total += c; if (w < warp) before += c; }
+        if (i < L) s_fl[i] = open ? F_OPEN : 0;
+        if (open) s_list[before + __popc(bal & ((1u << lane) - 1u))] = i;
+        n_open += total;
+    }
+    __syncthreads();
+    return n_open;
+}
+
+// One step of the transition rule.  `groups` CTAs per sequence: with two-pass row statistics (pos_lo given) every one of them
+// first lists the rows whose enclosure leaves the step's question open (the same list in each), they share the canonical
+// recomputation of those rows, warp by warp, adding integer partial sums to pos_sq, and the CTA that finishes last (a ticket)
+// goes on alone.  So the list, the recomputation and the choice are one launch: on 256 rows of 126464 logits the three kernels
+// they were took 6 + 9 + 11 us of a 45 us sfs_select call; DRAM has no part in it, the chain of block-wide steps bounds it.
+// Without two-pass statistics there is one CTA per sequence.
+// dynamic shared memory: keys u64[L] (before: the list of open rows) | flags u8[L]
 __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
 {
-    pdl_wait();
-    pdl_trigger();
     extern __shared__ unsigned long long s_keys[];
-    const int L = a.L, S = a.S, P = a.P, b = blockIdx.x, tid = threadIdx.x;
-    uint8_t *s_sel  = reinterpret_cast<uint8_t *>(s_keys + L);
-    uint8_t *s_high = s_sel + L;
+    const int L = a.L, S = a.S, P = a.P, b = blockIdx.x / a.groups, part = blockIdx.x - b * a.groups;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint8_t *s_fl = reinterpret_cast<uint8_t *>(s_keys + L);
     __shared__ int s_tmp[6 * (kSelThreads / 32)];
+    __shared__ unsigned long long s_min[kSelThreads / 32];
     __shared__ sfs_state st;
     __shared__ int s_last;
 
+    pdl_wait();
+    pdl_trigger();
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(&st)[tid] = reinterpret_cast<const int *>(a.state + b)[tid];
     __syncthreads();
 
-    int32_t *tok = a.tokens + (long long)b * S + P;
-    uint8_t *msk = a.mask + (long long)b * S + P;
-    unsigned long long *psq = a.pos_sq + (long long)b * S + P;
-    int32_t *parg = a.pos_arg + (long long)b * S + P;
+    const long long base = (long long)b * S + P;
+    int32_t *tok = a.tokens + base;
+    uint8_t *msk = a.mask + base;
+    unsigned long long *psq = a.pos_sq + base;
+    const int32_t *parg = a.pos_arg + base;
     const sfs_params &p = a.params;
+    const bool two_pass = a.pos_lo != nullptr;
 
     const bool active = !st.done && st.status == SFS_OK;
     const bool vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
+    if (a.groups > 1 && !active && part != 0) return;
+    if (two_pass && active) {
+        int32_t *s_list = reinterpret_cast<int32_t *>(s_keys);
+        const int n_open = list_open_rows(a, st, b, s_fl, s_list, s_tmp, s_min);
+        recompute_rows(a.lrows, s_list, n_open, a.pos_row + base, a.pos_max + base, psq, part * (kSelThreads / 32) + warp,
+                       a.groups * (kSelThreads / 32));
+        if (a.groups > 1) {
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) s_last = (atomicAdd(&a.seq_ticket[b], 1) == a.groups - 1) ? 1 : 0;
+            __syncthreads();
+            if (!s_last) return;
+            __threadfence();
+            if (tid == 0) a.seq_ticket[b] = 0;
+        } else {
+            __threadfence();
+            __syncthreads();
+        }
+    }
+
     int n_sel = 0, e_cand = -1, stable = 0;
     int rec_phase = st.phase, rec_s = st.s_cycle;
     int rec_hi = (st.phase == SFS_PHASE_SLOW) ? L : st.hi;
@@ -107,24 +222,31 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
         const int lo = vanilla ? blk.lo : (forced ? 0 : st.s_cycle);
         const int hi = vanilla ? blk.hi : (forced ? L : ((st.phase == SFS_PHASE_SLOW) ? L : st.hi));
 
-        // ---- candidates of this step and their statistics
+        // ---- candidates of this step and their statistics (consumed: a later step must bring its own)
         BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0};
+        unsigned long long kmin = kNoKey;
         for (int i = tid; i < L; i += kSelThreads) {
             const bool m = msk[i] != 0;
             const bool cand = m && i >= lo && i < hi;
             unsigned long long key = kNoKey;
-            uint8_t high = 0;
+            unsigned long long sq = __ldcg(&psq[i]);
+            if (two_pass) {
+                if (!(s_fl[i] & F_OPEN)) sq = __ldcg(&a.pos_lo[base + i]);
+                a.pos_lo[base + i] = 0;
+            }
+            psq[i] = 0;
+            uint8_t fl = m ? F_MASKED : 0;
             if (cand) {
-                const unsigned long long sq = psq[i];
                 if (sq == 0) r.missing++;
                 key = (sq << kPosBits) | (unsigned long long)i;
                 r.n_cand++;
                 r.min_cand = min(r.min_cand, i);
-                if (exceeds(sq, p.tau_min_conf)) r.max_above = max(r.max_above, i);
-                if (exceeds(sq, p.tau_high_conf)) { high = 1; r.n_high++; }
+                if (conf_exceeds(sq, p.tau_min_conf)) r.max_above = max(r.max_above, i);
+                if (conf_exceeds(sq, p.tau_high_conf)) { fl |= F_HIGH; r.n_high++; }
             }
+            kmin = min(kmin, key);
             r.n_masked += m ? 1 : 0;
-            s_keys[i] = key; s_high[i] = high; s_sel[i] = 0;
+            s_keys[i] = key; s_fl[i] = fl;
         }
         r = block_reduce(r, s_tmp);
 
@@ -145,22 +267,26 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             else { mode = MODE_TOPK; k_top = p.k_fast; }
 
             // ---- choose
+            const bool ranked = mode == MODE_TOPK && k_top > 1 && k_top < r.n_cand;      // (one or all: no ranking)
+            const unsigned long long top1 = (mode == MODE_TOPK && k_top == 1) ? block_min_u64(kmin, s_min) : 0ull;
             int my_sel = 0;
             for (int i = tid; i < L; i += kSelThreads) {
                 const unsigned long long key = s_keys[i];
                 if (key == kNoKey) continue;
                 bool sel;
                 if (mode == MODE_ALL) sel = true;
-                else if (mode == MODE_HIGH) sel = s_high[i] != 0;
+                else if (mode == MODE_HIGH) sel = (s_fl[i] & F_HIGH) != 0;
                 else if (mode == MODE_RANDOM)
                     sel = (unsigned long long)philox_first_word((uint32_t)i, (uint32_t)st.steps_done, (uint32_t)b, 0u, p.seed_lo, p.seed_hi)
                           * (unsigned long long)blk.k_b < (1ull << 32);
+                else if (k_top == 1) sel = key == top1;
+                else if (!ranked) sel = k_top > 0;
                 else {
                     int rank = 0;                           // candidates that are more confident (ties: smaller position)
                     for (int j = 0; j < L; ++j) rank += (s_keys[j] < key) ? 1 : 0;
                     sel = rank < k_top;
                 }
-                if (sel) { s_sel[i] = 1; my_sel++; tok[i] = parg[i]; msk[i] = 0; }
+                if (sel) { s_fl[i] = (uint8_t)((s_fl[i] | F_SEL) & ~F_MASKED); my_sel++; tok[i] = parg[i]; msk[i] = 0; }
             }
             n_sel = block_sum(my_sel, s_tmp);
 
@@ -197,7 +323,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             // ---- is the span clean?  (decides whether the next cycle starts)
             if (!vanilla && !forced && st.phase == SFS_PHASE_FAST) {
                 int cnt = 0;
-                for (int i = st.s_cycle + tid; i < st.hi && i < L; i += kSelThreads) cnt += msk[i] ? 1 : 0;
+                for (int i = st.s_cycle + tid; i < st.hi && i < L; i += kSelThreads) cnt += (s_fl[i] & F_MASKED) ? 1 : 0;
                 cnt = block_sum(cnt, s_tmp);
                 if (tid == 0 && cnt == 0 && st.n_masked > 0) {
                     st.s_cycle = st.hi; st.phase = SFS_PHASE_SLOW; st.hist_len = 0; st.step_count = 0; st.n_cycles++;
@@ -208,38 +334,42 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 if (st.n_masked > 0) st.status = SFS_ERR_STEP_LIMIT;
             }
         }
-        __syncthreads();
-        // the statistics of this step are consumed: a later step must bring its own
-        for (int i = tid; i < L; i += kSelThreads) psq[i] = 0;
-        if (a.pos_lo) for (int i = tid; i < L; i += kSelThreads) a.pos_lo[(long long)b * S + P + i] = 0;
     } else {
         // a finished (or stopped) sequence consumes the statistics supplied for it as well: nothing stale is left for a
         // later generation that reuses the scratch
-        for (int i = tid; i < L; i += kSelThreads) { s_sel[i] = 0; psq[i] = 0; if (a.pos_lo) a.pos_lo[(long long)b * S + P + i] = 0; }
+        for (int i = tid; i < L; i += kSelThreads) { s_fl[i] = 0; psq[i] = 0; if (two_pass) a.pos_lo[base + i] = 0; }
     }
     __syncthreads();
 
-    // ---- ordered outputs (warp 0: ballot scan): selected positions, and the rows of the next step
-    if (tid < 32) {
+    // ---- ordered outputs (ballots and per-warp counts): selected positions, and the rows of the next step
+    {
         const bool next_active = !st.done && st.status == SFS_OK;
         const bool nforced = !vanilla && st.k_remaining == 1;
         const BlockStep nblk = block_step(p, L, st.steps_done);
         const int nlo = vanilla ? nblk.lo : (nforced ? 0 : st.s_cycle);
         const int nhi = vanilla ? nblk.hi : (nforced ? L : ((st.phase == SFS_PHASE_SLOW) ? L : st.hi));
+        // a single sequence's list is the whole list
+        int32_t *const next = a.B == 1 ? a.next_rows : a.seq_rows + (long long)b * L;
         int n_out = 0, n_next = 0;
-        for (int base = 0; base < L; base += 32) {
-            const int i = base + tid;
-            const bool sel = i < L && s_sel[i];
-            const bool need = next_active && i < L && msk[i] && i >= nlo && i < nhi;
+        for (int i0 = 0; i0 < L; i0 += kSelThreads) {
+            const int i = i0 + tid;
+            const uint8_t fl = i < L ? s_fl[i] : 0;
+            const bool sel = (fl & F_SEL) != 0, need = next_active && (fl & F_MASKED) && i >= nlo && i < nhi;
             const unsigned bs = __ballot_sync(0xffffffffu, sel), bn = __ballot_sync(0xffffffffu, need);
-            const unsigned lt = (1u << tid) - 1u;
+            if (lane == 0) s_tmp[warp] = __popc(bs) | (__popc(bn) << 16);
+            __syncthreads();
+            int before = 0, total = 0;
+#pragma unroll
+            for (int w = 0; w < kSelThreads / 32; ++w) { const int c = s_tmp[w]; total += c; if (w < warp) before += c; }
+            const unsigned lt = (1u << lane) - 1u;
             if (sel && a.sel_pos) {
-                const int o = n_out + __popc(bs & lt);
+                const int o = n_out + (before & 0xFFFF) + __popc(bs & lt);
                 a.sel_pos[(long long)b * L + o] = i;
-                a.sel_tok[(long long)b * L + o] = tok[i];
+                a.sel_tok[(long long)b * L + o] = parg[i];
             }
-            if (need) a.seq_rows[(long long)b * L + n_next + __popc(bn & lt)] = b * S + P + i;
-            n_out += __popc(bs); n_next += __popc(bn);
+            if (need && next) next[n_next + (before >> 16) + __popc(bn & lt)] = b * S + P + i;
+            n_out += total & 0xFFFF; n_next += total >> 16;
+            __syncthreads();
         }
         if (tid == 0) {
             if (a.sel_count) a.sel_count[b] = n_out;
@@ -249,36 +379,38 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 t[0] = rec_phase; t[1] = rec_s; t[2] = rec_hi; t[3] = e_cand; t[4] = stable; t[5] = n_sel;
                 t[6] = st.n_masked; t[7] = st.k_remaining;
             }
+            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0);
         }
     }
-    __syncthreads();
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(a.state + b)[tid] = reinterpret_cast<const int *>(&st)[tid];
+    if (a.B == 1) return;
 
-    // ---- last CTA: concatenate the row lists, count the active sequences
+    // ---- last sequence: concatenate the row lists, count the active sequences
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = (atomicAdd(a.ticket, 1) == (int)gridDim.x - 1) ? 1 : 0;
+    if (tid == 0) s_last = (atomicAdd(a.ticket, 1) == a.B - 1) ? 1 : 0;
     __syncthreads();
-    if (s_last) {
-        __threadfence();
-        if (tid == 0) {
-            int total = 0, act = 0;
-            for (int q = 0; q < a.B; ++q) {
-                total += __ldcg(&a.seq_row_count[q]);
-                act += (__ldcg(&a.state[q].done) == 0 && __ldcg(&a.state[q].status) == SFS_OK) ? 1 : 0;
-            }
-            if (a.next_n_rows) *a.next_n_rows = total;
-            if (a.n_active) *a.n_active = act;
-            *a.ticket = 0;
+    if (!s_last) return;
+    __threadfence();
+    int off = 0, act = 0;
+    for (int q0 = 0; q0 < a.B; q0 += 32) {                  // every warp: offsets of 32 sequences; then each warp copies every 8th list
+        const int q = q0 + lane;
+        const int c = q < a.B ? __ldcg(&a.seq_row_count[q]) : 0;
+        act += (q < a.B && __ldcg(&a.state[q].done) == 0 && __ldcg(&a.state[q].status) == SFS_OK) ? 1 : 0;
+        int pre = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += t; }
+        for (int k = warp; k < 32 && q0 + k < a.B; k += kSelThreads / 32) {
+            const int ck = __shfl_sync(0xffffffffu, c, k), ok = off + __shfl_sync(0xffffffffu, pre, k) - ck;
+            if (a.next_rows)
+                for (int i = lane; i < ck; i += 32) a.next_rows[ok + i] = __ldcg(&a.seq_rows[(long long)(q0 + k) * L + i]);
         }
-        if (a.next_rows) {
-            int off = 0;
-            for (int q = 0; q < a.B; ++q) {
-                const int c = __ldcg(&a.seq_row_count[q]);
-                for (int i = tid; i < c; i += kSelThreads) a.next_rows[off + i] = __ldcg(&a.seq_rows[(long long)q * L + i]);
-                off += c;
-            }
-        }
+        off += __shfl_sync(0xffffffffu, pre, 31);
+    }
+    act = warp_sum_i32(act);
+    if (tid == 0) {
+        finish_step(a, off, act);
+        *a.ticket = 0;
     }
 }
 
@@ -297,14 +429,18 @@ __global__ void state_init_kernel(sfs_state *state, int B, int L, sfs_params p)
 
 }  // namespace
 
-int32_t launch_select(const SelectArgs &a, cudaStream_t stream)
+int32_t launch_select(const SelectArgs &args, cudaStream_t stream)
 {
-    const size_t smem = (size_t)a.L * (sizeof(unsigned long long) + 2);
+    SelectArgs a = args;
+    const size_t smem = (size_t)a.L * (sizeof(unsigned long long) + 1);
     SFS_REQUIRE(smem <= 200 * 1024, SFS_ERR_UNSUPPORTED, "gen_len %d too long for the selection kernel", a.L);
     if (smem > 48 * 1024) {
         SFS_CUDA(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     }
-    SFS_CUDA(launch_pdl(select_kernel, dim3((unsigned)(a.B)), dim3((unsigned)(kSelThreads)), (size_t)(smem), stream, a));
+    // two-pass statistics: two CTAs per SM over all sequences share the recomputation (k > 1 can ask for every row)
+    a.groups = 1;
+    if (a.pos_lo != nullptr) a.groups = a.B < 148 ? 296 / a.B : 1;
+    SFS_CUDA(launch_pdl(select_kernel, dim3((unsigned)(a.B * a.groups)), dim3((unsigned)(kSelThreads)), (size_t)(smem), stream, a));
     return SFS_OK;
 }
 

@@ -174,43 +174,46 @@ int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t voc
 // Row statistics for the selection step in two passes over long bf16 rows (the filter + exact form):
 //   pass 1 streams every row from HBM once and finds the exact maximum and argmax plus an APPROXIMATE denominator (special-
 //     function exponentials, fp32 sum) with a proven enclosure [lo, lo + w] of the canonical S_q;
-//   pass 2 looks, per sequence, at what the step's rule will ask of its rows (which threshold, which top-k), lists the rows
-//     whose enclosure leaves an answer open and recomputes the canonical S_q of those; every other candidate row gets its
-//     lower bound.
-// The selection kernel then runs unchanged on pos_sq, and its decisions equal those taken on all-canonical values.
-struct RefineArgs {
-    const int32_t *tokens_unused; const uint8_t *mask; int32_t B, S, P, L;
-    const sfs_state *state; sfs_params params;
-    unsigned long long *pos_lo, *pos_hi;                    // [B*S] enclosures written by pass 1 (lo == 0: no row supplied)
-    unsigned long long *pos_sq; int32_t *pos_arg;           // [B*S] what the selection kernel reads
+//   pass 2, inside the selection kernel, looks at what the step's rule will ask of a sequence's rows (which threshold, which
+//     top-k), recomputes the canonical S_q of those whose enclosure leaves an answer open and takes every other one's lower bound.
+// The decisions equal those taken on all-canonical values.
+struct BoundsScratch {
+    unsigned long long *pos_lo, *pos_hi;                    // [positions] enclosures written by pass 1 (lo == 0: no row supplied)
+    int32_t *pos_arg;                                       // [positions] what the selection kernel reads
     float *slice_partials; int32_t *row_tickets;            // scratch of pass 1: [max rows * 8 * 4] floats, [max rows] (zeroed)
-    int32_t *pos_row; float *pos_max;                       // [B*S] logits row and exact row maximum of each position (pass 1)
-    int32_t *refine_list, *refine_count;                    // [max rows], [1]: logits rows pass 2 recomputes
+    int32_t *pos_row; float *pos_max;                       // [positions] logits row and exact row maximum of each position (pass 1)
+    int32_t n_positions;
 };
 constexpr int kRowStatsSlices = 8;
 // true when the two-pass form applies to this logits layout (long bf16 rows, 16-byte aligned)
 bool row_stats_two_pass_applies(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld);
 int32_t launch_row_stats_two_pass(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,
-                                  const int32_t *d_rows, const RefineArgs &rf, int32_t *d_err, cudaStream_t stream);
+                                  const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err, cudaStream_t stream);
 // the same with pass 1 already taken by the LM head's epilogue: `stats` holds n_parts records per row (stats_ld apart)
-int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, const void *d_logits, int32_t vocab, int64_t ld,
-                                       const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const RefineArgs &rf, int32_t *d_err,
-                                       cudaStream_t stream);
+int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows,
+                                       const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err, cudaStream_t stream);
 // pass 1 alone, dense outputs by logits row (for tests): d_lo / d_hi enclose the canonical S_q
 int32_t launch_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,
                                 unsigned long long *d_lo, unsigned long long *d_hi, int32_t *d_argmax, int32_t *d_err, cudaStream_t stream);
 
+struct LogitsRows { const uint4 *base; long long ld; int32_t chunks; };          // bf16 logits as 16-byte chunks, ld chunks between rows
 struct SelectArgs {
     int32_t *tokens; uint8_t *mask; int32_t B, S, P, L;
     sfs_state *state; sfs_params params;
     unsigned long long *pos_sq; int32_t *pos_arg;          // [B*S] scratch written by the row-stats kernel
-    unsigned long long *pos_lo;                             // optional [B*S]: enclosures of the two-pass form, cleared with pos_sq
+    // two-pass form (pos_lo != NULL): the enclosures (pos_lo is cleared with pos_sq), and what recomputing a row takes
+    unsigned long long *pos_lo; const unsigned long long *pos_hi;           // [B*S]
+    const int32_t *pos_row; const float *pos_max;                           // [B*S]
+    LogitsRows lrows;
+    int32_t *seq_ticket;                                    // [B] scratch counters (zero between launches)
+    int32_t groups;                                         // CTAs per sequence (set by the launcher)
     int32_t *sel_count, *sel_pos, *sel_tok;                 // [B], [B,L], [B,L]   (optional)
     int32_t *seq_rows, *seq_row_count;                      // [B,L], [B] scratch: next step's rows per sequence
     int32_t *next_rows, *next_n_rows;                       // optional flat list (sequence-major) + count
     int32_t *n_active;                                      // optional: sequences not done after this step
     int32_t *ticket;                                        // scratch counter (zero between launches)
     int32_t *trace;                                         // optional [B, SFS_TRACE_INTS]
+    int32_t *host_active; int32_t host_step;                // optional: the host's mirror, and the step count to leave there
 };
 int32_t launch_select(const SelectArgs &a, cudaStream_t stream);
 int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, int32_t *seq_rows_unused,
