@@ -61,6 +61,7 @@ int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int
 // stores, C itself is not touched) and the consumer of the residual stream adds them in slab order (launch_rmsnorm does),
 // so the sum does not depend on which CTA finishes first.  ws must hold max_splits * M * ldc floats.
 int32_t gemm_plan_enable_split(GemmPlan *p, float *ws, int32_t max_splits, const GemmTune *tune);
+int gemm_num_sms();                                  // SMs of the device
 int32_t gemm_launch(const GemmPlan &p, const int32_t *d_m, const int32_t *d_active, int32_t *err, cudaStream_t stream);
 
 }  // namespace sfs

@@ -750,6 +750,8 @@ int stages_for_few(int bn, int nb)
 
 }  // namespace
 
+int gemm_num_sms() { return num_sms(); }
+
 int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int32_t K,
                          const void *const *Bs, int32_t n_maps, int32_t n_per_map, int64_t ldb,
                          int32_t mode, void *C, int64_t ldc, int32_t out_f32, float scale,
