@@ -165,13 +165,13 @@ static int32_t run_body(sfs_session *s, const int32_t *d_tokens, int32_t B, int3
     int32_t *err = device_status_word();
     SFS_REQUIRE(err != nullptr, SFS_ERR_OOM, "cannot allocate the device status word");
     int32_t rc;
-    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed(d_tokens, m->tok_emb, s->x, T, d, c.vocab, st); })) != SFS_OK) return rc;
+    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed_norm(d_tokens, m->tok_emb, c.vocab, s->x, m->attn_norm[0], s->h, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
     // A split-K projection leaves its partial products in s->partial; the next RMSNorm folds them into x.
     const long long pstride = (long long)T * d;
     int pending = 0;
     for (int l = 0; l < c.n_layers; ++l) {
         const LayerPlans &lp = s->layer_plans[l];
-        if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->attn_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
+        if (l > 0 && (rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->attn_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
         if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
         if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
         if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
@@ -278,13 +278,18 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
     if (n_sel_out) *n_sel_out = (rp && rr) ? S : n_sel;
     const int NR = B * n_sel;
 
-    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed(d_tokens, m->tok_emb, s->x, T, d, c.vocab, st); })) != SFS_OK) return rc;
     const float *pend = nullptr;
     // Rows whose residual stream this step keeps up to date: all of them, except that a single sequence whose prompt is not
     // refreshed needs only its response rows (nothing reads the prompt rows of x or h then).
     const int r_first = (B == 1 && !rp) ? P : 0, r_count = (B == 1 && !rp) ? L : T;
     // tokens whose fresh values are compared with the cached ones: the response of a single sequence (from an even index), else all
     const int sim_first = (B == 1) ? (P & ~1) : 0, sim_count = (B == 1) ? S - sim_first : T;
+    // the first layer's norm of those rows embeds their tokens
+    rc = timed_launch(s, SFS_K_EMBED, st, [&] {
+        return launch_embed_norm(d_tokens + r_first, m->tok_emb, c.vocab, s->x + (size_t)r_first * d, m->attn_norm[0], s->h + (size_t)r_first * d, r_count, d,
+                                 c.rms_eps, st);
+    });
+    if (rc != SFS_OK) return rc;
     auto norm_all = [&](const void *gain) {
         return timed_launch(s, SFS_K_RMSNORM, st, [&] {
             return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, pend ? 1 : 0, 0, gain,
@@ -296,7 +301,7 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
         for (int l = 0; l < c.n_layers; ++l) {
             const LayerPlans &lp = s->layer_plans[l];
             const CacheLayerPlans &cl = s->cache_plans[l];
-            if ((rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
+            if (l > 0 && (rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
             if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
             if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
             SFS_CUDA(cudaMemcpy2DAsync(s->Kc[l], (size_t)d * 2, s->qk + d, (size_t)2 * d * 2, (size_t)d * 2, (size_t)T, cudaMemcpyDeviceToDevice, st));
@@ -323,7 +328,7 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
         int n_pend = 0;
         for (int l = 0; l < c.n_layers; ++l) {
             const CacheLayerPlans &cl = s->cache_plans[l];
-            rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
+            if (l > 0) rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
                 return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, n_pend, inc_stride, m->attn_norm[l],
                                       s->h + (size_t)r_first * d, nullptr, nullptr, r_count, d, c.rms_eps, st);
             });

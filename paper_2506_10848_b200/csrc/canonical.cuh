@@ -69,10 +69,10 @@ __device__ __forceinline__ Consts2 canon_consts(float m) {
 }
 
 // Canonical S_q of the listed positions' logits rows (bf16, 16-byte aligned, a multiple of 8 entries), by `n_warps` warps of which
-// this one is `w`: a row is cut into items of kOpenChunks 16-byte chunks, eight loads of a lane in flight, and every item's
+// this one is `w`: a row is cut into items of kOpenChunks 16-byte chunks, four loads of a lane in flight, and every item's
 // integer sum is added to pos_sq of its position (which is zero before) — integer addition commutes, so the order of arrival
 // does not matter.  The rows come from L2: the first pass has just streamed them, or the LM head written them.
-constexpr int kOpenChunks = 256;
+constexpr int kOpenChunks = 128;
 __device__ __forceinline__ void recompute_rows(const LogitsRows &g, const int32_t *list, int n, const int32_t *pos_row, const float *pos_max,
                                                unsigned long long *pos_sq, int w, int n_warps)
 {

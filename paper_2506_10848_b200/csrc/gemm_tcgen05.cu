@@ -352,6 +352,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         s_abort = 0;
         tc::mbar_init_fence();
     }
+    if (threadIdx.x == 64) {                                // descriptors on their way while the kernel before this one runs
+        tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB0);
+        if (g.mode == GEMM_SWIGLU || g.n_per_map < g.N) { tc::tma_prefetch_desc(&tmB1); tc::tma_prefetch_desc(&tmB2); }
+    }
     __syncwarp();
     if (warp == 1) { tc::tmem_alloc_2cta(tc::smem_u32(tmem_slot), kTmemCols); tc::tmem_relinquish_2cta(); }
     tc::tc_fence_before();
@@ -376,7 +380,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // issued, so the latency of that poll overlaps the issue.
     if (warp == 0) {
         // ---------------- TMA producer (both CTAs; completion bytes are counted on the leader's barrier)
-        if (lane == 0) { tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB0); }
         uint32_t it = 0;
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);
@@ -525,6 +528,10 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         s_abort = 0;
         tc::mbar_init_fence();
     }
+    if (threadIdx.x == 64) {                                // descriptors on their way while the kernel before this one runs
+        tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB0);
+        if (g.mode == GEMM_SWIGLU || g.n_per_map < g.N) { tc::tma_prefetch_desc(&tmB1); tc::tma_prefetch_desc(&tmB2); }
+    }
     __syncwarp();
     if (warp == 1) { tc::tmem_alloc_2cta(tc::smem_u32(tmem_slot), kTmemCols); tc::tmem_relinquish_2cta(); }
     tc::tc_fence_before();
@@ -541,7 +548,6 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 
     if (warp == 0) {
         // ---------------- TMA producer (both CTAs; completion bytes are counted on the leader's barrier)
-        if (lane == 0) { tc::tma_prefetch_desc(&tmA); tc::tma_prefetch_desc(&tmB0); }
         uint32_t it = 0, s = 0, ph = 0;
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);

@@ -170,7 +170,13 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     float lmax = -INFINITY;
 #pragma unroll
     for (int j = 0; j < NV; ++j) lmax = fmaxf(lmax, chunk_max<T>(v[j]));
-    for (int c = c0 + NV * stride; c < rc.n; c += stride) lmax = fmaxf(lmax, chunk_max<T>(rc.load(c)));
+    for (int c = c0 + NV * stride; c < rc.n; c += 4 * stride) {                  // the rest of a longer row: four loads in flight
+        uint4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = rc.load(c + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) lmax = fmaxf(lmax, chunk_max<T>(q[u]));
+    }
     float m = warp_max(lmax);
     if (lane == 0) s_wmax[warp] = m;
     __syncthreads();
@@ -219,7 +225,13 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     unsigned long long acc = 0;
 #pragma unroll
     for (int j = 0; j < NV; ++j) acc += chunk_terms<T>(v[j], k);
-    for (int c = c0 + NV * stride; c < rc.n; c += stride) acc += chunk_terms<T>(rc.load(c), k);
+    for (int c = c0 + NV * stride; c < rc.n; c += 4 * stride) {
+        uint4 q[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) q[u] = rc.load(c + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc += chunk_terms<T>(q[u], k);
+    }
     acc = warp_sum_u64(acc);
     if (lane == 0) s_wsum[warp] = acc;
     __syncthreads();

@@ -17,38 +17,35 @@ constexpr int kPosBits = 17;                 // key = S_q << 17 | position  (S_q
 
 struct BlockRed {
     int n_cand, n_high, max_above, min_cand, n_masked, missing;
+    unsigned long long kmin;                                // smallest key
 };
 
-__device__ BlockRed block_reduce(BlockRed v, int *s_tmp /* [6 * 8] */) {
+__device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+__device__ BlockRed block_reduce(BlockRed v, int *s_tmp /* [6 * 8] */, unsigned long long *s_min /* [8] */) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     v.n_cand = warp_sum_i32(v.n_cand);   v.n_high = warp_sum_i32(v.n_high);
     v.max_above = warp_max_i32(v.max_above); v.min_cand = warp_min_i32(v.min_cand);
     v.n_masked = warp_sum_i32(v.n_masked);   v.missing = warp_sum_i32(v.missing);
+    v.kmin = warp_min_u64(v.kmin);
     __syncthreads();
     if (lane == 0) {
         s_tmp[warp * 6 + 0] = v.n_cand; s_tmp[warp * 6 + 1] = v.n_high; s_tmp[warp * 6 + 2] = v.max_above;
         s_tmp[warp * 6 + 3] = v.min_cand; s_tmp[warp * 6 + 4] = v.n_masked; s_tmp[warp * 6 + 5] = v.missing;
+        s_min[warp] = v.kmin;
     }
     __syncthreads();
-    BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0};
+    BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0, ~0ull};
+#pragma unroll
     for (int w = 0; w < kSelThreads / 32; ++w) {
         r.n_cand += s_tmp[w * 6 + 0]; r.n_high += s_tmp[w * 6 + 1];
         r.max_above = max(r.max_above, s_tmp[w * 6 + 2]); r.min_cand = min(r.min_cand, s_tmp[w * 6 + 3]);
-        r.n_masked += s_tmp[w * 6 + 4]; r.missing += s_tmp[w * 6 + 5];
+        r.n_masked += s_tmp[w * 6 + 4]; r.missing += s_tmp[w * 6 + 5]; r.kmin = min(r.kmin, s_min[w]);
     }
-    __syncthreads();
-    return r;
-}
-
-__device__ int block_sum(int v, int *s_tmp) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v = warp_sum_i32(v);
-    __syncthreads();
-    if (lane == 0) s_tmp[warp] = v;
-    __syncthreads();
-    int r = 0;
-    for (int w = 0; w < kSelThreads / 32; ++w) r += s_tmp[w];
-    __syncthreads();
     return r;
 }
 
@@ -81,18 +78,6 @@ __device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int
     }
 }
 
-__device__ unsigned long long block_min_u64(unsigned long long v, unsigned long long *s_tmp /* [8] */) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) s_tmp[threadIdx.x >> 5] = v;
-    __syncthreads();
-    unsigned long long r = s_tmp[0];
-#pragma unroll
-    for (int w = 1; w < kSelThreads / 32; ++w) r = min(r, s_tmp[w]);
-    return r;
-}
-
 // flags of a response position
 enum { F_MASKED = 1, F_HIGH = 2, F_SEL = 4, F_OPEN = 8 };
 
@@ -104,7 +89,9 @@ enum { F_MASKED = 1, F_HIGH = 2, F_SEL = 4, F_OPEN = 8 };
 //     U = the k-th smallest hi among the candidates: the k rows with the smallest hi all have S_q <= U, so a row with
 //     lo > U is not among the k most confident, and its lower bound (still > U) orders it behind them.  Only k = 1 is
 //     evaluated this way (U = the smallest hi); for k > 1 every candidate is recomputed.
-__device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, uint8_t *s_fl, int32_t *s_list, int *s_tmp, unsigned long long *s_min)
+// m0 / lo0 / hi0: mask and enclosure of position threadIdx.x, loaded by the caller beside the state.
+__device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, uint8_t m0, unsigned long long lo0, unsigned long long hi0, uint8_t *s_fl,
+                              int32_t *s_list, int *s_tmp, unsigned long long *s_min)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
     const StepAsk ask = step_ask(a.params, st, L);
@@ -114,29 +101,30 @@ __device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, u
     int k_top = 0;
     unsigned long long U = ~0ull;
     if (ask.rank_needed) {
-        int cnt = 0;
-        for (int j = ask.lo + tid; j < ask.hi; j += kSelThreads) {
-            if (!msk[j]) continue;
-            cnt++;
-            if (plo[j] != 0) U = min(U, phi[j]);
+        BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0, ~0ull};
+        for (int i = tid; i < ask.hi && i < L; i += kSelThreads) {
+            const bool first = i == tid;
+            if (i < ask.lo || !(first ? m0 : msk[i])) continue;
+            r.n_cand++;
+            if ((first ? lo0 : plo[i]) != 0) r.kmin = min(r.kmin, first ? hi0 : phi[i]);
         }
-        const int n_cand = block_sum(cnt, s_tmp);
-        U = block_min_u64(U, s_min);
+        r = block_reduce(r, s_tmp, s_min);
+        U = r.kmin;
         if (a.params.sampler == SFS_SAMPLER_LOW_CONFIDENCE) {
             const BlockStep blk = block_step(a.params, L, st.steps_done);
             const long long Lb = ask.hi - ask.lo, Nb = blk.steps_per_block;
-            k_top = (int)max(0ll, (Lb * (Nb - blk.k_b + 1)) / Nb - (Lb - n_cand));
+            k_top = (int)max(0ll, (Lb * (Nb - blk.k_b + 1)) / Nb - (Lb - r.n_cand));
         } else {
             k_top = (st.phase == SFS_PHASE_SLOW) ? a.params.k_slow : a.params.k_fast;
         }
-        if (k_top >= n_cand) k_top = 0;                     // everything is chosen: no ranking
+        if (k_top >= r.n_cand) k_top = 0;                   // everything is chosen: no ranking
     }
     int n_open = 0;
     for (int i0 = 0; i0 < L; i0 += kSelThreads) {
         const int i = i0 + tid;
         bool open = false;
-        if (i >= ask.lo && i < ask.hi && i < L && msk[i]) {
-            const unsigned long long lo = plo[i], hi = phi[i];
+        if (i >= ask.lo && i < ask.hi && i < L && (i0 == 0 ? m0 : msk[i])) {
+            const unsigned long long lo = i0 == 0 ? lo0 : plo[i], hi = i0 == 0 ? hi0 : phi[i];
             if (lo != 0) {                                  // 0: no row supplied for this candidate
                 if (ask.tau > 0.f) open = conf_exceeds(lo, ask.tau) && !conf_exceeds(hi, ask.tau);
                 if (k_top > 1) open = true;
@@ -176,25 +164,35 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     __shared__ sfs_state st;
     __shared__ int s_last;
 
-    pdl_wait();
-    pdl_trigger();
-    if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(&st)[tid] = reinterpret_cast<const int *>(a.state + b)[tid];
-    __syncthreads();
-
     const long long base = (long long)b * S + P;
     int32_t *tok = a.tokens + base;
     uint8_t *msk = a.mask + base;
     unsigned long long *psq = a.pos_sq + base;
     const int32_t *parg = a.pos_arg + base;
     const sfs_params &p = a.params;
-    const bool two_pass = a.pos_lo != nullptr;
+    const bool two_pass = a.pos_lo != nullptr, vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
+
+    pdl_wait();
+    pdl_trigger();
+    // the state and everything about position tid (all of a sequence, usually) in one round trip
+    uint8_t m0 = 0;
+    int32_t arg0 = 0;
+    unsigned long long lo0 = 0, hi0 = 0;                    // two-pass: the enclosure; else lo0 = S_q
+    if (tid < L) {
+        m0 = msk[tid]; arg0 = parg[tid];
+        if (two_pass) { lo0 = __ldcg(&a.pos_lo[base + tid]); hi0 = a.pos_hi[base + tid]; }
+        else lo0 = psq[tid];
+    }
+    if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(&st)[tid] = reinterpret_cast<const int *>(a.state + b)[tid];
+    __syncthreads();
 
     const bool active = !st.done && st.status == SFS_OK;
-    const bool vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
+    const int phase0 = st.phase, s0 = st.s_cycle, hi_fast = st.hi, steps0 = st.steps_done;
+    const bool forced = !vanilla && (st.k_remaining == 1);
     if (a.groups > 1 && !active && part != 0) return;
     if (two_pass && active) {
         int32_t *s_list = reinterpret_cast<int32_t *>(s_keys);
-        const int n_open = list_open_rows(a, st, b, s_fl, s_list, s_tmp, s_min);
+        const int n_open = list_open_rows(a, st, b, m0, lo0, hi0, s_fl, s_list, s_tmp, s_min);
         recompute_rows(a.lrows, s_list, n_open, a.pos_row + base, a.pos_max + base, psq, part * (kSelThreads / 32) + warp,
                        a.groups * (kSelThreads / 32));
         if (a.groups > 1) {
@@ -212,27 +210,27 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     }
 
     int n_sel = 0, e_cand = -1, stable = 0;
-    int rec_phase = st.phase, rec_s = st.s_cycle;
-    int rec_hi = (st.phase == SFS_PHASE_SLOW) ? L : st.hi;
-    const BlockStep blk = block_step(p, L, st.steps_done);
-    if (vanilla) { rec_phase = blk.j; rec_s = blk.lo; rec_hi = blk.hi; e_cand = blk.k_b; }
+    int rec_phase = phase0, rec_s = s0;
+    int rec_hi = (phase0 == SFS_PHASE_SLOW) ? L : hi_fast;
+    BlockStep blk{};
+    if (vanilla) { blk = block_step(p, L, steps0); rec_phase = blk.j; rec_s = blk.lo; rec_hi = blk.hi; e_cand = blk.k_b; }
 
     if (active) {
-        const bool forced = !vanilla && (st.k_remaining == 1);
-        const int lo = vanilla ? blk.lo : (forced ? 0 : st.s_cycle);
-        const int hi = vanilla ? blk.hi : (forced ? L : ((st.phase == SFS_PHASE_SLOW) ? L : st.hi));
+        const int lo = vanilla ? blk.lo : (forced ? 0 : s0);
+        const int hi = vanilla ? blk.hi : (forced ? L : ((phase0 == SFS_PHASE_SLOW) ? L : hi_fast));
 
         // ---- candidates of this step and their statistics (consumed: a later step must bring its own)
-        BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0};
-        unsigned long long kmin = kNoKey;
+        BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0, kNoKey};
         for (int i = tid; i < L; i += kSelThreads) {
-            const bool m = msk[i] != 0;
+            const bool m = (i == tid ? m0 : msk[i]) != 0;
             const bool cand = m && i >= lo && i < hi;
-            unsigned long long key = kNoKey;
-            unsigned long long sq = __ldcg(&psq[i]);
+            unsigned long long key = kNoKey, sq;
             if (two_pass) {
-                if (!(s_fl[i] & F_OPEN)) sq = __ldcg(&a.pos_lo[base + i]);
+                if (s_fl[i] & F_OPEN) sq = __ldcg(&psq[i]);
+                else sq = i == tid ? lo0 : __ldcg(&a.pos_lo[base + i]);
                 a.pos_lo[base + i] = 0;
+            } else {
+                sq = i == tid ? lo0 : psq[i];
             }
             psq[i] = 0;
             uint8_t fl = m ? F_MASKED : 0;
@@ -244,11 +242,11 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 if (conf_exceeds(sq, p.tau_min_conf)) r.max_above = max(r.max_above, i);
                 if (conf_exceeds(sq, p.tau_high_conf)) { fl |= F_HIGH; r.n_high++; }
             }
-            kmin = min(kmin, key);
+            r.kmin = min(r.kmin, key);
             r.n_masked += m ? 1 : 0;
             s_keys[i] = key; s_fl[i] = fl;
         }
-        r = block_reduce(r, s_tmp);
+        r = block_reduce(r, s_tmp, s_min);
 
         if (r.missing > 0 || (r.n_cand == 0 && !vanilla)) {
             // a needed row was not supplied (or the state is inconsistent): report, change nothing
@@ -262,54 +260,30 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 mode = MODE_TOPK; k_top = (int)max(0ll, target - (Lb - r.n_cand));
             } else if (p.sampler == SFS_SAMPLER_RANDOM) mode = MODE_RANDOM;
             else if (forced) mode = MODE_ALL;
-            else if (st.phase == SFS_PHASE_SLOW) { mode = MODE_TOPK; k_top = p.k_slow; }
+            else if (phase0 == SFS_PHASE_SLOW) { mode = MODE_TOPK; k_top = p.k_slow; }
             else if (r.n_high >= p.min_high_count) mode = MODE_HIGH;
             else { mode = MODE_TOPK; k_top = p.k_fast; }
 
-            // ---- choose
-            const bool ranked = mode == MODE_TOPK && k_top > 1 && k_top < r.n_cand;      // (one or all: no ranking)
-            const unsigned long long top1 = (mode == MODE_TOPK && k_top == 1) ? block_min_u64(kmin, s_min) : 0ull;
-            int my_sel = 0;
-            for (int i = tid; i < L; i += kSelThreads) {
-                const unsigned long long key = s_keys[i];
-                if (key == kNoKey) continue;
-                bool sel;
-                if (mode == MODE_ALL) sel = true;
-                else if (mode == MODE_HIGH) sel = (s_fl[i] & F_HIGH) != 0;
-                else if (mode == MODE_RANDOM)
-                    sel = (unsigned long long)philox_first_word((uint32_t)i, (uint32_t)st.steps_done, (uint32_t)b, 0u, p.seed_lo, p.seed_hi)
-                          * (unsigned long long)blk.k_b < (1ull << 32);
-                else if (k_top == 1) sel = key == top1;
-                else if (!ranked) sel = k_top > 0;
-                else {
-                    int rank = 0;                           // candidates that are more confident (ties: smaller position)
-                    for (int j = 0; j < L; ++j) rank += (s_keys[j] < key) ? 1 : 0;
-                    sel = rank < k_top;
-                }
-                if (sel) { s_fl[i] = (uint8_t)((s_fl[i] | F_SEL) & ~F_MASKED); my_sel++; tok[i] = parg[i]; msk[i] = 0; }
-            }
-            n_sel = block_sum(my_sel, s_tmp);
-
-            // ---- scheduler state (Algorithm 1), one thread
+            // ---- scheduler state (Algorithm 1), one thread: what does not depend on the choice
             if (tid == 0) {
-                st.n_masked = r.n_masked - n_sel;
                 st.steps_done++;
                 if (vanilla) {
                     st.k_remaining--;
                 } else if (forced) {
                     st.k_remaining = 0;
-                } else if (st.phase == SFS_PHASE_SLOW) {
+                } else if (phase0 == SFS_PHASE_SLOW) {
                     e_cand = (r.max_above >= 0) ? r.max_above : r.min_cand;
                     if (st.hist_len < p.w_hist) st.hist[st.hist_len++] = e_cand;
                     else { for (int h = 1; h < p.w_hist; ++h) st.hist[h - 1] = st.hist[h]; st.hist[p.w_hist - 1] = e_cand; }
                     st.k_remaining--; st.step_count++; st.n_slow++;
-                    long long sum = 0, sum2 = 0;
+                    int sum = 0;                                          // (at most 8 positions below 2^17)
+                    long long sum2 = 0;
                     for (int h = 0; h < st.hist_len; ++h) { sum += st.hist[h]; sum2 += (long long)st.hist[h] * st.hist[h]; }
-                    const long long n = st.hist_len;
-                    const long long num = n * sum2 - sum * sum;           // n^2 * population variance, exact
-                    if (st.hist_len >= p.w_hist && (double)num < (double)p.sigma2_stable * (double)(n * n)) {
+                    const int n = st.hist_len;
+                    const long long num = n * sum2 - (long long)sum * sum;               // n^2 * population variance, exact
+                    if (n >= p.w_hist && (double)num < (double)p.sigma2_stable * (double)((long long)n * n)) {
                         stable = 1;
-                        st.phase = SFS_PHASE_FAST; st.hi = (int)(sum / n) + 1;   // floor(mean(H_W)) + 1
+                        st.phase = SFS_PHASE_FAST; st.hi = sum / n + 1;   // floor(mean(H_W)) + 1
                     } else if (st.step_count >= p.k_max) {
                         st.phase = SFS_PHASE_FAST; st.hi = e_cand + 1;
                     }
@@ -319,19 +293,49 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 }
             }
             __syncthreads();
+            // is the span clean after this step?  (decides whether the next cycle starts)
+            const bool span = !vanilla && !forced && st.phase == SFS_PHASE_FAST;
+            const int span_hi = st.hi;
 
-            // ---- is the span clean?  (decides whether the next cycle starts)
-            if (!vanilla && !forced && st.phase == SFS_PHASE_FAST) {
-                int cnt = 0;
-                for (int i = st.s_cycle + tid; i < st.hi && i < L; i += kSelThreads) cnt += (s_fl[i] & F_MASKED) ? 1 : 0;
-                cnt = block_sum(cnt, s_tmp);
-                if (tid == 0 && cnt == 0 && st.n_masked > 0) {
+            // ---- choose
+            const bool ranked = mode == MODE_TOPK && k_top > 1 && k_top < r.n_cand;      // (one or all: no ranking)
+            int my_sel = 0, my_left = 0;
+            for (int i = tid; i < L; i += kSelThreads) {
+                const unsigned long long key = s_keys[i];
+                uint8_t fl = s_fl[i];
+                bool sel = false;
+                if (key != kNoKey) {
+                    if (mode == MODE_ALL) sel = true;
+                    else if (mode == MODE_HIGH) sel = (fl & F_HIGH) != 0;
+                    else if (mode == MODE_RANDOM)
+                        sel = (unsigned long long)philox_first_word((uint32_t)i, (uint32_t)steps0, (uint32_t)b, 0u, p.seed_lo, p.seed_hi)
+                              * (unsigned long long)blk.k_b < (1ull << 32);
+                    else if (k_top == 1) sel = key == r.kmin;
+                    else if (!ranked) sel = k_top > 0;
+                    else {
+                        int rank = 0;                           // candidates that are more confident (ties: smaller position)
+                        for (int j = 0; j < L; ++j) rank += (s_keys[j] < key) ? 1 : 0;
+                        sel = rank < k_top;
+                    }
+                }
+                if (sel) { fl = (uint8_t)((fl | F_SEL) & ~F_MASKED); s_fl[i] = fl; my_sel++; tok[i] = i == tid ? arg0 : parg[i]; msk[i] = 0; }
+                if ((fl & F_MASKED) && i >= s0 && i < span_hi) my_left++;
+            }
+            my_sel = warp_sum_i32(my_sel); my_left = warp_sum_i32(my_left);
+            if (lane == 0) { s_tmp[2 * warp] = my_sel; s_tmp[2 * warp + 1] = my_left; }
+            __syncthreads();
+            if (tid == 0) {
+                int left = 0;
+#pragma unroll
+                for (int w = 0; w < kSelThreads / 32; ++w) { n_sel += s_tmp[2 * w]; left += s_tmp[2 * w + 1]; }
+                st.n_masked = r.n_masked - n_sel;
+                if (span && left == 0 && st.n_masked > 0) {
                     st.s_cycle = st.hi; st.phase = SFS_PHASE_SLOW; st.hist_len = 0; st.step_count = 0; st.n_cycles++;
                 }
-            }
-            if (tid == 0 && (st.n_masked == 0 || st.k_remaining == 0)) {
-                st.done = 1;
-                if (st.n_masked > 0) st.status = SFS_ERR_STEP_LIMIT;
+                if (st.n_masked == 0 || st.k_remaining == 0) {
+                    st.done = 1;
+                    if (st.n_masked > 0) st.status = SFS_ERR_STEP_LIMIT;
+                }
             }
         }
     } else {
@@ -345,7 +349,8 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     {
         const bool next_active = !st.done && st.status == SFS_OK;
         const bool nforced = !vanilla && st.k_remaining == 1;
-        const BlockStep nblk = block_step(p, L, st.steps_done);
+        BlockStep nblk{};
+        if (vanilla) nblk = block_step(p, L, st.steps_done);
         const int nlo = vanilla ? nblk.lo : (nforced ? 0 : st.s_cycle);
         const int nhi = vanilla ? nblk.hi : (nforced ? L : ((st.phase == SFS_PHASE_SLOW) ? L : st.hi));
         // a single sequence's list is the whole list
@@ -365,7 +370,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             if (sel && a.sel_pos) {
                 const int o = n_out + (before & 0xFFFF) + __popc(bs & lt);
                 a.sel_pos[(long long)b * L + o] = i;
-                a.sel_tok[(long long)b * L + o] = parg[i];
+                a.sel_tok[(long long)b * L + o] = i == tid ? arg0 : parg[i];
             }
             if (need && next) next[n_next + (before >> 16) + __popc(bn & lt)] = b * S + P + i;
             n_out += total & 0xFFFF; n_next += total >> 16;
