@@ -107,6 +107,15 @@ static int32_t session_alloc_select(sfs_session *s)
     return SFS_OK;
 }
 
+// a projection by model weights (constant while the model is in use, so a kernel may request them early)
+template <typename... Args>
+static int32_t weight_plan_create(GemmPlan *p, Args... args)
+{
+    const int32_t rc = gemm_plan_create(p, args...);
+    p->args.b_static = 1;
+    return rc;
+}
+
 // (re)build the GEMM / attention plans of a model session for B sequences of S tokens
 static int32_t session_plan(sfs_session *s, int32_t B, int32_t S)
 {
@@ -121,17 +130,17 @@ static int32_t session_plan(sfs_session *s, int32_t B, int32_t S)
         LayerPlans &lp = s->layer_plans[l];
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
         // q | k go row-major into qk [T, 2d]; the v columns (>= 2d) go transposed into vt [d, T]
-        rc = gemm_plan_create(&lp.qkv, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
+        rc = weight_plan_create(&lp.qkv, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
-        rc = gemm_plan_create(&lp.o, s->attn, d, T, d, wo, 1, d, d, GEMM_RESIDUAL_F32, s->x, d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&lp.o, s->attn, d, T, d, wo, 1, d, d, GEMM_RESIDUAL_F32, s->x, d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         if ((rc = gemm_plan_enable_split(&lp.o, s->partial, kMaxSplits, nullptr)) != SFS_OK) return rc;
         const void *gu[2] = {m->w_gate[l], m->w_up[l]};
-        rc = gemm_plan_create(&lp.gate_up, s->h, d, T, d, gu, 2, ff, d, GEMM_SWIGLU, s->hid, ff, 0, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&lp.gate_up, s->h, d, T, d, gu, 2, ff, d, GEMM_SWIGLU, s->hid, ff, 0, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wd[1] = {m->w_down[l]};
-        rc = gemm_plan_create(&lp.down, s->hid, ff, T, ff, wd, 1, d, ff, GEMM_RESIDUAL_F32, s->x, d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&lp.down, s->hid, ff, T, ff, wd, 1, d, ff, GEMM_RESIDUAL_F32, s->x, d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         if ((rc = gemm_plan_enable_split(&lp.down, s->partial, kMaxSplits, nullptr)) != SFS_OK) return rc;
     }
@@ -203,14 +212,14 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
         // fresh values of the candidate rows, written transposed (every output column goes through the transposed store): the
         // response rows of a single sequence are one contiguous range; with several sequences every row is projected
         const int v_first = (B == 1) ? P : 0, v_rows = (B == 1) ? S - P : T;
-        rc = gemm_plan_create(&cp.vproj, s->h + (size_t)v_first * d, d, v_rows, d, wv, 1, d, d, GEMM_STORE, s->attn, d, 0, 1.0f, s->vnew_t + v_first, T, 0,
+        rc = weight_plan_create(&cp.vproj, s->h + (size_t)v_first * d, d, v_rows, d, wv, 1, d, d, GEMM_STORE, s->attn, d, 0, 1.0f, s->vnew_t + v_first, T, 0,
                               nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
-        rc = gemm_plan_create(&cp.o_store, s->attn, d, T, d, wo, 1, d, d, GEMM_STORE, s->Ac[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&cp.o_store, s->attn, d, T, d, wo, 1, d, d, GEMM_STORE, s->Ac[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wd[1] = {m->w_down[l]};
-        rc = gemm_plan_create(&cp.down_store, s->hid, ff, T, ff, wd, 1, d, ff, GEMM_STORE, s->Fc[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&cp.down_store, s->hid, ff, T, ff, wd, 1, d, ff, GEMM_STORE, s->Fc[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         rc = attn_plan_create_split(&cp.attn, s->qk, 2 * d, s->Kc[l], d, d, 0, s->Vtc[l], T, s->attn, d, B, S, c.n_heads, c.head_dim);
         if (rc != SFS_OK) return rc;
@@ -231,17 +240,17 @@ static int32_t gather_plan(sfs_session *s, int32_t NR, int32_t T, std::vector<Ga
     for (int l = 0; l < c.n_layers; ++l) {
         GatherLayerPlans &gp = v[l];
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
-        rc = gemm_plan_create(&gp.qkv, s->hg, d, NR, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
+        rc = weight_plan_create(&gp.qkv, s->hg, d, NR, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
-        rc = gemm_plan_create(&gp.o, s->attn, d, NR, d, wo, 1, d, d, GEMM_STORE, s->partial, d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&gp.o, s->attn, d, NR, d, wo, 1, d, d, GEMM_STORE, s->partial, d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         if ((rc = gemm_plan_enable_split(&gp.o, s->partial, kMaxSplits, nullptr)) != SFS_OK) return rc;   // few rows: K is split
         const void *gu[2] = {m->w_gate[l], m->w_up[l]};
-        rc = gemm_plan_create(&gp.gate_up, s->hg, d, NR, d, gu, 2, ff, d, GEMM_SWIGLU, s->hid, ff, 0, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&gp.gate_up, s->hg, d, NR, d, gu, 2, ff, d, GEMM_SWIGLU, s->hid, ff, 0, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wd[1] = {m->w_down[l]};
-        rc = gemm_plan_create(&gp.down, s->hid, ff, NR, ff, wd, 1, d, ff, GEMM_STORE, s->partial, d, 1, 1.0f, nullptr, 0, 0, nullptr);
+        rc = weight_plan_create(&gp.down, s->hid, ff, NR, ff, wd, 1, d, ff, GEMM_STORE, s->partial, d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         if ((rc = gemm_plan_enable_split(&gp.down, s->partial, kMaxSplits, nullptr)) != SFS_OK) return rc;
     }
@@ -560,7 +569,7 @@ int32_t sfs_forward(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t 
     if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, d_rows, d_n_rows, max_rows, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
     GemmPlan lm;
     const void *lmw[1] = {s->model->lm_head};
-    rc = gemm_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
+    rc = weight_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
                           logits_dtype == SFS_LOGITS_F32 ? 1 : 0, c.logit_scale, nullptr, 0, 0, nullptr);
     if (rc != SFS_OK) return rc;
     return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(lm, d_n_rows, nullptr, device_status_word(), st); });
@@ -694,7 +703,7 @@ int32_t sfs_forward_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, i
     if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, d_rows, d_n_rows, max_rows, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
     GemmPlan lm;
     const void *lmw[1] = {s->model->lm_head};
-    rc = gemm_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
+    rc = weight_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
                           logits_dtype == SFS_LOGITS_F32 ? 1 : 0, c.logit_scale, nullptr, 0, 0, nullptr);
     if (rc != SFS_OK) return rc;
     return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(lm, d_n_rows, nullptr, device_status_word(), st); });
@@ -716,7 +725,7 @@ int32_t sfs_generate_begin(sfs_session *s, const int32_t *d_prompt, int32_t B, i
     {   // the LM head sees at most B * gen_len rows: plan it for that many, not for all B * S tokens
         const sfs_config &c = s->model->cfg;
         const void *lm[1] = {s->model->lm_head};
-        rc = gemm_plan_create(&s->lm_plan, s->hfin, c.d_model, B * gen_len, c.d_model, lm, 1, c.vocab, c.d_model, GEMM_STORE,
+        rc = weight_plan_create(&s->lm_plan, s->hfin, c.d_model, B * gen_len, c.d_model, lm, 1, c.vocab, c.d_model, GEMM_STORE,
                               s->logits, c.vocab, 0, c.logit_scale, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         // Long bf16 rows: the LM head takes the first pass of the row statistics in its epilogue (one record per row,

@@ -29,6 +29,7 @@ struct GemmArgs {
     int n_col_tiles;         // column tiles over all B matrices
     int splits, kb_per_split;        // split-K: the k-blocks are cut into `splits` ranges, range s writes slab s of C
     long long split_stride;          // elements between slabs
+    int b_static;            // 1: B is a model weight, which no kernel in flight writes: it may be read before the dependent-launch wait
     int acc_bufs;            // accumulator buffers in tensor memory (2 when they fit: epilogue overlaps the next tile)
     // Optional (GEMM_STORE, bf16 output, no split): row statistics of the stored values, taken in the epilogue.  Per output
     // row, column tile (few rows: N-block and column half of it) and epilogue-warp parity one record (maximum, reference, sum

@@ -89,19 +89,29 @@ struct TileCoord {
 __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int m_groups)
 {
     TileCoord t;
-    const int rest = tile / m_groups;
-    t.m0 = (tile - rest * m_groups) * g.tile_rows;         // row groups fastest: pairs that share a weight tile run together
-    const int n_tile = rest / g.splits;
+    // row groups fastest: pairs that share a weight tile run together (divisions only where there is something to divide)
+    const int rest = m_groups == 1 ? tile : tile / m_groups;
+    t.m0 = (tile - rest * m_groups) * g.tile_rows;
+    const int n_tile = g.splits == 1 ? rest : rest / g.splits;
     t.split = rest - n_tile * g.splits;
     if (g.mode == GEMM_SWIGLU) {
         t.map_idx = 0; t.n_local = n_tile * g.tile_cols; t.ncol0 = t.n_local; t.ncols = min(g.tile_cols, g.N - t.ncol0);
     } else {
-        t.map_idx = n_tile / g.tiles_per_map;
+        t.map_idx = (n_tile >= g.tiles_per_map ? 1 : 0) + (n_tile >= 2 * g.tiles_per_map ? 1 : 0);      // at most three matrices
         t.n_local = (n_tile - t.map_idx * g.tiles_per_map) * g.tile_cols;
         t.ncol0 = t.map_idx * g.n_per_map + t.n_local;
         t.ncols = min(g.tile_cols, g.n_per_map - t.n_local);
     }
     return t;
+}
+
+// k-blocks of the pair's first tile whose weights are requested before the dependent-launch wait
+__device__ __forceinline__ int early_weights(const GemmArgs &g, int pair, int stages)
+{
+    const int num_kb = (g.K + BK - 1) / BK;
+    if (g.splits == 1) return min(stages, num_kb);
+    const int kb0 = tile_coord(g, pair, (g.M + g.tile_rows - 1) / g.tile_rows).split * g.kb_per_split;
+    return min(stages, min(num_kb, kb0 + g.kb_per_split) - kb0);
 }
 
 // ---- epilogue --------------------------------------------------------------------------------------------
@@ -163,7 +173,7 @@ struct EpiShare {
     uint32_t up;                 // SwiGLU: columns from a gate accumulator to its up accumulator
     int row0, row_block;         // output row of lane 0 in block 0, rows between blocks
     int col0, col_block;         // output column of the first accumulator column in block 0, columns between blocks
-    int blocks, seg;             // number of blocks, accumulator columns of each that may be valid
+    int blocks, seg;             // number of blocks (1 or 2), accumulator columns of each that may be valid
     int col_end;                 // columns at or beyond this belong to another tile or matrix
     int rec, rec_block;          // fused row statistics: record of block 0, records between blocks
     __device__ __forceinline__ int lim(int b) const { return min(col_end, col0 + b * col_block + seg); }
@@ -183,7 +193,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
         const int upb = (e.seg + 63) / 64;                                // units per block
         const int n_pieces = 2 * ((e.blocks * upb - par + 1) / 2);
         auto piece_addr = [&](int pc) {                                   // tensor-memory column of piece pc
-            const int u = par + 2 * (pc >> 1), b = u / upb, c = 64 * (u - b * upb);
+            const int u = par + 2 * (pc >> 1), b = u >= upb ? 1 : 0, c = 64 * (u - b * upb);
             return e.tmem + (uint32_t)b * e.tmem_block + (uint32_t)(c + 32 * (pc & 1));
         };
         uint32_t x0[32], x1[32];
@@ -201,7 +211,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
             if (grow < M) g.stats[(long long)grow * g.stats_ld + e.rec + st_b * e.rec_block + par] = make_float4(st_mx, st_ref, st_sum, __int_as_float(st_arg));
         };
         for (int pc = 0; pc < n_pieces; ++pc) {
-            const int u = par + 2 * (pc >> 1), b = u / upb, col0 = e.col0 + b * e.col_block + 64 * (u - b * upb);
+            const int u = par + 2 * (pc >> 1), b = u >= upb ? 1 : 0, col0 = e.col0 + b * e.col_block + 64 * (u - b * upb);
             uint32_t o[16];
             tc::tmem_ld_wait32(x0);
             if (swiglu) tc::tmem_ld_wait32(x1);
@@ -266,7 +276,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
         // ---- V columns of the QKV projection go out transposed: the 32 lanes hold 32 consecutive tokens of a feature
         const int upb = (e.seg + 31) / 32;
         const int n_pieces = (e.blocks * upb - par + 1) / 2;
-        auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u / upb; return 32 * (u - *b * upb); };
+        auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u >= upb ? 1 : 0; return 32 * (u - *b * upb); };
         uint32_t v[32];
         int b0;
         if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(e.tmem + (uint32_t)b0 * e.tmem_block + (uint32_t)c, v); }
@@ -291,7 +301,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
         // ---- fp32 output (residual add, split-K slab, or fp32 logits): units of 32 columns
         const int upb = (e.seg + 31) / 32;
         const int n_pieces = (e.blocks * upb - par + 1) / 2;
-        auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u / upb; return 32 * (u - *b * upb); };
+        auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u >= upb ? 1 : 0; return 32 * (u - *b * upb); };
         const bool scale = (g.mode != GEMM_RESIDUAL_F32 && g.scale != 1.0f);
         uint32_t v[32];
         int b0;
@@ -366,6 +376,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const uint32_t n_bufs = (uint32_t)g.acc_bufs, buf_stride = 256;     // two buffers only when MB * bn_pad <= 256
     const bool swiglu = (g.mode == GEMM_SWIGLU);
 
+    // Model weights do not depend on the kernel before this one: the first tile's weight rows are requested at once, as many
+    // k-blocks as the ring holds; their activation rows follow after the wait.
+    const int pre = (g.b_static && g.d_m == nullptr) ? early_weights(g, pair, STAGES) : 0;
+    if (warp == 0 && pre > 0) {
+        const TileCoord t = tile_coord(g, pair, (g.M + MB * 2 * BM - 1) / (MB * 2 * BM));
+        const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1) : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
+        const int brow = swiglu ? t.n_local : t.n_local + (int)rank * HALF, kb0 = t.split * g.kb_per_split;
+        for (int j = 0; j < pre; ++j) {
+            if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)STAGE_BYTES);
+            tc::tma_load_2d_2cta_elect(smem_base + j * STAGE_BYTES + MB * A_BYTES, mb, (kb0 + j) * BK, brow, lead_full + 8 * j);
+        }
+    }
     pdl_wait();                                             // the kernel before this one has completed: global memory from here on
     // nothing left to decode, or fewer rows than planned: the loops below find no tile (same values in both CTAs of the pair)
     const bool live = !(g.d_active && *g.d_active == 0);
@@ -399,12 +421,25 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
-                if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
+                const bool early = it < (uint32_t)pre;
+                if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 if (MB == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
-                tc::tma_load_2d_2cta_elect(sa + MB * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
+                if (!early) tc::tma_load_2d_2cta_elect(sa + MB * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
             }
         }
+        if (!live && pre > 0) {
+            // nothing left to decode: the stages requested above are completed and awaited, nobody reads them
+            for (int j = 0; j < pre; ++j) {
+                const uint32_t sa = smem_base + j * STAGE_BYTES;
+                tc::tma_load_2d_2cta_elect(sa, &tmA, 0, 0, lead_full + 8 * j);
+                if (MB == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, 0, 0, lead_full + 8 * j);
+            }
+            if (rank == 0) for (int j = 0; j < pre && tc::mbar_wait(bar_full + 8 * j, 0u, &s_abort); ++j) {}
+        }
+        // every stage has been released (by both CTAs' MMAs): no signal of the tensor core is on its way to this CTA when it leaves
+        if (ok)
+            for (uint32_t j = it > (uint32_t)STAGES ? it - (uint32_t)STAGES : 0u; j < it && tc::mbar_wait(bar_empty + 8 * (j % (uint32_t)STAGES), (j / (uint32_t)STAGES) & 1u, &s_abort); ++j) {}
         if (s_abort && rank == 0 && lane == 0) {
             // give copies already in flight (both CTAs') a bounded chance to land before the pair retires
             const uint32_t first = it > (uint32_t)STAGES ? it - (uint32_t)STAGES : 0u;
@@ -474,14 +509,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
+            if (lane == 0 && tile + (int)n_bufs * num_pairs < num_tiles) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);     // (if it is used again)
         }
     }
 
     // ---------------- teardown: no CTA of the pair leaves while the other may still signal its barriers
+    // (whatever one CTA signals the other has been waited for by then, unless a wait gave up: the barrier orders execution only)
     __syncwarp();                                           // the diverged roles rejoin their warps
     tc::tc_fence_before();
-    tc::cluster_sync();
+    if (s_abort) tc::cluster_sync(); else tc::cluster_sync_relaxed();
     if (warp == 1) { tc::tc_fence_after(); tc::tmem_dealloc_2cta(tmem_base, kTmemCols); }
     if (threadIdx.x == 0 && s_abort && g.err) atomicExch(g.err, SFS_ERR_TIMEOUT);
 }
@@ -540,6 +576,20 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
     const bool swiglu = (g.mode == GEMM_SWIGLU);
 
+    // the first tile's weight rows are requested before the wait (see the pair kernel)
+    const int pre = (g.b_static && g.d_m == nullptr) ? early_weights(g, pair, STAGES) : 0;
+    if (warp == 0 && pre > 0) {
+        const TileCoord t = tile_coord(g, pair, (g.M + 2 * FM - 1) / (2 * FM));
+        const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
+        const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
+        const int brow0 = t.n_local + (int)rank * HALF, brow1 = swiglu ? brow0 : brow0 + BN, kb0 = t.split * g.kb_per_split;
+        for (int j = 0; j < pre; ++j) {
+            const uint32_t sa = smem_base + j * STAGE_BYTES;
+            if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)STAGE_BYTES);
+            tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, (kb0 + j) * BK, brow0, lead_full + 8 * j);
+            if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, (kb0 + j) * BK, brow1, lead_full + 8 * j);
+        }
+    }
     pdl_wait();                                             // the kernel before this one has completed: global memory from here on
     const bool live = !(g.d_active && *g.d_active == 0);    // nothing left to decode: the loops below find no tile
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
@@ -565,13 +615,23 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint32_t ns = s + 1u == (uint32_t)STAGES ? 0u : s + 1u, nph = ns == 0u ? ph ^ 1u : ph;
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
-                if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
-                tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, kb * BK, brow0, lead_full + 8 * s);
-                if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, kb * BK, brow1, lead_full + 8 * s);
+                if (it >= (uint32_t)pre) {
+                    if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
+                    tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, kb * BK, brow0, lead_full + 8 * s);
+                    if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, kb * BK, brow1, lead_full + 8 * s);
+                }
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 s = ns; ph = nph;
             }
         }
+        if (!live && pre > 0) {
+            // nothing left to decode: the stages requested above are completed and awaited, nobody reads them
+            for (int j = 0; j < pre; ++j) tc::tma_load_2d_2cta_elect(smem_base + j * STAGE_BYTES, &tmA, 0, 0, lead_full + 8 * j);
+            if (rank == 0) for (int j = 0; j < pre && tc::mbar_wait(bar_full + 8 * j, 0u, &s_abort); ++j) {}
+        }
+        // every stage has been released (by both CTAs' MMAs): no signal of the tensor core is on its way to this CTA when it leaves
+        if (ok)
+            for (uint32_t j = it > (uint32_t)STAGES ? it - (uint32_t)STAGES : 0u; j < it && tc::mbar_wait(bar_empty + 8 * (j % (uint32_t)STAGES), (j / (uint32_t)STAGES) & 1u, &s_abort); ++j) {}
         if (s_abort && rank == 0 && lane == 0) {
             // give copies already in flight (both CTAs') a bounded chance to land before the pair retires
             const uint32_t first = it > (uint32_t)STAGES ? it - (uint32_t)STAGES : 0u;
@@ -641,14 +701,14 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
+            if (lane == 0 && tile + 2 * num_pairs < num_tiles) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
         }
     }
 
     // ---------------- teardown: no CTA of the pair leaves while the other may still signal its barriers
     __syncwarp();
     tc::tc_fence_before();
-    tc::cluster_sync();
+    if (s_abort) tc::cluster_sync(); else tc::cluster_sync_relaxed();
     if (warp == 1) { tc::tc_fence_after(); tc::tmem_dealloc_2cta(tmem_base, kTmemCols); }
     if (threadIdx.x == 0 && s_abort && g.err) atomicExch(g.err, SFS_ERR_TIMEOUT);
 }
@@ -830,6 +890,7 @@ int32_t gemm_plan_enable_split(GemmPlan *p, float *ws, int32_t max_splits, const
     int32_t rc = gemm_plan_create(&q, p->A, p->lda, g.M, g.K, p->Bs, p->n_maps, p->n_per_map, p->ldb, g.mode, g.C, g.ldc, g.out_f32,
                                   g.scale, g.vt, g.ldvt, g.vt_col0, &t2);
     if (rc != SFS_OK) return rc;
+    q.args.b_static = g.b_static;
     *p = q;
     GemmArgs &h = p->args;
     const int num_kb = (h.K + BK - 1) / BK;
