@@ -107,6 +107,12 @@ static int32_t session_alloc_select(sfs_session *s)
     return SFS_OK;
 }
 
+static void drop_graphs(sfs_session *s)
+{
+    for (auto &kv : s->graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+    s->graphs.clear();
+}
+
 // a projection by model weights (constant while the model is in use, so a kernel may request them early)
 template <typename... Args>
 static int32_t weight_plan_create(GemmPlan *p, Args... args)
@@ -124,6 +130,8 @@ static int32_t session_plan(sfs_session *s, int32_t B, int32_t S)
     const sfs_config &c = m->cfg;
     const int T = B * S, d = c.d_model, ff = c.d_ff;
     SFS_REQUIRE((S % 8) == 0, SFS_ERR_UNSUPPORTED, "sequence length %d must be a multiple of 8", S);
+    drop_graphs(s);
+    s->plan_B = s->plan_S = 0;
     s->layer_plans.resize(c.n_layers);
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
@@ -165,6 +173,39 @@ static int32_t timed_launch(sfs_session *s, int cls, cudaStream_t st, F &&f)
     return rc;
 }
 
+// Runs a body that reads and writes session buffers only.  Its launches are the same each time for the same plans, so from the
+// kGraphAfter-th time on they are one graph launch: a body of small kernels is bound by enqueueing them (18 launches of a tiny
+// step: 80 to 160 us of host time, by the host), and between two nodes of a graph the device loses less than between two launches
+// (8 layers at 104 rows 1184 -> 1137 us).  Recording and instantiating costs 1 to 3 ms, which a session that runs a few steps
+// does not get back.  The graph belongs to the session and its plans; a caller's own stream capture gets the plain launches.
+constexpr int kGraphAfter = 16;
+template <typename F>
+static int32_t run_recorded(sfs_session *s, long long key, cudaStream_t st, F &&enqueue)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (s->profile || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return enqueue(st);
+    BodyGraph &g = s->graphs[key];
+    if (g.exec == nullptr) {
+        if (g.uses < 0 || ++g.uses < kGraphAfter) return enqueue(st);
+        g.uses = -1;                                        // one attempt: if it fails the launches stay plain
+        if (s->record_stream == nullptr && cudaStreamCreateWithFlags(&s->record_stream, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
+        if (cudaStreamBeginCapture(s->record_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
+        const long long before = s->launches;
+        const int32_t rc = enqueue(s->record_stream);
+        g.kernels = s->launches - before;
+        s->launches = before;
+        cudaGraph_t graph = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(s->record_stream, &graph);
+        if (rc != SFS_OK || e != cudaSuccess || cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) g.exec = nullptr;
+        if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();
+        if (g.exec == nullptr) return enqueue(st);
+    }
+    SFS_CUDA(cudaGraphLaunch(g.exec, st));
+    s->launches += g.kernels;
+    return SFS_OK;
+}
+
 // the transformer body: tokens -> residual stream x [T, d]
 static int32_t run_body(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, const int32_t *d_active, cudaStream_t st)
 {
@@ -174,23 +215,30 @@ static int32_t run_body(sfs_session *s, const int32_t *d_tokens, int32_t B, int3
     int32_t *err = device_status_word();
     SFS_REQUIRE(err != nullptr, SFS_ERR_OOM, "cannot allocate the device status word");
     int32_t rc;
-    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed_norm(d_tokens, m->tok_emb, c.vocab, s->x, m->attn_norm[0], s->h, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
+    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed_norm(d_tokens, m->tok_emb, c.vocab, s->x, m->attn_norm[0], s->h, T, d, c.rms_eps, nullptr, nullptr, 0, st); })) != SFS_OK) return rc;
     // A split-K projection leaves its partial products in s->partial; the next RMSNorm folds them into x.
     const long long pstride = (long long)T * d;
-    int pending = 0;
-    for (int l = 0; l < c.n_layers; ++l) {
-        const LayerPlans &lp = s->layer_plans[l];
-        if (l > 0 && (rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->attn_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(lp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-        pending = lp.o.args.splits > 1 ? lp.o.args.splits : 0;
-        if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->mlp_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(lp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(lp.down, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-        pending = lp.down.args.splits > 1 ? lp.down.args.splits : 0;
-    }
+    rc = run_recorded(s, d_active ? 1 : 0, st, [&](cudaStream_t st) -> int32_t {
+        int32_t rc;
+        int pending = 0;
+        for (int l = 0; l < c.n_layers; ++l) {
+            const LayerPlans &lp = s->layer_plans[l];
+            if (l > 0 && (rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->attn_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(lp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+            pending = lp.o.args.splits > 1 ? lp.o.args.splits : 0;
+            if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->mlp_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(lp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(lp.down, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+            pending = lp.down.args.splits > 1 ? lp.down.args.splits : 0;
+        }
+        return SFS_OK;
+    });
+    if (rc != SFS_OK) return rc;
+    const LayerPlans &last = s->layer_plans[c.n_layers - 1];
+    const int pending = last.down.args.splits > 1 ? last.down.args.splits : 0;
     s->pending_ptr = s->partial; s->pending_n = pending; s->pending_stride = pstride;      // for the final RMSNorm of the caller
     return SFS_OK;
 }
@@ -203,6 +251,7 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
     const sfs_config &c = m->cfg;
     const int T = B * S, d = c.d_model, ff = c.d_ff;
     if ((int)s->cache_plans.size() == c.n_layers && s->cache_B == B && s->cache_S == S && s->cache_P == P) return SFS_OK;
+    drop_graphs(s);
     s->cache_plans.assign(c.n_layers, CacheLayerPlans());
     s->gather_plans.clear();
     int32_t rc;
@@ -293,92 +342,103 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
     const int r_first = (B == 1 && !rp) ? P : 0, r_count = (B == 1 && !rp) ? L : T;
     // tokens whose fresh values are compared with the cached ones: the response of a single sequence (from an even index), else all
     const int sim_first = (B == 1) ? (P & ~1) : 0, sim_count = (B == 1) ? S - sim_first : T;
-    // the first layer's norm of those rows embeds their tokens
+    // the first layer's norm of those rows embeds their tokens (and brings the states to where the body expects them)
     rc = timed_launch(s, SFS_K_EMBED, st, [&] {
         return launch_embed_norm(d_tokens + r_first, m->tok_emb, c.vocab, s->x + (size_t)r_first * d, m->attn_norm[0], s->h + (size_t)r_first * d, r_count, d,
-                                 c.rms_eps, st);
+                                 c.rms_eps, reinterpret_cast<const int32_t *>(d_state), reinterpret_cast<int32_t *>(s->state_in),
+                                 d_state ? B * (int)(sizeof(sfs_state) / 4) : 0, st);
     });
     if (rc != SFS_OK) return rc;
-    auto norm_all = [&](const void *gain) {
-        return timed_launch(s, SFS_K_RMSNORM, st, [&] {
-            return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, pend ? 1 : 0, 0, gain,
-                                  s->h + (size_t)r_first * d, nullptr, nullptr, r_count, d, c.rms_eps, st);
-        });
-    };
-    if (rp && rr) {
-        // everything is recomputed: the uncached layer pipeline, with the increments stored instead of added and K / V copied out
-        for (int l = 0; l < c.n_layers; ++l) {
-            const LayerPlans &lp = s->layer_plans[l];
-            const CacheLayerPlans &cl = s->cache_plans[l];
-            if (l > 0 && (rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
-            SFS_CUDA(cudaMemcpy2DAsync(s->Kc[l], (size_t)d * 2, s->qk + d, (size_t)2 * d * 2, (size_t)d * 2, (size_t)T, cudaMemcpyDeviceToDevice, st));
-            SFS_CUDA(cudaMemcpyAsync(s->Vtc[l], s->vt, (size_t)d * T * 2, cudaMemcpyDeviceToDevice, st));
-            if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(cl.o_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-            pend = s->Ac[l];
-            if ((rc = norm_all(m->mlp_norm[l])) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(lp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(cl.down_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-            pend = s->Fc[l];
-            if (d_sets) {   // the dump lists every token
-                CacheSelectArgs a{}; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T; a.refresh_p = 1; a.refresh_r = 1; a.n_sel = S;
-                a.sel_rows = d_sets + (size_t)l * B * S;
-                if ((rc = launch_cache_select(a, st)) != SFS_OK) return rc;
-            }
-        }
-    } else {
-        std::vector<GatherLayerPlans> *gps = nullptr;
-        if (NR > 0 && (rc = gather_plan(s, NR, T, &gps)) != SFS_OK) return rc;
-        // Here the attention increment of a layer stays pending through its MLP branch: the MLP norm reads x + A_l for the
-        // recomputed rows only (straight into the compact buffer), and the next layer's first norm folds A_l and F_l together.
-        const long long inc_stride = (long long)s->max_batch * s->max_seq * d;     // A_l -> F_l
-        int n_pend = 0;
-        for (int l = 0; l < c.n_layers; ++l) {
-            const CacheLayerPlans &cl = s->cache_plans[l];
-            if (l > 0) rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
-                return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, n_pend, inc_stride, m->attn_norm[l],
+    const sfs_state *state = d_state ? s->state_in : nullptr;
+    std::vector<GatherLayerPlans> *gps = nullptr;
+    if (!(rp && rr) && NR > 0 && (rc = gather_plan(s, NR, T, &gps)) != SFS_OK) return rc;
+    const long long inc_stride = (rp && rr) ? 0 : (long long)s->max_batch * s->max_seq * d;     // A_l -> F_l
+    int n_pend = 0;
+    auto body = [&](cudaStream_t st) -> int32_t {
+        int32_t rc = SFS_OK;
+        pend = nullptr; n_pend = 0;
+        auto norm_all = [&](const void *gain) {
+            return timed_launch(s, SFS_K_RMSNORM, st, [&] {
+                return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, pend ? 1 : 0, 0, gain,
                                       s->h + (size_t)r_first * d, nullptr, nullptr, r_count, d, c.rms_eps, st);
             });
-            if (rc != SFS_OK) return rc;
-            if (NR > 0) {
-                const GatherLayerPlans &gp = (*gps)[l];
-                if (!rr && n_adapt > 0) {
-                    if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(cl.vproj, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                    if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_sim_partial(s->vnew_t, s->Vtc[l], T, d, sim_first, sim_count, T, s->sim_partial, st); })) != SFS_OK) return rc;
+        };
+        if (rp && rr) {
+            // everything is recomputed: the uncached layer pipeline, with the increments stored instead of added and K / V copied out
+            for (int l = 0; l < c.n_layers; ++l) {
+                const LayerPlans &lp = s->layer_plans[l];
+                const CacheLayerPlans &cl = s->cache_plans[l];
+                if (l > 0 && (rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
+                SFS_CUDA(cudaMemcpy2DAsync(s->Kc[l], (size_t)d * 2, s->qk + d, (size_t)2 * d * 2, (size_t)d * 2, (size_t)T, cudaMemcpyDeviceToDevice, st));
+                SFS_CUDA(cudaMemcpyAsync(s->Vtc[l], s->vt, (size_t)d * T * 2, cudaMemcpyDeviceToDevice, st));
+                if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(cl.o_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                pend = s->Ac[l];
+                if ((rc = norm_all(m->mlp_norm[l])) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(lp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(cl.down_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                pend = s->Fc[l];
+                if (d_sets) {   // the dump lists every token
+                    CacheSelectArgs a{}; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T; a.refresh_p = 1; a.refresh_r = 1; a.n_sel = S;
+                    a.sel_rows = d_sets + (size_t)l * B * S;
+                    if ((rc = launch_cache_select(a, st)) != SFS_OK) return rc;
                 }
-                CacheSelectArgs a{};
-                a.partial = s->sim_partial; a.state = d_state; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T;
-                a.refresh_p = rp; a.refresh_r = rr; a.n_adapt = rr ? 0 : n_adapt; a.n_sel = n_sel; a.sel_rows = s->sel_rows;
-                a.sims_dump = (d_sims && !rr) ? d_sims + (size_t)l * B * L : nullptr;
-                a.sets_dump = d_sets ? d_sets + (size_t)l * NR : nullptr;
-                if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_cache_select(a, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_gather_rows_bf16(s->h, s->sel_rows, NR, d, s->hg, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(gp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope_scatter_kv(s->qk, 2 * d, NR, S, c.n_heads, c.head_dim, s->rope_table, s->sel_rows, s->Kc[l], s->vt, T, s->Vtc[l], T, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch_queries(cl.attn, n_sel, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(gp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
             }
-            pend = s->Ac[l]; n_pend = 2;
-            if (NR > 0) {
-                const GatherLayerPlans &gp = (*gps)[l];
-                // the O projection's slabs become the attention increments of the recomputed tokens, and the MLP's input rows
-                rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
-                    return launch_fold_norm_rows(s->partial, gp.o.args.splits, gp.o.args.split_stride, s->sel_rows, NR, s->x, s->Ac[l],
-                                                 m->mlp_norm[l], s->hg, d, c.rms_eps, st);
+        } else {
+            // Here the attention increment of a layer stays pending through its MLP branch: the MLP norm reads x + A_l for the
+            // recomputed rows only (straight into the compact buffer), and the next layer's first norm folds A_l and F_l together.
+            for (int l = 0; l < c.n_layers; ++l) {
+                const CacheLayerPlans &cl = s->cache_plans[l];
+                if (l > 0) rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
+                    return launch_rmsnorm(s->x + (size_t)r_first * d, pend ? pend + (size_t)r_first * d : nullptr, n_pend, inc_stride, m->attn_norm[l],
+                                          s->h + (size_t)r_first * d, nullptr, nullptr, r_count, d, c.rms_eps, st);
                 });
                 if (rc != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(gp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(gp.down, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_scatter_rows_f32(s->partial, gp.down.args.splits, gp.down.args.split_stride, s->sel_rows, NR, d, s->Fc[l], st); })) != SFS_OK) return rc;
+                if (NR > 0) {
+                    const GatherLayerPlans &gp = (*gps)[l];
+                    if (!rr && n_adapt > 0) {
+                        if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(cl.vproj, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                        if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_sim_partial(s->vnew_t, s->Vtc[l], T, d, sim_first, sim_count, T, s->sim_partial, st); })) != SFS_OK) return rc;
+                    }
+                    CacheSelectArgs a{};
+                    a.partial = s->sim_partial; a.state = state; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T;
+                    a.refresh_p = rp; a.refresh_r = rr; a.n_adapt = rr ? 0 : n_adapt; a.n_sel = n_sel; a.sel_rows = s->sel_rows;
+                    a.sims_dump = (d_sims && !rr) ? d_sims + (size_t)l * B * L : nullptr;
+                    a.sets_dump = d_sets ? d_sets + (size_t)l * NR : nullptr;
+                    if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_cache_select(a, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_gather_rows_bf16(s->h, s->sel_rows, NR, d, s->hg, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(gp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope_scatter_kv(s->qk, 2 * d, NR, S, c.n_heads, c.head_dim, s->rope_table, s->sel_rows, s->Kc[l], s->vt, T, s->Vtc[l], T, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch_queries(cl.attn, n_sel, d_active, err, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(gp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                }
+                pend = s->Ac[l]; n_pend = 2;
+                if (NR > 0) {
+                    const GatherLayerPlans &gp = (*gps)[l];
+                    // the O projection's slabs become the attention increments of the recomputed tokens, and the MLP's input rows
+                    rc = timed_launch(s, SFS_K_RMSNORM, st, [&] {
+                        return launch_fold_norm_rows(s->partial, gp.o.args.splits, gp.o.args.split_stride, s->sel_rows, NR, s->x, s->Ac[l],
+                                                     m->mlp_norm[l], s->hg, d, c.rms_eps, st);
+                    });
+                    if (rc != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(gp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(gp.down, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                    if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_scatter_rows_f32(s->partial, gp.down.args.splits, gp.down.args.split_stride, s->sel_rows, NR, d, s->Fc[l], st); })) != SFS_OK) return rc;
+                }
             }
         }
-        s->pending_ptr = pend; s->pending_n = pend ? n_pend : 0; s->pending_stride = inc_stride;
-        s->cache_t++;
         return SFS_OK;
-    }
-    s->pending_ptr = pend; s->pending_n = pend ? 1 : 0; s->pending_stride = 0;
+    };
+    // (a dump writes to the caller's buffers: not recorded)
+    const long long key = 2 + ((((long long)n_sel * 2 + rp) * 2 + rr) * 2 + (d_state ? 1 : 0)) * 2 + (d_active ? 1 : 0);
+    if (d_sets || d_sims) rc = body(st);
+    else rc = run_recorded(s, key, st, body);
+    if (rc != SFS_OK) return rc;
+    // what the last layer leaves pending: its MLP increment, or both increments
+    pend = (rp && rr) ? s->Fc[c.n_layers - 1] : s->Ac[c.n_layers - 1];
+    s->pending_ptr = pend; s->pending_n = (rp && rr) ? 1 : 2; s->pending_stride = inc_stride;
     s->cache_t++;
     return SFS_OK;
 }
@@ -483,6 +543,8 @@ int32_t sfs_session_destroy(sfs_session *s)
 {
     if (!s) return SFS_OK;
     cudaDeviceSynchronize();
+    drop_graphs(s);
+    if (s->record_stream) cudaStreamDestroy(s->record_stream);
     for (void *p : s->owned) cudaFree(p);
     if (s->host_active) cudaFreeHost(s->host_active);
     delete s;
@@ -662,6 +724,7 @@ int32_t sfs_cache_enable(sfs_session *s, const sfs_cache_params *p)
         if ((rc = dev_alloc(s, &s->vnew_t, T * d, true)) != SFS_OK) return rc;
         if ((rc = dev_alloc(s, &s->sim_partial, (size_t)kSimSlices * T * 3, true)) != SFS_OK) return rc;
         if ((rc = dev_alloc(s, &s->sel_rows, T, true)) != SFS_OK) return rc;
+        if ((rc = dev_alloc(s, &s->state_in, (size_t)s->max_batch, true)) != SFS_OK) return rc;
         SFS_CUDA(cudaDeviceSynchronize());
     }
     s->cache_params = *p;

@@ -17,11 +17,14 @@ __global__ void __launch_bounds__(NT)
 rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_partial, long long partial_stride,
                const __nv_bfloat16 *__restrict__ gain, __nv_bfloat16 *__restrict__ h,
                const int32_t *__restrict__ rows, const int32_t *__restrict__ n_rows_ptr, int max_rows, int d, float eps,
-               const int32_t *__restrict__ tokens, const __nv_bfloat16 *__restrict__ emb, int vocab)
+               const int32_t *__restrict__ tokens, const __nv_bfloat16 *__restrict__ emb, int vocab, const int32_t *__restrict__ copy_src,
+               int32_t *__restrict__ copy_dst, int copy_n)
 {
     constexpr int kNormThreads = NT;
     pdl_wait();
     pdl_trigger();
+    if (EMBED && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < copy_n; i += kNormThreads) copy_dst[i] = copy_src[i];
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
     __shared__ float s_part[kNormThreads / 32];
     const int chunks = d / 4;
@@ -162,7 +165,8 @@ static int norm_threads(int rows, int d)
 
 template <bool EMBED>
 static int32_t launch_norm(float *x, const float *partial, int n_partial, long long partial_stride, const void *gain, void *h, const int32_t *rows,
-                           const int32_t *n_rows, int max_rows, int d, float eps, const int32_t *tokens, const void *emb, int vocab, cudaStream_t s)
+                           const int32_t *n_rows, int max_rows, int d, float eps, const int32_t *tokens, const void *emb, int vocab, const int32_t *copy_src, int32_t *copy_dst, int copy_n,
+                           cudaStream_t s)
 {
     if (max_rows <= 0) return SFS_OK;
     const int grid = max_rows < 148 * 16 ? max_rows : 148 * 16, nt = norm_threads(max_rows, d);
@@ -170,7 +174,7 @@ static int32_t launch_norm(float *x, const float *partial, int n_partial, long l
     auto go = [&](auto kernel, int threads) {
         return launch_pdl(kernel, dim3(grid), dim3(threads), 0, s, x, partial ? partial : x, n_partial, partial_stride,
                           reinterpret_cast<const __nv_bfloat16 *>(gain), reinterpret_cast<__nv_bfloat16 *>(h), rows, n_rows, max_rows, d, eps, tokens,
-                          reinterpret_cast<const __nv_bfloat16 *>(emb), vocab);
+                          reinterpret_cast<const __nv_bfloat16 *>(emb), vocab, copy_src, copy_dst, copy_n);
     };
     if (nt == 1024) SFS_CUDA(go(rmsnorm_kernel<1024, EMBED>, 1024));
     else if (nt == 512) SFS_CUDA(go(rmsnorm_kernel<512, EMBED>, 512));
@@ -180,15 +184,16 @@ static int32_t launch_norm(float *x, const float *partial, int n_partial, long l
     return SFS_OK;
 }
 
-int32_t launch_embed_norm(const int32_t *tokens, const void *emb, int vocab, float *x, const void *gain, void *h, int T, int d, float eps, cudaStream_t s)
+int32_t launch_embed_norm(const int32_t *tokens, const void *emb, int vocab, float *x, const void *gain, void *h, int T, int d, float eps, const int32_t *copy_src,
+                          int32_t *copy_dst, int copy_n, cudaStream_t s)
 {
-    return launch_norm<true>(x, nullptr, 0, 0, gain, h, nullptr, nullptr, T, d, eps, tokens, emb, vocab, s);
+    return launch_norm<true>(x, nullptr, 0, 0, gain, h, nullptr, nullptr, T, d, eps, tokens, emb, vocab, copy_src, copy_dst, copy_n, s);
 }
 
 int32_t launch_rmsnorm(float *x, const float *partial, int n_partial, long long partial_stride, const void *gain, void *h,
                        const int32_t *rows, const int32_t *n_rows, int max_rows, int d, float eps, cudaStream_t s)
 {
-    return launch_norm<false>(x, partial, n_partial, partial_stride, gain, h, rows, n_rows, max_rows, d, eps, nullptr, nullptr, 0, s);
+    return launch_norm<false>(x, partial, n_partial, partial_stride, gain, h, rows, n_rows, max_rows, d, eps, nullptr, nullptr, 0, nullptr, nullptr, 0, s);
 }
 
 int32_t launch_rope_table(float2 *table, int positions, int head_dim, float theta, cudaStream_t s)

@@ -3,8 +3,10 @@
 #include "sfs_common.cuh"
 
 namespace sfs {
-// the start of a forward pass: x[t,:] = the embedding of tokens[t] as fp32, h[t,:] = bf16(RMSNorm(x[t,:]) * gain) of the first layer
-int32_t launch_embed_norm(const int32_t *tokens, const void *emb, int vocab, float *x, const void *gain, void *h, int T, int d, float eps, cudaStream_t s);
+// the start of a forward pass: x[t,:] = the embedding of tokens[t] as fp32, h[t,:] = bf16(RMSNorm(x[t,:]) * gain) of the first layer;
+// copy_n integers are copied from copy_src to copy_dst on the way
+int32_t launch_embed_norm(const int32_t *tokens, const void *emb, int vocab, float *x, const void *gain, void *h, int T, int d, float eps, const int32_t *copy_src,
+                          int32_t *copy_dst, int copy_n, cudaStream_t s);
 // h[r,:] = bf16(RMSNorm(y[rows ? rows[r] : r, :]) * gain) with y = x + the n_partial slabs of `partial` (partial_stride
 // floats apart, added in slab order; may be NULL).  Without a row list y is written back to x.  The row count may
 // come from the device (n_rows).

@@ -19,6 +19,9 @@ struct CacheLayerPlans { sfs::GemmPlan vproj, o_store, down_store; sfs::AttnPlan
 // cached mode: projections over the compact buffer of recomputed rows, per layer, for one row count
 struct GatherLayerPlans { sfs::GemmPlan qkv, o, gate_up, down; };
 
+// A transformer body as a CUDA graph: recorded once the same body has been run kGraphAfter times, replayed from then on
+struct BodyGraph { cudaGraphExec_t exec = nullptr; int uses = 0; long long kernels = 0; };
+
 struct sfs_session {
     sfs_model *model = nullptr;          // NULL: a selection-only session
     int32_t max_batch = 0, max_seq = 0, vocab = 0;
@@ -57,6 +60,9 @@ struct sfs_session {
     sfs::AttnPlan attn_plan;
     sfs::GemmPlan lm_plan;
     float4 *lm_stats = nullptr; size_t lm_stats_cap = 0;     // row-statistics records the LM head's epilogue leaves (fused first pass)
+    std::map<long long, BodyGraph> graphs;   // by kind of body; dropped with the plans they were recorded from
+    cudaStream_t record_stream = nullptr;    // recording happens here, never on a caller's stream
+    sfs_state *state_in = nullptr;           // [max_batch] the caller's scheduler states, where a recorded body finds them
     // what the next RMSNorm must fold into x: n slabs `pending_stride` floats apart (split-K partials or a cached increment)
     const float *pending_ptr = nullptr; int pending_n = 0; long long pending_stride = 0;
     // feature cache (dLLM-Cache-style), allocated by sfs_cache_enable
