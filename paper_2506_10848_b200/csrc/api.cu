@@ -444,7 +444,7 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
 }
 
 __global__ void generate_init_kernel(const int32_t *prompt, int32_t *tokens, uint8_t *mask, int32_t *rows, int32_t *ctrl,
-                                     int32_t *host_active, unsigned long long *pos_sq, int B, int P, int L, int mask_id)
+                                     int32_t *host_active, unsigned long long *pos_sq, sfs_state *state, int max_steps, int B, int P, int L, int mask_id)
 {
     const int S = P + L;
     const long long n = (long long)B * S;
@@ -455,6 +455,7 @@ __global__ void generate_init_kernel(const int32_t *prompt, int32_t *tokens, uin
         pos_sq[i] = 0;
         if (pos >= P) rows[(long long)b * L + (pos - P)] = (int)i;         // first step: every response row, sequence-major
     }
+    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) state[b] = initial_state(L, max_steps);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         ctrl[0] = B * L; ctrl[1] = 0; ctrl[2] = (L > 0) ? B : 0;
         *host_active = (L > 0) ? B : 0;
@@ -597,7 +598,7 @@ int32_t sfs_session_create(sfs_model *m, int32_t max_batch, int32_t max_seq, sfs
     if ((rc = dev_alloc(s, &s->rows[0], T, true)) != SFS_OK) return fail(rc);
     if ((rc = dev_alloc(s, &s->rows[1], T, true)) != SFS_OK) return fail(rc);
     if ((rc = dev_alloc(s, &s->ctrl, 16, true)) != SFS_OK) return fail(rc);
-    if (cudaHostAlloc(reinterpret_cast<void **>(&s->host_active), 64, cudaHostAllocMapped) != cudaSuccess ||
+    if (cudaHostAlloc(reinterpret_cast<void **>(&s->host_active), 64 + (size_t)max_batch * sizeof(sfs_state), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void **>(&s->host_active_dev), s->host_active, 0) != cudaSuccess) {
         set_error("pinned host allocation failed");
         return fail(SFS_ERR_OOM);
@@ -809,9 +810,8 @@ int32_t sfs_generate_begin(sfs_session *s, const int32_t *d_prompt, int32_t B, i
         }
     }
     generate_init_kernel<<<64, 256, 0, st>>>(d_prompt, s->tokens, s->mask, s->rows[0], s->ctrl, s->host_active_dev, s->pos_sq,
-                                             B, P, gen_len, s->model->cfg.mask_id);
+                                             s->state, params->max_steps, B, P, gen_len, s->model->cfg.mask_id);
     SFS_LAUNCH_CHECK();
-    if ((rc = launch_state_init(s->state, B, gen_len, *params, nullptr, st)) != SFS_OK) return rc;
     s->gen_B = B; s->gen_P = P; s->gen_L = gen_len; s->gen_cur = 0; s->gen_steps = 0;
     s->gen_max_steps = params->max_steps > 0 ? params->max_steps : gen_len;
     s->gen_params = *params;
@@ -874,12 +874,18 @@ int32_t sfs_generate_end(sfs_session *s, int32_t *d_out_tokens, sfs_state *d_sta
     const int B = s->gen_B, S = s->gen_P + s->gen_L;
     if (d_out_tokens) SFS_CUDA(cudaMemcpyAsync(d_out_tokens, s->tokens, (size_t)B * S * 4, cudaMemcpyDeviceToDevice, st));
     if (d_state_out) SFS_CUDA(cudaMemcpyAsync(d_state_out, s->state, (size_t)B * sizeof(sfs_state), cudaMemcpyDeviceToDevice, st));
-    std::vector<sfs_state> hs((size_t)B);
-    SFS_CUDA(cudaMemcpyAsync(hs.data(), s->state, (size_t)B * sizeof(sfs_state), cudaMemcpyDeviceToHost, st));
-    int32_t dev = sfs_check_device_status(stream);                 // synchronises
+    // states and status word into pinned memory, one synchronisation for everything
+    int32_t *err = device_status_word(), *h_err = s->host_active + 2;
+    SFS_REQUIRE(err != nullptr, SFS_ERR_OOM, "cannot allocate the device status word");
+    const sfs_state *hs = reinterpret_cast<const sfs_state *>(s->host_active + 16);
+    SFS_CUDA(cudaMemcpyAsync(s->host_active + 16, s->state, (size_t)B * sizeof(sfs_state), cudaMemcpyDeviceToHost, st));
+    SFS_CUDA(cudaMemcpyAsync(h_err, err, 4, cudaMemcpyDeviceToHost, st));
+    SFS_CUDA(cudaStreamSynchronize(st));
+    const int32_t dev = *h_err != 0 ? sfs_check_device_status(stream) : SFS_OK;      // (clears the word and words the error)
     if (steps_enqueued) *steps_enqueued = s->gen_steps;
     int act = 0, bad = SFS_OK;
-    for (const sfs_state &h : hs) {
+    for (int b = 0; b < B; ++b) {
+        const sfs_state &h = hs[b];
         if (!h.done && h.status == SFS_OK) act++;
         if (h.status != SFS_OK && bad == SFS_OK) bad = h.status;
     }

@@ -160,6 +160,20 @@ __global__ void gather_rows_bf16_kernel(const uint4 *__restrict__ src, const int
     for (int c = threadIdx.x; c < chunks; c += blockDim.x) o[c] = s[c];
 }
 
+// the split-K partial products of one 16-byte chunk, added in slab order; up to six slabs are one round trip
+constexpr int kSlabRegs = 6;
+__device__ __forceinline__ float4 sum_slabs(const float4 *s, int n_slabs, long long slab_chunks)
+{
+    float4 p[kSlabRegs];
+#pragma unroll
+    for (int k = 0; k < kSlabRegs; ++k) if (k < n_slabs) p[k] = s[(long long)k * slab_chunks];
+    float4 v = p[0];
+#pragma unroll
+    for (int k = 1; k < kSlabRegs; ++k) if (k < n_slabs) { v.x += p[k].x; v.y += p[k].y; v.z += p[k].z; v.w += p[k].w; }
+    for (int k = kSlabRegs; k < n_slabs; ++k) { const float4 q = s[(long long)k * slab_chunks]; v.x += q.x; v.y += q.y; v.z += q.z; v.w += q.w; }
+    return v;
+}
+
 __global__ void scatter_rows_f32_kernel(const float4 *__restrict__ src, int n_slabs, long long slab_chunks, const int32_t *__restrict__ rows,
                                         int chunks, float4 *__restrict__ dst)
 {
@@ -169,12 +183,7 @@ __global__ void scatter_rows_f32_kernel(const float4 *__restrict__ src, int n_sl
     const float4 *s = src + (long long)j * chunks;
     float4 *o = dst + (long long)rows[j] * chunks;
     for (int c = blockIdx.y * blockDim.x + threadIdx.x; c < chunks; c += gridDim.y * blockDim.x) {
-        float4 v = s[c];
-        for (int k = 1; k < n_slabs; ++k) {                  // split-K partial products, added in slab order
-            const float4 p = s[(long long)k * slab_chunks + c];
-            v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
-        }
-        o[c] = v;
+        o[c] = sum_slabs(s + c, n_slabs, slab_chunks);
     }
 }
 
@@ -275,13 +284,8 @@ fold_norm_rows_kernel(const float *__restrict__ slabs, int n_slabs, long long sl
     extern __shared__ float4 s_y[];                            // the row, kept between the two passes
     float ss = 0.f;
     for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-        float4 v = sp[c];
-        for (int k = 1; k < n_slabs; ++k) {
-            const float4 p = sp[(long long)k * (slab_stride / 4) + c];
-            v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
-        }
+        const float4 xv = xr[c], v = sum_slabs(sp + c, n_slabs, slab_stride / 4);
         ir[c] = v;
-        const float4 xv = xr[c];
         const float4 y = make_float4(xv.x + v.x, xv.y + v.y, xv.z + v.z, xv.w + v.w);
         s_y[c] = y;
         ss += y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w;

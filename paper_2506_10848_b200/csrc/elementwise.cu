@@ -2,6 +2,7 @@
 // gather), rotary position embedding, and the RoPE table.  All of them move 16 bytes per thread per access.
 #include "sfs_common.cuh"
 #include "elementwise.cuh"
+#include <type_traits>
 
 namespace sfs {
 namespace {
@@ -10,9 +11,10 @@ namespace {
 // The partial products of a split-K projection are added in slab order (the sum does not depend on which CTA of the
 // projection finished first); without a row list y is written back to x, so the residual stream is complete again.
 // EMBED: y is the embedding of the row's token (bf16 -> fp32, written to x: the residual stream begins here).
-// A thread keeps its part of the row in registers between the two passes (rows of up to NT * 16 elements).
-constexpr int kNormRegChunks = 4;                          // float4 chunks a thread keeps
-template <int NT, bool EMBED>
+// A thread keeps its part of the row in registers between the two passes (kNormRegChunks 16-byte chunks of it).
+// NP bounds the number of slabs: all of a thread's loads are issued before the first addition (summed slab by slab in a loop,
+// 512 rows of 4096 with four slabs took 8.5 us, four dependent round trips per chunk).
+template <int NT, int NP, bool EMBED>
 __global__ void __launch_bounds__(NT)
 rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_partial, long long partial_stride,
                const __nv_bfloat16 *__restrict__ gain, __nv_bfloat16 *__restrict__ h,
@@ -20,7 +22,7 @@ rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_p
                const int32_t *__restrict__ tokens, const __nv_bfloat16 *__restrict__ emb, int vocab, const int32_t *__restrict__ copy_src,
                int32_t *__restrict__ copy_dst, int copy_n)
 {
-    constexpr int kNormThreads = NT;
+    constexpr int kNormThreads = NT, kNormRegChunks = NT == 256 ? 4 : (NT == 1024 ? 1 : 2);
     pdl_wait();
     pdl_trigger();
     if (EMBED && blockIdx.x == 0)
@@ -45,21 +47,40 @@ rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_p
                 const uint2 e = er[c];
                 return make_float4(bf16_bits_to_f32(e.x & 0xFFFFu), bf16_bits_to_f32(e.x >> 16), bf16_bits_to_f32(e.y & 0xFFFFu), bf16_bits_to_f32(e.y >> 16));
             }
-            float4 v = xr[c];
-            for (int s = 0; s < n_partial; ++s) {
-                const float4 p = pr[(long long)s * pstride4 + c];
-                v.x += p.x; v.y += p.y; v.z += p.z; v.w += p.w;
-            }
+            float4 v = xr[c], p[NP > 0 ? NP : 1];
+#pragma unroll
+            for (int s = 0; s < NP; ++s) if (s < n_partial) p[s] = pr[(long long)s * pstride4 + c];
+#pragma unroll
+            for (int s = 0; s < NP; ++s) if (s < n_partial) { v.x += p[s].x; v.y += p[s].y; v.z += p[s].z; v.w += p[s].w; }
             return v;
         };
         // the first kNormRegChunks chunks of a thread stay in registers (statically indexed); longer rows re-read the rest
         float4 keep[kNormRegChunks];
         float ss = 0.f;
+        if (EMBED || NP == 0) {
 #pragma unroll
-        for (int k = 0; k < kNormRegChunks; ++k) {
-            const int c = threadIdx.x + k * kNormThreads;
-            keep[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c < chunks) keep[k] = load(c);
+            for (int k = 0; k < kNormRegChunks; ++k) {
+                const int c = threadIdx.x + k * kNormThreads;
+                keep[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c < chunks) keep[k] = load(c);
+            }
+        } else {
+            float4 p[NP > 0 ? NP : 1][kNormRegChunks];
+#pragma unroll
+            for (int k = 0; k < kNormRegChunks; ++k) {
+                const int c = threadIdx.x + k * kNormThreads;
+                keep[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (c < chunks) keep[k] = xr[c];
+#pragma unroll
+                for (int s = 0; s < NP; ++s) {
+                    p[s][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (s < n_partial && c < chunks) p[s][k] = pr[(long long)s * pstride4 + c];
+                }
+            }
+#pragma unroll
+            for (int s = 0; s < NP; ++s)
+#pragma unroll
+                for (int k = 0; k < kNormRegChunks; ++k) { keep[k].x += p[s][k].x; keep[k].y += p[s][k].y; keep[k].z += p[s][k].z; keep[k].w += p[s][k].w; }
         }
 #pragma unroll
         for (int k = 0; k < kNormRegChunks; ++k) {
@@ -176,11 +197,16 @@ static int32_t launch_norm(float *x, const float *partial, int n_partial, long l
                           reinterpret_cast<const __nv_bfloat16 *>(gain), reinterpret_cast<__nv_bfloat16 *>(h), rows, n_rows, max_rows, d, eps, tokens,
                           reinterpret_cast<const __nv_bfloat16 *>(emb), vocab, copy_src, copy_dst, copy_n);
     };
-    if (nt == 1024) SFS_CUDA(go(rmsnorm_kernel<1024, EMBED>, 1024));
-    else if (nt == 512) SFS_CUDA(go(rmsnorm_kernel<512, EMBED>, 512));
-    else if (nt == 256) SFS_CUDA(go(rmsnorm_kernel<256, EMBED>, 256));
-    else if (nt == 128) SFS_CUDA(go(rmsnorm_kernel<128, EMBED>, 128));
-    else SFS_CUDA(go(rmsnorm_kernel<64, EMBED>, 64));
+    auto pick = [&](auto np) {
+        constexpr int NP = decltype(np)::value;
+        return nt == 1024 ? go(rmsnorm_kernel<1024, NP, EMBED>, 1024) : (nt == 512 ? go(rmsnorm_kernel<512, NP, EMBED>, 512)
+             : (nt == 256 ? go(rmsnorm_kernel<256, NP, EMBED>, 256) : (nt == 128 ? go(rmsnorm_kernel<128, NP, EMBED>, 128) : go(rmsnorm_kernel<64, NP, EMBED>, 64))));
+    };
+    SFS_REQUIRE(n_partial <= 6, SFS_ERR_UNSUPPORTED, "norm: %d slabs", n_partial);
+    if (n_partial == 0) SFS_CUDA(pick(std::integral_constant<int, 0>()));
+    else if (EMBED || n_partial <= 2) SFS_CUDA(pick(std::integral_constant<int, EMBED ? 0 : 2>()));
+    else if (n_partial <= 4) SFS_CUDA(pick(std::integral_constant<int, EMBED ? 0 : 4>()));
+    else SFS_CUDA(pick(std::integral_constant<int, EMBED ? 0 : 6>()));
     return SFS_OK;
 }
 

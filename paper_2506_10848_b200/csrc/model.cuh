@@ -52,7 +52,7 @@ struct sfs_session {
     sfs_state *state = nullptr;              // [max_batch]
     int32_t *rows[2] = {nullptr, nullptr};   // [T] row lists of the current / next step
     int32_t *ctrl = nullptr;                 // [0..1] row counts (double buffer), [2] active sequences
-    int32_t *host_active = nullptr;          // pinned, device-mapped mirror of ctrl[2]
+    int32_t *host_active = nullptr;          // pinned, device-mapped: [0] mirror of ctrl[2], [1] steps finished, [2] status word, [16..] states at the end
     int32_t *host_active_dev = nullptr;      // its device address
     // plans for the shapes of the current call
     int32_t plan_B = 0, plan_S = 0;

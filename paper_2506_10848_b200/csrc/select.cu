@@ -72,9 +72,9 @@ __device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int
     if (a.next_n_rows) *a.next_n_rows = n_next;
     if (a.n_active) *a.n_active = n_active;
     if (a.host_active) {
-        a.host_active[1] = a.host_step;
+        a.host_active[0] = n_active;                        // before the step count: who sees the step sees whether it was the last
         __threadfence_system();
-        a.host_active[0] = n_active;
+        a.host_active[1] = a.host_step;
     }
 }
 
@@ -423,13 +423,7 @@ __global__ void state_init_kernel(sfs_state *state, int B, int L, sfs_params p)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    sfs_state s;
-    memset(&s, 0, sizeof(s));
-    s.phase = SFS_PHASE_SLOW;
-    s.k_remaining = p.max_steps > 0 ? p.max_steps : L;
-    s.n_masked = L;
-    s.done = (L == 0) ? 1 : 0;
-    state[b] = s;
+    state[b] = initial_state(L, p.max_steps);
 }
 
 }  // namespace

@@ -104,6 +104,18 @@ __device__ __forceinline__ int warp_sum_i32(int v) { return __reduce_add_sync(0x
 __device__ __forceinline__ int warp_min_i32(int v) { return __reduce_min_sync(0xffffffffu, v); }
 __device__ __forceinline__ int warp_max_i32(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
+// Algorithm 1's initial state of a sequence with L masked positions
+__device__ __forceinline__ sfs_state initial_state(int L, int max_steps)
+{
+    sfs_state s;
+    memset(&s, 0, sizeof(s));
+    s.phase = SFS_PHASE_SLOW;
+    s.k_remaining = max_steps > 0 ? max_steps : L;
+    s.n_masked = L;
+    s.done = (L == 0) ? 1 : 0;
+    return s;
+}
+
 // block structure of the LLaDA strategies: which positions the step with index t works on, and the block's countdown
 struct BlockStep { int j, lo, hi, k_b, steps_per_block; };
 __device__ __forceinline__ BlockStep block_step(const sfs_params &p, int L, int t)
