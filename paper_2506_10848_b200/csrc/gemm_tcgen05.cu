@@ -373,18 +373,21 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     tc::tc_fence_after();
     const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t *>(tmem_slot);
     const uint32_t bn_pad = (uint32_t)((BN + 31) & ~31);
-    const uint32_t n_bufs = (uint32_t)g.acc_bufs, buf_stride = 256;     // two buffers only when MB * bn_pad <= 256
+    const uint32_t buf_stride = 256;
     const bool swiglu = (g.mode == GEMM_SWIGLU);
 
     // Model weights do not depend on the kernel before this one: the first tile's weight rows are requested at once, as many
     // k-blocks as the ring holds; their activation rows follow after the wait.
     const int pre = (g.b_static && g.d_m == nullptr) ? early_weights(g, pair, STAGES) : 0;
+    // 256-row blocks of a tile that hold rows at all: the last one of an odd number of blocks, and every tile when the device's
+    // row count is below the planned one, is half as high (an LM head planned for 512 rows and given 256 took 370 us, 1.9x)
+    auto blocks_of = [&](const TileCoord &t, int rows) { return MB == 2 && t.m0 + 2 * BM < rows ? 2 : 1; };
     if (warp == 0 && pre > 0) {
         const TileCoord t = tile_coord(g, pair, (g.M + MB * 2 * BM - 1) / (MB * 2 * BM));
         const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1) : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
         const int brow = swiglu ? t.n_local : t.n_local + (int)rank * HALF, kb0 = t.split * g.kb_per_split;
         for (int j = 0; j < pre; ++j) {
-            if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)STAGE_BYTES);
+            if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)(STAGE_BYTES - (MB - blocks_of(t, g.M)) * A_BYTES));
             tc::tma_load_2d_2cta_elect(smem_base + j * STAGE_BYTES + MB * A_BYTES, mb, (kb0 + j) * BK, brow, lead_full + 8 * j);
         }
     }
@@ -394,6 +397,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
     const int m_groups = (M + MB * 2 * BM - 1) / (MB * 2 * BM);
     const int num_tiles = live ? m_groups * g.n_col_tiles * g.splits : 0;
+    const uint32_t n_bufs = M <= 2 * BM ? 2u : (uint32_t)g.acc_bufs;    // two buffers when a tile's blocks leave room for them
 
     // The producer and MMA loops are run by all 32 lanes of their warp with warp-uniform operands; one elected lane
     // issues each asynchronous instruction.  (Issued from a single-lane branch, every tcgen05.mma cost the thread
@@ -411,7 +415,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1)
                                            : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
             const int brow = swiglu ? t.n_local : t.n_local + (int)rank * HALF;
-            const int arow = t.m0 + (int)rank * BM;
+            const int arow = t.m0 + (int)rank * BM, mbt = blocks_of(t, M);
             const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
                 const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
@@ -422,18 +426,19 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
                 const bool early = it < (uint32_t)pre;
-                if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
+                if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)(STAGE_BYTES - (MB - mbt) * A_BYTES));
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
-                if (MB == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
+                if (mbt == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
                 if (!early) tc::tma_load_2d_2cta_elect(sa + MB * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
             }
         }
         if (!live && pre > 0) {
             // nothing left to decode: the stages requested above are completed and awaited, nobody reads them
+            const int mbt = blocks_of(tile_coord(g, pair, m_groups), g.M);
             for (int j = 0; j < pre; ++j) {
                 const uint32_t sa = smem_base + j * STAGE_BYTES;
                 tc::tma_load_2d_2cta_elect(sa, &tmA, 0, 0, lead_full + 8 * j);
-                if (MB == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, 0, 0, lead_full + 8 * j);
+                if (mbt == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, 0, 0, lead_full + 8 * j);
             }
             if (rank == 0) for (int j = 0; j < pre && tc::mbar_wait(bar_full + 8 * j, 0u, &s_abort); ++j) {}
         }
@@ -462,7 +467,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * buf_stride;
-                const int kb0 = tile_coord(g, tile, m_groups).split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
+                const TileCoord t = tile_coord(g, tile, m_groups);
+                const bool second = blocks_of(t, M) == 2;
+                const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
                 for (int kb = kb0; kb < kb1; ++kb, ++it) {
                     const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
                     if (!ready) ready = tc::mbar_wait(bar_full + 8 * s, ph, &s_abort);
@@ -477,7 +484,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     tc::mma_bf16_2cta_elect(d_tmem, da, db, idesc, acc);
 #pragma unroll
                     for (int kk = 1; kk < BK / 16; ++kk) tc::mma_bf16_2cta_elect(d_tmem, da + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, 1u);
-                    if (MB == 2) {
+                    if (second) {
                         const uint64_t da1 = tc::smem_desc_sw128(sa + A_BYTES);
                         tc::mma_bf16_2cta_elect(d_tmem + bn_pad, da1, db, idesc, acc);
 #pragma unroll
@@ -503,7 +510,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             EpiShare e;
             e.tmem = tmem_base + buf * buf_stride + ((uint32_t)(q * 32) << 16); e.tmem_block = bn_pad; e.up = (uint32_t)HALF;
             e.row0 = t.m0 + (int)rank * BM + q * 32; e.row_block = 2 * BM;
-            e.col0 = t.ncol0; e.col_block = 0; e.blocks = MB; e.seg = STATS ? BN : t.ncols;      // (every record is written)
+            e.col0 = t.ncol0; e.col_block = 0; e.blocks = blocks_of(t, M); e.seg = STATS ? BN : t.ncols;      // (every record is written)
             e.col_end = min(t.ncol0 + t.ncols, g.N);
             e.rec = 2 * (t.ncol0 / BN); e.rec_block = 0;
             epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
