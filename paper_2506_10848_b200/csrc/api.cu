@@ -257,6 +257,10 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
         CacheLayerPlans &cp = s->cache_plans[l];
+        // a full refresh writes the values straight into the cache (and the rotary kernel the keys)
+        const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
+        rc = weight_plan_create(&cp.qkv_store, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->Vtc[l], T, 2 * d, nullptr);
+        if (rc != SFS_OK) return rc;
         const void *wv[1] = {m->wv[l]};
         // fresh values of the candidate rows, written transposed (every output column goes through the transposed store): the
         // response rows of a single sequence are one contiguous range; with several sequences every row is projected
@@ -364,16 +368,14 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
             });
         };
         if (rp && rr) {
-            // everything is recomputed: the uncached layer pipeline, with the increments stored instead of added and K / V copied out
+            // everything is recomputed: the uncached layer pipeline, with the increments stored instead of added and K / V going to the cache
             for (int l = 0; l < c.n_layers; ++l) {
                 const LayerPlans &lp = s->layer_plans[l];
                 const CacheLayerPlans &cl = s->cache_plans[l];
                 if (l > 0 && (rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
-                SFS_CUDA(cudaMemcpy2DAsync(s->Kc[l], (size_t)d * 2, s->qk + d, (size_t)2 * d * 2, (size_t)d * 2, (size_t)T, cudaMemcpyDeviceToDevice, st));
-                SFS_CUDA(cudaMemcpyAsync(s->Vtc[l], s->vt, (size_t)d * T * 2, cudaMemcpyDeviceToDevice, st));
-                if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(cl.qkv_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, s->Kc[l], st); })) != SFS_OK) return rc;
+                if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(cl.attn, d_active, err, st); })) != SFS_OK) return rc;
                 if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(cl.o_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
                 pend = s->Ac[l];
                 if ((rc = norm_all(m->mlp_norm[l])) != SFS_OK) return rc;

@@ -54,95 +54,110 @@ sim_partial_kernel(const __nv_bfloat16 *__restrict__ a, const __nv_bfloat16 *__r
     }
 }
 
+__device__ __forceinline__ float ld_nc(const float *p) {              // (volatile: issued where it stands, not where it is used)
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
 __device__ __forceinline__ uint32_t float_order_key(float f) {       // monotone map float -> uint32
     const uint32_t u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// one CTA per sequence; dynamic shared memory: u64 keys[L], u8 chosen[L]
-__global__ void __launch_bounds__(1024) cache_select_kernel(CacheSelectArgs a)
+// One CTA per sequence; dynamic shared memory: u32 keys[L].  The similarities of a position are summed by two lanes; the k-th
+// smallest key is found bit by bit (one block-wide count per bit), the chosen positions are those below it and the first of those
+// equal to it, and their slots are running counts.  It is one link of every layer's chain: 512 positions took 18 us when each
+// candidate's rank was counted over all keys (262 thousand 64-bit comparisons on one SM).
+constexpr int kChoiceThreads = 1024;
+__global__ void __launch_bounds__(kChoiceThreads) cache_select_kernel(CacheSelectArgs a)
 {
     pdl_wait();
     pdl_trigger();
-    extern __shared__ __align__(16) unsigned long long s_key[];
-    const int b = blockIdx.x, tid = threadIdx.x, L = a.L, P = a.P, S = a.S;
+    extern __shared__ __align__(16) uint32_t s_key[];
+    __shared__ int s_cnt[kChoiceThreads / 32], s_last;
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L, P = a.P, S = a.S;
     int32_t *out = a.sel_rows + (long long)b * a.n_sel;
     int base = 0;
     if (a.refresh_p) {
-        for (int i = tid; i < P; i += blockDim.x) out[i] = b * S + i;
+        for (int i = tid; i < P; i += kChoiceThreads) out[i] = b * S + i;
         base = P;
     }
     if (a.refresh_r) {
-        for (int i = tid; i < L; i += blockDim.x) out[base + i] = b * S + P + i;
+        for (int i = tid; i < L; i += kChoiceThreads) out[base + i] = b * S + P + i;
     } else if (a.n_adapt > 0) {
         int lo = 0, hi = L;
         if (a.state != nullptr && a.state[b].phase == SFS_PHASE_FAST && !a.state[b].done) { lo = a.state[b].s_cycle; hi = a.state[b].hi; }
         lo = max(0, min(lo, L)); hi = max(lo, min(hi, L));
-        for (int i = tid; i < L; i += blockDim.x) {
-            float dot = 0.f, na = 0.f, nb = 0.f;
-            const long long t = (long long)b * S + P + i;
-            const float *__restrict__ part = a.partial;
-            float pd[kSimSlices], pa[kSimSlices], pb[kSimSlices];
+        constexpr int HS = kSimSlices / 2;
+        for (int it = tid; it < 2 * L; it += kChoiceThreads) {        // (2 L is even: both lanes of a position are there)
+            const int i = it >> 1, half = it & 1;
+            const float *__restrict__ p = a.partial + ((long long)(half * HS) * a.T + (long long)b * S + P + i) * 3;
+            float pd[HS], pa[HS], pb[HS];
 #pragma unroll
-            for (int sl = 0; sl < kSimSlices; ++sl) {                // all loads first: one latency, not kSimSlices of them
-                const float *p = part + ((long long)sl * a.T + t) * 3;
-                pd[sl] = __ldg(p); pa[sl] = __ldg(p + 1); pb[sl] = __ldg(p + 2);
+            for (int sl = 0; sl < HS; ++sl) {                        // all loads first: one latency, not HS of them
+                const float *q = p + (long long)sl * a.T * 3;
+                pd[sl] = ld_nc(q); pa[sl] = ld_nc(q + 1); pb[sl] = ld_nc(q + 2);
             }
+            float dot = 0.f, na = 0.f, nb = 0.f;
 #pragma unroll
-            for (int sl = 0; sl < kSimSlices; ++sl) { dot += pd[sl]; na += pa[sl]; nb += pb[sl]; }   // fixed order
+            for (int sl = 0; sl < HS; ++sl) { dot += pd[sl]; na += pa[sl]; nb += pb[sl]; }           // fixed order
+            const unsigned both = 3u << (lane & 30);
+            dot += __shfl_xor_sync(both, dot, 1); na += __shfl_xor_sync(both, na, 1); nb += __shfl_xor_sync(both, nb, 1);
             const float den = __fmul_rn(__fsqrt_rn(na), __fsqrt_rn(nb));
             const float sim = den > 0.f ? __fdiv_rn(dot, den) : 0.f;
-            if (a.sims_dump) a.sims_dump[(long long)b * L + i] = sim;
-            s_key[i] = (i >= lo && i < hi) ? (((unsigned long long)float_order_key(sim) << 32) | (unsigned)i) : ~0ull;
-        }
-        const int Lp = (L + 1) & ~1;                               // keys are scanned two at a time: an odd L gets a sentinel
-        if (tid == 0 && Lp != L) s_key[L] = ~0ull;
-        __syncthreads();
-        const int n_cand = hi - lo;
-        const int k = min(a.n_adapt, n_cand);
-        __shared__ int s_last, s_wcnt[32];
-        if (tid == 0) s_last = -1;
-        // rank by counting: candidate i is chosen when fewer than k candidate keys are smaller.  `parts` adjacent lanes share
-        // a candidate, each counting over its own range of the keys (16-byte loads, two keys each).
-        uint8_t *s_sel = reinterpret_cast<uint8_t *>(s_key + Lp);
-        int parts = 1;
-        while (parts < 32 && (long long)L * parts * 2 <= (long long)blockDim.x) parts *= 2;
-        const int span = ((Lp / 2 + parts - 1) / parts) * 2;      // keys per part (even)
-        const ulonglong2 *k2 = reinterpret_cast<const ulonglong2 *>(s_key);
-        const int items = ((L * parts + 31) / 32) * 32;           // whole warps take part in the shuffles
-        for (int it = tid; it < items; it += blockDim.x) {
-            const int i = it / parts, part = it - i * parts;
-            const unsigned long long ki = i < L ? s_key[i] : ~0ull;
-            int rank = 0;
-            if (ki != ~0ull) {
-                const int j0 = part * span, j1 = min(Lp, j0 + span);
-                for (int j = j0; j < j1; j += 2) { const ulonglong2 kk = k2[j >> 1]; rank += (kk.x < ki ? 1 : 0) + (kk.y < ki ? 1 : 0); }
+            if (half == 0) {
+                if (a.sims_dump) a.sims_dump[(long long)b * L + i] = sim;
+                s_key[i] = float_order_key(sim);
             }
-            for (int o = 1; o < parts; o <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
-            if (part == 0 && i < L) s_sel[i] = (ki != ~0ull && rank < k) ? 1 : 0;
         }
+        if (tid == 0) s_last = -1;
         __syncthreads();
-        // its slot in the ascending list is the number of chosen positions before it (ballots and per-warp counts)
-        const int lane = tid & 31, warp = tid >> 5, n_warps = (int)blockDim.x >> 5;
-        int run = 0;
-        for (int i0 = 0; i0 < L; i0 += blockDim.x) {
-            const int i = i0 + tid;
-            const bool chosen = i < L && s_sel[i] != 0;
-            const unsigned bal = __ballot_sync(0xffffffffu, chosen);
-            if (lane == 0) s_wcnt[warp] = __popc(bal);
+        const int n_cand = hi - lo, k = min(a.n_adapt, n_cand);
+        // candidates whose key is below v
+        auto count_below = [&](uint32_t v) {
+            if (L <= kChoiceThreads) return __syncthreads_count(tid >= lo && tid < hi && s_key[tid] < v);
+            int c = 0;
+            for (int i = lo + tid; i < hi; i += kChoiceThreads) c += s_key[i] < v ? 1 : 0;
+            c = warp_sum_i32(c);
             __syncthreads();
-            int before = run, total = 0;
-            for (int w = 0; w < n_warps; ++w) { const int cnt = s_wcnt[w]; total += cnt; if (w < warp) before += cnt; }
-            if (chosen) {
-                const int slot = before + __popc(bal & ((1u << lane) - 1u));
+            if (lane == 0) s_cnt[warp] = c;
+            __syncthreads();
+            return warp_sum_i32(s_cnt[lane]);
+        };
+        uint32_t kth = 0xFFFFFFFFu;                                  // the k-th smallest key, when not all are chosen
+        int need = n_cand;                                           // how many of those equal to it are chosen
+        if (k > 0 && k < n_cand) {
+            kth = 0;
+            for (int bit = 31; bit >= 0; --bit) {
+                const uint32_t v = kth | (1u << bit);
+                if (count_below(v) < k) kth = v;
+            }
+            need = k - count_below(kth);
+        }
+        int run_less = 0, run_eq = 0;
+        for (int i0 = 0; i0 < L && k > 0; i0 += kChoiceThreads) {
+            const int i = i0 + tid;
+            const bool cand = i >= lo && i < hi, all = k == n_cand;
+            const uint32_t key = cand ? s_key[i] : 0u;
+            const bool less = cand && !all && key < kth, eq = cand && (all || key == kth);
+            const unsigned bl = __ballot_sync(0xffffffffu, less), be = __ballot_sync(0xffffffffu, eq);
+            __syncthreads();
+            if (lane == 0) s_cnt[warp] = __popc(bl) | (__popc(be) << 16);
+            __syncthreads();
+            const int c = s_cnt[lane];
+            const int before = warp_sum_i32(lane < warp ? c : 0), total = warp_sum_i32(c);
+            const unsigned lt = (1u << lane) - 1u;
+            const int n_less = run_less + (before & 0xFFFF) + __popc(bl & lt), n_eq = run_eq + (before >> 16) + __popc(be & lt);
+            if (less || (eq && n_eq < need)) {
+                const int slot = n_less + min(n_eq, need);
                 out[base + slot] = b * S + P + i;
                 if (slot == k - 1) s_last = b * S + P + i;
             }
-            run += total;
-            __syncthreads();
+            run_less += total & 0xFFFF; run_eq += total >> 16;
         }
+        __syncthreads();
         const int pad = (k > 0) ? s_last : b * S + P;                  // nothing to choose from: recompute the first response row
-        for (int j = k + tid; j < a.n_adapt; j += blockDim.x) out[base + j] = pad;
+        for (int j = k + tid; j < a.n_adapt; j += kChoiceThreads) out[base + j] = pad;
     }
     if (a.sets_dump) {
         __syncthreads();
@@ -347,8 +362,8 @@ int32_t launch_sim_partial(const void *vnew_t, const void *vold_t, long long ld,
 
 int32_t launch_cache_select(const CacheSelectArgs &a, cudaStream_t s)
 {
-    // 1024 threads: the ranking is O(L^2 / threads); shared memory: the keys (an even number of them), then one byte per position
-    SFS_CUDA(launch_pdl(cache_select_kernel, dim3((unsigned)(a.B)), dim3((unsigned)(1024)), (size_t)((size_t)(a.L + 1) * 9 + 16), s, a));
+    if ((size_t)a.L * 4 > 48 * 1024) SFS_CUDA(cudaFuncSetAttribute(cache_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, a.L * 4));
+    SFS_CUDA(launch_pdl(cache_select_kernel, dim3((unsigned)(a.B)), dim3(kChoiceThreads), (size_t)a.L * 4, s, a));
     return SFS_OK;
 }
 

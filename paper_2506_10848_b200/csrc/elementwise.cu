@@ -133,9 +133,10 @@ __global__ void rope_table_kernel(float2 *table, int positions, int half, double
     table[idx] = make_float2((float)cos(ang), (float)sin(ang));
 }
 
-// in place on q and k: pairs (j, j + dh/2) of every head rotate by the angle of the token's position
+// in place on q, and in place on k or (k_dst given) into the K cache [T, n_heads * dh]: pairs (j, j + dh/2) of every head rotate by
+// the angle of the token's position
 __global__ void rope_kernel(__nv_bfloat16 *__restrict__ qk, long long ld, int T, int S, int n_heads, int dh,
-                            const float2 *__restrict__ table, const int32_t *__restrict__ rows)
+                            const float2 *__restrict__ table, __nv_bfloat16 *__restrict__ k_dst)
 {
     // one thread handles 8 consecutive j of one (token, q-or-k, head)
     pdl_wait();
@@ -149,7 +150,7 @@ __global__ void rope_kernel(__nv_bfloat16 *__restrict__ qk, long long ld, int T,
     const unsigned rem = idx - (unsigned)t * per_token;
     const int hh = (int)(rem / (unsigned)groups);              // q heads then k heads: contiguous columns
     const int g = (int)(rem - (unsigned)hh * (unsigned)groups);
-    const int pos = (rows ? rows[t] : t) % S;              // compact rows carry the token index they came from
+    const int pos = t % S;
     __nv_bfloat16 *base = qk + (long long)t * ld + (long long)hh * dh + g * 8;
     uint4 lo = *reinterpret_cast<uint4 *>(base), hi = *reinterpret_cast<uint4 *>(base + half);
     const float2 *tb = table + (long long)pos * half + g * 8;
@@ -169,6 +170,7 @@ __global__ void rope_kernel(__nv_bfloat16 *__restrict__ qk, long long ld, int T,
         lw[w] = *reinterpret_cast<uint32_t *>(&a);
         hw[w] = *reinterpret_cast<uint32_t *>(&b2);
     }
+    if (k_dst != nullptr && hh >= n_heads) base = k_dst + (long long)t * n_heads * dh + (long long)(hh - n_heads) * dh + g * 8;
     *reinterpret_cast<uint4 *>(base) = lo;
     *reinterpret_cast<uint4 *>(base + half) = hi;
 }
@@ -230,12 +232,12 @@ int32_t launch_rope_table(float2 *table, int positions, int head_dim, float thet
     return SFS_OK;
 }
 
-int32_t launch_rope(void *qk, int64_t ld, int T, int S, int n_heads, int head_dim, const float2 *table, const int32_t *rows, cudaStream_t s)
+int32_t launch_rope(void *qk, int64_t ld, int T, int S, int n_heads, int head_dim, const float2 *table, void *k_dst, cudaStream_t s)
 {
     const long long total = (long long)T * 2 * n_heads * (head_dim / 16);
     SFS_REQUIRE(total < (1LL << 31), SFS_ERR_INVALID_ARG, "rope: %lld items do not fit a 32-bit index", total);
     SFS_CUDA(launch_pdl(rope_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, reinterpret_cast<__nv_bfloat16 *>(qk), (long long)ld, T, S,
-                        n_heads, head_dim, table, rows));
+                        n_heads, head_dim, table, reinterpret_cast<__nv_bfloat16 *>(k_dst)));
     return SFS_OK;
 }
 
