@@ -74,7 +74,7 @@ static int32_t dev_alloc(sfs_session *s, T **out, size_t count, bool zero)
 // whose second pass the selection kernel takes; the all-canonical kernels otherwise.  `a` learns which.
 static int32_t step_row_stats(sfs_session *s, const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
                               const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, int32_t B, int32_t S, SelectArgs *a,
-                              cudaStream_t st, const float4 *lm_stats = nullptr, int32_t lm_stats_ld = 0)
+                              cudaStream_t st, const GemmArgs *lm = nullptr)
 {
     int32_t *err = device_status_word();
     if (max_rows <= 0 || !row_stats_two_pass_applies(d_logits, logits_dtype, vocab, ld))
@@ -83,8 +83,11 @@ static int32_t step_row_stats(sfs_session *s, const void *d_logits, int32_t logi
     a->pos_lo = s->pos_lo; a->pos_hi = s->pos_hi; a->pos_row = s->pos_row; a->pos_max = s->pos_max; a->seq_ticket = s->seq_ticket;
     a->lrows = {reinterpret_cast<const uint4 *>(d_logits), (long long)(ld / 8), vocab / 8};
     const BoundsScratch bs = {s->pos_lo, s->pos_hi, s->pos_arg, s->slice_partials, s->row_tickets, s->pos_row, s->pos_max, B * S};
-    if (lm_stats != nullptr)       // the LM head's epilogue has taken the first pass: the logits are read only for the open rows
-        return launch_row_stats_from_partials(lm_stats, lm_stats_ld, lm_stats_ld, vocab, d_n_rows, max_rows, d_rows, bs, err, st);
+    if (lm != nullptr && lm->stats != nullptr) {   // the LM head's epilogue has taken the first pass: the logits are read only for the open rows
+        const int block = lm->few ? lm->bn / 2 : lm->bn;    // (few rows: an N-block's column halves are blocks of their own)
+        const StatsLayout lay = {block, 64 * (((block + 63) / 64 + 1) / 2)};
+        return launch_row_stats_from_partials(lm->stats, lm->stats_ld, lm->stats_ld, lay, d_logits, ld, vocab, d_n_rows, max_rows, d_rows, bs, err, st);
+    }
     return launch_row_stats_two_pass(d_logits, vocab, ld, d_n_rows, max_rows, d_rows, bs, err, st);
 }
 
@@ -851,8 +854,7 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
         }
         SelectArgs a{};
         if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
-                 return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, s->lm_plan.args.stats,
-                                       s->lm_plan.args.stats_ld); })) != SFS_OK) return rc;
+                 return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, &s->lm_plan.args); })) != SFS_OK) return rc;
         a.tokens = s->tokens; a.mask = s->mask; a.B = B; a.S = S; a.P = P; a.L = L;
         a.state = s->state; a.params = s->gen_params;
         a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;

@@ -338,13 +338,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // uniform over the pair, before any barrier or allocation: pairs beyond the tiles of even the largest row count
     if (pair >= ((g.M + MB * 2 * BM - 1) / (MB * 2 * BM)) * g.n_col_tiles * g.splits) return;
 
-    const int BN = g.bn, STAGES = g.stages, HALF = BN >> 1;
-    const int STAGE_BYTES = MB * A_BYTES + HALF * BK * 2;   // per CTA: MB blocks of 128 A rows, half of the weight rows
+    const int BN = g.bn, HALF = BN >> 1;
+    int STAGES = g.stages, STAGE_BYTES = MB * A_BYTES + HALF * BK * 2;      // per CTA: MB blocks of 128 A rows, half of the weight rows
+    const int ring_bytes = STAGES * STAGE_BYTES;
     const uint32_t rank = tc::cluster_ctarank();            // 0 = leader (issues the MMAs), 1 = peer
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + ring_bytes);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + 2 * kMaxStages + 4);
     __shared__ int s_abort;
 
@@ -357,7 +358,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const uint32_t lead_full = tc::mapa(bar_full, 0), lead_acc_empty = tc::mapa(bar_acc_empty, 0);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) { tc::mbar_init(bar_full + 8 * s, 1); tc::mbar_init(bar_empty + 8 * s, 1); }
+        for (int s = 0; s < kMaxStages; ++s) { tc::mbar_init(bar_full + 8 * s, 1); tc::mbar_init(bar_empty + 8 * s, 1); }
         for (int b = 0; b < 2; ++b) { tc::mbar_init(bar_acc_full + 8 * b, 1); tc::mbar_init(bar_acc_empty + 8 * b, 2 * kEpiWarps); }
         s_abort = 0;
         tc::mbar_init_fence();
@@ -397,7 +398,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
     const int m_groups = (M + MB * 2 * BM - 1) / (MB * 2 * BM);
     const int num_tiles = live ? m_groups * g.n_col_tiles * g.splits : 0;
-    const uint32_t n_bufs = M <= 2 * BM ? 2u : (uint32_t)g.acc_bufs;    // two buffers when a tile's blocks leave room for them
+    // Fewer rows than planned, one block in use: two accumulators fit tensor memory, and the ring holds more, smaller stages
+    // (256 rows of an LM head planned for 512: 250 us with the four stages of two blocks).
+    const bool one_block = g.d_m != nullptr && M <= 2 * BM;
+    const uint32_t n_bufs = one_block ? 2u : (uint32_t)g.acc_bufs;
+    const int MBS = one_block ? 1 : MB;                     // blocks a stage has room for
+    if (one_block) { STAGE_BYTES = A_BYTES + HALF * BK * 2; STAGES = min(kMaxStages, ring_bytes / STAGE_BYTES); }
 
     // The producer and MMA loops are run by all 32 lanes of their warp with warp-uniform operands; one elected lane
     // issues each asynchronous instruction.  (Issued from a single-lane branch, every tcgen05.mma cost the thread
@@ -426,10 +432,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
                 const bool early = it < (uint32_t)pre;
-                if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)(STAGE_BYTES - (MB - mbt) * A_BYTES));
+                if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)(STAGE_BYTES - (MBS - mbt) * A_BYTES));
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 if (mbt == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
-                if (!early) tc::tma_load_2d_2cta_elect(sa + MB * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
+                if (!early) tc::tma_load_2d_2cta_elect(sa + MBS * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
             }
         }
         if (!live && pre > 0) {
@@ -479,7 +485,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
                     ready = tc::mbar_test(bar_full + 8 * ns, nph);
                     const uint32_t sa = smem_base + s * STAGE_BYTES;
-                    const uint64_t da = tc::smem_desc_sw128(sa), db = tc::smem_desc_sw128(sa + MB * A_BYTES);
+                    const uint64_t da = tc::smem_desc_sw128(sa), db = tc::smem_desc_sw128(sa + MBS * A_BYTES);
                     const uint32_t acc = kb != kb0 ? 1u : 0u;
                     tc::mma_bf16_2cta_elect(d_tmem, da, db, idesc, acc);
 #pragma unroll
@@ -498,7 +504,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     } else {
         // ---------------- epilogue: 8 warps; warp w reads TMEM lanes 32*(w%4).., the column units of parity (w-2)/4
         const int q = warp & 3, par = (warp - 2) >> 2;
-        const uint32_t stage = smem_base + STAGES * STAGE_BYTES + kBarBytes + (uint32_t)(warp - 2) * (32 * 128);
+        const uint32_t stage = smem_base + ring_bytes + kBarBytes + (uint32_t)(warp - 2) * (32 * 128);
         uint32_t lt = 0;
         bool ok = true;
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {

@@ -427,7 +427,7 @@ struct BoundsOut {
 };
 
 // the enclosure of the canonical S_q from the approximate sum `tot` (relative to the row maximum m), and the scattered outputs
-__device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, float tot, int arg, float m, bool open, int vocab)
+__device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, float tot, int arg, float m, bool open, int vocab, bool certain = false)
 {
     if (arg == 0x7FFFFFFF) arg = 0;
     const double Sd = (double)tot * (double)(1u << SFS_CONF_QBITS);
@@ -436,6 +436,7 @@ __device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, f
     unsigned long long lo = dlo > (double)floor_q ? (unsigned long long)dlo : floor_q;
     unsigned long long hi = (unsigned long long)dhi + 1ull;
     if (open || !(tot >= 0.999f) || !(tot <= 3.0e38f)) { lo = 1ull; hi = ~0ull >> 1; }
+    if (certain) lo = hi = floor_q;
     if (out.lo) out.lo[row] = lo;
     if (out.hi) out.hi[row] = hi;
     if (out.argmax) out.argmax[row] = arg;
@@ -451,11 +452,14 @@ __device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, f
 
 // Pass 1 when the LM head has already taken the statistics in its epilogue: per row, n_parts records (maximum, reference,
 // sum of 2^((x - reference) log2 e), first position of the maximum) are combined exactly like the slices of the streaming
-// kernel — one warp per row, the lanes' shares added in a fixed order — into the row's argmax and enclosure.  The logits are
-// not read.
+// kernel — one warp per row, the lanes' shares added in a fixed order — into the row's argmax and enclosure.  Of the logits
+// only the columns of the record that holds the maximum are read: with the other records' maxima they give the second largest
+// logit, and when that is more than 19.5 below the maximum every other term of the canonical S_q is trunc(2^28 exp(< -19.5)) = 0
+// (2^28 exp(-19.5) = 0.91), so S_q is 2^28 exactly.  Such rows (confidence above 0.9996, most of a confident model's) all lie in
+// each other's enclosures otherwise, and a ranking step recomputed every one of them (256 rows: 50 us).
 __global__ void __launch_bounds__(128)
 combine_partials_kernel(const float4 *__restrict__ stats, int stats_ld, int n_parts, const int32_t *__restrict__ n_rows_ptr, int max_rows,
-                        int vocab, BoundsOut out)
+                        int vocab, BoundsOut out, const __nv_bfloat16 *__restrict__ logits, long long ld, StatsLayout lay)
 {
     pdl_wait();
     pdl_trigger();
@@ -482,7 +486,25 @@ combine_partials_kernel(const float4 *__restrict__ stats, int stats_ld, int n_pa
     tot = warp_sum(tot);
     arg = warp_min_i32(arg);
     open = warp_max_i32(open);
-    if (lane == 0) write_enclosure(out, row, tot, arg, m, open != 0, vocab);
+    // the second largest logit: the other records' maxima, and the other columns of the record that holds position arg
+    float m2 = -INFINITY;
+    int own = -1;
+    for (int q = lane; q < n_parts; q += 32) {
+        const float4 r = __ldg(&ps[q]);
+        if (r.x == m && __float_as_int(r.w) == arg) own = q;
+        else m2 = fmaxf(m2, r.x);
+    }
+    own = warp_max_i32(own);
+    if (own >= 0) {
+        const __nv_bfloat16 *rp = logits + (long long)row * ld;
+        for (int i = lane; i < lay.per_part; i += 32) {
+            const int c = lay.column(own, i);
+            if (c >= 0 && c < vocab && c != arg) m2 = fmaxf(m2, __bfloat162float(rp[c]));
+        }
+    }
+    m2 = warp_max(m2);
+    const bool certain = own >= 0 && fabsf(m) <= 3.0e38f && m2 - m < -19.5f;
+    if (lane == 0) write_enclosure(out, row, tot, arg, m, open != 0, vocab, certain);
 }
 
 __device__ __forceinline__ uint32_t chunk_max2(const uint4 &v) {
@@ -774,13 +796,14 @@ int32_t launch_row_stats_two_pass(const void *d_logits, int32_t vocab, int64_t l
     return SFS_OK;
 }
 
-int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err,
+int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, const StatsLayout &lay, const void *d_logits, int64_t ld, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err,
                                        cudaStream_t stream)
 {
     if (max_rows <= 0) return SFS_OK;
     BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.n_positions, d_err,
                  nullptr, nullptr};
-    SFS_CUDA(launch_pdl(combine_partials_kernel, dim3((unsigned)((max_rows + 3) / 4)), dim3((unsigned)(128)), (size_t)(0), stream, reinterpret_cast<const float4 *>(stats), stats_ld, n_parts, d_n_rows, max_rows, vocab, bo));
+    SFS_CUDA(launch_pdl(combine_partials_kernel, dim3((unsigned)((max_rows + 3) / 4)), dim3((unsigned)(128)), (size_t)(0), stream, reinterpret_cast<const float4 *>(stats), stats_ld, n_parts, d_n_rows, max_rows, vocab, bo,
+                        reinterpret_cast<const __nv_bfloat16 *>(d_logits), (long long)ld, lay));
     return SFS_OK;
 }
 

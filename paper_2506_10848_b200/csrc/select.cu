@@ -84,6 +84,7 @@ enum { F_MASKED = 1, F_HIGH = 2, F_SEL = 4, F_OPEN = 8 };
 // Which candidate rows of a step must be recomputed canonically (two-pass statistics): flags them F_OPEN and lists their logits
 // rows, in position order, in s_list; returns how many.  Every other candidate row's enclosure [lo, hi] answers what the step's
 // rule asks, and its lower bound stands for it:
+//   * a row whose enclosure is one value is never open;
 //   * a threshold is open when lo and hi fall on different sides of it;
 //   * the ranking (k most confident candidates, smallest S_q first) is open for every candidate whose lo does not exceed
 //     U = the k-th smallest hi among the candidates: the k rows with the smallest hi all have S_q <= U, so a row with
@@ -125,7 +126,7 @@ __device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, u
         bool open = false;
         if (i >= ask.lo && i < ask.hi && i < L && (i0 == 0 ? m0 : msk[i])) {
             const unsigned long long lo = i0 == 0 ? lo0 : plo[i], hi = i0 == 0 ? hi0 : phi[i];
-            if (lo != 0) {                                  // 0: no row supplied for this candidate
+            if (lo != 0 && lo != hi) {                      // 0: no row supplied for this candidate
                 if (ask.tau > 0.f) open = conf_exceeds(lo, ask.tau) && !conf_exceeds(hi, ask.tau);
                 if (k_top > 1) open = true;
                 else if (k_top == 1) open = open || lo <= U;

@@ -189,8 +189,18 @@ constexpr int kRowStatsSlices = 8;
 bool row_stats_two_pass_applies(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld);
 int32_t launch_row_stats_two_pass(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,
                                   const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err, cudaStream_t stream);
+// Which columns a record of the LM head's statistics covers: blocks of `block` columns, each with two records (epilogue-warp
+// parities) that take its 64-column units in turn; record 2 b + p holds the units p, p + 2, ... of block b.
+struct StatsLayout {
+    int block, per_part;                                    // columns of a block, columns a record covers at most
+    __host__ __device__ int column(int rec, int i) const    // i-th column of a record, -1 beyond its block
+    {
+        const int c = 64 * ((rec & 1) + 2 * (i >> 6)) + (i & 63);
+        return c < block ? (rec >> 1) * block + c : -1;
+    }
+};
 // the same with pass 1 already taken by the LM head's epilogue: `stats` holds n_parts records per row (stats_ld apart)
-int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows,
+int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int32_t n_parts, const StatsLayout &lay, const void *d_logits, int64_t ld, int32_t vocab, const int32_t *d_n_rows, int32_t max_rows,
                                        const int32_t *d_rows, const BoundsScratch &rf, int32_t *d_err, cudaStream_t stream);
 // pass 1 alone, dense outputs by logits row (for tests): d_lo / d_hi enclose the canonical S_q
 int32_t launch_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,

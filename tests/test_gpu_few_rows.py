@@ -27,13 +27,14 @@ def test_linear_edges(M, N, K):
         assert np.all(err <= 4.0 * K * K * 2.0 ** -24 + (2.0 ** -8 * np.abs(ref) if out_dtype == 0 else 0.0)), float(err.max())
 
 
-@pytest.mark.parametrize("B,L,vocab", [(1, 24, 70008), (2, 61, 65536), (1, 128, 99992)])
-def test_generation_with_few_long_rows_is_reproduced_by_the_oracle(B, L, vocab):
-    """Long vocabulary rows, at most 128 of them (ragged last column tile): the decisions come from the LM head's own records."""
+@pytest.mark.parametrize("B,L,vocab,scale", [(1, 24, 70008, 60.0), (2, 61, 65536, 60.0), (1, 128, 99992, 60.0), (1, 40, 70008, 600.0), (2, 131, 65544, 600.0)])
+def test_generation_with_few_long_rows_is_reproduced_by_the_oracle(B, L, vocab, scale):
+    """Long vocabulary rows, at most 128 of them (ragged last column tile): the decisions come from the LM head's own records.  At the
+    larger scale most rows' other terms all truncate to zero (several rows tie exactly at S_q = 2^28); the last case has more rows."""
     P = 8 - L % 8
     S = P + L
     shape = W.Shape(n_layers=1, d_model=256, n_heads=2, head_dim=128, d_ff=512, vocab=vocab, mask_id=vocab - 1, rms_eps=1e-5,
-                    rope_theta=10000.0, logit_scale=60.0)
+                    rope_theta=10000.0, logit_scale=scale)
     w = W.model_weights(shape, seed=9, device=DEV)
     model = sfs.Model(shape, w)
     session = sfs.sfs_session_create(model, B, S)
