@@ -112,7 +112,10 @@ static int32_t session_alloc_select(sfs_session *s)
 
 static void drop_graphs(sfs_session *s)
 {
-    for (auto &kv : s->graphs) if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+    for (auto &kv : s->graphs) {
+        if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
+        if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
+    }
     s->graphs.clear();
 }
 
@@ -176,52 +179,107 @@ static int32_t timed_launch(sfs_session *s, int cls, cudaStream_t st, F &&f)
     return rc;
 }
 
-// Runs a body that reads and writes session buffers only.  Its launches are the same each time for the same plans, so from the
-// kGraphAfter-th time on they are one graph launch: a body of small kernels is bound by enqueueing them (18 launches of a tiny
-// step: 80 to 160 us of host time, by the host), and between two nodes of a graph the device loses less than between two launches
-// (8 layers at 104 rows 1184 -> 1137 us).  Recording and instantiating costs 1 to 3 ms, which a session that runs a few steps
-// does not get back.  The graph belongs to the session and its plans; a caller's own stream capture gets the plain launches.
-constexpr int kGraphAfter = 16;
-template <typename F>
-static int32_t run_recorded(sfs_session *s, long long key, cudaStream_t st, F &&enqueue)
+cudaError_t note_recorded_node(NodeSink *sink, cudaStream_t stream)
 {
+    cudaStreamCaptureStatus cs;
+    const cudaGraphNode_t *deps = nullptr;
+    const cudaGraphEdgeData *edges = nullptr;
+    size_t n = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo_v3(stream, &cs, nullptr, nullptr, &deps, &edges, &n);
+    if (e == cudaSuccess && (cs != cudaStreamCaptureStatusActive || n != 1)) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) sink->nodes->push_back(deps[0]);
+    return e;
+}
+
+// Runs a step in three parts: `head` and `tail` enqueue the launches that see a caller's pointers or the step's number, `body`
+// those that work on session buffers only and are the same every time for the same plans.  From the kGraphAfter-th step of a kind
+// on it is one graph launch, before which the head's and tail's nodes get this call's arguments: a step of small kernels is
+// bound by enqueueing them (18 launches of a tiny step: 80 to 160 us of host time, by the host; as a graph 30), and the device
+// loses less between two nodes than between two launches (8 layers at 104 rows 1184 -> 1137 us).  Recording and instantiating costs 1
+// to 3 ms, which a session that runs a few steps does not get back.  The graph belongs to the session and its plans; profiling
+// and a caller's own stream capture get the plain launches.
+constexpr int kGraphAfter = 16;
+constexpr size_t kMaxGraphs = 32;
+struct StepMode {
+    bool plain = false;                      // never as a graph
+    // head and tail see nothing of a caller's either: their arguments need not be set as long as these bytes are those recorded with
+    // (a graph whose nodes have just been changed costs the device ~15 us more to start)
+    const std::vector<char> *fixed = nullptr;
+};
+template <typename Head, typename Body, typename Tail>
+static int32_t run_step(sfs_session *s, const StepKey &key, const StepMode &mode, cudaStream_t st, Head &&head, Body &&body, Tail &&tail)
+{
+    auto enqueue = [&](cudaStream_t q, NodeSink *sink) -> int32_t {
+        g_node_sink = sink;
+        int32_t rc = head(q);
+        g_node_sink = nullptr;
+        if (rc == SFS_OK && !(sink && sink->exec)) rc = body(q);
+        if (rc != SFS_OK) return rc;
+        g_node_sink = sink;
+        rc = tail(q);
+        g_node_sink = nullptr;
+        return rc;
+    };
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (s->profile || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return enqueue(st);
-    BodyGraph &g = s->graphs[key];
+    if (mode.plain || s->profile || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return enqueue(st, nullptr);
+    if (s->graphs.size() >= kMaxGraphs && s->graphs.find(key) == s->graphs.end()) drop_graphs(s);
+    StepGraph &g = s->graphs[key];
+    if (mode.fixed && g.exec && g.sig != *mode.fixed) {      // recorded for other parameters: start over
+        cudaGraphExecDestroy(g.exec);
+        cudaGraphDestroy(g.graph);
+        g = StepGraph();
+    }
+    const long long before = s->launches;
     if (g.exec == nullptr) {
-        if (g.uses < 0 || ++g.uses < kGraphAfter) return enqueue(st);
+        if (g.uses < 0 || ++g.uses < kGraphAfter) return enqueue(st, nullptr);
         g.uses = -1;                                        // one attempt: if it fails the launches stay plain
-        if (s->record_stream == nullptr && cudaStreamCreateWithFlags(&s->record_stream, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-        if (cudaStreamBeginCapture(s->record_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return enqueue(st); }
-        const long long before = s->launches;
-        const int32_t rc = enqueue(s->record_stream);
+        if (s->record_stream == nullptr && cudaStreamCreateWithFlags(&s->record_stream, cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); return enqueue(st, nullptr); }
+        if (cudaStreamBeginCapture(s->record_stream, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return enqueue(st, nullptr); }
+        NodeSink sink;
+        sink.nodes = &g.nodes;
+        if (mode.fixed) g.sig = *mode.fixed;
+        const int32_t rc = enqueue(s->record_stream, mode.fixed ? nullptr : &sink);
         g.kernels = s->launches - before;
         s->launches = before;
-        cudaGraph_t graph = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(s->record_stream, &graph);
-        if (rc != SFS_OK || e != cudaSuccess || cudaGraphInstantiate(&g.exec, graph, 0) != cudaSuccess) g.exec = nullptr;
-        if (graph) cudaGraphDestroy(graph);
+        const cudaError_t e = cudaStreamEndCapture(s->record_stream, &g.graph);
+        if (rc != SFS_OK || e != cudaSuccess || cudaGraphInstantiate(&g.exec, g.graph, 0) != cudaSuccess) g.exec = nullptr;
         cudaGetLastError();
-        if (g.exec == nullptr) return enqueue(st);
+        if (g.exec == nullptr) return enqueue(st, nullptr);
+    } else if (!mode.fixed) {
+        NodeSink sink;
+        sink.exec = g.exec; sink.nodes = &g.nodes;
+        const int32_t rc = enqueue(st, &sink);
+        s->launches = before;
+        if (rc != SFS_OK || sink.next != g.nodes.size()) {   // the arguments do not fit the recorded nodes: plain launches from now on
+            cudaGetLastError();
+            cudaGraphExecDestroy(g.exec);
+            g.exec = nullptr; g.uses = -1;
+            return enqueue(st, nullptr);
+        }
     }
     SFS_CUDA(cudaGraphLaunch(g.exec, st));
     s->launches += g.kernels;
     return SFS_OK;
 }
 
-// the transformer body: tokens -> residual stream x [T, d]
-static int32_t run_body(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, const int32_t *d_active, cudaStream_t st)
+// One step through the transformer: tokens -> residual stream x [T, d], then `tail` (final norm, LM head and what follows)
+template <typename Tail>
+static int32_t run_uncached(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, const int32_t *d_active, long long tail_kind, const StepMode &mode, cudaStream_t st,
+                            Tail &&tail)
 {
     const sfs_model *m = s->model;
     const sfs_config &c = m->cfg;
     const int T = B * S, d = c.d_model;
     int32_t *err = device_status_word();
     SFS_REQUIRE(err != nullptr, SFS_ERR_OOM, "cannot allocate the device status word");
-    int32_t rc;
-    if ((rc = timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed_norm(d_tokens, m->tok_emb, c.vocab, s->x, m->attn_norm[0], s->h, T, d, c.rms_eps, nullptr, nullptr, 0, st); })) != SFS_OK) return rc;
     // A split-K projection leaves its partial products in s->partial; the next RMSNorm folds them into x.
     const long long pstride = (long long)T * d;
-    rc = run_recorded(s, d_active ? 1 : 0, st, [&](cudaStream_t st) -> int32_t {
+    const LayerPlans &last = s->layer_plans[c.n_layers - 1];
+    s->pending_ptr = s->partial; s->pending_n = last.down.args.splits > 1 ? last.down.args.splits : 0; s->pending_stride = pstride;      // for the final RMSNorm
+    auto head = [&](cudaStream_t st) {
+        return timed_launch(s, SFS_K_EMBED, st, [&] { return launch_embed_norm(d_tokens, m->tok_emb, c.vocab, s->x, m->attn_norm[0], s->h, T, d, c.rms_eps, nullptr, nullptr, 0, st); });
+    };
+    auto body = [&](cudaStream_t st) -> int32_t {
         int32_t rc;
         int pending = 0;
         for (int l = 0; l < c.n_layers; ++l) {
@@ -238,12 +296,8 @@ static int32_t run_body(sfs_session *s, const int32_t *d_tokens, int32_t B, int3
             pending = lp.down.args.splits > 1 ? lp.down.args.splits : 0;
         }
         return SFS_OK;
-    });
-    if (rc != SFS_OK) return rc;
-    const LayerPlans &last = s->layer_plans[c.n_layers - 1];
-    const int pending = last.down.args.splits > 1 ? last.down.args.splits : 0;
-    s->pending_ptr = s->partial; s->pending_n = pending; s->pending_stride = pstride;      // for the final RMSNorm of the caller
-    return SFS_OK;
+    };
+    return run_step(s, StepKey{0, tail_kind, d_active ? 1 : 0, 0, 0}, mode, st, head, body, tail);
 }
 
 // ---- cached steps --------------------------------------------------------------------------------------
@@ -316,9 +370,10 @@ static int32_t gather_plan(sfs_session *s, int32_t NR, int32_t T, std::vector<Ga
 }
 
 // One cached step of the transformer body (the rule is stated with sfs_cache_params in sfs.h): tokens -> x [T, d],
-// leaving the last layer's MLP increment pending for the caller's final RMSNorm.
-static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, int32_t P, const sfs_state *d_state,
-                               const int32_t *d_active, int32_t *d_sets, float *d_sims, int32_t *n_sel_out, cudaStream_t st)
+// leaving the last layer's MLP increment pending for the final RMSNorm in `tail`.
+template <typename Tail>
+static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, int32_t P, const sfs_state *d_state, const int32_t *d_active,
+                          int32_t *d_sets, float *d_sims, int32_t *n_sel_out, long long tail_kind, const StepMode &mode, cudaStream_t st, Tail &&tail)
 {
     const sfs_model *m = s->model;
     const sfs_config &c = m->cfg;
@@ -350,12 +405,11 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
     // tokens whose fresh values are compared with the cached ones: the response of a single sequence (from an even index), else all
     const int sim_first = (B == 1) ? (P & ~1) : 0, sim_count = (B == 1) ? S - sim_first : T;
     // the first layer's norm of those rows embeds their tokens (and brings the states to where the body expects them)
-    rc = timed_launch(s, SFS_K_EMBED, st, [&] {
+    auto head = [&](cudaStream_t st) { return timed_launch(s, SFS_K_EMBED, st, [&] {
         return launch_embed_norm(d_tokens + r_first, m->tok_emb, c.vocab, s->x + (size_t)r_first * d, m->attn_norm[0], s->h + (size_t)r_first * d, r_count, d,
                                  c.rms_eps, reinterpret_cast<const int32_t *>(d_state), reinterpret_cast<int32_t *>(s->state_in),
                                  d_state ? B * (int)(sizeof(sfs_state) / 4) : 0, st);
-    });
-    if (rc != SFS_OK) return rc;
+    }); };
     const sfs_state *state = d_state ? s->state_in : nullptr;
     std::vector<GatherLayerPlans> *gps = nullptr;
     if (!(rp && rr) && NR > 0 && (rc = gather_plan(s, NR, T, &gps)) != SFS_OK) return rc;
@@ -436,14 +490,12 @@ static int32_t run_body_cached(sfs_session *s, const int32_t *d_tokens, int32_t 
         }
         return SFS_OK;
     };
-    // (a dump writes to the caller's buffers: not recorded)
-    const long long key = 2 + ((((long long)n_sel * 2 + rp) * 2 + rr) * 2 + (d_state ? 1 : 0)) * 2 + (d_active ? 1 : 0);
-    if (d_sets || d_sims) rc = body(st);
-    else rc = run_recorded(s, key, st, body);
-    if (rc != SFS_OK) return rc;
     // what the last layer leaves pending: its MLP increment, or both increments
-    pend = (rp && rr) ? s->Fc[c.n_layers - 1] : s->Ac[c.n_layers - 1];
-    s->pending_ptr = pend; s->pending_n = (rp && rr) ? 1 : 2; s->pending_stride = inc_stride;
+    s->pending_ptr = (rp && rr) ? s->Fc[c.n_layers - 1] : s->Ac[c.n_layers - 1];
+    s->pending_n = (rp && rr) ? 1 : 2; s->pending_stride = inc_stride;
+    // (a dump writes to the caller's buffers: not recorded)
+    const StepKey key{1, tail_kind, d_active ? 1 : 0, n_sel, (rp ? 1 : 0) + (rr ? 2 : 0) + (d_state ? 4 : 0)};
+    if ((rc = run_step(s, key, {mode.plain || d_sets || d_sims, mode.fixed}, st, head, body, tail)) != SFS_OK) return rc;
     s->cache_t++;
     return SFS_OK;
 }
@@ -462,7 +514,7 @@ __global__ void generate_init_kernel(const int32_t *prompt, int32_t *tokens, uin
     }
     for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < B; b += gridDim.x * blockDim.x) state[b] = initial_state(L, max_steps);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        ctrl[0] = B * L; ctrl[1] = 0; ctrl[2] = (L > 0) ? B : 0;
+        ctrl[0] = B * L; ctrl[2] = (L > 0) ? B : 0; ctrl[3] = 0;
         *host_active = (L > 0) ? B : 0;
     }
 }
@@ -600,8 +652,7 @@ int32_t sfs_session_create(sfs_model *m, int32_t max_batch, int32_t max_seq, sfs
     if ((rc = dev_alloc(s, &s->tokens, T, true)) != SFS_OK) return fail(rc);
     if ((rc = dev_alloc(s, &s->mask, T, true)) != SFS_OK) return fail(rc);
     if ((rc = dev_alloc(s, &s->state, (size_t)max_batch, true)) != SFS_OK) return fail(rc);
-    if ((rc = dev_alloc(s, &s->rows[0], T, true)) != SFS_OK) return fail(rc);
-    if ((rc = dev_alloc(s, &s->rows[1], T, true)) != SFS_OK) return fail(rc);
+    if ((rc = dev_alloc(s, &s->rows, T, true)) != SFS_OK) return fail(rc);
     if ((rc = dev_alloc(s, &s->ctrl, 16, true)) != SFS_OK) return fail(rc);
     if (cudaHostAlloc(reinterpret_cast<void **>(&s->host_active), 64 + (size_t)max_batch * sizeof(sfs_state), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer(reinterpret_cast<void **>(&s->host_active_dev), s->host_active, 0) != cudaSuccess) {
@@ -614,6 +665,26 @@ int32_t sfs_session_create(sfs_model *m, int32_t max_batch, int32_t max_seq, sfs
     if (cudaDeviceSynchronize() != cudaSuccess) { set_error("device synchronisation failed after session set-up"); return fail(SFS_ERR_CUDA); }
     *out = s;
     return SFS_OK;
+}
+
+// the end of a forward call: listed rows -> final norm -> LM head into the caller's logits
+static int32_t logits_plan(sfs_session *s, GemmPlan *lm, int32_t max_rows, void *d_logits, int32_t logits_dtype)
+{
+    const sfs_config &c = s->model->cfg;
+    const void *lmw[1] = {s->model->lm_head};
+    return weight_plan_create(lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
+                              logits_dtype == SFS_LOGITS_F32 ? 1 : 0, c.logit_scale, nullptr, 0, 0, nullptr);
+}
+static long long logits_kind(int32_t max_rows, int32_t logits_dtype, const int32_t *d_n_rows)
+{
+    return ((long long)max_rows * 2 + (logits_dtype == SFS_LOGITS_F32 ? 1 : 0)) * 2 + (d_n_rows ? 1 : 0);
+}
+static int32_t enqueue_logits(sfs_session *s, const GemmPlan &lm, const int32_t *d_rows, const int32_t *d_n_rows, int32_t max_rows, cudaStream_t st)
+{
+    const sfs_config &c = s->model->cfg;
+    int32_t rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, d_rows, d_n_rows, max_rows, c.d_model, c.rms_eps, st); });
+    if (rc != SFS_OK) return rc;
+    return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(lm, d_n_rows, nullptr, device_status_word(), st); });
 }
 
 // ---- single steps ---------------------------------------------------------------------------------------
@@ -630,17 +701,12 @@ int32_t sfs_forward(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t 
     SFS_REQUIRE(d_rows != nullptr || (max_rows == B * S && d_n_rows == nullptr), SFS_ERR_INVALID_ARG,
                 "forward: without a row list all B*S rows are produced");
     cudaStream_t st = (cudaStream_t)stream;
-    const sfs_config &c = s->model->cfg;
     int32_t rc = session_plan(s, B, S);
     if (rc != SFS_OK) return rc;
-    if ((rc = run_body(s, d_tokens, B, S, nullptr, st)) != SFS_OK) return rc;
-    if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, d_rows, d_n_rows, max_rows, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
     GemmPlan lm;
-    const void *lmw[1] = {s->model->lm_head};
-    rc = weight_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
-                          logits_dtype == SFS_LOGITS_F32 ? 1 : 0, c.logit_scale, nullptr, 0, 0, nullptr);
-    if (rc != SFS_OK) return rc;
-    return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(lm, d_n_rows, nullptr, device_status_word(), st); });
+    if ((rc = logits_plan(s, &lm, max_rows, d_logits, logits_dtype)) != SFS_OK) return rc;
+    return run_uncached(s, d_tokens, B, S, nullptr, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
+                        [&](cudaStream_t st) { return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st); });
 }
 
 int32_t sfs_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
@@ -766,16 +832,11 @@ int32_t sfs_forward_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, i
     SFS_REQUIRE(d_rows != nullptr || (max_rows == B * S && d_n_rows == nullptr), SFS_ERR_INVALID_ARG,
                 "forward_cached: without a row list all B*S rows are produced");
     cudaStream_t st = (cudaStream_t)stream;
-    const sfs_config &c = s->model->cfg;
-    int32_t rc = run_body_cached(s, d_tokens, B, S, P, d_state, nullptr, d_sets, d_sims, n_sel, st);
-    if (rc != SFS_OK) return rc;
-    if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, d_rows, d_n_rows, max_rows, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
     GemmPlan lm;
-    const void *lmw[1] = {s->model->lm_head};
-    rc = weight_plan_create(&lm, s->hfin, c.d_model, max_rows, c.d_model, lmw, 1, c.vocab, c.d_model, GEMM_STORE, d_logits, c.vocab,
-                          logits_dtype == SFS_LOGITS_F32 ? 1 : 0, c.logit_scale, nullptr, 0, 0, nullptr);
+    const int32_t rc = logits_plan(s, &lm, max_rows, d_logits, logits_dtype);
     if (rc != SFS_OK) return rc;
-    return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(lm, d_n_rows, nullptr, device_status_word(), st); });
+    return run_cached(s, d_tokens, B, S, P, d_state, nullptr, d_sets, d_sims, n_sel, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
+                      [&](cudaStream_t st) { return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st); });
 }
 
 // ---- the whole loop -------------------------------------------------------------------------------------
@@ -814,10 +875,10 @@ int32_t sfs_generate_begin(sfs_session *s, const int32_t *d_prompt, int32_t B, i
             s->lm_plan.args.stats = s->lm_stats; s->lm_plan.args.stats_ld = parts;
         }
     }
-    generate_init_kernel<<<64, 256, 0, st>>>(d_prompt, s->tokens, s->mask, s->rows[0], s->ctrl, s->host_active_dev, s->pos_sq,
+    generate_init_kernel<<<64, 256, 0, st>>>(d_prompt, s->tokens, s->mask, s->rows, s->ctrl, s->host_active_dev, s->pos_sq,
                                              s->state, params->max_steps, B, P, gen_len, s->model->cfg.mask_id);
     SFS_LAUNCH_CHECK();
-    s->gen_B = B; s->gen_P = P; s->gen_L = gen_len; s->gen_cur = 0; s->gen_steps = 0;
+    s->gen_B = B; s->gen_P = P; s->gen_L = gen_len; s->gen_steps = 0;
     s->gen_max_steps = params->max_steps > 0 ? params->max_steps : gen_len;
     s->gen_params = *params;
     s->cache_t = 0;                                          // a new generation starts with a full refresh
@@ -839,32 +900,42 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
     int32_t rc;
     for (int i = 0; i < n_steps; ++i) {
         if (s->gen_steps >= s->gen_max_steps) break;                 // every sequence is done by construction
-        const int cur = s->gen_cur, nxt = cur ^ 1;
-        const int32_t *d_active = s->ctrl + 2;
-        const int32_t *rows = s->rows[cur], *n_rows = s->ctrl + cur;
-        if (s->cache_on) rc = run_body_cached(s, s->tokens, B, S, P, s->state, d_active, s->dump_sets, s->dump_sims, nullptr, st);
-        else rc = run_body(s, s->tokens, B, S, d_active, st);
-        if (rc != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, rows, n_rows, B * L, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(s->lm_plan, n_rows, d_active, err, st); })) != SFS_OK) return rc;
-        if (d_logits_dump) {
-            SFS_CUDA(cudaMemcpyAsync(d_logits_dump, s->logits, (size_t)B * L * c.vocab * 2, cudaMemcpyDeviceToDevice, st));
-            if (d_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_rows_dump, rows, (size_t)B * L * 4, cudaMemcpyDeviceToDevice, st));
-            if (d_n_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_n_rows_dump, n_rows, 4, cudaMemcpyDeviceToDevice, st));
+        const int32_t *d_active = s->ctrl + 2, *rows = s->rows, *n_rows = s->ctrl;
+        // final norm, LM head, row statistics, selection
+        auto tail = [&](cudaStream_t st) -> int32_t {
+            int32_t rc;
+            if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, rows, n_rows, B * L, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
+            if ((rc = timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(s->lm_plan, n_rows, d_active, err, st); })) != SFS_OK) return rc;
+            if (d_logits_dump) {
+                SFS_CUDA(cudaMemcpyAsync(d_logits_dump, s->logits, (size_t)B * L * c.vocab * 2, cudaMemcpyDeviceToDevice, st));
+                if (d_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_rows_dump, rows, (size_t)B * L * 4, cudaMemcpyDeviceToDevice, st));
+                if (d_n_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_n_rows_dump, n_rows, 4, cudaMemcpyDeviceToDevice, st));
+            }
+            SelectArgs a{};
+            if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
+                     return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, &s->lm_plan.args); })) != SFS_OK) return rc;
+            a.tokens = s->tokens; a.mask = s->mask; a.B = B; a.S = S; a.P = P; a.L = L;
+            a.state = s->state; a.params = s->gen_params;
+            a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;
+            a.seq_rows = s->seq_rows; a.seq_row_count = s->seq_row_count;
+            a.next_rows = s->rows; a.next_n_rows = s->ctrl; a.n_active = s->ctrl + 2;
+            a.ticket = s->ticket;
+            a.trace = (d_trace && s->gen_steps < max_trace_steps) ? d_trace + (size_t)s->gen_steps * B * SFS_TRACE_INTS : nullptr;
+            a.host_active = s->host_active_dev; a.step_count = s->ctrl + 3;
+            return timed_launch(s, SFS_K_SELECT, st, [&] { return launch_select(a, st); });
+        };
+        // (the tails of forward calls have kinds >= 0; without a trace a step's launches are all the same within a generation)
+        const long long kind = -2 * L - (d_trace ? 1 : 2);
+        std::vector<char> fixed;
+        if (!d_trace) {
+            const void *stats = s->lm_plan.args.stats;
+            fixed.assign(reinterpret_cast<const char *>(&s->gen_params), reinterpret_cast<const char *>(&s->gen_params) + sizeof(s->gen_params));
+            fixed.insert(fixed.end(), reinterpret_cast<const char *>(&stats), reinterpret_cast<const char *>(&stats) + sizeof(stats));
         }
-        SelectArgs a{};
-        if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
-                 return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, &s->lm_plan.args); })) != SFS_OK) return rc;
-        a.tokens = s->tokens; a.mask = s->mask; a.B = B; a.S = S; a.P = P; a.L = L;
-        a.state = s->state; a.params = s->gen_params;
-        a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;
-        a.seq_rows = s->seq_rows; a.seq_row_count = s->seq_row_count;
-        a.next_rows = s->rows[nxt]; a.next_n_rows = s->ctrl + nxt; a.n_active = s->ctrl + 2;
-        a.ticket = s->ticket;
-        a.trace = (d_trace && s->gen_steps < max_trace_steps) ? d_trace + (size_t)s->gen_steps * B * SFS_TRACE_INTS : nullptr;
-        a.host_active = s->host_active_dev; a.host_step = s->gen_steps + 1;
-        if ((rc = timed_launch(s, SFS_K_SELECT, st, [&] { return launch_select(a, st); })) != SFS_OK) return rc;
-        s->gen_cur = nxt;
+        const StepMode mode = {d_logits_dump != nullptr, d_trace ? nullptr : &fixed};
+        if (s->cache_on) rc = run_cached(s, s->tokens, B, S, P, s->state, d_active, s->dump_sets, s->dump_sims, nullptr, kind, mode, st, tail);
+        else rc = run_uncached(s, s->tokens, B, S, d_active, kind, mode, st, tail);
+        if (rc != SFS_OK) return rc;
         s->gen_steps++;
     }
     return SFS_OK;

@@ -3,6 +3,7 @@
 #include "sfs_common.cuh"
 #include "gemm.cuh"
 #include "attention.cuh"
+#include <array>
 #include <vector>
 #include <map>
 
@@ -19,8 +20,9 @@ struct CacheLayerPlans { sfs::GemmPlan qkv_store, vproj, o_store, down_store; sf
 // cached mode: projections over the compact buffer of recomputed rows, per layer, for one row count
 struct GatherLayerPlans { sfs::GemmPlan qkv, o, gate_up, down; };
 
-// A transformer body as a CUDA graph: recorded once the same body has been run kGraphAfter times, replayed from then on
-struct BodyGraph { cudaGraphExec_t exec = nullptr; int uses = 0; long long kernels = 0; };
+// A step as a CUDA graph: recorded once steps of the same shape have been run kGraphAfter times, replayed from then on
+typedef std::array<long long, 5> StepKey;
+struct StepGraph { cudaGraph_t graph = nullptr; cudaGraphExec_t exec = nullptr; std::vector<cudaGraphNode_t> nodes; std::vector<char> sig; int uses = 0; long long kernels = 0; };
 
 struct sfs_session {
     sfs_model *model = nullptr;          // NULL: a selection-only session
@@ -50,8 +52,8 @@ struct sfs_session {
     int32_t *tokens = nullptr;               // [T]
     uint8_t *mask = nullptr;                 // [T]
     sfs_state *state = nullptr;              // [max_batch]
-    int32_t *rows[2] = {nullptr, nullptr};   // [T] row lists of the current / next step
-    int32_t *ctrl = nullptr;                 // [0..1] row counts (double buffer), [2] active sequences
+    int32_t *rows = nullptr;                 // [T] row list of the step (the selection, a step's last kernel, writes the next one)
+    int32_t *ctrl = nullptr;                 // [0] its row count, [2] active sequences, [3] steps finished
     int32_t *host_active = nullptr;          // pinned, device-mapped: [0] mirror of ctrl[2], [1] steps finished, [2] status word, [16..] states at the end
     int32_t *host_active_dev = nullptr;      // its device address
     // plans for the shapes of the current call
@@ -60,7 +62,7 @@ struct sfs_session {
     sfs::AttnPlan attn_plan;
     sfs::GemmPlan lm_plan;
     float4 *lm_stats = nullptr; size_t lm_stats_cap = 0;     // row-statistics records the LM head's epilogue leaves (fused first pass)
-    std::map<long long, BodyGraph> graphs;   // by kind of body; dropped with the plans they were recorded from
+    std::map<StepKey, StepGraph> graphs;     // by kind of step; dropped with the plans they were recorded from
     cudaStream_t record_stream = nullptr;    // recording happens here, never on a caller's stream
     sfs_state *state_in = nullptr;           // [max_batch] the caller's scheduler states, where a recorded body finds them
     // what the next RMSNorm must fold into x: n slabs `pending_stride` floats apart (split-K partials or a cached increment)
@@ -79,7 +81,7 @@ struct sfs_session {
     std::vector<CacheLayerPlans> cache_plans;
     std::map<int, std::vector<GatherLayerPlans>> gather_plans;
     // generation bookkeeping (host)
-    int32_t gen_B = 0, gen_P = 0, gen_L = 0, gen_cur = 0, gen_steps = 0, gen_max_steps = 0;
+    int32_t gen_B = 0, gen_P = 0, gen_L = 0, gen_steps = 0, gen_max_steps = 0;
     sfs_params gen_params;
     bool generating = false;
     std::vector<void *> owned;               // device allocations to free at destroy

@@ -74,7 +74,7 @@ __device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int
     if (a.host_active) {
         a.host_active[0] = n_active;                        // before the step count: who sees the step sees whether it was the last
         __threadfence_system();
-        a.host_active[1] = a.host_step;
+        a.host_active[1] = ++*a.step_count;
     }
 }
 

@@ -6,6 +6,9 @@
 #include <stdint.h>
 #include <stdio.h>
 #include <stdarg.h>
+#include <tuple>
+#include <utility>
+#include <vector>
 
 #include "../../include/sfs.h"
 
@@ -54,21 +57,54 @@ int32_t *device_status_word_if_any();
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Launches whose arguments change from call to call (a caller's pointers, step counts) inside a recorded graph: while a sink is
+// installed on the thread, launch_pdl either notes the node it has just recorded, or sets that node's arguments instead of launching.
+struct NodeSink {
+    cudaGraphExec_t exec = nullptr;          // NULL: recording
+    std::vector<cudaGraphNode_t> *nodes = nullptr;
+    size_t next = 0;
+};
+inline thread_local NodeSink *g_node_sink = nullptr;
+cudaError_t note_recorded_node(NodeSink *sink, cudaStream_t stream);
+template <typename Tuple, size_t... I>
+static inline cudaError_t set_node_args(NodeSink *sink, void *kernel, dim3 grid, dim3 block, size_t smem, Tuple &vals, std::index_sequence<I...>)
+{
+    void *ptrs[] = {(void *)&std::get<I>(vals)...};
+    cudaKernelNodeParams p = {};
+    p.func = kernel; p.gridDim = grid; p.blockDim = block; p.sharedMemBytes = (unsigned)smem; p.kernelParams = ptrs;
+    if (sink->next >= sink->nodes->size()) return cudaErrorInvalidValue;
+    return cudaGraphExecKernelNodeSetParams(sink->exec, (*sink->nodes)[sink->next++], &p);
+}
+template <typename... KArgs, typename... Args>
+static inline bool redirect_launch(cudaError_t *e, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args)
+{
+    if (g_node_sink == nullptr || g_node_sink->exec == nullptr) return false;
+    std::tuple<KArgs...> vals{static_cast<KArgs>(args)...};
+    *e = set_node_args(g_node_sink, (void *)kernel, grid, block, smem, vals, std::index_sequence_for<KArgs...>());
+    return true;
+}
+
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
 {
+    cudaError_t e;
+    if (redirect_launch(&e, kernel, grid, block, smem, args...)) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    return (e == cudaSuccess && g_node_sink) ? note_recorded_node(g_node_sink, stream) : e;
 }
 // the same with clusters of `cluster` CTAs
 template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args... args)
 {
+    cudaError_t e;
+    if (redirect_launch(&e, kernel, grid, block, smem, args...)) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr[2];
@@ -77,7 +113,8 @@ static inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), int clust
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr; cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    e = cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+    return (e == cudaSuccess && g_node_sink) ? note_recorded_node(g_node_sink, stream) : e;
 }
 #endif
 
@@ -223,7 +260,7 @@ struct SelectArgs {
     int32_t *n_active;                                      // optional: sequences not done after this step
     int32_t *ticket;                                        // scratch counter (zero between launches)
     int32_t *trace;                                         // optional [B, SFS_TRACE_INTS]
-    int32_t *host_active; int32_t host_step;                // optional: the host's mirror, and the step count to leave there
+    int32_t *host_active, *step_count;                      // optional: the host's mirror, and the device's count of steps
 };
 int32_t launch_select(const SelectArgs &a, cudaStream_t stream);
 int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, int32_t *seq_rows_unused,
