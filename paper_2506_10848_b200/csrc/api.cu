@@ -6,6 +6,7 @@
 #include "attention.cuh"
 #include "elementwise.cuh"
 #include "cache.cuh"
+#include "small_gemm.cuh"
 #include <math.h>
 
 #include <new>
@@ -262,6 +263,78 @@ static int32_t run_step(sfs_session *s, const StepKey &key, const StepMode &mode
     return SFS_OK;
 }
 
+// Small models and few rows take kernels that do the row-wise work of the neighbours too (see small_gemm.cu), up to seven or so tiles
+// of the widest projection per SM: a whole step of the 2-layer d 256, d_ff 688 model takes, us against the tensor-memory kernels,
+// 64 rows 55 / 71, 256 63 / 83, 448 75 / 87, 768 97 / 105, 1024 105 / 103, 2048 167 / 120.
+static bool small_step(const sfs_config &c, int rows)
+{
+    return small_gemm_fits(c.d_model, c.d_ff, c.head_dim) && (long long)((rows + 31) / 32) * ((c.d_ff + 15) / 16) <= 1056;
+}
+static SmallGemmArgs small_args(sfs_session *s, int M, int N, int K, const int32_t *d_active)
+{
+    const sfs_config &c = s->model->cfg;
+    SmallGemmArgs g{};
+    g.M = M; g.N = N; g.K = K; g.d_active = d_active; g.x = s->x; g.eps = c.rms_eps; g.head_dim = c.head_dim; g.n_per_map = N; g.scale = 1.0f;
+    return g;
+}
+static const __nv_bfloat16 *bf(const void *p) { return reinterpret_cast<const __nv_bfloat16 *>(p); }
+// `cache`: the step also fills the feature cache (keys, values and both increments of every layer)
+static int32_t small_qkv(sfs_session *s, int l, int B, int S, const int32_t *d_tokens, const int32_t *d_active, bool cache, cudaStream_t st)
+{
+    const sfs_model *m = s->model;
+    const sfs_config &c = m->cfg;
+    SmallGemmArgs g = small_args(s, B * S, 0, c.d_model, d_active);
+    g.n_per_map = c.d_model; g.gain = bf(m->attn_norm[l]); g.B[0] = bf(m->wq[l]); g.B[1] = bf(m->wk[l]); g.B[2] = bf(m->wv[l]);
+    g.out = s->qk; g.ldc = 2 * c.d_model; g.vt = s->vt; g.ldvt = B * S; g.table = s->rope_table; g.S = S;
+    g.tokens = d_tokens; g.emb = bf(m->tok_emb); g.vocab = c.vocab;
+    if (cache) { g.k_dst = s->Kc[l]; g.vt = s->Vtc[l]; }
+    return launch_small_gemm(d_tokens ? SMALL_EMBED : SMALL_NORM, SMALL_QKV, g, st);
+}
+static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active, bool cache, cudaStream_t st)
+{
+    const sfs_model *m = s->model;
+    const sfs_config &c = m->cfg;
+    const int T = B * S, d = c.d_model, ff = c.d_ff;
+    int32_t rc;
+    for (int l = 0; l < c.n_layers; ++l) {
+        if (l > 0 && (rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, l, B, S, nullptr, d_active, cache, st); })) != SFS_OK) return rc;
+        if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(cache ? s->cache_plans[l].attn : s->attn_plan, d_active, device_status_word(), st); })) != SFS_OK) return rc;
+        rc = timed_launch(s, SFS_K_GEMM_O, st, [&] {
+            SmallGemmArgs g = small_args(s, T, d, d, d_active);
+            g.a = s->attn; g.lda = d; g.B[0] = bf(m->wo[l]); g.inc = cache ? s->Ac[l] : nullptr;
+            return launch_small_gemm(SMALL_BF16, SMALL_RESIDUAL, g, st);
+        });
+        if (rc != SFS_OK) return rc;
+        rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] {
+            SmallGemmArgs g = small_args(s, T, ff, d, d_active);
+            g.gain = bf(m->mlp_norm[l]); g.B[0] = bf(m->w_gate[l]); g.B[1] = bf(m->w_up[l]); g.out = s->hid; g.ldc = ff;
+            return launch_small_gemm(SMALL_NORM, SMALL_SWIGLU, g, st);
+        });
+        if (rc != SFS_OK) return rc;
+        rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] {
+            SmallGemmArgs g = small_args(s, T, d, ff, d_active);
+            g.a = s->hid; g.lda = ff; g.B[0] = bf(m->w_down[l]); g.inc = cache ? s->Fc[l] : nullptr;
+            return launch_small_gemm(SMALL_BF16, SMALL_RESIDUAL, g, st);
+        });
+        if (rc != SFS_OK) return rc;
+    }
+    return SFS_OK;
+}
+// final norm + LM head of up to max_rows listed rows in one launch, for vocabularies whose statistics the LM head does not take
+static bool small_logits(const sfs_config &c, int max_rows, int T) { return small_step(c, max_rows) && small_step(c, T) && c.vocab <= 16384; }
+static int32_t enqueue_small_logits(sfs_session *s, const int32_t *d_rows, const int32_t *d_n_rows, int max_rows, void *d_logits, int32_t logits_dtype,
+                                    const int32_t *d_active, cudaStream_t st)
+{
+    const sfs_config &c = s->model->cfg;
+    return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] {
+        SmallGemmArgs g = small_args(s, max_rows, c.vocab, c.d_model, d_active);
+        g.d_m = d_n_rows; g.rows = d_rows; g.gain = bf(s->model->final_norm); g.B[0] = bf(s->model->lm_head); g.scale = c.logit_scale; g.ldc = c.vocab;
+        if (logits_dtype == SFS_LOGITS_F32) g.out_f32 = reinterpret_cast<float *>(d_logits);
+        else g.out = reinterpret_cast<__nv_bfloat16 *>(d_logits);
+        return launch_small_gemm(SMALL_NORM, SMALL_STORE, g, st);
+    });
+}
+
 // One step through the transformer: tokens -> residual stream x [T, d], then `tail` (final norm, LM head and what follows)
 template <typename Tail>
 static int32_t run_uncached(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t S, const int32_t *d_active, long long tail_kind, const StepMode &mode, cudaStream_t st,
@@ -297,6 +370,12 @@ static int32_t run_uncached(sfs_session *s, const int32_t *d_tokens, int32_t B, 
         }
         return SFS_OK;
     };
+    if (small_step(c, T)) {
+        s->pending_n = 0;
+        return run_step(s, StepKey{0, tail_kind, d_active ? 1 : 0, 0, 0}, mode, st,
+                        [&](cudaStream_t st) { return timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, 0, B, S, d_tokens, d_active, false, st); }); },
+                        [&](cudaStream_t st) { return small_body(s, B, S, d_active, false, st); }, tail);
+    }
     return run_step(s, StepKey{0, tail_kind, d_active ? 1 : 0, 0, 0}, mode, st, head, body, tail);
 }
 
@@ -415,6 +494,11 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
     if (!(rp && rr) && NR > 0 && (rc = gather_plan(s, NR, T, &gps)) != SFS_OK) return rc;
     const long long inc_stride = (rp && rr) ? 0 : (long long)s->max_batch * s->max_seq * d;     // A_l -> F_l
     int n_pend = 0;
+    auto dump_all = [&](int l, cudaStream_t st) {          // a full refresh's dump lists every token
+        CacheSelectArgs a{}; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T; a.refresh_p = 1; a.refresh_r = 1; a.n_sel = S;
+        a.sel_rows = d_sets + (size_t)l * B * S;
+        return launch_cache_select(a, st);
+    };
     auto body = [&](cudaStream_t st) -> int32_t {
         int32_t rc = SFS_OK;
         pend = nullptr; n_pend = 0;
@@ -439,11 +523,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
                 if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return gemm_launch(lp.gate_up, nullptr, d_active, err, st); })) != SFS_OK) return rc;
                 if ((rc = timed_launch(s, SFS_K_GEMM_DOWN, st, [&] { return gemm_launch(cl.down_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
                 pend = s->Fc[l];
-                if (d_sets) {   // the dump lists every token
-                    CacheSelectArgs a{}; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T; a.refresh_p = 1; a.refresh_r = 1; a.n_sel = S;
-                    a.sel_rows = d_sets + (size_t)l * B * S;
-                    if ((rc = launch_cache_select(a, st)) != SFS_OK) return rc;
-                }
+                if (d_sets && (rc = dump_all(l, st)) != SFS_OK) return rc;
             }
         } else {
             // Here the attention increment of a layer stays pending through its MLP branch: the MLP norm reads x + A_l for the
@@ -494,6 +574,20 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
     s->pending_ptr = (rp && rr) ? s->Fc[c.n_layers - 1] : s->Ac[c.n_layers - 1];
     s->pending_n = (rp && rr) ? 1 : 2; s->pending_stride = inc_stride;
     // (a dump writes to the caller's buffers: not recorded)
+    if (rp && rr && small_step(c, T)) {
+        // everything is recomputed: the kernels of an uncached step (also of its logits, see the callers), which fill the cache as they go
+        s->pending_n = 0;
+        rc = run_step(s, StepKey{2, tail_kind, d_active ? 1 : 0, 0, 0}, {mode.plain || d_sets || d_sims, mode.fixed}, st,
+                      [&](cudaStream_t st) { return timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, 0, B, S, d_tokens, d_active, true, st); }); },
+                      [&](cudaStream_t st) -> int32_t {
+                          int32_t rc = small_body(s, B, S, d_active, true, st);
+                          for (int l = 0; l < c.n_layers && rc == SFS_OK && d_sets; ++l) rc = dump_all(l, st);
+                          return rc;
+                      }, tail);
+        if (rc != SFS_OK) return rc;
+        s->cache_t++;
+        return SFS_OK;
+    }
     const StepKey key{1, tail_kind, d_active ? 1 : 0, n_sel, (rp ? 1 : 0) + (rr ? 2 : 0) + (d_state ? 4 : 0)};
     if ((rc = run_step(s, key, {mode.plain || d_sets || d_sims, mode.fixed}, st, head, body, tail)) != SFS_OK) return rc;
     s->cache_t++;
@@ -705,6 +799,9 @@ int32_t sfs_forward(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t 
     if (rc != SFS_OK) return rc;
     GemmPlan lm;
     if ((rc = logits_plan(s, &lm, max_rows, d_logits, logits_dtype)) != SFS_OK) return rc;
+    if (small_logits(s->model->cfg, max_rows, B * S))
+        return run_uncached(s, d_tokens, B, S, nullptr, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
+                            [&](cudaStream_t st) { return enqueue_small_logits(s, d_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st); });
     return run_uncached(s, d_tokens, B, S, nullptr, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
                         [&](cudaStream_t st) { return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st); });
 }
@@ -836,7 +933,11 @@ int32_t sfs_forward_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, i
     const int32_t rc = logits_plan(s, &lm, max_rows, d_logits, logits_dtype);
     if (rc != SFS_OK) return rc;
     return run_cached(s, d_tokens, B, S, P, d_state, nullptr, d_sets, d_sims, n_sel, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
-                      [&](cudaStream_t st) { return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st); });
+                      [&](cudaStream_t st) {
+                          if (s->pending_n == 0 && small_logits(s->model->cfg, max_rows, B * S))
+                              return enqueue_small_logits(s, d_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st);
+                          return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st);
+                      });
 }
 
 // ---- the whole loop -------------------------------------------------------------------------------------
@@ -904,8 +1005,10 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
         // final norm, LM head, row statistics, selection
         auto tail = [&](cudaStream_t st) -> int32_t {
             int32_t rc;
-            if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, rows, n_rows, B * L, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(s->lm_plan, n_rows, d_active, err, st); })) != SFS_OK) return rc;
+            if (s->pending_n == 0 && small_logits(c, B * L, B * S)) {
+                if ((rc = enqueue_small_logits(s, rows, n_rows, B * L, s->logits, SFS_LOGITS_BF16, d_active, st)) != SFS_OK) return rc;
+            } else if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, rows, n_rows, B * L, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
+            else if ((rc = timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(s->lm_plan, n_rows, d_active, err, st); })) != SFS_OK) return rc;
             if (d_logits_dump) {
                 SFS_CUDA(cudaMemcpyAsync(d_logits_dump, s->logits, (size_t)B * L * c.vocab * 2, cudaMemcpyDeviceToDevice, st));
                 if (d_rows_dump) SFS_CUDA(cudaMemcpyAsync(d_rows_dump, rows, (size_t)B * L * 4, cudaMemcpyDeviceToDevice, st));

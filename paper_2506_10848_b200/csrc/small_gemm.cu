@@ -1,0 +1,235 @@
+// Projections of small models and few rows, where a step is bound by the number and the length of its launches: each kernel takes
+// in the row-wise work before it (embedding, RMSNorm, row gather) and after it (rotary embedding, SwiGLU, residual add).
+//
+// A 64 x 256 x 256 product has 8 MFLOP; the tcgen05 kernel needs 4 us for it after its inputs are there (pair set-up, TMA round
+// trip, tensor-memory hand-overs), its norm and its rotary kernel 1.5 to 1.7 each, and every launch in a chain 1.4 us on
+// top.  Here a CTA of four warps computes a 32 x 32 tile with mma.sync from shared memory that holds all of K at once: the weight
+// rows are requested before the dependent-launch wait, the activation rows are normalised on the way in (every column tile
+// repeats that for its 32 rows, from L2), and the accumulators of a warp pair up what the epilogue needs together (gate and up,
+// the two halves of a rotary pair).  A layer is five launches instead of eight.
+// Bound: the latency of one memory round trip, K / 16 dependent MMAs and the launch.
+#include "sfs_common.cuh"
+#include "small_gemm.cuh"
+
+namespace sfs {
+namespace {
+
+constexpr int TILE = 32, kThreads = 128;
+
+__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void ldmatrix4(uint32_t *r, uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16816(float *c, const uint32_t *a, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&h);
+}
+__device__ __forceinline__ float round_bf16(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+__device__ __forceinline__ float silu(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
+
+// NCH: 16-byte chunks of a row per lane (SRC_NORM, SRC_EMBED: rows of up to NCH * 128 elements)
+template <int SRC, int EPI, int NCH>
+__global__ void __launch_bounds__(kThreads)
+small_gemm_kernel(SmallGemmArgs g)
+{
+    pdl_trigger();
+    extern __shared__ __align__(16) __nv_bfloat16 s_mem[];
+    const int K = g.K, Kp = (K + 15) & ~15, ld = Kp + 8;          // rows 16 bytes apart modulo 128: ldmatrix is conflict-free
+    __nv_bfloat16 *sA = s_mem, *sB = s_mem + TILE * ld;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockIdx.x, m0 = blockIdx.y * TILE;
+
+    // ---- which weight rows: rows 0-15 and 16-31 of the tile are the two halves the epilogue combines
+    const int half = g.head_dim / 2, tiles_per_map = g.n_per_map / TILE, per_head = g.head_dim / TILE;
+    const int map = EPI == SMALL_QKV ? nt / tiles_per_map : 0, tt = EPI == SMALL_QKV ? nt - map * tiles_per_map : nt;
+    const bool rotated = EPI == SMALL_QKV && map < 2;
+    const int head = rotated ? tt / per_head : 0, j0 = rotated ? 16 * (tt - head * per_head) : 0;
+    auto weight_row = [&](int r) -> const __nv_bfloat16 * {
+        const int hi = r >> 4, q = r & 15;
+        if (EPI == SMALL_SWIGLU) {
+            const int n = nt * 16 + q;
+            return n < g.N ? (hi ? g.B[1] : g.B[0]) + (long long)n * K : nullptr;
+        }
+        if (rotated) return (map ? g.B[1] : g.B[0]) + (long long)(head * g.head_dim + hi * half + j0 + q) * K;
+        const int n = tt * TILE + r;
+        return n < g.n_per_map ? (map == 2 ? g.B[2] : g.B[0]) + (long long)n * K : nullptr;
+    };
+    const int chunks = Kp / 8;
+    const uint4 zero = make_uint4(0, 0, 0, 0);
+    for (int i = tid; i < TILE * chunks; i += kThreads) {
+        const int r = i / chunks, c = i - r * chunks;
+        const __nv_bfloat16 *src = weight_row(r);
+        if (src != nullptr && c * 8 < K) cp_async16(sB + r * ld + c * 8, src + c * 8);
+        else *reinterpret_cast<uint4 *>(sB + r * ld + c * 8) = zero;
+    }
+
+    pdl_wait();                                             // weights are constant; everything else may come from the kernel before
+    const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
+    if ((g.d_active && *g.d_active == 0) || m0 >= M) { cp_async_wait(); return; }
+
+    // ---- activation rows
+    if (SRC == SMALL_BF16) {
+        for (int i = tid; i < TILE * chunks; i += kThreads) {
+            const int r = i / chunks, c = i - r * chunks;
+            if (m0 + r < M && c * 8 < K) cp_async16(sA + r * ld + c * 8, g.a + (long long)(m0 + r) * g.lda + c * 8);
+            else *reinterpret_cast<uint4 *>(sA + r * ld + c * 8) = zero;
+        }
+    } else {
+        constexpr int ROWS = 16 / NCH;                      // rows of a warp in flight: 16 loads per lane
+        const int q4 = K / 4;
+#pragma unroll
+        for (int r0 = 0; r0 < 8; r0 += ROWS) {
+            float4 v[ROWS][NCH];
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                const int m = m0 + warp * 8 + r0 + u;
+                const long long src = m < M ? (g.rows ? g.rows[m] : m) : 0;
+                const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
+                const uint2 *er = nullptr;
+                if (SRC == SMALL_EMBED) {
+                    int id = g.tokens[src];
+                    id = id < 0 ? 0 : (id >= g.vocab ? g.vocab - 1 : id);     // out-of-range ids are clamped, never dereferenced
+                    er = reinterpret_cast<const uint2 *>(g.emb + (long long)id * K);
+                }
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) {
+                    const int c = lane + 32 * k;
+                    v[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (m < M && c < q4) {
+                        if (SRC == SMALL_EMBED) {
+                            const uint2 e = er[c];
+                            v[u][k] = make_float4(bf16_bits_to_f32(e.x & 0xFFFFu), bf16_bits_to_f32(e.x >> 16), bf16_bits_to_f32(e.y & 0xFFFFu),
+                                                  bf16_bits_to_f32(e.y >> 16));
+                        } else v[u][k] = xr[c];
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                const int r = warp * 8 + r0 + u, m = m0 + r;
+                float ss = 0.f;
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) ss += v[u][k].x * v[u][k].x + v[u][k].y * v[u][k].y + v[u][k].z * v[u][k].z + v[u][k].w * v[u][k].w;
+                const float inv = rsqrtf(warp_sum(ss) / (float)K + g.eps);
+#pragma unroll
+                for (int k = 0; k < NCH; ++k) {
+                    const int c = lane + 32 * k;
+                    if (c >= q4) continue;
+                    if (SRC == SMALL_EMBED && nt == 0 && m < M) reinterpret_cast<float4 *>(g.x)[(long long)m * q4 + c] = v[u][k];      // the residual stream begins
+                    const uint2 gn = reinterpret_cast<const uint2 *>(g.gain)[c];
+                    *reinterpret_cast<uint2 *>(sA + r * ld + 4 * c) =
+                        make_uint2(pack2(v[u][k].x * inv * bf16_bits_to_f32(gn.x & 0xFFFFu), v[u][k].y * inv * bf16_bits_to_f32(gn.x >> 16)),
+                                   pack2(v[u][k].z * inv * bf16_bits_to_f32(gn.y & 0xFFFFu), v[u][k].w * inv * bf16_bits_to_f32(gn.y >> 16)));
+                }
+            }
+        }
+        if (K < Kp) for (int r = tid; r < TILE; r += kThreads) *reinterpret_cast<uint4 *>(sA + r * ld + K) = zero;      // K is a multiple of 8
+    }
+    cp_async_wait();
+    __syncthreads();
+
+    // ---- 16 rows x (8 + 8) columns per warp; even and odd k-steps accumulate apart, which halves the chain
+    const int wm = warp & 1, wn = warp >> 1;
+    const uint32_t a_addr = smem_addr(sA + (wm * 16 + (lane & 15)) * ld + (lane >> 4) * 8);
+    const uint32_t b_addr = smem_addr(sB + ((lane >> 4) * 16 + wn * 8 + (lane & 7)) * ld + ((lane >> 3) & 1) * 8);
+    float acc[2][2][4] = {};
+    const int steps = Kp / 16;
+    int k = 0;
+    for (; k + 2 <= steps; k += 2)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            uint32_t a[4], b[4];
+            ldmatrix4(a, a_addr + (k + u) * 32); ldmatrix4(b, b_addr + (k + u) * 32);
+            mma_16816(acc[u][0], a, b[0], b[1]);
+            mma_16816(acc[u][1], a, b[2], b[3]);
+        }
+    if (k < steps) {
+        uint32_t a[4], b[4];
+        ldmatrix4(a, a_addr + k * 32); ldmatrix4(b, b_addr + k * 32);
+        mma_16816(acc[0][0], a, b[0], b[1]);
+        mma_16816(acc[0][1], a, b[2], b[3]);
+    }
+
+    // ---- epilogue: a thread holds, of both halves, rows lane / 4 and + 8, columns 2 (lane % 4) and + 1
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int m = m0 + wm * 16 + (lane >> 2) + 8 * h, q = wn * 8 + 2 * (lane & 3);
+        if (m >= M) continue;
+        const float x0 = acc[0][0][2 * h] + acc[1][0][2 * h], x1 = acc[0][0][2 * h + 1] + acc[1][0][2 * h + 1];
+        const float y0 = acc[0][1][2 * h] + acc[1][1][2 * h], y1 = acc[0][1][2 * h + 1] + acc[1][1][2 * h + 1];
+        if (EPI == SMALL_SWIGLU) {
+            const int n = nt * 16 + q;
+            if (n < g.N) *reinterpret_cast<uint32_t *>(g.out + (long long)m * g.ldc + n) = pack2(silu(x0) * y0, silu(x1) * y1);       // N is even
+        } else if (EPI == SMALL_RESIDUAL) {
+            float2 *p0 = reinterpret_cast<float2 *>(g.x + (long long)m * g.N + nt * TILE + q), *p1 = p0 + 8;
+            float2 *i0 = reinterpret_cast<float2 *>(g.inc + (long long)m * g.N + nt * TILE + q), *i1 = i0 + 8;
+            if (nt * TILE + q < g.N) { float2 t = *p0; t.x += x0; t.y += x1; *p0 = t; if (g.inc) *i0 = make_float2(x0, x1); }
+            if (nt * TILE + 16 + q < g.N) { float2 t = *p1; t.x += y0; t.y += y1; *p1 = t; if (g.inc) *i1 = make_float2(y0, y1); }
+        } else if (EPI == SMALL_QKV) {
+            if (rotated) {
+                // the projection's result is rounded to bf16 and so is the rotated one, as when the two are kernels of their own
+                const float a0 = round_bf16(x0), a1 = round_bf16(x1), b0 = round_bf16(y0), b1 = round_bf16(y1);
+                const float4 cs = *reinterpret_cast<const float4 *>(g.table + (long long)(m % g.S) * half + j0 + q);       // two (cos, sin)
+                __nv_bfloat16 *dst = (map && g.k_dst ? g.k_dst + (long long)m * g.n_per_map : g.out + (long long)m * g.ldc + map * g.n_per_map)
+                                     + head * g.head_dim + j0 + q;
+                *reinterpret_cast<uint32_t *>(dst) = pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
+                *reinterpret_cast<uint32_t *>(dst + half) = pack2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
+            } else {
+                __nv_bfloat16 *dst = g.vt + (long long)(tt * TILE + q) * g.ldvt + m;       // values go out transposed
+                dst[0] = __float2bfloat16_rn(x0); dst[g.ldvt] = __float2bfloat16_rn(x1);
+                dst[16 * g.ldvt] = __float2bfloat16_rn(y0); dst[17 * g.ldvt] = __float2bfloat16_rn(y1);
+            }
+        } else {
+            const float v[4] = {x0 * g.scale, x1 * g.scale, y0 * g.scale, y1 * g.scale};
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int n = nt * TILE + 16 * u + q;
+                if (n >= g.N) continue;                     // N is even
+                if (g.out_f32 != nullptr) *reinterpret_cast<float2 *>(g.out_f32 + (long long)m * g.ldc + n) = make_float2(v[2 * u], v[2 * u + 1]);
+                else *reinterpret_cast<uint32_t *>(g.out + (long long)m * g.ldc + n) = pack2(v[2 * u], v[2 * u + 1]);
+            }
+        }
+    }
+}
+
+size_t smem_bytes(int K) { return (size_t)2 * TILE * (((K + 15) & ~15) + 8) * 2; }
+
+template <int SRC, int EPI, int NCH>
+int32_t launch(const SmallGemmArgs &g, int n_tiles, cudaStream_t s)
+{
+    const size_t smem = smem_bytes(g.K);
+    static size_t configured[kMaxDevices] = {};
+    size_t &done = configured[current_device_slot()];
+    if (smem > 48 * 1024 && smem > done) {
+        SFS_CUDA(cudaFuncSetAttribute(small_gemm_kernel<SRC, EPI, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        done = smem;
+    }
+    SFS_CUDA(launch_pdl(small_gemm_kernel<SRC, EPI, NCH>, dim3((unsigned)n_tiles, (unsigned)((g.M + TILE - 1) / TILE)), dim3(kThreads), smem, s, g));
+    return SFS_OK;
+}
+
+}  // namespace
+
+bool small_gemm_fits(int d_model, int d_ff, int head_dim) { return d_model <= 512 && smem_bytes(d_ff) <= 200 * 1024 && (d_model % 32) == 0 && (head_dim % 32) == 0; }
+
+int32_t launch_small_gemm(int src, int epi, const SmallGemmArgs &g, cudaStream_t s)
+{
+    const int n_tiles = epi == SMALL_SWIGLU ? (g.N + 15) / 16 : (epi == SMALL_QKV ? 3 * (g.n_per_map / TILE) : (g.N + TILE - 1) / TILE);
+    const bool wide = g.K > 256;
+    if (src == SMALL_EMBED) return wide ? launch<SMALL_EMBED, SMALL_QKV, 4>(g, n_tiles, s) : launch<SMALL_EMBED, SMALL_QKV, 2>(g, n_tiles, s);
+    if (src == SMALL_BF16) return launch<SMALL_BF16, SMALL_RESIDUAL, 2>(g, n_tiles, s);
+    switch (epi) {
+        case SMALL_QKV: return wide ? launch<SMALL_NORM, SMALL_QKV, 4>(g, n_tiles, s) : launch<SMALL_NORM, SMALL_QKV, 2>(g, n_tiles, s);
+        case SMALL_SWIGLU: return wide ? launch<SMALL_NORM, SMALL_SWIGLU, 4>(g, n_tiles, s) : launch<SMALL_NORM, SMALL_SWIGLU, 2>(g, n_tiles, s);
+        default: return wide ? launch<SMALL_NORM, SMALL_STORE, 4>(g, n_tiles, s) : launch<SMALL_NORM, SMALL_STORE, 2>(g, n_tiles, s);
+    }
+}
+
+}  // namespace sfs

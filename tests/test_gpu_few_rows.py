@@ -4,11 +4,13 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import forward as F
 from oracle import rowstats as RS
 from oracle.scheduler import SlowFastState, rows_needed, slowfast_step
 from paper_2506_10848_b200 import binding as sfs
 from paper_2506_10848_b200 import workloads as W
 
+from bf16_reference import forward_bf16_points
 from helpers import params_pair
 from test_gpu_linear import run
 
@@ -61,6 +63,37 @@ def test_generation_with_few_long_rows_is_reproduced_by_the_oracle(B, L, vocab, 
                 rec = slowfast_step(ost[b], {i: int(st["argmax"][j]) for i, j in idx.items()}, {i: int(st["sq"][j]) for i, j in idx.items()}, po)
                 assert trace[step, b].tolist()[:6] == [rec.phase, rec.s, rec.hi, rec.e_cand, rec.stable, len(rec.positions)], (step, b)
         sfs.sfs_check_device_status()
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
+
+
+# small models (fused 32 x 32 tiles): rows below, at and across a tile; both head widths; a d_ff whose K tail is 8; a ragged vocabulary;
+# the last shape has one row tile more than these kernels take
+@pytest.mark.parametrize("dims", [dict(d_model=256, n_heads=4, head_dim=64, d_ff=1000, vocab=1000), dict(d_model=384, n_heads=3, head_dim=128, d_ff=264, vocab=4104)])
+@pytest.mark.parametrize("B,S", [(1, 8), (3, 8), (1, 40), (2, 24), (1, 536)])
+def test_small_model_edges(dims, B, S):
+    shape = W.Shape(n_layers=2, mask_id=dims["vocab"] - 1, rms_eps=1e-5, rope_theta=10000.0, logit_scale=8.0, **dims)
+    w = W.model_weights(shape, seed=6, gain_std=0.2)
+    wd = {k: (v.to(DEV) if k != "layers" else [{kk: vv.to(DEV) for kk, vv in lw.items()} for lw in v]) for k, v in w.items()}
+    model = sfs.Model(shape, wd)
+    session = sfs.sfs_session_create(model, B, S)
+    try:
+        tok = W.prompt_ids(B, S, shape.vocab, seed=S)
+        picked = [(b, t) for b in range(B) for t in range(0, S, max(1, S // 9))]
+        n, cap = len(picked), B * S                              # fewer rows than the call allows for
+        rows = torch.zeros(cap, dtype=torch.int32); rows[:n] = torch.tensor([b * S + t for b, t in picked])
+        for dtype in (sfs.LOGITS_F32, sfs.LOGITS_BF16):
+            lg = torch.full((cap, shape.vocab), 7.0, dtype=torch.float32 if dtype else torch.bfloat16, device=DEV)
+            sfs.sfs_forward(session, tok.to(DEV), B, S, rows.to(DEV), torch.tensor([n], dtype=torch.int32, device=DEV), cap, lg, dtype)
+            sfs.sfs_check_device_status()
+            assert torch.all(lg[n:] == 7.0)                       # rows beyond the device's count untouched
+            got = lg[:n].float().cpu().double().numpy()
+            ref = F.forward(F.ModelConfig(**shape.asdict()), W.weights_to_numpy(w, np.float64), tok.numpy(), rows=picked, dtype=np.float64)
+            # what rounding to bf16 at the stored operands alone gives, plus 10 % (and the rounding of a stored bf16 logit: 2^-9 rms)
+            emu = np.concatenate([forward_bf16_points(F.ModelConfig(**shape.asdict()), w, tok[b].numpy(), [t for bb, t in picked if bb == b]) for b in range(B)])
+            rel, rel_model = np.linalg.norm(got - ref) / np.linalg.norm(ref), np.linalg.norm(emu - ref) / np.linalg.norm(ref)
+            assert rel <= 1.10 * rel_model + (0.0 if dtype else 2.0 ** -9), (rel, rel_model)
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
