@@ -17,9 +17,15 @@ struct AttnArgs {
     const int32_t *d_active;           // optional: the kernel does nothing when *d_active == 0
 };
 
+// what the kernel for short sequences reads directly
+struct AttnShort {
+    const __nv_bfloat16 *q, *k, *vt; long long ld_q, ld_k, ld_vt;
+};
+
 struct AttnPlan {
     CUtensorMap tmQ, tmK, tmVt;
     AttnArgs args;
+    AttnShort direct;
     int head_dim;
 };
 
@@ -33,6 +39,9 @@ int32_t attn_plan_create(AttnPlan *p, const void *qkv, int64_t ld_qkv, const voi
 int32_t attn_plan_create_split(AttnPlan *p, const void *q, int64_t ld_q, const void *k, int64_t ld_k, int32_t k_cols, int32_t k_col0,
                                const void *vt, int64_t ld_vt, void *out, int64_t ld_out, int32_t B, int32_t S, int32_t n_heads, int32_t head_dim);
 int32_t attn_launch_queries(const AttnPlan &p, int32_t kq, const int32_t *d_active, int32_t *err, cudaStream_t stream);
+// Short sequences: whether kq query rows each take the kernel for them, and that kernel (attn_launch and attn_launch_queries decide)
+bool attn_is_short(const AttnPlan &p, int32_t kq);
+int32_t attn_launch_short(const AttnPlan &p, int32_t kq, const int32_t *d_active, cudaStream_t stream);
 int32_t attn_launch(const AttnPlan &p, const int32_t *d_active, int32_t *err, cudaStream_t stream);
 
 }  // namespace sfs

@@ -359,6 +359,7 @@ int32_t attn_plan_create_split(AttnPlan *p, const void *q, int64_t ld_q, const v
     a.scale_log2 = 1.4426950408889634f / sqrtf((float)head_dim);
     a.out = reinterpret_cast<__nv_bfloat16 *>(out); a.ld_out = ld_out;
     p->head_dim = head_dim;
+    p->direct = {reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<const __nv_bfloat16 *>(k) + k_col0, reinterpret_cast<const __nv_bfloat16 *>(vt), ld_q, ld_k, ld_vt};
     return SFS_OK;
 }
 
@@ -377,6 +378,7 @@ int32_t attn_launch(const AttnPlan &p, const int32_t *d_active, int32_t *err, cu
 int32_t attn_launch_queries(const AttnPlan &p, int32_t kq, const int32_t *d_active, int32_t *err, cudaStream_t stream)
 {
     const int rows = kq > 0 ? kq : p.args.kq, nkv = (p.args.S + KT - 1) / KT;
+    if (attn_is_short(p, rows)) return attn_launch_short(p, rows, d_active, stream);
     const long long heads = (long long)p.args.n_heads * p.args.B, sms = gemm_num_sms();
     // waves of CTAs x (tile pairs of a CTA + 3, about what its set-up, first loads and final store cost).  32 heads, pair against
     // split in us: 512 tokens 13.9 / 9.8, 1000 23.2 / 27.4, 1536 57.8 / 50.9, 2048 74.6 / 83.2, 8 x 768 108.7 / 124.4.

@@ -332,7 +332,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 {
     // This kernel may have been scheduled while the one before it in the stream still runs (programmatic dependent launch):
     // everything up to pdl_wait() touches only this CTA's shared and tensor memory.
-    pdl_trigger();
     const int MB = g.mb;
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     // uniform over the pair, before any barrier or allocation: pairs beyond the tiles of even the largest row count
@@ -513,6 +512,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
+            if (tile + num_pairs >= num_tiles) pdl_trigger();
             EpiShare e;
             e.tmem = tmem_base + buf * buf_stride + ((uint32_t)(q * 32) << 16); e.tmem_block = bn_pad; e.up = (uint32_t)HALF;
             e.row0 = t.m0 + (int)rank * BM + q * 32; e.row_block = 2 * BM;
@@ -551,7 +551,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                 const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, GemmArgs g)
 {
-    pdl_trigger();
     const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
     if (pair >= ((g.M + 2 * FM - 1) / (2 * FM)) * g.n_col_tiles * g.splits) return;      // beyond the tiles of even the largest row count
 
@@ -705,6 +704,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
+            if (tile + num_pairs >= num_tiles) pdl_trigger();
             EpiShare e;
             e.tmem = tmem_base + buf * 256u + ((uint32_t)(q * 32) << 16); e.tmem_block = (uint32_t)HALF; e.up = (uint32_t)HALF;
             e.row0 = t.m0 + (int)rank * FM + (q & 1) * 32; e.row_block = 0;

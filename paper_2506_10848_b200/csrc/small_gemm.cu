@@ -40,7 +40,6 @@ template <int SRC, int EPI, int NCH>
 __global__ void __launch_bounds__(kThreads)
 small_gemm_kernel(SmallGemmArgs g)
 {
-    pdl_trigger();
     extern __shared__ __align__(16) __nv_bfloat16 s_mem[];
     const int K = g.K, Kp = (K + 15) & ~15, ld = Kp + 8;          // rows 16 bytes apart modulo 128: ldmatrix is conflict-free
     __nv_bfloat16 *sA = s_mem, *sB = s_mem + TILE * ld;
@@ -70,17 +69,40 @@ small_gemm_kernel(SmallGemmArgs g)
         else *reinterpret_cast<uint4 *>(sB + r * ld + c * 8) = zero;
     }
 
+    // constant too: the gains of this lane's columns, the rotary angles of its rows
+    const int wm = warp & 1, wn = warp >> 1, em = m0 + wm * 16 + (lane >> 2), eq = wn * 8 + 2 * (lane & 3);      // epilogue: rows em and em + 8, columns eq, eq + 1 of both halves
+    uint2 gain[NCH];
+    float4 angle[2];
+    if (SRC != SMALL_BF16)
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) gain[k] = lane + 32 * k < K / 4 ? reinterpret_cast<const uint2 *>(g.gain)[lane + 32 * k] : make_uint2(0, 0);
+    if (EPI == SMALL_QKV && rotated)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) angle[h] = *reinterpret_cast<const float4 *>(g.table + (long long)((em + 8 * h) % g.S) * half + j0 + eq);       // two (cos, sin)
+
     pdl_wait();                                             // weights are constant; everything else may come from the kernel before
+    pdl_trigger();
+    // the row count and the flag are used only after the loads below have been issued (which stay within g.M rows)
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
-    if ((g.d_active && *g.d_active == 0) || m0 >= M) { cp_async_wait(); return; }
+    const bool active = g.d_active == nullptr || *g.d_active != 0;
+    float2 xr[2][2];
+    if (EPI == SMALL_RESIDUAL)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int n = nt * TILE + 16 * u + eq;
+                xr[h][u] = (em + 8 * h < g.M && n < g.N) ? *reinterpret_cast<const float2 *>(g.x + (long long)(em + 8 * h) * g.N + n) : make_float2(0.f, 0.f);
+            }
 
     // ---- activation rows
     if (SRC == SMALL_BF16) {
         for (int i = tid; i < TILE * chunks; i += kThreads) {
             const int r = i / chunks, c = i - r * chunks;
-            if (m0 + r < M && c * 8 < K) cp_async16(sA + r * ld + c * 8, g.a + (long long)(m0 + r) * g.lda + c * 8);
+            if (m0 + r < g.M && c * 8 < K) cp_async16(sA + r * ld + c * 8, g.a + (long long)(m0 + r) * g.lda + c * 8);
             else *reinterpret_cast<uint4 *>(sA + r * ld + c * 8) = zero;
         }
+        if (!active || m0 >= M) { cp_async_wait(); return; }
     } else {
         constexpr int ROWS = 16 / NCH;                      // rows of a warp in flight: 16 loads per lane
         const int q4 = K / 4;
@@ -90,7 +112,8 @@ small_gemm_kernel(SmallGemmArgs g)
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
                 const int m = m0 + warp * 8 + r0 + u;
-                const long long src = m < M ? (g.rows ? g.rows[m] : m) : 0;
+                const int listed = g.rows && m < g.M ? g.rows[m] : 0;
+                const long long src = g.rows ? (m < M ? listed : 0) : (m < g.M ? m : 0);
                 const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
                 const uint2 *er = nullptr;
                 if (SRC == SMALL_EMBED) {
@@ -102,7 +125,7 @@ small_gemm_kernel(SmallGemmArgs g)
                 for (int k = 0; k < NCH; ++k) {
                     const int c = lane + 32 * k;
                     v[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (m < M && c < q4) {
+                    if (m < g.M && c < q4) {
                         if (SRC == SMALL_EMBED) {
                             const uint2 e = er[c];
                             v[u][k] = make_float4(bf16_bits_to_f32(e.x & 0xFFFFu), bf16_bits_to_f32(e.x >> 16), bf16_bits_to_f32(e.y & 0xFFFFu),
@@ -111,6 +134,7 @@ small_gemm_kernel(SmallGemmArgs g)
                     }
                 }
             }
+            if (r0 == 0 && (!active || m0 >= M)) { cp_async_wait(); return; }
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
                 const int r = warp * 8 + r0 + u, m = m0 + r;
@@ -123,7 +147,7 @@ small_gemm_kernel(SmallGemmArgs g)
                     const int c = lane + 32 * k;
                     if (c >= q4) continue;
                     if (SRC == SMALL_EMBED && nt == 0 && m < M) reinterpret_cast<float4 *>(g.x)[(long long)m * q4 + c] = v[u][k];      // the residual stream begins
-                    const uint2 gn = reinterpret_cast<const uint2 *>(g.gain)[c];
+                    const uint2 gn = gain[k];
                     *reinterpret_cast<uint2 *>(sA + r * ld + 4 * c) =
                         make_uint2(pack2(v[u][k].x * inv * bf16_bits_to_f32(gn.x & 0xFFFFu), v[u][k].y * inv * bf16_bits_to_f32(gn.x >> 16)),
                                    pack2(v[u][k].z * inv * bf16_bits_to_f32(gn.y & 0xFFFFu), v[u][k].w * inv * bf16_bits_to_f32(gn.y >> 16)));
@@ -136,7 +160,6 @@ small_gemm_kernel(SmallGemmArgs g)
     __syncthreads();
 
     // ---- 16 rows x (8 + 8) columns per warp; even and odd k-steps accumulate apart, which halves the chain
-    const int wm = warp & 1, wn = warp >> 1;
     const uint32_t a_addr = smem_addr(sA + (wm * 16 + (lane & 15)) * ld + (lane >> 4) * 8);
     const uint32_t b_addr = smem_addr(sB + ((lane >> 4) * 16 + wn * 8 + (lane & 7)) * ld + ((lane >> 3) & 1) * 8);
     float acc[2][2][4] = {};
@@ -160,7 +183,7 @@ small_gemm_kernel(SmallGemmArgs g)
     // ---- epilogue: a thread holds, of both halves, rows lane / 4 and + 8, columns 2 (lane % 4) and + 1
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-        const int m = m0 + wm * 16 + (lane >> 2) + 8 * h, q = wn * 8 + 2 * (lane & 3);
+        const int m = em + 8 * h, q = eq;
         if (m >= M) continue;
         const float x0 = acc[0][0][2 * h] + acc[1][0][2 * h], x1 = acc[0][0][2 * h + 1] + acc[1][0][2 * h + 1];
         const float y0 = acc[0][1][2 * h] + acc[1][1][2 * h], y1 = acc[0][1][2 * h + 1] + acc[1][1][2 * h + 1];
@@ -170,13 +193,13 @@ small_gemm_kernel(SmallGemmArgs g)
         } else if (EPI == SMALL_RESIDUAL) {
             float2 *p0 = reinterpret_cast<float2 *>(g.x + (long long)m * g.N + nt * TILE + q), *p1 = p0 + 8;
             float2 *i0 = reinterpret_cast<float2 *>(g.inc + (long long)m * g.N + nt * TILE + q), *i1 = i0 + 8;
-            if (nt * TILE + q < g.N) { float2 t = *p0; t.x += x0; t.y += x1; *p0 = t; if (g.inc) *i0 = make_float2(x0, x1); }
-            if (nt * TILE + 16 + q < g.N) { float2 t = *p1; t.x += y0; t.y += y1; *p1 = t; if (g.inc) *i1 = make_float2(y0, y1); }
+            if (nt * TILE + q < g.N) { *p0 = make_float2(xr[h][0].x + x0, xr[h][0].y + x1); if (g.inc) *i0 = make_float2(x0, x1); }
+            if (nt * TILE + 16 + q < g.N) { *p1 = make_float2(xr[h][1].x + y0, xr[h][1].y + y1); if (g.inc) *i1 = make_float2(y0, y1); }
         } else if (EPI == SMALL_QKV) {
             if (rotated) {
                 // the projection's result is rounded to bf16 and so is the rotated one, as when the two are kernels of their own
                 const float a0 = round_bf16(x0), a1 = round_bf16(x1), b0 = round_bf16(y0), b1 = round_bf16(y1);
-                const float4 cs = *reinterpret_cast<const float4 *>(g.table + (long long)(m % g.S) * half + j0 + q);       // two (cos, sin)
+                const float4 cs = angle[h];
                 __nv_bfloat16 *dst = (map && g.k_dst ? g.k_dst + (long long)m * g.n_per_map : g.out + (long long)m * g.ldc + map * g.n_per_map)
                                      + head * g.head_dim + j0 + q;
                 *reinterpret_cast<uint32_t *>(dst) = pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
