@@ -3,7 +3,7 @@
 //
 // A 64 x 256 x 256 product has 8 MFLOP; the tcgen05 kernel needs 4 us for it after its inputs are there (pair set-up, TMA round
 // trip, tensor-memory hand-overs), its norm and its rotary kernel 1.5 to 1.7 each, and every launch in a chain 1.4 us on
-// top.  Here a CTA of four warps computes a 32 x 32 tile with mma.sync from shared memory that holds all of K at once: the weight
+// top.  Here a CTA of eight warps computes a 32 x 32 tile with mma.sync from shared memory that holds all of K at once: the weight
 // rows are requested before the dependent-launch wait, the activation rows are normalised on the way in (every column tile
 // repeats that for its 32 rows, from L2), and the accumulators of a warp pair up what the epilogue needs together (gate and up,
 // the two halves of a rotary pair).  A layer is five launches instead of eight.
@@ -14,7 +14,7 @@
 namespace sfs {
 namespace {
 
-constexpr int TILE = 32, kThreads = 128;
+constexpr int TILE = 32, kThreads = 256, kWarps = kThreads / 32;
 
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -25,7 +25,7 @@ __device__ __forceinline__ void ldmatrix4(uint32_t *r, uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void mma_16816(float *c, const uint32_t *a, uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
@@ -62,15 +62,15 @@ small_gemm_kernel(SmallGemmArgs g)
     };
     const int chunks = Kp / 8;
     const uint4 zero = make_uint4(0, 0, 0, 0);
-    for (int i = tid; i < TILE * chunks; i += kThreads) {
-        const int r = i / chunks, c = i - r * chunks;
+    for (int r = warp; r < TILE; r += kWarps) {
         const __nv_bfloat16 *src = weight_row(r);
-        if (src != nullptr && c * 8 < K) cp_async16(sB + r * ld + c * 8, src + c * 8);
-        else *reinterpret_cast<uint4 *>(sB + r * ld + c * 8) = zero;
+        for (int c = lane; c < chunks; c += 32)
+            if (src != nullptr && c * 8 < K) cp_async16(sB + r * ld + c * 8, src + c * 8);
+            else *reinterpret_cast<uint4 *>(sB + r * ld + c * 8) = zero;
     }
 
     // constant too: the gains of this lane's columns, the rotary angles of its rows
-    const int wm = warp & 1, wn = warp >> 1, em = m0 + wm * 16 + (lane >> 2), eq = wn * 8 + 2 * (lane & 3);      // epilogue: rows em and em + 8, columns eq, eq + 1 of both halves
+    const int wm = warp & 1, wn = (warp >> 1) & 1, wk = warp >> 2, em = m0 + wm * 16 + (lane >> 2), eq = wn * 8 + 2 * (lane & 3);      // epilogue: rows em and em + 8, columns eq, eq + 1 of both halves
     uint2 gain[NCH];
     float4 angle[2];
     if (SRC != SMALL_BF16)
@@ -97,21 +97,20 @@ small_gemm_kernel(SmallGemmArgs g)
 
     // ---- activation rows
     if (SRC == SMALL_BF16) {
-        for (int i = tid; i < TILE * chunks; i += kThreads) {
-            const int r = i / chunks, c = i - r * chunks;
-            if (m0 + r < g.M && c * 8 < K) cp_async16(sA + r * ld + c * 8, g.a + (long long)(m0 + r) * g.lda + c * 8);
-            else *reinterpret_cast<uint4 *>(sA + r * ld + c * 8) = zero;
-        }
+        for (int r = warp; r < TILE; r += kWarps)
+            for (int c = lane; c < chunks; c += 32)
+                if (m0 + r < g.M && c * 8 < K) cp_async16(sA + r * ld + c * 8, g.a + (long long)(m0 + r) * g.lda + c * 8);
+                else *reinterpret_cast<uint4 *>(sA + r * ld + c * 8) = zero;
         if (!active || m0 >= M) { cp_async_wait(); return; }
     } else {
-        constexpr int ROWS = 16 / NCH;                      // rows of a warp in flight: 16 loads per lane
+        constexpr int PER = TILE / kWarps, ROWS = PER;      // rows of a warp, all in flight
         const int q4 = K / 4;
 #pragma unroll
-        for (int r0 = 0; r0 < 8; r0 += ROWS) {
+        for (int r0 = 0; r0 < PER; r0 += ROWS) {
             float4 v[ROWS][NCH];
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
-                const int m = m0 + warp * 8 + r0 + u;
+                const int m = m0 + warp * PER + r0 + u;
                 const int listed = g.rows && m < g.M ? g.rows[m] : 0;
                 const long long src = g.rows ? (m < M ? listed : 0) : (m < g.M ? m : 0);
                 const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
@@ -137,7 +136,7 @@ small_gemm_kernel(SmallGemmArgs g)
             if (r0 == 0 && (!active || m0 >= M)) { cp_async_wait(); return; }
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
-                const int r = warp * 8 + r0 + u, m = m0 + r;
+                const int r = warp * PER + r0 + u, m = m0 + r;
                 float ss = 0.f;
 #pragma unroll
                 for (int k = 0; k < NCH; ++k) ss += v[u][k].x * v[u][k].x + v[u][k].y * v[u][k].y + v[u][k].z * v[u][k].z + v[u][k].w * v[u][k].w;
@@ -159,13 +158,14 @@ small_gemm_kernel(SmallGemmArgs g)
     cp_async_wait();
     __syncthreads();
 
-    // ---- 16 rows x (8 + 8) columns per warp; even and odd k-steps accumulate apart, which halves the chain
+    // ---- 16 rows x (8 + 8) columns and half of k per warp; even and odd k-steps accumulate apart, which halves the chain again
     const uint32_t a_addr = smem_addr(sA + (wm * 16 + (lane & 15)) * ld + (lane >> 4) * 8);
     const uint32_t b_addr = smem_addr(sB + ((lane >> 4) * 16 + wn * 8 + (lane & 7)) * ld + ((lane >> 3) & 1) * 8);
     float acc[2][2][4] = {};
-    const int steps = Kp / 16;
-    int k = 0;
-    for (; k + 2 <= steps; k += 2)
+    const int steps = Kp / 16, mid = (steps + 1) / 2, end = wk ? steps : mid;
+    int k = wk ? mid : 0;
+#pragma unroll 2
+    for (; k + 2 <= end; k += 2)
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             uint32_t a[4], b[4];
@@ -173,11 +173,24 @@ small_gemm_kernel(SmallGemmArgs g)
             mma_16816(acc[u][0], a, b[0], b[1]);
             mma_16816(acc[u][1], a, b[2], b[3]);
         }
-    if (k < steps) {
+    if (k < end) {
         uint32_t a[4], b[4];
         ldmatrix4(a, a_addr + k * 32); ldmatrix4(b, b_addr + k * 32);
         mma_16816(acc[0][0], a, b[0], b[1]);
         mma_16816(acc[0][1], a, b[2], b[3]);
+    }
+    float4 sum[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+        sum[u] = make_float4(acc[0][u][0] + acc[1][u][0], acc[0][u][1] + acc[1][u][1], acc[0][u][2] + acc[1][u][2], acc[0][u][3] + acc[1][u][3]);
+    __shared__ float4 s_half[2][kThreads / 2];
+    if (wk) { s_half[0][tid - kThreads / 2] = sum[0]; s_half[1][tid - kThreads / 2] = sum[1]; }
+    __syncthreads();
+    if (wk) return;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        const float4 o = s_half[u][tid];
+        sum[u].x += o.x; sum[u].y += o.y; sum[u].z += o.z; sum[u].w += o.w;
     }
 
     // ---- epilogue: a thread holds, of both halves, rows lane / 4 and + 8, columns 2 (lane % 4) and + 1
@@ -185,8 +198,7 @@ small_gemm_kernel(SmallGemmArgs g)
     for (int h = 0; h < 2; ++h) {
         const int m = em + 8 * h, q = eq;
         if (m >= M) continue;
-        const float x0 = acc[0][0][2 * h] + acc[1][0][2 * h], x1 = acc[0][0][2 * h + 1] + acc[1][0][2 * h + 1];
-        const float y0 = acc[0][1][2 * h] + acc[1][1][2 * h], y1 = acc[0][1][2 * h + 1] + acc[1][1][2 * h + 1];
+        const float x0 = h ? sum[0].z : sum[0].x, x1 = h ? sum[0].w : sum[0].y, y0 = h ? sum[1].z : sum[1].x, y1 = h ? sum[1].w : sum[1].y;
         if (EPI == SMALL_SWIGLU) {
             const int n = nt * 16 + q;
             if (n < g.N) *reinterpret_cast<uint32_t *>(g.out + (long long)m * g.ldc + n) = pack2(silu(x0) * y0, silu(x1) * y1);       // N is even
