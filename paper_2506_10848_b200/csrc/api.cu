@@ -263,12 +263,12 @@ static int32_t run_step(sfs_session *s, const StepKey &key, const StepMode &mode
     return SFS_OK;
 }
 
-// Small models and few rows take kernels that do the row-wise work of the neighbours too (see small_gemm.cu), up to seven or so tiles
-// of the widest projection per SM: a whole step of the 2-layer d 256, d_ff 688 model takes, us against the tensor-memory kernels,
-// 64 rows 55 / 71, 256 63 / 83, 448 75 / 87, 768 97 / 105, 1024 105 / 103, 2048 167 / 120.
+// Small models and few rows take kernels that do the row-wise work of the neighbours too (see small_gemm.cu), up to nine or so
+// tiles of the widest projection per SM: a whole step of the 2-layer d 256, d_ff 688 model takes, us against the tensor-memory
+// kernels, 64 rows 35 / 67, 512 61 / 84, 768 86 / 104, 1024 100 / 110, 1280 120 / 116, 8 x 224 139 / 113.
 static bool small_step(const sfs_config &c, int rows)
 {
-    return small_gemm_fits(c.d_model, c.d_ff, c.head_dim) && (long long)((rows + 31) / 32) * ((c.d_ff + 15) / 16) <= 1056;
+    return small_gemm_fits(c.d_model, c.d_ff, c.head_dim) && (long long)((rows + 31) / 32) * ((c.d_ff + 15) / 16) <= 1408;
 }
 static SmallGemmArgs small_args(sfs_session *s, int M, int N, int K, const int32_t *d_active)
 {

@@ -158,12 +158,10 @@ int32_t launch(const AttnPlan &p, const AttnArgs &a, int mt, cudaStream_t s)
 }  // namespace
 
 // Heads of 64 and at most one wave of CTAs of two tiles.  4 heads, us per launch back to back, against the tcgen05 kernel: 64 tokens
-// 2.5 / 4.6, 224 3.5 / 5.4, 2 x 224 4.1 / 5.6, 512 6.5 / 7.7, 8 x 256 (two waves) 7.7 / 5.9.  Heads of 128 gain nothing: 32 of them,
-// 104 tokens 5.1 / 5.8, 192 tokens 11.5 / 6.8.
+// 2.6 / 4.6, 224 3.5 / 5.4, 4 x 224 4.4 / 5.6, 512 6.4 / 7.7, 3 x 512 (two waves) 10.9 / 7.8; in the chain of a step 192 tokens
+// 2.4 / 6.0.  Heads of 128 gain nothing: 32 of them, 104 tokens 5.1 / 5.8, 192 tokens 11.5 / 6.8.
 bool attn_is_short(const AttnPlan &p, int32_t kq)
 {
-    static const int lim = getenv("SFS_SHORT") ? atoi(getenv("SFS_SHORT")) : 100000;
-    if (lim < 100000) return p.head_dim == DH && p.args.S <= lim;
     return p.head_dim == DH && p.args.S <= 512 && (long long)((kq + 31) / 32) * p.args.n_heads * p.args.B <= gemm_num_sms();
 }
 

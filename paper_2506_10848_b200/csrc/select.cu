@@ -66,15 +66,15 @@ __device__ __forceinline__ uint32_t philox_first_word(uint32_t c0, uint32_t c1, 
 }
 
 // what the whole step leaves: the size of the next row list, the number of sequences still decoding and, in a generation, the
-// host's mirror of it (host_active[0]: sequences still decoding; host_active[1]: denoising steps finished)
-__device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int n_active)
+// host's mirror of it (host_active[0]: sequences still decoding; host_active[1]: denoising steps finished; one 8-byte write, so
+// that who sees the step sees whether it was the last, without a system-wide fence between two)
+__device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int n_active, int steps_before)
 {
     if (a.next_n_rows) *a.next_n_rows = n_next;
     if (a.n_active) *a.n_active = n_active;
     if (a.host_active) {
-        a.host_active[0] = n_active;                        // before the step count: who sees the step sees whether it was the last
-        __threadfence_system();
-        a.host_active[1] = ++*a.step_count;
+        *reinterpret_cast<volatile unsigned long long *>(a.host_active) = (unsigned long long)(uint32_t)n_active | (unsigned long long)(uint32_t)(steps_before + 1) << 32;
+        *a.step_count = steps_before + 1;
     }
 }
 
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
 
     pdl_wait();
     pdl_trigger();
+    const int steps_before = tid == 0 && a.step_count ? *a.step_count : 0;      // (of the whole generation)
     // the state and everything about position tid (all of a sequence, usually) in one round trip
     uint8_t m0 = 0;
     int32_t arg0 = 0;
@@ -385,7 +386,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                 t[0] = rec_phase; t[1] = rec_s; t[2] = rec_hi; t[3] = e_cand; t[4] = stable; t[5] = n_sel;
                 t[6] = st.n_masked; t[7] = st.k_remaining;
             }
-            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0);
+            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0, steps_before);
         }
     }
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(a.state + b)[tid] = reinterpret_cast<const int *>(&st)[tid];
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     }
     act = warp_sum_i32(act);
     if (tid == 0) {
-        finish_step(a, off, act);
+        finish_step(a, off, act, steps_before);
         *a.ticket = 0;
     }
 }
