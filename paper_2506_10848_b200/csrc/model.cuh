@@ -74,7 +74,6 @@ struct sfs_session {
     std::vector<__nv_bfloat16 *> Kc, Vtc;    // per layer: rotated keys [T, d], values transposed [d, T]
     std::vector<float *> Ac, Fc;             // per layer: residual increments of the attention and MLP branches [T, d]
     __nv_bfloat16 *hg = nullptr;             // [T, d] gathered normalised rows
-    __nv_bfloat16 *vnew_t = nullptr;         // [d, T] fresh values of every row, transposed
     float *sim_partial = nullptr;            // [kSimSlices, T, 3]
     int32_t *sel_rows = nullptr;             // [T] rows recomputed in the current layer
     int32_t *dump_sets = nullptr; float *dump_sims = nullptr;   // caller's buffers for the sets / similarities of generate steps
