@@ -195,27 +195,55 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
             ok = tc::mbar_wait(bar_s + 8 * w, (uint32_t)i & 1u, &s_abort);      // (P V of the tile before has finished too)
             if (!ok) break;
             tc::tc_fence_after();
-            uint32_t v[KT];
-#pragma unroll
-            for (int q = 0; q < KT / 32; ++q) tc::tmem_ld32(ts + q * 32, v + q * 32);
-#pragma unroll
-            for (int q = 0; q < KT / 32; ++q) tc::tmem_ld_wait32(v + q * 32);
+            uint32_t v[64], pk[32];
             const int valid = S - key_tile(w, i) * KT;     // keys of this tile that belong to the sequence
-            if (valid < KT) {
+            auto load = [&](int q) {                       // 64 scores, those beyond the sequence -inf
+                tc::tmem_ld32(ts + q * 64, v); tc::tmem_ld32(ts + q * 64 + 32, v + 32);
+                tc::tmem_ld_wait32(v); tc::tmem_ld_wait32(v + 32);
+                if (valid < KT) {
 #pragma unroll
-                for (int k = 0; k < KT; ++k)
-                    if (k >= valid) v[k] = 0xFF800000u;    // -inf: probability 0
-            }
-            float mx[4];
+                    for (int k = 0; k < 64; ++k)
+                        if (q * 64 + k >= valid) v[k] = 0xFF800000u;    // probability 0
+                }
+            };
+            auto row_max = [&]() {
+                float mx[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) mx[k] = __uint_as_float(v[k]);
+                for (int k = 0; k < 4; ++k) mx[k] = __uint_as_float(v[k]);
 #pragma unroll
-            for (int k = 4; k + 7 < KT; k += 8)
+                for (int k = 4; k + 7 < 64; k += 8)
 #pragma unroll
-                for (int e = 0; e < 4; ++e) mx[e] = tc::max3(mx[e], __uint_as_float(v[k + e]), __uint_as_float(v[k + 4 + e]));
+                    for (int e = 0; e < 4; ++e) mx[e] = tc::max3(mx[e], __uint_as_float(v[k + e]), __uint_as_float(v[k + 4 + e]));
 #pragma unroll
-            for (int e = 0; e < 4; ++e) mx[e] = fmaxf(mx[e], __uint_as_float(v[KT - 4 + e]));
-            const float m_row = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+                for (int e = 0; e < 4; ++e) mx[e] = fmaxf(mx[e], __uint_as_float(v[60 + e]));
+                return fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3]));
+            };
+            unsigned long long sum2[2];
+            auto half = [&]() {                            // 64 keys: 32 columns of packed pairs
+                const float mc = m * c;
+                const unsigned long long c2 = tc::pack_f32x2(c, c), mc2 = tc::pack_f32x2(-mc, -mc);
+#pragma unroll
+                for (int k = 0; k < 32; ++k) {
+                    float e0, e1;
+                    tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1])), c2, mc2), e0, e1);
+                    const float p0 = tc::ex2_approx(e0), p1 = tc::ex2_approx(e1);
+                    sum2[k & 1] = tc::add_f32x2(sum2[k & 1], tc::pack_f32x2(p0, p1));
+                    __nv_bfloat162 hh = __floats2bfloat162_rn(p0, p1);
+                    pk[k] = *reinterpret_cast<uint32_t *>(&hh);
+                }
+            };
+            auto hand = [&](int q) {
+                tc::tmem_st32(ts + q * 32, pk);
+                tc::tmem_st_wait();
+                tc::tc_fence_before();                     // S has been read, this half of P written, O rescaled
+                tc::mbar_arrive(bar_p + 16 * w + 8 * q);
+            };
+            // the maximum of the second half first (the first half is then in registers for its exponentials)
+            load(1);
+            const float m_hi = row_max();
+            load(0);
+            sum2[0] = sum2[1] = 0ull;
+            const float m_row = fmaxf(row_max(), m_hi);
             if (i == 0) {
                 m = m_row;
             } else {
@@ -234,26 +262,11 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
                     if (move) { l *= alpha; m = m_row; }
                 }
             }
-            const float mc = m * c;
-            const unsigned long long c2 = tc::pack_f32x2(c, c), mc2 = tc::pack_f32x2(-mc, -mc);
-            unsigned long long sum2[2] = {0ull, 0ull};
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {                  // 64 keys: 32 columns of packed pairs
-                uint32_t pk[32];
-#pragma unroll
-                for (int k = 0; k < 32; ++k) {
-                    float e0, e1;
-                    tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[q * 64 + 2 * k]), __uint_as_float(v[q * 64 + 2 * k + 1])), c2, mc2), e0, e1);
-                    const float p0 = tc::ex2_approx(e0), p1 = tc::ex2_approx(e1);
-                    sum2[k & 1] = tc::add_f32x2(sum2[k & 1], tc::pack_f32x2(p0, p1));
-                    __nv_bfloat162 hh = __floats2bfloat162_rn(p0, p1);
-                    pk[k] = *reinterpret_cast<uint32_t *>(&hh);
-                }
-                tc::tmem_st32(ts + q * 32, pk);
-                tc::tmem_st_wait();
-                tc::tc_fence_before();                     // S has been read, this half of P written, O rescaled
-                tc::mbar_arrive(bar_p + 16 * w + 8 * q);
-            }
+            half();
+            hand(0);
+            load(1);
+            half();
+            hand(1);
             float s0, s1;
             tc::unpack_f32x2(tc::add_f32x2(sum2[0], sum2[1]), s0, s1);
             l += s0 + s1;
