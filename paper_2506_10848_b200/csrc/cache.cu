@@ -212,27 +212,6 @@ __global__ void scatter_rows_f32_kernel(const float4 *__restrict__ src, int n_sl
     }
 }
 
-// K rows: block j copies compact row j to its token row
-__global__ void scatter_k_kernel(const __nv_bfloat16 *__restrict__ qk, long long ld_src, int col0, const int32_t *__restrict__ rows,
-                                 int d, __nv_bfloat16 *__restrict__ k_dst)
-{
-    const int j = blockIdx.x;
-    const uint4 *s = reinterpret_cast<const uint4 *>(qk + (long long)j * ld_src + col0);
-    uint4 *o = reinterpret_cast<uint4 *>(k_dst + (long long)rows[j] * d);
-    for (int c = threadIdx.x; c < d / 8; c += blockDim.x) o[c] = s[c];
-}
-
-// V^T columns: a block owns 8 features; compact rows run fastest over the threads, so the reads are contiguous
-__global__ void scatter_vt_kernel(const __nv_bfloat16 *__restrict__ vt_src, long long ld_vt_src, const int32_t *__restrict__ rows, int n_rows,
-                                  int d, __nv_bfloat16 *__restrict__ vt_dst, long long ld_vt_dst)
-{
-    const int f0 = blockIdx.x * 8;
-    for (int idx = threadIdx.x; idx < 8 * n_rows; idx += blockDim.x) {
-        const int f = f0 + idx / n_rows, j = idx - (idx / n_rows) * n_rows;
-        if (f < d) vt_dst[(long long)f * ld_vt_dst + rows[j]] = vt_src[(long long)f * ld_vt_src + j];
-    }
-}
-
 // One launch for what follows the QKV projection of the recomputed rows: the rotary embedding of q and k (in place, on the
 // compact rows; the arithmetic of rope_kernel), the rotated k also written to the token's row of the K cache, and the new
 // value columns scattered into V^T.  Blocks [0, rope_blocks) rotate, the rest scatter values (8 features per block).
@@ -392,19 +371,6 @@ int32_t launch_scatter_rows_f32(const float *src, int n_slabs, long long slab_st
     if (n_rows <= 0) return SFS_OK;
     SFS_CUDA(launch_pdl(scatter_rows_f32_kernel, dim3((unsigned)n_rows, 4, 1), dim3((unsigned)(256)), (size_t)(0), s, reinterpret_cast<const float4 *>(src), n_slabs < 1 ? 1 : n_slabs, slab_stride / 4, rows, d / 4,
                                                    reinterpret_cast<float4 *>(dst)));
-    return SFS_OK;
-}
-
-int32_t launch_scatter_kv(const void *qk_src, long long ld_src, int col0, const void *vt_src, long long ld_vt_src,
-                          const int32_t *rows, int n_rows, int d, void *k_dst, void *vt_dst, long long ld_vt_dst, cudaStream_t s)
-{
-    if (n_rows <= 0) return SFS_OK;
-    scatter_k_kernel<<<n_rows, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(qk_src), ld_src, col0, rows, d,
-                                            reinterpret_cast<__nv_bfloat16 *>(k_dst));
-    SFS_LAUNCH_CHECK();
-    scatter_vt_kernel<<<(d + 7) / 8, 256, 0, s>>>(reinterpret_cast<const __nv_bfloat16 *>(vt_src), ld_vt_src, rows, n_rows, d,
-                                                  reinterpret_cast<__nv_bfloat16 *>(vt_dst), ld_vt_dst);
-    SFS_LAUNCH_CHECK();
     return SFS_OK;
 }
 

@@ -34,10 +34,6 @@ int32_t launch_gather_rows_bf16(const void *src, const int32_t *rows, int n_rows
 // products of a split-K projection, added in slab order)
 int32_t launch_scatter_rows_f32(const float *src, int n_slabs, long long slab_stride, const int32_t *rows, int n_rows, int d, float *dst,
                                 cudaStream_t s);
-// K rows: dst[rows[j], 0:d] = src[j, col0 : col0 + d] (bf16, src ld = ld_src);  V columns: dst_t[f, rows[j]] = src_t[f, j]
-int32_t launch_scatter_kv(const void *qk_src, long long ld_src, int col0, const void *vt_src, long long ld_vt_src,
-                          const int32_t *rows, int n_rows, int d, void *k_dst, void *vt_dst, long long ld_vt_dst, cudaStream_t s);
-
 // rope (as launch_rope, on the compact rows) + rotated k rows into the K cache + new value columns into V^T, one launch
 int32_t launch_rope_scatter_kv(void *qk, long long ld, int n_rows, int S, int n_heads, int head_dim, const float2 *table, const int32_t *rows,
                                void *k_dst, const void *vt_src, long long ld_vt_src, void *vt_dst, long long ld_vt_dst, cudaStream_t s);

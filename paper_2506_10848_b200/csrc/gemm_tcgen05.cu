@@ -512,7 +512,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
-            if (tile + num_pairs >= num_tiles) pdl_trigger();
+            if (tile + num_pairs >= num_tiles) pdl_trigger();   // the rest takes about as long as a launch (see pdl_trigger)
             EpiShare e;
             e.tmem = tmem_base + buf * buf_stride + ((uint32_t)(q * 32) << 16); e.tmem_block = bn_pad; e.up = (uint32_t)HALF;
             e.row0 = t.m0 + (int)rank * BM + q * 32; e.row_block = 2 * BM;
@@ -704,7 +704,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
             tc::tc_fence_after();
-            if (tile + num_pairs >= num_tiles) pdl_trigger();
+            if (tile + num_pairs >= num_tiles) pdl_trigger();   // the rest takes about as long as a launch (see pdl_trigger)
             EpiShare e;
             e.tmem = tmem_base + buf * 256u + ((uint32_t)(q * 32) << 16); e.tmem_block = (uint32_t)HALF; e.up = (uint32_t)HALF;
             e.row0 = t.m0 + (int)rank * FM + (q & 1) * 32; e.row_block = 0;

@@ -512,7 +512,7 @@ __device__ __forceinline__ uint32_t chunk_max2(const uint4 &v) {
     return *reinterpret_cast<uint32_t *>(&m);
 }
 
-template <int kInFlight, bool PACKED, bool PIPE>
+template <int kInFlight>
 __global__ void __launch_bounds__(kBoundsThreads)
 rowstats_bounds_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nchunks, int vocab,
                      const int32_t *__restrict__ n_rows_ptr, int max_rows, int slices, BoundsOut out)
@@ -545,7 +545,6 @@ rowstats_bounds_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
     float cref = warp_max(fm);
     if (!(fabsf(cref) <= 3.0e38f)) cref = 0.f;
     const float nc = __fmul_rn(-cref, kLog2e);
-    const f32x2 l2e2 = pack2(kLog2e, kLog2e), nc2 = pack2(nc, nc);
 
     float mx = -INFINITY, a0 = 0.f, a1 = 0.f;
     int best_c = -1;
@@ -556,45 +555,23 @@ rowstats_bounds_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
         float e[8];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (PACKED) {
-                const f32x2 t = fma2(pack2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xFFFF0000u)), l2e2, nc2);
-                uint32_t t0, t1;
-                unpack2(t, t0, t1);
-                e[2 * k] = ex2_fast(__uint_as_float(t0)); e[2 * k + 1] = ex2_fast(__uint_as_float(t1));
-            } else {
-                e[2 * k] = ex2_fast(__fmaf_rn(__uint_as_float(w[k] << 16), kLog2e, nc));
-                e[2 * k + 1] = ex2_fast(__fmaf_rn(__uint_as_float(w[k] & 0xFFFF0000u), kLog2e, nc));
-            }
+            e[2 * k] = ex2_fast(__fmaf_rn(__uint_as_float(w[k] << 16), kLog2e, nc));
+            e[2 * k + 1] = ex2_fast(__fmaf_rn(__uint_as_float(w[k] & 0xFFFF0000u), kLog2e, nc));
         }
         a0 += (e[0] + e[1]) + (e[2] + e[3]); a1 += (e[4] + e[5]) + (e[6] + e[7]);
     };
-    if (PIPE) {
-        // software pipeline: the next batch is in flight while the current one is evaluated (chunks past the slice are -inf:
-        // they add nothing and never win the maximum)
-        for (int cur = c0 + tid; cur < c1; cur += kInFlight * kBoundsThreads) {
-            uint4 w2[kInFlight];
-            const int c2 = cur + 2 * kInFlight * kBoundsThreads;
+    int cur = c0 + tid;
 #pragma unroll
-            for (int u = 0; u < kInFlight; ++u) { const int cc = c2 + u * kBoundsThreads; w2[u] = cc < c1 ? ld_stream(rp + cc) : neg; }
+    for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(v[u], cur + u * kBoundsThreads);
+    cur += kInFlight * kBoundsThreads;
 #pragma unroll
-            for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(v[u], cur + u * kBoundsThreads);
+    for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(nx[u], cur + u * kBoundsThreads);
+    cur += kInFlight * kBoundsThreads;
+    for (; cur < c1; cur += kInFlight * kBoundsThreads) {
 #pragma unroll
-            for (int u = 0; u < kInFlight; ++u) { v[u] = nx[u]; nx[u] = w2[u]; }
-        }
-    } else {
-        int cur = c0 + tid;
+        for (int u = 0; u < kInFlight; ++u) { const int cc = cur + u * kBoundsThreads; v[u] = cc < c1 ? ld_stream(rp + cc) : neg; }
 #pragma unroll
         for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(v[u], cur + u * kBoundsThreads);
-        cur += kInFlight * kBoundsThreads;
-#pragma unroll
-        for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(nx[u], cur + u * kBoundsThreads);
-        cur += kInFlight * kBoundsThreads;
-        for (; cur < c1; cur += kInFlight * kBoundsThreads) {
-#pragma unroll
-            for (int u = 0; u < kInFlight; ++u) { const int cc = cur + u * kBoundsThreads; v[u] = cc < c1 ? ld_stream(rp + cc) : neg; }
-#pragma unroll
-            for (int u = 0; u < kInFlight; ++u) if (cur + u * kBoundsThreads < c1) eat(v[u], cur + u * kBoundsThreads);
-        }
     }
 
     // ---- slice maximum, its first position, slice sum
@@ -691,7 +668,7 @@ int32_t launch_bounds(const uint4 *logits, long long ld_chunks, int nchunks, int
         const double fill = (double)ctas / (double)(waves * per_wave);
         if (fill > best + 0.02) { best = fill; slices = sl; }
     }
-    SFS_CUDA(launch_pdl(rowstats_bounds_bf16<4, false, false>, dim3((unsigned)(max_rows * slices)), dim3(kBoundsThreads), 0, stream, logits, ld_chunks,
+    SFS_CUDA(launch_pdl(rowstats_bounds_bf16<4>, dim3((unsigned)(max_rows * slices)), dim3(kBoundsThreads), 0, stream, logits, ld_chunks,
                         nchunks, vocab, d_n_rows, max_rows, slices, out));
     return SFS_OK;
 }

@@ -53,7 +53,11 @@ int32_t *device_status_word_if_any();
 // ---- programmatic dependent launch -----------------------------------------------------------------------
 // A kernel launched with launch_pdl may start (be scheduled, run its prologue) while the kernel before it in the stream is
 // still running; it calls pdl_wait() before its first access to global memory, which returns once that kernel has completed
-// and its writes are visible.  pdl_trigger() tells the runtime that the kernels after this one may be scheduled.
+// and its writes are visible.  pdl_trigger() tells the runtime that the kernels after this one may be scheduled.  Kernels call it
+// when about one launch latency of their own work is left: after their wait if they are short, before the last epilogue if they
+// are GEMMs.  Called first thing, a whole row of kernels becomes resident, and each reaches its wait so long before its input is
+// there that the code behind the wait has left the instruction cache by then (small projection after attention, 192 tokens: 4.9
+// us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -7,7 +7,11 @@
 // rows are requested before the dependent-launch wait, the activation rows are normalised on the way in (every column tile
 // repeats that for its 32 rows, from L2), and the accumulators of a warp pair up what the epilogue needs together (gate and up,
 // the two halves of a rotary pair).  A layer is five launches instead of eight.
-// Bound: the latency of one memory round trip, K / 16 dependent MMAs and the launch.
+// Bound: the latency of one memory round trip, K / 32 dependent MMAs per warp and the launch: 2.0 to 2.6 us from wait to end at 64
+// rows, 0.95 us from one kernel's end to the next one's wait.  2-layer d 256 step, before with the tensor-memory kernels / now: 64
+// rows 70.6 / 34.8 us, 192 - / 43, 512 84 / 61.  All layers in one launch (a cluster of 16 CTAs per sequence, cluster barriers
+// between the projections) took 54.8 us at 64 rows when this took 55.3, and twice this at 224: a barrier behind global stores and
+// the first loads of lines that other SMs have just written cost as much as a launch.
 #include "sfs_common.cuh"
 #include "small_gemm.cuh"
 
@@ -81,7 +85,7 @@ small_gemm_kernel(SmallGemmArgs g)
         for (int h = 0; h < 2; ++h) angle[h] = *reinterpret_cast<const float4 *>(g.table + (long long)((em + 8 * h) % g.S) * half + j0 + eq);       // two (cos, sin)
 
     pdl_wait();                                             // weights are constant; everything else may come from the kernel before
-    pdl_trigger();
+    pdl_trigger();                                          // (not earlier: see pdl_trigger)
     // the row count and the flag are used only after the loads below have been issued (which stay within g.M rows)
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
     const bool active = g.d_active == nullptr || *g.d_active != 0;
