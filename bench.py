@@ -300,12 +300,12 @@ def run_epilogue(torch, sfs, W, shape, dev, peaks):
     out["epilogue"] = {"workload": f"bf16 logits [{R}, {V}], planted winners, seed 1; cold (4 rotating copies > L2)", "row_stats_us": us,
                        "hbm_gbs": gbs, "frac_of_measured_hbm_peak": gbs / peaks["hbm_gbs"],
                        "kernel": "rowstats_bounds_bf16: the one pass over HBM of the selection step (exact argmax, enclosure of S_q); rows whose "
-                                 "enclosure leaves the step's comparisons open are recomputed canonically from L2 by a second launch",
+                                 "enclosure leaves the step's comparisons open are recomputed canonically from L2 in the selection's launch",
                        "canonical_all_rows_us": us_canonical, "canonical_all_rows_hbm_gbs": R * V * 2 / us_canonical * 1e-3,
                        "select_slow_step_us": slow_us, "select_fast_step_us": fast_us,
                        "select_slow_step_enqueue_bound_us": slow_chain_us, "select_fast_step_enqueue_bound_us": fast_chain_us,
-                       "select_step_note": "whole sfs_select call (four launches: streaming pass, decision, canonical recompute of the listed rows, "
-                                           "selection): one call timed alone, launch latency included; and 12 calls enqueued back to back, which is "
+                       "select_step_note": "whole sfs_select call (two launches: streaming pass; listing, canonical recompute of the listed rows "
+                                           "and selection): one call timed alone, launch latency included; and 12 calls enqueued back to back, which is "
                                            "bound by the host's enqueue rate through the Python binding, not by the device (per-kernel device times: "
                                            "profiles/rowstats_bounds_256x126464.md)",
                        "span": [lo, hi]}

@@ -542,6 +542,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 // k-block an SM pulls 64 + NB * BN / 2 rows and the ring holds up to nine k-blocks of wide tiles.  Measured at 128 rows, 8B
 // widths, weights from HBM, QKV / O / gate-up / down in us: 24.8 / 12.0 / 40.2 / 24.0 (the HBM floor at 6458 GB/s: 15.6 / 5.2 /
 // 31.2 / 15.6); single-CTA 128 x BN tiles, which pull 128 + BN rows for BN weight rows, took 29.1 / 12.0 / 42.3 / 24.7.
+// In a step, where the first weights arrive while the kernel ahead still runs: 20.7 / 10.4 / 36.5 / 19.5 from wait to end.  Two
+// k-blocks per stage with the epilogue parked in the idle ring (fewer hand-overs): 8 layers 1142 -> 1209 us, not taken.
 // SwiGLU: N-block 0
 // holds gate rows, N-block 1 the up rows of the same features.  Of an N-block's accumulators every CTA holds its 64 rows:
 // tensor-memory lanes 0-63 the columns [0, BN/2), lanes 64-127 the columns [BN/2, BN), in BN/2 tensor-memory columns.
