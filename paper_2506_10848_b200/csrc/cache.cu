@@ -95,9 +95,9 @@ __global__ void __launch_bounds__(kChoiceThreads) cache_select_kernel(CacheSelec
     if (a.refresh_r) {
         for (int i = tid; i < L; i += kChoiceThreads) out[base + i] = b * S + P + i;
     } else if (a.n_adapt > 0) {
-        int lo = 0, hi = L;
-        if (a.state != nullptr && a.state[b].phase == SFS_PHASE_FAST && !a.state[b].done) { lo = a.state[b].s_cycle; hi = a.state[b].hi; }
-        lo = max(0, min(lo, L)); hi = max(lo, min(hi, L));
+        // (the four fields in one round trip, beside that of the similarities)
+        int4 span = make_int4(SFS_PHASE_SLOW, 0, 0, L);              // phase, done, first, end
+        if (a.state != nullptr) span = make_int4(a.state[b].phase, a.state[b].done, a.state[b].s_cycle, a.state[b].hi);
         constexpr int HS = kSimSlices / 2;
         for (int it = tid; it < 2 * L; it += kChoiceThreads) {        // (2 L is even: both lanes of a position are there)
             const int i = it >> 1, half = it & 1;
@@ -120,6 +120,8 @@ __global__ void __launch_bounds__(kChoiceThreads) cache_select_kernel(CacheSelec
                 s_key[i] = float_order_key(sim);
             }
         }
+        const bool fast = span.x == SFS_PHASE_FAST && !span.y;
+        const int lo = fast ? max(0, min(span.z, L)) : 0, hi = fast ? max(lo, min(span.w, L)) : L;
         if (tid == 0) s_last = -1;
         __syncthreads();
         const int n_cand = hi - lo, k = min(a.n_adapt, n_cand);

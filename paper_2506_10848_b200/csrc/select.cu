@@ -13,6 +13,7 @@ namespace {
 
 constexpr int kSelThreads = 256;
 constexpr unsigned long long kNoKey = ~0ull;
+constexpr int kGoesOn = 1 << 30;             // beside a sequence's row count: its next step will hardly be its last
 constexpr int kPosBits = 17;                 // key = S_q << 17 | position  (S_q < 2^47, position < 2^17)
 
 struct BlockRed {
@@ -67,13 +68,14 @@ __device__ __forceinline__ uint32_t philox_first_word(uint32_t c0, uint32_t c1, 
 
 // what the whole step leaves: the size of the next row list, the number of sequences still decoding and, in a generation, the
 // host's mirror of it (host_active[0]: sequences still decoding; host_active[1]: denoising steps finished; one 8-byte write, so
-// that who sees the step sees whether it was the last, without a system-wide fence between two)
-__device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int n_active, int steps_before)
+// that who sees the step sees whether it was the last, without a system-wide fence between two; kMayEnd is set in the step count when
+// the next step may well be the last, and the host then waits for it instead of enqueueing another one behind it)
+__device__ __forceinline__ void finish_step(const SelectArgs &a, int n_next, int n_active, int steps_before, bool may_end)
 {
     if (a.next_n_rows) *a.next_n_rows = n_next;
     if (a.n_active) *a.n_active = n_active;
     if (a.host_active) {
-        *reinterpret_cast<volatile unsigned long long *>(a.host_active) = (unsigned long long)(uint32_t)n_active | (unsigned long long)(uint32_t)(steps_before + 1) << 32;
+        *reinterpret_cast<volatile unsigned long long *>(a.host_active) = (unsigned long long)(uint32_t)n_active | (unsigned long long)(uint32_t)((steps_before + 1) | (may_end ? kMayEnd : 0)) << 32;
         *a.step_count = steps_before + 1;
     }
 }
@@ -211,7 +213,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
         }
     }
 
-    int n_sel = 0, e_cand = -1, stable = 0;
+    int n_sel = 0, e_cand = -1, stable = 0, n_sure = 0;    // n_sure: candidates above the high threshold
     int rec_phase = phase0, rec_s = s0;
     int rec_hi = (phase0 == SFS_PHASE_SLOW) ? L : hi_fast;
     BlockStep blk{};
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             s_keys[i] = key; s_fl[i] = fl;
         }
         r = block_reduce(r, s_tmp, s_min);
+        n_sure = r.n_high;
 
         if (r.missing > 0 || (r.n_cand == 0 && !vanilla)) {
             // a needed row was not supplied (or the state is inconsistent): report, change nothing
@@ -380,13 +383,18 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
         }
         if (tid == 0) {
             if (a.sel_count) a.sel_count[b] = n_out;
-            a.seq_row_count[b] = n_next;
+            // May the next step finish the sequence?  It does when the budget ends.  Before that (SlowFast) its rows must be all that
+            // is masked, and no more than its ranking unmasks or, in the fast phase, twice what has just been unmasked or was sure.
+            const int reach = st.phase == SFS_PHASE_SLOW ? p.k_slow : max(p.k_fast, 2 * max(n_sel, n_sure));
+            const bool may_end = st.k_remaining <= 1 || (!vanilla && n_next == st.n_masked && reach >= st.n_masked);
+            const bool goes_on = next_active && !may_end;
+            a.seq_row_count[b] = n_next | (goes_on ? kGoesOn : 0);
             if (a.trace) {
                 int32_t *t = a.trace + (long long)b * SFS_TRACE_INTS;
                 t[0] = rec_phase; t[1] = rec_s; t[2] = rec_hi; t[3] = e_cand; t[4] = stable; t[5] = n_sel;
                 t[6] = st.n_masked; t[7] = st.k_remaining;
             }
-            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0, steps_before);
+            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0, steps_before, !goes_on);
         }
     }
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(a.state + b)[tid] = reinterpret_cast<const int *>(&st)[tid];
@@ -399,10 +407,11 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    int off = 0, act = 0;
+    int off = 0, act = 0, on = 0;
     for (int q0 = 0; q0 < a.B; q0 += 32) {                  // every warp: offsets of 32 sequences; then each warp copies every 8th list
         const int q = q0 + lane;
-        const int c = q < a.B ? __ldcg(&a.seq_row_count[q]) : 0;
+        const int cw = q < a.B ? __ldcg(&a.seq_row_count[q]) : 0, c = cw & ~kGoesOn;
+        on |= cw & kGoesOn;
         act += (q < a.B && __ldcg(&a.state[q].done) == 0 && __ldcg(&a.state[q].status) == SFS_OK) ? 1 : 0;
         int pre = c;
 #pragma unroll
@@ -415,8 +424,9 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
         off += __shfl_sync(0xffffffffu, pre, 31);
     }
     act = warp_sum_i32(act);
+    on = __any_sync(0xffffffffu, on != 0);
     if (tid == 0) {
-        finish_step(a, off, act, steps_before);
+        finish_step(a, off, act, steps_before, !on);
         *a.ticket = 0;
     }
 }

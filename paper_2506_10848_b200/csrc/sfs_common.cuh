@@ -248,6 +248,7 @@ int32_t launch_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld,
                                 unsigned long long *d_lo, unsigned long long *d_hi, int32_t *d_argmax, int32_t *d_err, cudaStream_t stream);
 
 struct LogitsRows { const uint4 *base; long long ld; int32_t chunks; };          // bf16 logits as 16-byte chunks, ld chunks between rows
+constexpr int32_t kMayEnd = 1 << 30;
 struct SelectArgs {
     int32_t *tokens; uint8_t *mask; int32_t B, S, P, L;
     sfs_state *state; sfs_params params;
@@ -264,6 +265,7 @@ struct SelectArgs {
     int32_t *n_active;                                      // optional: sequences not done after this step
     int32_t *ticket;                                        // scratch counter (zero between launches)
     int32_t *trace;                                         // optional [B, SFS_TRACE_INTS]
+    // host_active: [0] sequences still decoding, [1] steps finished, with kMayEnd when the next one may be the last
     int32_t *host_active, *step_count;                      // optional: the host's mirror, and the device's count of steps
 };
 int32_t launch_select(const SelectArgs &a, cudaStream_t stream);
