@@ -97,3 +97,78 @@ def test_small_model_edges(dims, B, S):
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
+
+
+# heads of 64, short sequences: one key block, blocks that end inside a warp's share, keys over 4 and 8 warps, one and two row tiles
+# per CTA, a last row tile of 8 rows, the longest of them
+@pytest.mark.parametrize("B,S,H", [(1, 8, 1), (2, 40, 3), (1, 128, 4), (1, 136, 4), (4, 224, 4), (8, 64, 8), (1, 512, 4), (2, 264, 8)])
+def test_short_attention_edges(B, S, H):
+    d = H * 64
+    g = torch.Generator().manual_seed(S)
+    q, k, v = (torch.randn((B * S, d), generator=g).to(torch.bfloat16) for _ in range(3))
+    out = torch.zeros((B * S, d), dtype=torch.bfloat16, device=DEV)
+    sfs.sfs_attention(torch.cat([2 * q, k], dim=1).contiguous().to(DEV), v.t().contiguous().to(DEV), out, B, S, H, 64)
+    sfs.sfs_check_device_status()
+    got = out.cpu().double().numpy()
+    for b in range(B):
+        sl = slice(b * S, (b + 1) * S)
+        qq, kk, vv = (t[sl].double().numpy().reshape(S, H, 64) for t in (2 * q, k, v))
+        ref, mag = F.attention(qq, kk, vv).reshape(S, d), F.attention(qq, kk, np.abs(vv)).reshape(S, d)
+        # probabilities and the output rounded to bf16 (unit roundoff 2^-8 each), exponentials to about 2^-20
+        assert np.all(np.abs(got[sl] - ref) <= 2.0 ** -8 * (mag + np.abs(ref)) + 2.0 ** -16), b
+
+
+@pytest.mark.parametrize("scale,B,L,kw", [(60.0, 1, 64, {}), (60.0, 3, 40, {}), (1.0, 2, 24, {}), (8.0, 1, 1, {}),
+                                          (60.0, 1, 32, dict(sampler=sfs.SAMPLER_RANDOM, max_steps=4)), (8.0, 2, 16, dict(k_slow=5, k_fast=3))])
+def test_generation_enqueues_what_it_needs(scale, B, L, kw):
+    """The host runs ahead of the device except where a step may be the last: the same tokens as step by step, at most one step more."""
+    dct = W.TINY.asdict()
+    dct["logit_scale"] = scale
+    shape, P = W.Shape(**dct), 8 - L % 8
+    model = sfs.Model(shape, W.model_weights(shape, seed=4, device=DEV))
+    session = sfs.sfs_session_create(model, B, P + L)
+    try:
+        prompt = W.prompt_ids(B, P, shape.vocab - 2, seed=2).to(DEV)
+        params = sfs.Params.default(**kw)
+        one, whole = (torch.zeros((B, P + L), dtype=torch.int32, device=DEV) for _ in range(2))
+        state = torch.zeros((B, sfs.STATE_INTS), dtype=torch.int32, device=DEV)
+        sfs.sfs_generate_begin(session, prompt, B, P, L, params)
+        before, steps, active = sfs.sfs_profile(session, False, read=False)[2], 0, B
+        while active:
+            sfs.sfs_generate_steps(session, 1)
+            active, steps = sfs.sfs_generate_end(session, one)
+        per_step = (sfs.sfs_profile(session, False, read=False)[2] - before) / steps
+        for _ in range(3):
+            before = sfs.sfs_profile(session, False, read=False)[2]
+            sfs.sfs_generate(session, prompt, B, P, L, params, whole, state_out=state)
+            enqueued = round((sfs.sfs_profile(session, False, read=False)[2] - before) / per_step)
+            done = int(state[:, sfs.STATE_FIELDS.index("steps_done")].max())
+            assert done == steps and done <= enqueued <= done + 1, (steps, done, enqueued)
+            assert torch.equal(one, whole)
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
+
+
+@pytest.mark.parametrize("P,L", [(16, 24), (19, 197), (8, 712)])
+def test_similarities_of_unchanged_tokens(P, L):
+    """Fresh values come as slabs over ranges of K (as many as the row count makes worth while), from an even token: with nothing changed
+    they are the cached ones up to the order of summation, two bf16 roundings of the same sums (they differ by an ulp at most, 2^-7: 1 - cos <= 2^-15)."""
+    shape = W.Shape(n_layers=1, d_model=2048, n_heads=16, head_dim=128, d_ff=256, vocab=1024, mask_id=1023, rms_eps=1e-5,
+                    rope_theta=10000.0, logit_scale=1.0)
+    model = sfs.Model(shape, W.model_weights(shape, seed=3, device=DEV))
+    S = P + L
+    session = sfs.sfs_session_create(model, 1, S)
+    try:
+        sfs.sfs_cache_enable(session, 100, 100, 0.25)
+        tok = W.prompt_ids(1, S, shape.vocab, seed=5).to(DEV)
+        rows = torch.arange(P, S, dtype=torch.int32, device=DEV)
+        lg = torch.zeros((L, shape.vocab), dtype=torch.bfloat16, device=DEV)
+        sims = torch.zeros((1, 1, L), dtype=torch.float32, device=DEV)
+        for step in range(2):
+            sfs.sfs_forward_cached(session, tok, 1, S, P, None, rows, None, L, lg, sfs.LOGITS_BF16, sims=sims if step else None)
+        sfs.sfs_check_device_status()
+        assert float((1.0 - sims).abs().max()) <= 2.0 ** -15
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
