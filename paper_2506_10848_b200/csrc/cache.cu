@@ -33,8 +33,8 @@ sim_partial_kernel(const float *__restrict__ a, long long lda, long long stride,
             acc[0] = fmaf(a0, b0, acc[0]); acc[1] = fmaf(a0, a0, acc[1]); acc[2] = fmaf(b0, b0, acc[2]);
             acc[3] = fmaf(a1, b1, acc[3]); acc[4] = fmaf(a1, a1, acc[4]); acc[5] = fmaf(b1, b1, acc[5]);
         };
-        constexpr int U = 4;
-        for (int f = f0 + warp; f < f1; f += 8 * U) {                // four features per round, all their loads in flight
+        constexpr int U = 8;
+        for (int f = f0 + warp; f < f1; f += 8 * U) {                // eight features per round, all their loads in flight
             float2 v[U][NS];
             uint32_t wb[U];
 #pragma unroll

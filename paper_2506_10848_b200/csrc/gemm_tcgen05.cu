@@ -411,7 +411,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // issued, so the latency of that poll overlaps the issue.
     if (warp == 0) {
         // ---------------- TMA producer (both CTAs; completion bytes are counted on the leader's barrier)
-        uint32_t it = 0;
+        uint32_t it = 0, s = 0, ph = 0;                     // stage and phase are counted along: dividing by STAGES in both loops cost 256 + 256 tokens 6 %
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
@@ -423,11 +423,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const int arow = t.m0 + (int)rank * BM, mbt = blocks_of(t, M);
             const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
                 if (!ready) ready = tc::mbar_wait(bar_empty + 8 * s, ph ^ 1u, &s_abort);
                 ok = __all_sync(0xffffffffu, ready);
                 if (!ok) break;
-                const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
+                const uint32_t ns = s + 1u == (uint32_t)STAGES ? 0u : s + 1u, nph = ns == 0u ? ph ^ 1u : ph;
                 ready = tc::mbar_test(bar_empty + 8 * ns, nph ^ 1u);
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
                 const bool early = it < (uint32_t)pre;
@@ -435,6 +434,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 if (mbt == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
                 if (!early) tc::tma_load_2d_2cta_elect(sa + MBS * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
+                s = ns; ph = nph;
             }
         }
         if (!live && pre > 0) {
@@ -462,7 +462,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (rank == 0) {
             // ---------------- MMA issuer (leader CTA only)
             const uint32_t idesc = tc::idesc_bf16_f32(2 * BM, BN);
-            uint32_t it = 0, lt = 0;
+            uint32_t s = 0, ph = 0, lt = 0;
             bool ok = true;
             bool ready = tc::mbar_test(bar_full, 0u);
             for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {
@@ -475,13 +475,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const TileCoord t = tile_coord(g, tile, m_groups);
                 const bool second = blocks_of(t, M) == 2;
                 const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
-                for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const uint32_t s = it % (uint32_t)STAGES, ph = (it / (uint32_t)STAGES) & 1u;
+                for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ready) ready = tc::mbar_wait(bar_full + 8 * s, ph, &s_abort);
                     ok = __all_sync(0xffffffffu, ready);
                     if (!ok) break;
                     tc::tc_fence_after();
-                    const uint32_t nx = it + 1u, ns = nx % (uint32_t)STAGES, nph = (nx / (uint32_t)STAGES) & 1u;
+                    const uint32_t ns = s + 1u == (uint32_t)STAGES ? 0u : s + 1u, nph = ns == 0u ? ph ^ 1u : ph;
                     ready = tc::mbar_test(bar_full + 8 * ns, nph);
                     const uint32_t sa = smem_base + s * STAGE_BYTES;
                     const uint64_t da = tc::smem_desc_sw128(sa), db = tc::smem_desc_sw128(sa + MBS * A_BYTES);
@@ -496,6 +495,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         for (int kk = 1; kk < BK / 16; ++kk) tc::mma_bf16_2cta_elect(d_tmem + bn_pad, da1 + (uint64_t)(kk * 2), db + (uint64_t)(kk * 2), idesc, 1u);
                     }
                     tc::mma_commit_2cta_elect(bar_empty + 8 * s);     // frees the stage in both CTAs once these MMAs have read it
+                    s = ns; ph = nph;
                 }
                 tc::mma_commit_2cta_elect(bar_acc_full + 8 * buf);    // accumulator complete (or abandoned), both CTAs
             }
