@@ -754,9 +754,11 @@ int stages_for(int mb, int bn)
 }
 
 // Modelled clocks of one candidate: waves x (k-blocks x clocks per k-block + exposed epilogue), per pair of SMs.
-// Per k-block and CTA the tensor core needs MB*bn*2 clocks (8192 FLOP/clk/SM); the operand stream is
-// (MB*128 + bn/2) rows x 128 B at the ~40 B/clk an SM sustains from L2 when every SM streams; below ~750 clocks the
-// k-block time stops shrinking with the tile (load latency over the bytes a CTA can keep in flight).  All measured.
+// Per k-block and CTA the tensor core needs MB*bn*2 clocks (8192 FLOP/clk/SM) and some 80 pass between k-blocks; the operand
+// stream is (MB*128 + bn/2) rows x 128 B at the ~54 B/clk an SM sustains from L2 when every SM streams; below 540 (MB = 1) or 980
+// clocks the k-block time stops shrinking with the tile.  Fitted to sweeps of MB, bn and the split at 512 to 2048 rows with operands
+// that do not heat the part; what it changed against the calibration before (40 B/clk, 750 clocks), us: down 512 rows 40.7 -> 37.1
+// (240 x 2 ranges instead of 512 x 240 x 4), QKV 1000 rows 70.4 -> 61.9, 1536 rows 90.8 -> 82.9, gate / up 1536 rows 168 -> 153.
 // The epilogue hides behind the next tile when two accumulators fit tensor memory, except for a pair's last tile.
 // Splitting K pays for few rows only: the slabs grow with M, the idle pairs they avoid do not.
 long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int mb, int bn, int splits)
@@ -765,9 +767,9 @@ long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int pa
     const int m_groups = (M + mb * 2 * BM - 1) / (mb * 2 * BM);
     const long long tiles = (long long)m_groups * col_tiles(mode, n_maps, n_per_map, mode == GEMM_SWIGLU ? bn / 2 : bn) * ((num_kb + kbps - 1) / kbps);
     const long long waves = (tiles + pairs - 1) / pairs;
-    const long long mma = (long long)mb * bn * 2, load = (long long)(mb * BM + bn / 2) * 128 / 40;
+    const long long mma = (long long)mb * bn * 2 + 80, load = (long long)(mb * BM + bn / 2) * 128 / 54, least = mb == 1 ? 540 : 980;
     long long kb_clk = mma > load ? mma : load;
-    if (kb_clk < 750) kb_clk = 750;
+    if (kb_clk < least) kb_clk = least;
     const long long epi = (long long)mb * bn * 16 + 3000;
     const bool hidden = mb * ((bn + 31) & ~31) <= 256;
     // a split K also costs the fp32 slab that the next RMSNorm reads back: M x N x 4 bytes, measured at ~1.2e-3 clocks per element
