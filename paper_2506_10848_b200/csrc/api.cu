@@ -1091,7 +1091,7 @@ int32_t sfs_generate(sfs_session *s, const int32_t *d_prompt, int32_t B, int32_t
             const int32_t w = (int32_t)(seen >> 32), ahead = s->gen_steps - (w & ~kMayEnd);
             more = (int32_t)seen != 0;
             if (!more || ahead <= 0 || (ahead == 1 && !(w & kMayEnd))) break;
-            if (++spins > (1ll << 34) || ((spins & 0xFFFFF) == 0 && cudaStreamQuery((cudaStream_t)stream) == cudaSuccess)) break;   // the stream drained or stalled
+            if (++spins > (1ll << 34) || ((spins & 0xFFFFF) == 0 && cudaStreamQuery((cudaStream_t)stream) != cudaErrorNotReady)) break;   // the stream drained or failed
         }
         if (more && (rc = sfs_generate_steps(s, 1, d_trace, max_trace_steps, nullptr, nullptr, nullptr, stream)) != SFS_OK) return rc;
     }
