@@ -14,6 +14,11 @@ namespace {
 // A thread keeps its part of the row in registers between the two passes (kNormRegChunks 16-byte chunks of it).
 // NP bounds the number of slabs: all of a thread's loads are issued before the first addition (summed slab by slab in a loop,
 // 512 rows of 4096 with four slabs took 8.5 us, four dependent round trips per chunk).
+// Whatever NT is, the squares are added in the order of 256 threads that take every 256th chunk each: how many threads share a
+// row depends on how many rows a launch has, and a row must not (a cached step compares the values of a few rows with those of a
+// launch over all of them, where the last bit decides).  Blocks of more than 256 threads pass the chunks' sums through shared
+// memory for that; narrower ones have a thread per chunk at least.  (A chunk's four squares are spelled out: contracted by the compiler,
+// two instances rounded them differently.)
 template <int NT, int NP, bool EMBED>
 __global__ void __launch_bounds__(NT)
 rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_partial, long long partial_stride,
@@ -22,13 +27,14 @@ rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_p
                const int32_t *__restrict__ tokens, const __nv_bfloat16 *__restrict__ emb, int vocab, const int32_t *__restrict__ copy_src,
                int32_t *__restrict__ copy_dst, int copy_n)
 {
-    constexpr int kNormThreads = NT, kNormRegChunks = NT == 256 ? 4 : (NT == 1024 ? 1 : 2);
+    constexpr int kNormThreads = NT, kNormRegChunks = NT == 256 ? 4 : (NT == 512 ? 2 : 1), kSumThreads = NT < 256 ? NT : 256;
+    extern __shared__ float s_sq[];                          // NT > 256: [chunks] sums of squares
     pdl_wait();
     pdl_trigger();
     if (EMBED && blockIdx.x == 0)
         for (int i = threadIdx.x; i < copy_n; i += kNormThreads) copy_dst[i] = copy_src[i];
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
-    __shared__ float s_part[kNormThreads / 32];
+    __shared__ float s_part[kSumThreads / 32];
     const int chunks = d / 4;
     for (int r = blockIdx.x; r < n_rows; r += gridDim.x) {
         const long long src = rows ? rows[r] : r;
@@ -57,6 +63,11 @@ rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_p
         // the first kNormRegChunks chunks of a thread stay in registers (statically indexed); longer rows re-read the rest
         float4 keep[kNormRegChunks];
         float ss = 0.f;
+        auto add = [&](int c, const float4 &v) {
+            const float q = __fmaf_rn(v.w, v.w, __fmaf_rn(v.z, v.z, __fmaf_rn(v.y, v.y, __fmul_rn(v.x, v.x))));
+            if (NT <= 256) ss += q;
+            else if (c < chunks) s_sq[c] = q;
+        };
         if (EMBED || NP == 0) {
 #pragma unroll
             for (int k = 0; k < kNormRegChunks; ++k) {
@@ -87,19 +98,25 @@ rmsnorm_kernel(float *__restrict__ x, const float *__restrict__ partial, int n_p
             const int c = threadIdx.x + k * kNormThreads;
             const float4 v = keep[k];
             if (c < chunks && write_x) xr[c] = v;
-            ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+            add(c, v);
         }
         for (int c = threadIdx.x + kNormRegChunks * kNormThreads; c < chunks; c += kNormThreads) {
             const float4 v = load(c);
             if (write_x) xr[c] = v;
-            ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+            add(c, v);
         }
-        ss = warp_sum(ss);
-        if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;
+        if (NT > 256) {
+            __syncthreads();
+            if (threadIdx.x < 256) for (int c = threadIdx.x; c < chunks; c += 256) ss += s_sq[c];
+        }
+        if (threadIdx.x < kSumThreads) {
+            ss = warp_sum(ss);
+            if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = ss;
+        }
         __syncthreads();
         float tot = 0.f;
 #pragma unroll
-        for (int w = 0; w < kNormThreads / 32; ++w) tot += s_part[w];
+        for (int w = 0; w < kSumThreads / 32; ++w) tot += s_part[w];
         const float inv = rsqrtf(tot / (float)d + eps);
         const uint2 *gp = reinterpret_cast<const uint2 *>(gain);
         uint2 *hp = reinterpret_cast<uint2 *>(h + (long long)r * d);
@@ -178,12 +195,12 @@ __global__ void rope_kernel(__nv_bfloat16 *__restrict__ qk, long long ld, int T,
 }  // namespace
 
 // Threads per row: 256 while the rows fill the machine, up to one 16-byte chunk per thread when they do not (a row is then one
-// round trip instead of four: 104 rows of 4096 with three slabs 6.8 -> 4.9 us), and no more threads than chunks.
+// round trip instead of four: 104 rows of 4096 with three slabs 6.8 -> 4.9 us), and no more threads than it takes.
 static int norm_threads(int rows, int d)
 {
     const int chunks = d / 4;
-    if (rows > 2 * 148) return 256;
-    return chunks >= 1024 ? 1024 : (chunks >= 512 ? 512 : (chunks >= 256 ? 256 : (chunks >= 128 ? 128 : 64)));
+    if (rows > 2 * 148 || d > 32768) return 256;          // (wider rows: their sums would not fit the shared memory of a plain launch)
+    return chunks >= 1024 ? 1024 : (chunks >= 512 ? 512 : (chunks > 128 ? 256 : (chunks > 64 ? 128 : 64)));
 }
 
 template <bool EMBED>
@@ -195,7 +212,7 @@ static int32_t launch_norm(float *x, const float *partial, int n_partial, long l
     const int grid = max_rows < 148 * 16 ? max_rows : 148 * 16, nt = norm_threads(max_rows, d);
     if (partial == nullptr) n_partial = 0;
     auto go = [&](auto kernel, int threads) {
-        return launch_pdl(kernel, dim3(grid), dim3(threads), 0, s, x, partial ? partial : x, n_partial, partial_stride,
+        return launch_pdl(kernel, dim3(grid), dim3(threads), threads > 256 ? (size_t)d : 0, s, x, partial ? partial : x, n_partial, partial_stride,
                           reinterpret_cast<const __nv_bfloat16 *>(gain), reinterpret_cast<__nv_bfloat16 *>(h), rows, n_rows, max_rows, d, eps, tokens,
                           reinterpret_cast<const __nv_bfloat16 *>(emb), vocab, copy_src, copy_dst, copy_n);
     };

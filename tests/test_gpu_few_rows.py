@@ -172,3 +172,30 @@ def test_similarities_of_unchanged_tokens(P, L):
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
+
+
+# the widths at which rows have fewer, as many and more 16-byte chunks than a block has threads
+@pytest.mark.parametrize("d,head_dim,d_ff,S", [(384, 128, 1536, 480), (640, 128, 256, 304), (2048, 128, 256, 304), (2560, 128, 256, 304), (4096, 128, 256, 304),
+                                               (5120, 128, 256, 304)])
+def test_norm_of_a_row_does_not_depend_on_how_many_rows_there_are(d, head_dim, d_ff, S):
+    """The full refresh normalises all tokens, a partial step the response, a call the rows it is asked for: each row must come out the
+    same, bit for bit (the identity as head shows the final norm's output)."""
+    shape = W.Shape(n_layers=1, d_model=d, n_heads=d // head_dim, head_dim=head_dim, d_ff=d_ff, vocab=d, mask_id=d - 1, rms_eps=1e-5, rope_theta=10000.0,
+                    logit_scale=1.0)
+    w = W.model_weights(shape, seed=d, gain_std=0.2, device=DEV)
+    w["lm_head"].copy_(torch.eye(d, device=DEV))
+    model = sfs.Model(shape, w)
+    session = sfs.sfs_session_create(model, 1, S)
+    try:
+        tok = W.prompt_ids(1, S, d, seed=1).to(DEV)
+        every = torch.zeros((S, d), dtype=torch.float32, device=DEV)
+        sfs.sfs_forward(session, tok, 1, S, None, None, S, every, sfs.LOGITS_F32)
+        for n in (1, 50, 288):
+            rows = torch.randperm(S, generator=torch.Generator().manual_seed(n))[:n].to(torch.int32).to(DEV)
+            some = torch.zeros((n, d), dtype=torch.float32, device=DEV)
+            sfs.sfs_forward(session, tok, 1, S, rows, None, n, some, sfs.LOGITS_F32)
+            sfs.sfs_check_device_status()
+            assert torch.equal(some, every[rows.long()]), (n, int((some != every[rows.long()]).sum()))
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
