@@ -108,14 +108,22 @@ __global__ void __launch_bounds__(kChoiceThreads) cache_select_kernel(CacheSelec
                 const float *q = p + (long long)sl * a.T * 3;
                 pd[sl] = ld_nc(q); pa[sl] = ld_nc(q + 1); pb[sl] = ld_nc(q + 2);
             }
+            // added in slice order, the odd lane going on where the even one stopped: equal vectors' last bits decide among unchanged rows
             float dot = 0.f, na = 0.f, nb = 0.f;
-#pragma unroll
-            for (int sl = 0; sl < HS; ++sl) { dot += pd[sl]; na += pa[sl]; nb += pb[sl]; }           // fixed order
             const unsigned both = 3u << (lane & 30);
-            dot += __shfl_xor_sync(both, dot, 1); na += __shfl_xor_sync(both, na, 1); nb += __shfl_xor_sync(both, nb, 1);
+#pragma unroll
+            for (int turn = 0; turn < 2; ++turn) {
+                if (half == turn)
+#pragma unroll
+                    for (int sl = 0; sl < HS; ++sl) { dot += pd[sl]; na += pa[sl]; nb += pb[sl]; }
+                if (turn == 0) {
+                    const float d0 = __shfl_sync(both, dot, lane & 30), a0 = __shfl_sync(both, na, lane & 30), b0 = __shfl_sync(both, nb, lane & 30);
+                    if (half == 1) { dot = d0; na = a0; nb = b0; }
+                }
+            }
             const float den = __fmul_rn(__fsqrt_rn(na), __fsqrt_rn(nb));
             const float sim = den > 0.f ? __fdiv_rn(dot, den) : 0.f;
-            if (half == 0) {
+            if (half == 1) {
                 if (a.sims_dump) a.sims_dump[(long long)b * L + i] = sim;
                 s_key[i] = float_order_key(sim);
             }
