@@ -397,13 +397,13 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
         rc = weight_plan_create(&cp.qkv_store, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->Vtc[l], T, 2 * d, nullptr);
         if (rc != SFS_OK) return rc;
-        // Fresh values of the candidate rows, transposed because the weights take the part of the rows (V^T = W_v h^T), for the similarities
-        // only: fp32 slabs over ranges of K, which the similarity kernel adds.  512 rows, 8B width: 33 -> 22 us, and 4 -> 6 in the similarities.  The response rows of a single
-        // sequence are one contiguous range (from an even token); with several sequences every row is projected.
+        // Fresh values of the candidate rows, for the similarities only: V^T = W_v h^T, the weights taking the part of the rows, so that they
+        // leave in the cached values' layout.  Not split over K: an unchanged row has to get its cached values again, bit for bit, which
+        // the QKV projection summed over all of K (in two ranges, 512 rows at the 8B width: 22 us instead of 24, but other rows chosen).  The
+        // response rows of a single sequence are one contiguous range (from an even token); with several sequences every row is projected.
         const int v_first = (B == 1) ? (P & ~1) : 0, v_rows = T - v_first;
         const void *h[1] = {s->h + (size_t)v_first * d};
-        rc = gemm_plan_create(&cp.vproj, m->wv[l], d, d, d, h, 1, v_rows, d, GEMM_STORE, s->partial, T, 1, 1.0f, nullptr, 0, 0, nullptr);
-        if (rc == SFS_OK) rc = gemm_plan_enable_split(&cp.vproj, s->partial, kSimSlabs < kMaxSplits ? kSimSlabs : kMaxSplits, nullptr);
+        rc = gemm_plan_create(&cp.vproj, m->wv[l], d, d, d, h, 1, v_rows, d, GEMM_STORE, s->vt, T, 0, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
         rc = weight_plan_create(&cp.o_store, s->attn, d, T, d, wo, 1, d, d, GEMM_STORE, s->Ac[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
@@ -540,7 +540,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
                     const GatherLayerPlans &gp = (*gps)[l];
                     if (!rr && n_adapt > 0) {
                         if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(cl.vproj, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                        if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_sim_partial(s->partial, T, cl.vproj.args.splits, cl.vproj.args.split_stride, s->Vtc[l], T, d, sim_first, sim_count, T, s->sim_partial, st); })) != SFS_OK) return rc;
+                        if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_sim_partial(s->vt, T, s->Vtc[l], T, d, sim_first, sim_count, T, s->sim_partial, st); })) != SFS_OK) return rc;
                     }
                     CacheSelectArgs a{};
                     a.partial = s->sim_partial; a.state = state; a.B = B; a.S = S; a.P = P; a.L = L; a.T = T;

@@ -7,47 +7,41 @@
 namespace sfs {
 namespace {
 
-// Fresh values come as NS fp32 slabs (the value projection's ranges of K), features x tokens, `stride` floats apart; they are summed in
-// slab order and rounded to bf16, as the cached ones are.
+// Fresh (a) and cached (b) values are bf16, features x tokens; a's columns begin with token t_first.  An unchanged row's fresh values
+// equal its cached ones bit for bit (one sum over all of K gives both), so its three sums are one number.
 // grid (ceil(tokens / 64), kSimSlices), 256 threads: lane = two neighbouring tokens, warp = every 8th feature of the slice
-template <int NS>
 __global__ void __launch_bounds__(256)
-sim_partial_kernel(const float *__restrict__ a, long long lda, long long stride, const __nv_bfloat16 *__restrict__ b, long long ldb, int d, int t_first,
-                   int t_end, int T, float *__restrict__ partial)
+sim_partial_kernel(const __nv_bfloat16 *__restrict__ a, long long lda, const __nv_bfloat16 *__restrict__ b, long long ldb, int d, int t_first, int t_end, int T,
+                   float *__restrict__ partial)
 {
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int t0 = t_first + blockIdx.x * 64 + 2 * lane;             // t_first is even: the loads of two tokens stay aligned
+    const int t0 = t_first + blockIdx.x * 64 + 2 * lane;             // t_first is even: 4-byte loads of two tokens stay aligned
     const int per = (d + kSimSlices - 1) / kSimSlices;
     const int f0 = blockIdx.y * per, f1 = min(d, f0 + per);
     float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (t0 < t_end) {
-        const float *ap = a + (t0 - t_first);                        // slab columns begin with token t_first
-        auto term = [&](const float2 *v, uint32_t wb) {
-            float2 x = v[0];
-#pragma unroll
-            for (int i = 1; i < NS; ++i) { x.x += v[i].x; x.y += v[i].y; }
-            const float a0 = __bfloat162float(__float2bfloat16_rn(x.x)), a1 = __bfloat162float(__float2bfloat16_rn(x.y));
+        const __nv_bfloat16 *ap = a + (t0 - t_first);
+        auto term = [&](uint32_t wa, uint32_t wb) {
+            const float a0 = bf16_bits_to_f32(wa & 0xFFFFu), a1 = bf16_bits_to_f32(wa >> 16);
             const float b0 = bf16_bits_to_f32(wb & 0xFFFFu), b1 = bf16_bits_to_f32(wb >> 16);
             acc[0] = fmaf(a0, b0, acc[0]); acc[1] = fmaf(a0, a0, acc[1]); acc[2] = fmaf(b0, b0, acc[2]);
             acc[3] = fmaf(a1, b1, acc[3]); acc[4] = fmaf(a1, a1, acc[4]); acc[5] = fmaf(b1, b1, acc[5]);
         };
         constexpr int U = 8;
         for (int f = f0 + warp; f < f1; f += 8 * U) {                // eight features per round, all their loads in flight
-            float2 v[U][NS];
-            uint32_t wb[U];
+            uint32_t wa[U], wb[U];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int fu = f + 8 * u;
                 if (fu < f1) {
-#pragma unroll
-                    for (int i = 0; i < NS; ++i) v[u][i] = *reinterpret_cast<const float2 *>(ap + i * stride + (long long)fu * lda);
+                    wa[u] = *reinterpret_cast<const uint32_t *>(ap + (long long)fu * lda);
                     wb[u] = *reinterpret_cast<const uint32_t *>(b + (long long)fu * ldb + t0);
                 }
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u) if (f + 8 * u < f1) term(v[u], wb[u]);
+            for (int u = 0; u < U; ++u) if (f + 8 * u < f1) term(wa[u], wb[u]);
         }
     }
     __shared__ float s[8][32][6];
@@ -348,16 +342,14 @@ int32_t launch_fold_norm_rows(const float *slabs, int n_slabs, long long slab_st
     return SFS_OK;
 }
 
-int32_t launch_sim_partial(const float *vnew_t, long long ld_new, int n_slabs, long long slab_stride, const void *vold_t, long long ld_old, int d,
-                           int t_first, int t_count, int T, float *partial, cudaStream_t s)
+int32_t launch_sim_partial(const void *vnew_t, long long ld_new, const void *vold_t, long long ld_old, int d, int t_first, int t_count, int T,
+                           float *partial, cudaStream_t s)
 {
     if (t_count <= 0) return SFS_OK;
-    SFS_REQUIRE((t_first % 2) == 0 && (ld_new % 2) == 0 && (ld_old % 2) == 0 && n_slabs >= 1 && n_slabs <= kSimSlabs, SFS_ERR_INVALID_ARG,
-                "similarity: first token and row strides must be even, at most %d slabs", kSimSlabs);
-    auto *kernel = n_slabs == 1 ? sim_partial_kernel<1> : (n_slabs == 2 ? sim_partial_kernel<2> : sim_partial_kernel<3>);
+    SFS_REQUIRE((t_first % 2) == 0 && (ld_new % 2) == 0 && (ld_old % 2) == 0, SFS_ERR_INVALID_ARG, "similarity: first token and row strides must be even");
     dim3 grid((unsigned)((t_count + 63) / 64), kSimSlices, 1);
-    SFS_CUDA(launch_pdl(kernel, grid, dim3((unsigned)(256)), (size_t)(0), s, vnew_t, ld_new, slab_stride, reinterpret_cast<const __nv_bfloat16 *>(vold_t), ld_old,
-                        d, t_first, t_first + t_count, T, partial));
+    SFS_CUDA(launch_pdl(sim_partial_kernel, grid, dim3((unsigned)(256)), (size_t)(0), s, reinterpret_cast<const __nv_bfloat16 *>(vnew_t), ld_new,
+                        reinterpret_cast<const __nv_bfloat16 *>(vold_t), ld_old, d, t_first, t_first + t_count, T, partial));
     return SFS_OK;
 }
 

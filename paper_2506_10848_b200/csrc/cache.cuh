@@ -7,11 +7,10 @@ namespace sfs {
 constexpr int kSimSlices = 32;         // the feature dimension is cut into this many slices for the similarity sums
 
 // partial[slice][t][0..2] = sum over the slice's features of (v_new * v_old, v_new^2, v_old^2) for the tokens
-// t_first <= t < t_first + t_count (t_first even); both operands are feature-major bf16 [d, T] with ld elements between
-// feature rows; partial is [kSimSlices, T, 3] whatever the token range.
-constexpr int kSimSlabs = 3;           // fresh values: fp32 slabs to add, at most; their columns begin with token t_first
-int32_t launch_sim_partial(const float *vnew_t, long long ld_new, int n_slabs, long long slab_stride, const void *vold_t, long long ld_old, int d,
-                           int t_first, int t_count, int T, float *partial, cudaStream_t s);
+// t_first <= t < t_first + t_count (t_first even); both operands are feature-major bf16 with ld elements between feature rows, the
+// new values' columns beginning with token t_first; partial is [kSimSlices, T, 3] whatever the token range.
+int32_t launch_sim_partial(const void *vnew_t, long long ld_new, const void *vold_t, long long ld_old, int d, int t_first, int t_count, int T,
+                           float *partial, cudaStream_t s);
 
 struct CacheSelectArgs {
     const float *partial;              // [kSimSlices, T, 3]
