@@ -278,7 +278,7 @@ static SmallGemmArgs small_args(sfs_session *s, int M, int N, int K, const int32
     return g;
 }
 static const __nv_bfloat16 *bf(const void *p) { return reinterpret_cast<const __nv_bfloat16 *>(p); }
-// `cache`: the step also fills the feature cache (keys, values and both increments of every layer)
+// `cache`: the step also fills the feature cache (keys and both increments of every layer; its values come from cache_values)
 static int32_t small_qkv(sfs_session *s, int l, int B, int S, const int32_t *d_tokens, const int32_t *d_active, bool cache, cudaStream_t st)
 {
     const sfs_model *m = s->model;
@@ -287,8 +287,18 @@ static int32_t small_qkv(sfs_session *s, int l, int B, int S, const int32_t *d_t
     g.n_per_map = c.d_model; g.gain = bf(m->attn_norm[l]); g.B[0] = bf(m->wq[l]); g.B[1] = bf(m->wk[l]); g.B[2] = bf(m->wv[l]);
     g.out = s->qk; g.ldc = 2 * c.d_model; g.vt = s->vt; g.ldvt = B * S; g.table = s->rope_table; g.S = S;
     g.tokens = d_tokens; g.emb = bf(m->tok_emb); g.vocab = c.vocab;
-    if (cache) { g.k_dst = s->Kc[l]; g.vt = s->Vtc[l]; }
+    if (cache) g.k_dst = s->Kc[l];
     return launch_small_gemm(d_tokens ? SMALL_EMBED : SMALL_NORM, SMALL_QKV, g, st);
+}
+// The values a small model's full refresh caches: not those of its own projection, which adds its products in another order than the
+// one the partial steps take fresh values from, but the latter's for all tokens.  An unchanged row then gets them again bit for bit.
+// Two launches per layer (2-layer model, 32 + 32 tokens: 34.8 -> 49.2 us a refresh; with the tensor-memory kernels throughout 95).
+static int32_t cache_values(sfs_session *s, int l, int T, const int32_t *d_active, cudaStream_t st)
+{
+    const sfs_config &c = s->model->cfg;
+    const int32_t rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, nullptr, 0, 0, s->model->attn_norm[l], s->h, nullptr, nullptr, T, c.d_model, c.rms_eps, st); });
+    if (rc != SFS_OK) return rc;
+    return timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(s->cache_plans[l].v_store, nullptr, d_active, device_status_word(), st); });
 }
 static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active, bool cache, cudaStream_t st)
 {
@@ -298,7 +308,8 @@ static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active,
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
         if (l > 0 && (rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, l, B, S, nullptr, d_active, cache, st); })) != SFS_OK) return rc;
-        if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(cache ? s->cache_plans[l].attn : s->attn_plan, d_active, device_status_word(), st); })) != SFS_OK) return rc;
+        if (cache && (rc = cache_values(s, l, T, d_active, st)) != SFS_OK) return rc;
+        if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, device_status_word(), st); })) != SFS_OK) return rc;
         rc = timed_launch(s, SFS_K_GEMM_O, st, [&] {
             SmallGemmArgs g = small_args(s, T, d, d, d_active);
             g.a = s->attn; g.lda = d; g.B[0] = bf(m->wo[l]); g.inc = cache ? s->Ac[l] : nullptr;
@@ -405,6 +416,11 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
         const void *h[1] = {s->h + (size_t)v_first * d};
         rc = gemm_plan_create(&cp.vproj, m->wv[l], d, d, d, h, 1, v_rows, d, GEMM_STORE, s->vt, T, 0, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
+        if (small_step(c, T)) {                                // (see cache_values)
+            const void *all[1] = {s->h};
+            rc = gemm_plan_create(&cp.v_store, m->wv[l], d, d, d, all, 1, T, d, GEMM_STORE, s->Vtc[l], T, 0, 1.0f, nullptr, 0, 0, nullptr);
+            if (rc != SFS_OK) return rc;
+        }
         const void *wo[1] = {m->wo[l]};
         rc = weight_plan_create(&cp.o_store, s->attn, d, T, d, wo, 1, d, d, GEMM_STORE, s->Ac[l], d, 1, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;

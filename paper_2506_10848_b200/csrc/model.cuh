@@ -16,7 +16,7 @@ struct sfs_model {
 
 struct LayerPlans { sfs::GemmPlan qkv, o, gate_up, down; };
 // cached mode: per layer, independent of how many rows are recomputed
-struct CacheLayerPlans { sfs::GemmPlan qkv_store, vproj, o_store, down_store; sfs::AttnPlan attn; };
+struct CacheLayerPlans { sfs::GemmPlan qkv_store, v_store, vproj, o_store, down_store; sfs::AttnPlan attn; };
 // cached mode: projections over the compact buffer of recomputed rows, per layer, for one row count
 struct GatherLayerPlans { sfs::GemmPlan qkv, o, gate_up, down; };
 

@@ -216,10 +216,14 @@ small_gemm_kernel(SmallGemmArgs g)
                 // the projection's result is rounded to bf16 and so is the rotated one, as when the two are kernels of their own
                 const float a0 = round_bf16(x0), a1 = round_bf16(x1), b0 = round_bf16(y0), b1 = round_bf16(y1);
                 const float4 cs = angle[h];
-                __nv_bfloat16 *dst = (map && g.k_dst ? g.k_dst + (long long)m * g.n_per_map : g.out + (long long)m * g.ldc + map * g.n_per_map)
-                                     + head * g.head_dim + j0 + q;
-                *reinterpret_cast<uint32_t *>(dst) = pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w);
-                *reinterpret_cast<uint32_t *>(dst + half) = pack2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
+                const uint32_t lo = pack2(a0 * cs.x - b0 * cs.y, a1 * cs.z - b1 * cs.w), hi = pack2(b0 * cs.x + a0 * cs.y, b1 * cs.z + a1 * cs.w);
+                const int col = head * g.head_dim + j0 + q;
+                __nv_bfloat16 *dst = g.out + (long long)m * g.ldc + map * g.n_per_map + col;
+                *reinterpret_cast<uint32_t *>(dst) = lo; *reinterpret_cast<uint32_t *>(dst + half) = hi;
+                if (map && g.k_dst) {
+                    dst = g.k_dst + (long long)m * g.n_per_map + col;
+                    *reinterpret_cast<uint32_t *>(dst) = lo; *reinterpret_cast<uint32_t *>(dst + half) = hi;
+                }
             } else {
                 __nv_bfloat16 *dst = g.vt + (long long)(tt * TILE + q) * g.ldvt + m;       // values go out transposed
                 dst[0] = __float2bfloat16_rn(x0); dst[g.ldvt] = __float2bfloat16_rn(x1);

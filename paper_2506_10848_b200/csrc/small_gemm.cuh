@@ -19,7 +19,7 @@ struct SmallGemmArgs {
     __nv_bfloat16 *out; float *out_f32; long long ldc; float scale;
     float *inc;                              // SMALL_RESIDUAL, optional [M, N]: receives what is added to x
     __nv_bfloat16 *vt; long long ldvt;       // SMALL_QKV: q and k rotated into out [M, 2 n_per_map], v transposed into vt [n_per_map, M]
-    __nv_bfloat16 *k_dst;                    // SMALL_QKV, optional [M, n_per_map]: k goes there instead
+    __nv_bfloat16 *k_dst;                    // SMALL_QKV, optional [M, n_per_map]: k goes there as well
     const float2 *table; int S, head_dim;    // rotary table, tokens per sequence
 };
 // combinations: (EMBED | NORM, QKV), (BF16, RESIDUAL), (NORM, SWIGLU), (NORM, STORE)

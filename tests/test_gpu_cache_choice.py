@@ -64,8 +64,10 @@ def similarity(a, b):
     return ordered_sum(a, b) / (np.sqrt(ordered_sum(a, a)) * np.sqrt(ordered_sum(b, b)))
 
 
-# one sequence (odd and even first response token) and two; row counts at which splitting K would pay; the long prompt
-@pytest.mark.parametrize("d,head_dim,B,P,L", [(2048, 128, 1, 19, 197), (2048, 128, 1, 64, 256), (2048, 128, 2, 40, 120), (4096, 128, 1, 1024, 512), (4096, 128, 1, 24, 768)])
+# one sequence (odd and even first response token) and two; a small model; as many K ranges as a planner might like for few rows; the
+# long prompt; a width that is no multiple of 8 slices
+@pytest.mark.parametrize("d,head_dim,B,P,L", [(256, 64, 1, 32, 64), (256, 64, 2, 24, 40), (384, 128, 1, 9, 55), (2048, 128, 1, 19, 197), (2048, 128, 1, 64, 256),
+                                              (2048, 128, 2, 40, 120), (4096, 128, 1, 1024, 512), (4096, 128, 1, 24, 768)])
 def test_row_sets_are_those_of_the_unsplit_values(d, head_dim, B, P, L):
     nl, S, rho = 2, P + L, 0.25
     shape, w = silent_model(d, head_dim, nl, 256, 1024, seed=d + L)
