@@ -333,13 +333,14 @@ static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active,
 }
 // final norm + LM head of up to max_rows listed rows in one launch, for vocabularies whose statistics the LM head does not take
 static bool small_logits(const sfs_config &c, int max_rows, int T) { return small_step(c, max_rows) && small_step(c, T) && c.vocab <= 16384; }
-static int32_t enqueue_small_logits(sfs_session *s, const int32_t *d_rows, const int32_t *d_n_rows, int max_rows, void *d_logits, int32_t logits_dtype,
+// (`known`: entries of d_rows that may be read whatever *d_n_rows says)
+static int32_t enqueue_small_logits(sfs_session *s, const int32_t *d_rows, int known, const int32_t *d_n_rows, int max_rows, void *d_logits, int32_t logits_dtype,
                                     const int32_t *d_active, cudaStream_t st)
 {
     const sfs_config &c = s->model->cfg;
     return timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] {
         SmallGemmArgs g = small_args(s, max_rows, c.vocab, c.d_model, d_active);
-        g.d_m = d_n_rows; g.rows = d_rows; g.gain = bf(s->model->final_norm); g.B[0] = bf(s->model->lm_head); g.scale = c.logit_scale; g.ldc = c.vocab;
+        g.d_m = d_n_rows; g.rows = d_rows; g.rows_known = known; g.gain = bf(s->model->final_norm); g.B[0] = bf(s->model->lm_head); g.scale = c.logit_scale; g.ldc = c.vocab;
         if (logits_dtype == SFS_LOGITS_F32) g.out_f32 = reinterpret_cast<float *>(d_logits);
         else g.out = reinterpret_cast<__nv_bfloat16 *>(d_logits);
         return launch_small_gemm(SMALL_NORM, SMALL_STORE, g, st);
@@ -818,7 +819,7 @@ int32_t sfs_forward(sfs_session *s, const int32_t *d_tokens, int32_t B, int32_t 
     if ((rc = logits_plan(s, &lm, max_rows, d_logits, logits_dtype)) != SFS_OK) return rc;
     if (small_logits(s->model->cfg, max_rows, B * S))
         return run_uncached(s, d_tokens, B, S, nullptr, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
-                            [&](cudaStream_t st) { return enqueue_small_logits(s, d_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st); });
+                            [&](cudaStream_t st) { return enqueue_small_logits(s, d_rows, d_n_rows ? 0 : max_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st); });
     return run_uncached(s, d_tokens, B, S, nullptr, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
                         [&](cudaStream_t st) { return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st); });
 }
@@ -951,7 +952,7 @@ int32_t sfs_forward_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, i
     return run_cached(s, d_tokens, B, S, P, d_state, nullptr, d_sets, d_sims, n_sel, logits_kind(max_rows, logits_dtype, d_n_rows), StepMode{}, st,
                       [&](cudaStream_t st) {
                           if (s->pending_n == 0 && small_logits(s->model->cfg, max_rows, B * S))
-                              return enqueue_small_logits(s, d_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st);
+                              return enqueue_small_logits(s, d_rows, d_n_rows ? 0 : max_rows, d_n_rows, max_rows, d_logits, logits_dtype, nullptr, st);
                           return enqueue_logits(s, lm, d_rows, d_n_rows, max_rows, st);
                       });
 }
@@ -1022,7 +1023,7 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
         auto tail = [&](cudaStream_t st) -> int32_t {
             int32_t rc;
             if (s->pending_n == 0 && small_logits(c, B * L, B * S)) {
-                if ((rc = enqueue_small_logits(s, rows, n_rows, B * L, s->logits, SFS_LOGITS_BF16, d_active, st)) != SFS_OK) return rc;
+                if ((rc = enqueue_small_logits(s, rows, B * L, n_rows, B * L, s->logits, SFS_LOGITS_BF16, d_active, st)) != SFS_OK) return rc;
             } else if ((rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->pending_ptr, s->pending_n, s->pending_stride, s->model->final_norm, s->hfin, rows, n_rows, B * L, c.d_model, c.rms_eps, st); })) != SFS_OK) return rc;
             else if ((rc = timed_launch(s, SFS_K_GEMM_LM_HEAD, st, [&] { return gemm_launch(s->lm_plan, n_rows, d_active, err, st); })) != SFS_OK) return rc;
             if (d_logits_dump) {

@@ -86,7 +86,8 @@ small_gemm_kernel(SmallGemmArgs g)
 
     pdl_wait();                                             // weights are constant; everything else may come from the kernel before
     pdl_trigger();                                          // (not earlier: see pdl_trigger)
-    // the row count and the flag are used only after the loads below have been issued (which stay within g.M rows)
+    // the row count and the flag are used only after the loads below have been issued (which stay within g.M rows), but for a caller's
+    // row list, which ends with the count
     const int M = g.d_m ? min(*g.d_m, g.M) : g.M;
     const bool active = g.d_active == nullptr || *g.d_active != 0;
     float2 xr[2][2];
@@ -112,11 +113,22 @@ small_gemm_kernel(SmallGemmArgs g)
 #pragma unroll
         for (int r0 = 0; r0 < PER; r0 += ROWS) {
             float4 v[ROWS][NCH];
+            int listed[ROWS];                               // (all rows' entries at once: row by row, each would be a round trip)
+#pragma unroll
+            for (int u = 0; u < ROWS; ++u) {
+                const int e = list_entry_early(g, m0 + warp * PER + r0 + u);
+                listed[u] = e >= 0 ? g.rows[e] : 0;
+            }
+            if (g.rows != nullptr && g.rows_known < M)
+#pragma unroll
+                for (int u = 0; u < ROWS; ++u) {
+                    const int e = list_entry_late(g, m0 + warp * PER + r0 + u, M);
+                    if (e >= 0) listed[u] = g.rows[e];
+                }
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
                 const int m = m0 + warp * PER + r0 + u;
-                const int listed = g.rows && m < g.M ? g.rows[m] : 0;
-                const long long src = g.rows ? (m < M ? listed : 0) : (m < g.M ? m : 0);
+                const long long src = g.rows ? (m < M ? listed[u] : 0) : (m < g.M ? m : 0);
                 const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
                 const uint2 *er = nullptr;
                 if (SRC == SMALL_EMBED) {

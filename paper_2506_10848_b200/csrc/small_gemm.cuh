@@ -13,7 +13,8 @@ struct SmallGemmArgs {
     const __nv_bfloat16 *a; long long lda;   // SMALL_BF16: activation rows
     float *x;                                // fp32 residual stream [., K] (read by SMALL_NORM, written by SMALL_EMBED), [., N] for SMALL_RESIDUAL
     const __nv_bfloat16 *gain; float eps;
-    const int32_t *rows;                     // optional: row m is row rows[m] of x
+    const int32_t *rows;                     // optional: row m is row rows[m] of x, for m below the row count
+    int rows_known;                          // entries of `rows` that are there whatever *d_m says
     const int32_t *tokens; const __nv_bfloat16 *emb; int vocab;      // SMALL_EMBED
     const __nv_bfloat16 *B[3]; int n_per_map;                        // weights [n_per_map, K] each (model weights: constant)
     __nv_bfloat16 *out; float *out_f32; long long ldc; float scale;
@@ -22,6 +23,10 @@ struct SmallGemmArgs {
     __nv_bfloat16 *k_dst;                    // SMALL_QKV, optional [M, n_per_map]: k goes there as well
     const float2 *table; int S, head_dim;    // rotary table, tokens per sequence
 };
+// The entry of the row list that output row m reads before the device's row count has arrived, and the one it reads after it (M);
+// -1: none.  A caller's list ends with the count, so nothing beyond it may be touched, not even to throw the value away.
+__host__ __device__ inline int list_entry_early(const SmallGemmArgs &g, int m) { return g.rows != nullptr && m < g.rows_known ? m : -1; }
+__host__ __device__ inline int list_entry_late(const SmallGemmArgs &g, int m, int M) { return g.rows != nullptr && m >= g.rows_known && m < M ? m : -1; }
 // combinations: (EMBED | NORM, QKV), (BF16, RESIDUAL), (NORM, SWIGLU), (NORM, STORE)
 int32_t launch_small_gemm(int src, int epi, const SmallGemmArgs &g, cudaStream_t s);
 // whether a model's widths fit these kernels (all of K in shared memory, a row's norm in a warp's registers)
