@@ -111,8 +111,20 @@ static int32_t session_alloc_select(sfs_session *s)
     return SFS_OK;
 }
 
+// While a stream capture goes on elsewhere in the process (on another stream of this thread, or, by default, on any thread), calls
+// like cudaGraphInstantiate are refused to this thread and end that capture.  What the library records, it records on a stream of its
+// own: nothing of it conflicts with anybody's capture, so the thread says so while it handles its graphs.
+struct OwnCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    OwnCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~OwnCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    OwnCapture(const OwnCapture &) = delete;
+    OwnCapture &operator=(const OwnCapture &) = delete;
+};
+
 static void drop_graphs(sfs_session *s)
 {
+    OwnCapture own;
     for (auto &kv : s->graphs) {
         if (kv.second.exec) cudaGraphExecDestroy(kv.second.exec);
         if (kv.second.graph) cudaGraphDestroy(kv.second.graph);
@@ -223,6 +235,7 @@ static int32_t run_step(sfs_session *s, const StepKey &key, const StepMode &mode
     };
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (mode.plain || s->profile || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return enqueue(st, nullptr);
+    OwnCapture own;
     if (s->graphs.size() >= kMaxGraphs && s->graphs.find(key) == s->graphs.end()) drop_graphs(s);
     StepGraph &g = s->graphs[key];
     if (mode.fixed && g.exec && g.sig != *mode.fixed) {      // recorded for other parameters: start over

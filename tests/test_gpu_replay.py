@@ -1,5 +1,7 @@
 """Steps replayed as recorded graphs against the same steps launched one by one (a session that is being profiled never replays): from
 its sixteenth use on a kind of step sets the arguments of recorded launches, and everything a call brings has to reach them."""
+import threading
+
 import pytest
 import torch
 
@@ -79,3 +81,48 @@ def test_replayed_cached_steps_take_every_argument_of_their_call(shape, B, P, L,
             kept.append((d_tok, state, rows, n, p.both(lambda s, o: sfs.sfs_forward_cached(s, d_tok, B, S, P, state, rows, n, 24, o, sfs.LOGITS_BF16), 24, shape.vocab,
                                                        sfs.LOGITS_BF16)))
             kept = kept[-9:]
+
+
+@pytest.mark.parametrize("where", ["same thread", "other thread"])
+def test_recording_does_not_end_a_capture_that_goes_on_elsewhere(where):
+    """A program captures work of its own (in the mode that watches all threads) while steps run on another stream: their recording, replay
+    and the loss of a recording when the length changes leave that capture alone, and the capture leaves them alone."""
+    shape = W.TINY
+    with Pair(shape, 1, 64) as p:
+        session, stream = p.sessions[0], torch.cuda.Stream()
+        tok = W.prompt_ids(1, 64, shape.vocab, seed=1).to(DEV)
+        out, plain = {}, {}
+        for S in (64, 56):
+            out[S], plain[S] = (torch.zeros((S, shape.vocab), dtype=torch.bfloat16, device=DEV) for _ in range(2))
+            sfs.sfs_forward(p.sessions[1], tok, 1, S, None, None, S, plain[S], sfs.LOGITS_BF16)
+        raised = []
+
+        def calls(S, n):
+            try:
+                torch.cuda.set_device(0)
+                for _ in range(n):
+                    sfs.sfs_forward(session, tok, 1, S, None, None, S, out[S], sfs.LOGITS_BF16, stream=stream)
+            except Exception as e:  # noqa: BLE001
+                raised.append(e)
+
+        def steps():
+            calls(64, 30)
+            calls(56, 30)
+            calls(64, 3)
+
+        calls(64, 3)                                            # what a first call sets up is set up
+        torch.cuda.synchronize()
+        x, g = torch.zeros(1000, device=DEV), torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=torch.cuda.Stream(), capture_error_mode="global"):
+            x += 1
+            if where == "same thread":
+                steps()
+            else:
+                t = threading.Thread(target=steps)
+                t.start()
+                t.join()
+            x += 1
+        g.replay()
+        torch.cuda.synchronize()
+        assert not raised and torch.all(x == 2.0)
+        assert all(torch.equal(out[S], plain[S]) for S in out)
