@@ -336,7 +336,7 @@ int32_t launch_fold_norm_rows(const float *slabs, int n_slabs, long long slab_st
     if (n_rows <= 0) return SFS_OK;
     SFS_REQUIRE((size_t)d * 4 <= 96 * 1024, SFS_ERR_UNSUPPORTED, "d_model %d too wide for the fused fold + norm", d);
     const size_t smem = (size_t)d * 4;
-    if (smem > 48 * 1024) SFS_CUDA(cudaFuncSetAttribute(fold_norm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    SFS_CUDA(allow_shared(fold_norm_rows_kernel, smem));
     SFS_CUDA(launch_pdl(fold_norm_rows_kernel, dim3((unsigned)(n_rows)), dim3((unsigned)(d >= 4096 ? 1024 : (d >= 2048 ? 512 : 256))), (size_t)(smem), s, slabs, n_slabs < 1 ? 1 : n_slabs, slab_stride, rows, x, inc, reinterpret_cast<const __nv_bfloat16 *>(gain),
                                                     reinterpret_cast<__nv_bfloat16 *>(h), d, eps));
     return SFS_OK;
@@ -355,7 +355,7 @@ int32_t launch_sim_partial(const void *vnew_t, long long ld_new, const void *vol
 
 int32_t launch_cache_select(const CacheSelectArgs &a, cudaStream_t s)
 {
-    if ((size_t)a.L * 4 > 48 * 1024) SFS_CUDA(cudaFuncSetAttribute(cache_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, a.L * 4));
+    SFS_CUDA(allow_shared(cache_select_kernel, (size_t)a.L * 4));
     SFS_CUDA(launch_pdl(cache_select_kernel, dim3((unsigned)(a.B)), dim3(kChoiceThreads), (size_t)a.L * 4, s, a));
     return SFS_OK;
 }

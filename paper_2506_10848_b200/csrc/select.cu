@@ -445,9 +445,7 @@ int32_t launch_select(const SelectArgs &args, cudaStream_t stream)
     SelectArgs a = args;
     const size_t smem = (size_t)a.L * (sizeof(unsigned long long) + 1);
     SFS_REQUIRE(smem <= 200 * 1024, SFS_ERR_UNSUPPORTED, "gen_len %d too long for the selection kernel", a.L);
-    if (smem > 48 * 1024) {
-        SFS_CUDA(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    }
+    SFS_CUDA(allow_shared(select_kernel, smem));
     // two-pass statistics: two CTAs per SM over all sequences share the recomputation (k > 1 can ask for every row)
     a.groups = 1;
     if (a.pos_lo != nullptr) a.groups = a.B < 148 ? 296 / a.B : 1;

@@ -122,6 +122,17 @@ static inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), int clust
 }
 #endif
 
+// A launch may use 48 KB of shared memory unasked, static arrays included (these kernels have a few KB of them at most): more is asked
+// for here.  Comparing the dynamic part alone with 48 KB left a band of sizes just below it that no launch accepted.
+#ifdef __CUDACC__
+constexpr size_t kUnaskedShared = 40 * 1024;
+template <typename... KArgs>
+static inline cudaError_t allow_shared(void (*kernel)(KArgs...), size_t dynamic)
+{
+    return dynamic > kUnaskedShared ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic) : cudaSuccess;
+}
+#endif
+
 // ---- device helpers ---------------------------------------------------------------------------------
 #ifdef __CUDACC__
 __device__ __forceinline__ float bf16_bits_to_f32(uint32_t h16) { return __uint_as_float(h16 << 16); }

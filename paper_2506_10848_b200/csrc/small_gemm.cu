@@ -262,8 +262,8 @@ int32_t launch(const SmallGemmArgs &g, int n_tiles, cudaStream_t s)
     const size_t smem = smem_bytes(g.K);
     static size_t configured[kMaxDevices] = {};
     size_t &done = configured[current_device_slot()];
-    if (smem > 48 * 1024 && smem > done) {
-        SFS_CUDA(cudaFuncSetAttribute(small_gemm_kernel<SRC, EPI, NCH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    if (smem > done) {
+        SFS_CUDA(allow_shared(small_gemm_kernel<SRC, EPI, NCH>, smem));
         done = smem;
     }
     SFS_CUDA(launch_pdl(small_gemm_kernel<SRC, EPI, NCH>, dim3((unsigned)n_tiles, (unsigned)((g.M + TILE - 1) / TILE)), dim3(kThreads), smem, s, g));

@@ -110,3 +110,27 @@ def test_row_sets_are_those_of_the_unsplit_values(d, head_dim, B, P, L):
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
+
+
+# a candidate takes 4 bytes of the choice's shared memory, a recomputed row 4 per feature: both sides of the 48 KB that a launch has unasked
+@pytest.mark.parametrize("d,P,L", [(128, 8, 10240), (128, 8, 12256), (128, 8, 12280), (128, 8, 12288), (12288, 8, 8)])
+def test_shared_memory_of_long_responses_and_wide_models(d, P, L):
+    shape = W.Shape(n_layers=1, d_model=d, n_heads=d // 128, head_dim=128, d_ff=128, vocab=64, mask_id=63, rms_eps=1e-5, rope_theta=10000.0, logit_scale=1.0)
+    model = sfs.Model(shape, W.model_weights(shape, seed=1, device=DEV))
+    session = sfs.sfs_session_create(model, 1, P + L)
+    try:
+        sfs.sfs_cache_enable(session, 100, 100, 0.25)
+        tok = W.prompt_ids(1, P + L, shape.vocab, seed=2).to(DEV)
+        rows = torch.arange(P + L - 8, P + L, dtype=torch.int32, device=DEV)
+        lg = [torch.zeros((8, shape.vocab), dtype=torch.float32, device=DEV) for _ in range(2)]
+        sets, sims = torch.zeros(P + L, dtype=torch.int32, device=DEV), torch.zeros(L, dtype=torch.float32, device=DEV)
+        for step in range(2):
+            if step:
+                tok[0, P:P + L // 8] = 1
+            n_sel = sfs.sfs_forward_cached(session, tok, 1, P + L, P, None, rows, None, 8, lg[step], sfs.LOGITS_F32, sets=sets, sims=sims)
+        sfs.sfs_check_device_status()
+        assert sorted(int(r) - P for r in sets[:n_sel]) == C.least_similar(sims.cpu().numpy(), list(range(L)), C.adaptive_count(0.25, L))
+        assert bool(torch.isfinite(lg[1]).all())
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()

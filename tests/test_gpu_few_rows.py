@@ -1,5 +1,9 @@
 """Projections of at most 128 rows (CTA pairs, tensor-memory tiles of 64 rows per CTA): edges of the row, column and K tiles, and the
 row statistics the LM head leaves when a generation has that few response rows."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -103,6 +107,25 @@ def test_small_model_edges(dims, B, S):
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
+
+
+# d_ff 344 to 368: tiles near the 48 KB of shared memory that a launch has unasked.  A process of its own: what a launch has once asked
+# for stays granted, and other tests ask for more.
+@pytest.mark.parametrize("d_ff", [312, 336, 344, 368, 376])
+def test_small_model_is_the_first_to_use_its_shared_memory(d_ff):
+    code = f"""if True:
+        import torch
+        from paper_2506_10848_b200 import binding as sfs, workloads as W
+        shape = W.Shape(n_layers=1, d_model=128, n_heads=2, head_dim=64, d_ff={d_ff}, vocab=512, mask_id=511, rms_eps=1e-5, rope_theta=10000.0, logit_scale=1.0)
+        model = sfs.Model(shape, W.model_weights(shape, seed=1, device="cuda:0"))
+        session = sfs.sfs_session_create(model, 1, 64)
+        out = torch.full((64, 512), float("nan"), device="cuda:0")
+        sfs.sfs_forward(session, W.prompt_ids(1, 64, 512, seed=1).to("cuda:0"), 1, 64, None, None, 64, out, sfs.LOGITS_F32)
+        sfs.sfs_check_device_status()
+        assert bool(torch.isfinite(out).all())
+    """
+    r = subprocess.run([sys.executable, "-c", code], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))), capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
 
 
 # heads of 64, short sequences: one key block, blocks that end inside a warp's share, keys over 4 and 8 warps, one and two row tiles

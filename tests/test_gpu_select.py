@@ -100,6 +100,12 @@ def test_lockstep_default_params(seed):
     assert steps < 48                                       # parallel unmasking happened
 
 
+# a position takes 9 bytes of the selection's shared memory: both sides of the 48 KB that a launch has unasked
+@pytest.mark.parametrize("L", [4544, 4552, 5416, 5440, 5456, 5464])
+def test_lockstep_long_responses(L):
+    run_lockstep(B=1, P=8, L=L, V=64, pkw=dict(max_steps=3), seed=L)
+
+
 @pytest.mark.parametrize("seed,pkw", [
     (10, dict(k_max=3, w_hist=3, sigma2_stable=30.0, k_slow=2, k_fast=3)),
     (11, dict(k_max=1, w_hist=1, k_slow=4, min_high_count=3)),
