@@ -344,8 +344,16 @@ static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active,
     }
     return SFS_OK;
 }
-// final norm + LM head of up to max_rows listed rows in one launch, for vocabularies whose statistics the LM head does not take
-static bool small_logits(const sfs_config &c, int max_rows, int T) { return small_step(c, max_rows) && small_step(c, T) && c.vocab <= 16384; }
+// final norm + LM head of up to max_rows listed rows in one launch, for vocabularies whose statistics the LM head does not take, while
+// its 32 x 32 tiles are about one wave (a model wider than 256 has half as many on an SM: more of K in shared memory).  Whole
+// steps in us, against norm and tensor-memory projection: d 256 with 512 tiles (vocabulary 1000 / 4096 / 16384) 62 / 64, 41 / 43,
+// 37 / 39, with 768 84 / 86, 47 / 45, with 2048 (128 rows of 16384) 55 / 43; d 512 with 256 tiles 43 / 45 (64 rows of 4096), with 512
+// 51 / 49 (128 rows), with 1024 63 / 56 (256 rows of 4096: 80 / 71); 1024 rows of 16384 took 2.1 to 2.6 times as long at every width.
+static bool small_logits(const sfs_config &c, int max_rows, int T)
+{
+    const long long tiles = (long long)((max_rows + 31) / 32) * ((c.vocab + 31) / 32);
+    return small_step(c, T) && c.vocab <= 16384 && tiles <= (c.d_model <= 256 ? 4 : 2) * gemm_num_sms();
+}
 // (`known`: entries of d_rows that may be read whatever *d_n_rows says)
 static int32_t enqueue_small_logits(sfs_session *s, const int32_t *d_rows, int known, const int32_t *d_n_rows, int max_rows, void *d_logits, int32_t logits_dtype,
                                     const int32_t *d_active, cudaStream_t st)

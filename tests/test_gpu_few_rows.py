@@ -74,7 +74,9 @@ def test_generation_with_few_long_rows_is_reproduced_by_the_oracle(B, L, vocab, 
 
 # small models (fused 32 x 32 tiles): rows below, at and across a tile; both head widths; a d_ff whose K tail is 8; a ragged vocabulary;
 # the last shape has one row tile more than these kernels take
-@pytest.mark.parametrize("dims", [dict(d_model=256, n_heads=4, head_dim=64, d_ff=1000, vocab=1000), dict(d_model=384, n_heads=3, head_dim=128, d_ff=264, vocab=4104)])
+@pytest.mark.parametrize("dims", [dict(d_model=256, n_heads=4, head_dim=64, d_ff=1000, vocab=1000), dict(d_model=384, n_heads=3, head_dim=128, d_ff=264, vocab=4104),
+                                  # more LM-head tiles than one wave: the projections in front stay fused, the LM head is the tensor-memory kernel's
+                                  dict(d_model=256, n_heads=2, head_dim=128, d_ff=264, vocab=10000)])
 @pytest.mark.parametrize("B,S", [(1, 8), (3, 8), (1, 40), (2, 24), (1, 712)])
 def test_small_model_edges(dims, B, S):
     shape = W.Shape(n_layers=2, mask_id=dims["vocab"] - 1, rms_eps=1e-5, rope_theta=10000.0, logit_scale=8.0, **dims)
