@@ -113,22 +113,24 @@ small_gemm_kernel(SmallGemmArgs g)
 #pragma unroll
         for (int r0 = 0; r0 < PER; r0 += ROWS) {
             float4 v[ROWS][NCH];
-            int listed[ROWS];                               // (all rows' entries at once: row by row, each would be a round trip)
-#pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                const int e = list_entry_early(g, m0 + warp * PER + r0 + u);
-                listed[u] = e >= 0 ? g.rows[e] : 0;
-            }
-            if (g.rows != nullptr && g.rows_known < M)
+            int listed[ROWS] = {};                          // (all rows' entries at once: row by row, each would be a round trip)
+            if (EPI == SMALL_STORE) {                       // only the LM head takes a row list
 #pragma unroll
                 for (int u = 0; u < ROWS; ++u) {
-                    const int e = list_entry_late(g, m0 + warp * PER + r0 + u, M);
-                    if (e >= 0) listed[u] = g.rows[e];
+                    const int e = list_entry_early(g, m0 + warp * PER + r0 + u);
+                    listed[u] = e >= 0 ? g.rows[e] : 0;
                 }
+                if (g.rows != nullptr && g.rows_known < M)
+#pragma unroll
+                    for (int u = 0; u < ROWS; ++u) {
+                        const int e = list_entry_late(g, m0 + warp * PER + r0 + u, M);
+                        if (e >= 0) listed[u] = g.rows[e];
+                    }
+            }
 #pragma unroll
             for (int u = 0; u < ROWS; ++u) {
                 const int m = m0 + warp * PER + r0 + u;
-                const long long src = g.rows ? (m < M ? listed[u] : 0) : (m < g.M ? m : 0);
+                const long long src = EPI == SMALL_STORE && g.rows ? (m < M ? listed[u] : 0) : (m < g.M ? m : 0);
                 const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
                 const uint2 *er = nullptr;
                 if (SRC == SMALL_EMBED) {

@@ -13,7 +13,7 @@ struct SmallGemmArgs {
     const __nv_bfloat16 *a; long long lda;   // SMALL_BF16: activation rows
     float *x;                                // fp32 residual stream [., K] (read by SMALL_NORM, written by SMALL_EMBED), [., N] for SMALL_RESIDUAL
     const __nv_bfloat16 *gain; float eps;
-    const int32_t *rows;                     // optional: row m is row rows[m] of x, for m below the row count
+    const int32_t *rows;                     // SMALL_STORE, optional: row m is row rows[m] of x, for m below the row count
     int rows_known;                          // entries of `rows` that are there whatever *d_m says
     const int32_t *tokens; const __nv_bfloat16 *emb; int vocab;      // SMALL_EMBED
     const __nv_bfloat16 *B[3]; int n_per_map;                        // weights [n_per_map, K] each (model weights: constant)
