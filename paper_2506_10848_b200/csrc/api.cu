@@ -276,13 +276,22 @@ static int32_t run_step(sfs_session *s, const StepKey &key, const StepMode &mode
     return SFS_OK;
 }
 
-// Small models and few rows take kernels that do the row-wise work of the neighbours too (see small_gemm.cu), up to nine or so
-// tiles of the widest projection per SM: a whole step of the 2-layer d 256, d_ff 688 model takes, us against the tensor-memory
-// kernels, 64 rows 35 / 67, 512 61 / 84, 768 86 / 104, 1024 100 / 110, 1280 120 / 116, 8 x 224 139 / 113.
-static bool small_step(const sfs_config &c, int rows)
+// Small models and few rows take kernels that do the row-wise work of the neighbours too (see small_gemm.cu): up to nine or so tiles of
+// the widest projection per SM, and up to a number of multiply-adds in a layer's projections, beyond which mma.sync loses to the
+// tensor-memory kernels what the saved launches gain (a model wider than 256 has half as many tiles on an SM).  A whole step of
+// two layers, us against those kernels, on both sides of where they are level:
+//   d 128, d_ff 512: 1408 rows 87 / 105, 2048 111 / 123.  d 256: d_ff 128 2048 110 / 127, 2816 144 / 142, 5632 331 / 281; d_ff 256 2048 119 / 128,
+//   2560 146 / 138; d_ff 688 1024 96 / 105, 1280 115 / 110; d_ff 1024 704 92 / 100, 1024 113 / 107.
+//   d 384: d_ff 192 768 93 / 103, 1024 115 / 109; d_ff 384 640 92 / 96, 768 107 / 105; d_ff 1024 384 94 / 96, 512 110 / 100.
+//   d 512: d_ff 256 512 88 / 92, 640 99 / 94; d_ff 512 384 82 / 91, 512 100 / 96; d_ff 1368 192 66 / 80, 256 86 / 84, 512 140 / 100.
+// `part`: a full refresh of the feature cache has two launches more a layer and is level at half the work: d 256, d_ff 688 512 rows
+// 76 / 81, 1024 117 / 106; d 384, d_ff 384 384 91 / 95, 512 102 / 98; d 512, d_ff 1368 128 76 / 84, 224 100 / 86.
+static bool small_step(const sfs_config &c, int rows, int part = 1)
 {
-    return small_gemm_fits(c.d_model, c.d_ff, c.head_dim) && (long long)((rows + 31) / 32) * ((c.d_ff + 15) / 16) <= 1408;
+    const long long row_tiles = (rows + 31) / 32, d = c.d_model, work = 32 * row_tiles * (4 * d * d + 3 * d * c.d_ff);
+    return small_gemm_fits(c.d_model, c.d_ff, c.head_dim) && row_tiles * ((c.d_ff + 15) / 16) <= 1408 && work * part <= (d <= 256 ? 970000000ll : 740000000ll);
 }
+static bool small_refresh(const sfs_config &c, int rows) { return small_step(c, rows, 2); }
 static SmallGemmArgs small_args(sfs_session *s, int M, int N, int K, const int32_t *d_active)
 {
     const sfs_config &c = s->model->cfg;
@@ -438,7 +447,7 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
         const void *h[1] = {s->h + (size_t)v_first * d};
         rc = gemm_plan_create(&cp.vproj, m->wv[l], d, d, d, h, 1, v_rows, d, GEMM_STORE, s->vt, T, 0, 1.0f, nullptr, 0, 0, nullptr);
         if (rc != SFS_OK) return rc;
-        if (small_step(c, T)) {                                // (see cache_values)
+        if (small_refresh(c, T)) {                             // (see cache_values)
             const void *all[1] = {s->h};
             rc = gemm_plan_create(&cp.v_store, m->wv[l], d, d, d, all, 1, T, d, GEMM_STORE, s->Vtc[l], T, 0, 1.0f, nullptr, 0, 0, nullptr);
             if (rc != SFS_OK) return rc;
@@ -613,7 +622,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
     s->pending_ptr = (rp && rr) ? s->Fc[c.n_layers - 1] : s->Ac[c.n_layers - 1];
     s->pending_n = (rp && rr) ? 1 : 2; s->pending_stride = inc_stride;
     // (a dump writes to the caller's buffers: not recorded)
-    if (rp && rr && small_step(c, T)) {
+    if (rp && rr && small_refresh(c, T)) {
         // everything is recomputed: the kernels of an uncached step (also of its logits, see the callers), which fill the cache as they go
         s->pending_n = 0;
         rc = run_step(s, StepKey{2, tail_kind, d_active ? 1 : 0, 0, 0}, {mode.plain || d_sets || d_sims, mode.fixed}, st,
