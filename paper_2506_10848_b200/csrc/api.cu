@@ -74,16 +74,19 @@ static int32_t dev_alloc(sfs_session *s, T **out, size_t count, bool zero)
 // Row statistics of one selection step into the session's scratch: the first of two passes (filter + exact) for long bf16 rows,
 // whose second pass the selection kernel takes; the all-canonical kernels otherwise.  `a` learns which.
 static int32_t step_row_stats(sfs_session *s, const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
-                              const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, int32_t B, int32_t S, SelectArgs *a,
+                              const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows, int32_t B, int32_t S, int32_t P, SelectArgs *a,
                               cudaStream_t st, const GemmArgs *lm = nullptr)
 {
+    const TokenGrid grid = {B * S, S, P};
+    const int32_t rc = select_fits(S - P);                  // (statistics that no selection consumes would stay behind)
+    if (rc != SFS_OK) return rc;
     int32_t *err = device_status_word();
     if (max_rows <= 0 || !row_stats_two_pass_applies(d_logits, logits_dtype, vocab, ld))
         return launch_row_stats(d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, nullptr, nullptr, nullptr,
-                                s->pos_sq, s->pos_arg, B * S, err, st);
+                                s->pos_sq, s->pos_arg, grid, err, st);
     a->pos_lo = s->pos_lo; a->pos_hi = s->pos_hi; a->pos_row = s->pos_row; a->pos_max = s->pos_max; a->seq_ticket = s->seq_ticket;
     a->lrows = {reinterpret_cast<const uint4 *>(d_logits), (long long)(ld / 8), vocab / 8};
-    const BoundsScratch bs = {s->pos_lo, s->pos_hi, s->pos_arg, s->slice_partials, s->row_tickets, s->pos_row, s->pos_max, B * S};
+    const BoundsScratch bs = {s->pos_lo, s->pos_hi, s->pos_arg, s->slice_partials, s->row_tickets, s->pos_row, s->pos_max, grid};
     if (lm != nullptr && lm->stats != nullptr) {   // the LM head's epilogue has taken the first pass: the logits are read only for the open rows
         const int block = lm->few ? lm->bn / 2 : lm->bn;    // (few rows: an N-block's column halves are blocks of their own)
         const StatsLayout lay = {block, 64 * (((block + 63) / 64 + 1) / 2)};
@@ -865,7 +868,7 @@ int32_t sfs_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab,
     SFS_REQUIRE(max_rows >= 0, SFS_ERR_INVALID_ARG, "max_rows %d", max_rows);
     SFS_REQUIRE(aligned_to(d_logits, logits_dtype == SFS_LOGITS_BF16 ? 2 : 4), SFS_ERR_INVALID_ARG, "d_logits misaligned");
     return launch_row_stats(d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, nullptr, d_argmax,
-                            reinterpret_cast<unsigned long long *>(d_sq), d_conf, nullptr, nullptr, 0, device_status_word_if_any(),
+                            reinterpret_cast<unsigned long long *>(d_sq), d_conf, nullptr, nullptr, TokenGrid{0, 1, 0}, device_status_word_if_any(),
                             (cudaStream_t)stream);
 }
 
@@ -906,7 +909,7 @@ int32_t sfs_select(sfs_session *s, const void *d_logits, int32_t logits_dtype, i
     if (rc != SFS_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     SelectArgs a{};
-    rc = step_row_stats(s, d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, B, S, &a, st);
+    rc = step_row_stats(s, d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, B, S, P, &a, st);
     if (rc != SFS_OK) return rc;
     a.tokens = d_tokens; a.mask = d_mask; a.B = B; a.S = S; a.P = P; a.L = S - P;
     a.state = d_state; a.params = *params;
@@ -1063,7 +1066,7 @@ int32_t sfs_generate_steps(sfs_session *s, int32_t n_steps, int32_t *d_trace, in
             }
             SelectArgs a{};
             if ((rc = timed_launch(s, SFS_K_ROW_STATS, st, [&] {
-                     return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, &a, st, &s->lm_plan.args); })) != SFS_OK) return rc;
+                     return step_row_stats(s, s->logits, SFS_LOGITS_BF16, c.vocab, c.vocab, n_rows, B * L, rows, B, S, P, &a, st, &s->lm_plan.args); })) != SFS_OK) return rc;
             a.tokens = s->tokens; a.mask = s->mask; a.B = B; a.S = S; a.P = P; a.L = L;
             a.state = s->state; a.params = s->gen_params;
             a.pos_sq = s->pos_sq; a.pos_arg = s->pos_arg;

@@ -37,7 +37,7 @@ struct RowOut {
     const int32_t *rows;            // flat token index per logits row, or null
     int32_t *argmax; unsigned long long *sq; float *conf;       // dense by logits row (optional)
     unsigned long long *pos_sq; int32_t *pos_arg;               // scattered by flat token index (optional)
-    int32_t n_positions;                                        // size of the scattered arrays
+    TokenGrid grid;                                             // positions of the scattered arrays
     int32_t *err;                                               // device status word (optional)
 };
 
@@ -47,9 +47,8 @@ __device__ __forceinline__ void write_row(const RowOut &o, int row, int arg, uns
     if (o.conf) o.conf[row] = (float)((double)(1u << SFS_CONF_QBITS) / (double)S);
     if (o.rows && o.pos_sq) {
         const int p = o.rows[row];
-        if ((unsigned)p < (unsigned)o.n_positions) {
-            o.pos_sq[p] = S;
-            o.pos_arg[p] = arg;
+        if (o.grid.inside(p)) {
+            if (o.grid.response(p)) { o.pos_sq[p] = S; o.pos_arg[p] = arg; }
         } else if (o.err) {
             atomicExch(o.err, SFS_ERR_INVALID_ARG);               // a row index outside the token grid: skipped, reported
         }
@@ -421,7 +420,7 @@ struct BoundsOut {
     unsigned long long *pos_lo, *pos_hi; int32_t *pos_arg;  // scattered by flat token index (optional)
     int32_t *pos_row;                                       // with them: the logits row a position's statistics came from
     float *pos_max;                                         //            and the exact row maximum
-    int32_t n_positions; int32_t *err;
+    TokenGrid grid; int32_t *err;
     float4 *partial;                                        // scratch [max_rows * kSlices]: (slice max, reference, sum, argmax bits)
     int32_t *tickets;                                       // scratch [max_rows], zero between launches
 };
@@ -442,7 +441,8 @@ __device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, f
     if (out.argmax) out.argmax[row] = arg;
     if (out.rows && out.pos_lo) {
         const int p = out.rows[row];
-        if ((unsigned)p < (unsigned)out.n_positions) {
+        if (out.grid.inside(p)) {
+            if (!out.grid.response(p)) return;
             out.pos_lo[p] = lo; out.pos_hi[p] = hi; out.pos_arg[p] = arg; out.pos_row[p] = row; out.pos_max[p] = m;
         } else if (out.err) {
             atomicExch(out.err, SFS_ERR_INVALID_ARG);
@@ -708,11 +708,11 @@ int32_t launch_rows(const void *logits, long long ld, int vocab, const int32_t *
 int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
                          const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows,
                          int32_t *d_argmax, unsigned long long *d_sq, float *d_conf,
-                         unsigned long long *d_pos_sq, int32_t *d_pos_arg, int32_t n_positions, int32_t *d_err,
+                         unsigned long long *d_pos_sq, int32_t *d_pos_arg, TokenGrid grid, int32_t *d_err,
                          cudaStream_t stream)
 {
     if (max_rows <= 0) return SFS_OK;
-    RowOut out{d_rows, d_argmax, d_sq, d_conf, d_pos_sq, d_pos_arg, n_positions, d_err};
+    RowOut out{d_rows, d_argmax, d_sq, d_conf, d_pos_sq, d_pos_arg, grid, d_err};
     const bool fast = logits_dtype == SFS_LOGITS_BF16 && (vocab % 8) == 0 && (ld % 8) == 0 && aligned_to(d_logits, 16);
     if (fast) {
         const int nchunks = vocab / 8;
@@ -757,7 +757,7 @@ int32_t launch_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld,
         SFS_CUDA(cudaMemset(s_tickets[dev], 0, (size_t)max_rows * sizeof(int32_t)));
         s_rows[dev] = max_rows;
     }
-    BoundsOut out{nullptr, d_lo, d_hi, d_argmax, nullptr, nullptr, nullptr, nullptr, nullptr, 0, d_err, s_partial[dev], s_tickets[dev]};
+    BoundsOut out{nullptr, d_lo, d_hi, d_argmax, nullptr, nullptr, nullptr, nullptr, nullptr, TokenGrid{0, 1, 0}, d_err, s_partial[dev], s_tickets[dev]};
     return launch_bounds(reinterpret_cast<const uint4 *>(d_logits), ld / 8, vocab / 8, vocab, d_n_rows, max_rows, out, stream);
 }
 
@@ -766,7 +766,7 @@ int32_t launch_row_stats_two_pass(const void *d_logits, int32_t vocab, int64_t l
 {
     if (max_rows <= 0) return SFS_OK;
     const uint4 *lp = reinterpret_cast<const uint4 *>(d_logits);
-    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.n_positions, d_err,
+    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.grid, d_err,
                  reinterpret_cast<float4 *>(rf.slice_partials), rf.row_tickets};
     int32_t rc = launch_bounds(lp, ld / 8, vocab / 8, vocab, d_n_rows, max_rows, bo, stream);
     if (rc != SFS_OK) return rc;
@@ -777,7 +777,7 @@ int32_t launch_row_stats_from_partials(const void *stats, int32_t stats_ld, int3
                                        cudaStream_t stream)
 {
     if (max_rows <= 0) return SFS_OK;
-    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.n_positions, d_err,
+    BoundsOut bo{d_rows, nullptr, nullptr, nullptr, rf.pos_lo, rf.pos_hi, rf.pos_arg, rf.pos_row, rf.pos_max, rf.grid, d_err,
                  nullptr, nullptr};
     SFS_CUDA(launch_pdl(combine_partials_kernel, dim3((unsigned)((max_rows + 3) / 4)), dim3((unsigned)(128)), (size_t)(0), stream, reinterpret_cast<const float4 *>(stats), stats_ld, n_parts, d_n_rows, max_rows, vocab, bo,
                         reinterpret_cast<const __nv_bfloat16 *>(d_logits), (long long)ld, lay));

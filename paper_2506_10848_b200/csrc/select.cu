@@ -440,11 +440,19 @@ __global__ void state_init_kernel(sfs_state *state, int B, int L, sfs_params p)
 
 }  // namespace
 
+static size_t select_shared(int32_t L) { return (size_t)L * (sizeof(unsigned long long) + 1); }
+int32_t select_fits(int32_t L)
+{
+    SFS_REQUIRE(select_shared(L) <= 200 * 1024, SFS_ERR_UNSUPPORTED, "gen_len %d too long for the selection kernel", L);
+    return SFS_OK;
+}
+
 int32_t launch_select(const SelectArgs &args, cudaStream_t stream)
 {
     SelectArgs a = args;
-    const size_t smem = (size_t)a.L * (sizeof(unsigned long long) + 1);
-    SFS_REQUIRE(smem <= 200 * 1024, SFS_ERR_UNSUPPORTED, "gen_len %d too long for the selection kernel", a.L);
+    const size_t smem = select_shared(a.L);
+    const int32_t rc = select_fits(a.L);
+    if (rc != SFS_OK) return rc;
     SFS_CUDA(allow_shared(select_kernel, smem));
     // two-pass statistics: two CTAs per SM over all sequences share the recomputation (k > 1 can ask for every row)
     a.groups = 1;

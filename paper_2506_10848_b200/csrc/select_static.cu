@@ -95,7 +95,7 @@ extern "C" int32_t sfs_select_static(int32_t vocab, const void *d_logits, int32_
     SFS_CUDA(cudaMemsetAsync(sc->pos_sq, 0, sizeof(unsigned long long) * (size_t)B * S, st));
     SFS_CUDA(cudaMemsetAsync(sc->ticket, 0, sizeof(sc->ticket) + sizeof(sc->status), st));
     rc = launch_row_stats(d_logits, logits_dtype, vocab, ld, d_n_rows, max_rows, d_rows, nullptr, nullptr, nullptr,
-                          sc->pos_sq, sc->pos_arg, B * S, sc->status, st);
+                          sc->pos_sq, sc->pos_arg, TokenGrid{B * S, S, P}, sc->status, st);
     if (rc != SFS_OK) return rc;
     SelectArgs a{};
     a.tokens = d_tokens; a.mask = d_mask; a.B = B; a.S = S; a.P = P; a.L = S - P;

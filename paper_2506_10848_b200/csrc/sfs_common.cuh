@@ -213,14 +213,25 @@ __device__ __forceinline__ bool conf_exceeds(unsigned long long sq, float tau) {
 #endif
 
 // ---- internal launchers (defined in the .cu files) --------------------------------------------------
+// The token positions that statistics are scattered to: n = B * S of them, the first P of every S a prompt's.  Rows of prompt positions
+// are left out: the selection reads, and clears again, response positions only, and what stayed behind would be taken for the
+// statistics of a later call whose prompt is shorter (with a logits row that may lie beyond that call's buffer).
+struct TokenGrid {
+    int32_t n, S, P;
+#ifdef __CUDACC__
+    __device__ __forceinline__ bool inside(int p) const { return (unsigned)p < (unsigned)n; }
+    __device__ __forceinline__ bool response(int p) const { return p % S >= P; }
+#endif
+};
+
 // Row statistics (Section 3.1: greedy token and confidence).  Results are written densely by logits row
 // (d_argmax/d_sq/d_conf, each optional) and, when d_rows is given, scattered to d_pos_sq/d_pos_arg at the
-// flat token index of each row; an index outside [0, n_positions) is skipped and reported as SFS_ERR_INVALID_ARG
+// flat token index of each row; an index outside the grid is skipped and reported as SFS_ERR_INVALID_ARG
 // in *d_err (a device status word, optional), as is a bounded wait that gives up (SFS_ERR_TIMEOUT).
 int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
                          const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows,
                          int32_t *d_argmax, unsigned long long *d_sq, float *d_conf,
-                         unsigned long long *d_pos_sq, int32_t *d_pos_arg, int32_t n_positions, int32_t *d_err,
+                         unsigned long long *d_pos_sq, int32_t *d_pos_arg, TokenGrid grid, int32_t *d_err,
                          cudaStream_t stream);
 
 // Row statistics for the selection step in two passes over long bf16 rows (the filter + exact form):
@@ -234,7 +245,7 @@ struct BoundsScratch {
     int32_t *pos_arg;                                       // [positions] what the selection kernel reads
     float *slice_partials; int32_t *row_tickets;            // scratch of pass 1: [max rows * 8 * 4] floats, [max rows] (zeroed)
     int32_t *pos_row; float *pos_max;                       // [positions] logits row and exact row maximum of each position (pass 1)
-    int32_t n_positions;
+    TokenGrid grid;
 };
 constexpr int kRowStatsSlices = 8;
 // true when the two-pass form applies to this logits layout (long bf16 rows, 16-byte aligned)
@@ -279,6 +290,7 @@ struct SelectArgs {
     // host_active: [0] sequences still decoding, [1] steps finished, with kMayEnd when the next one may be the last
     int32_t *host_active, *step_count;                      // optional: the host's mirror, and the device's count of steps
 };
+int32_t select_fits(int32_t L);                             // SFS_OK, or the error of a response too long (before any statistics are written)
 int32_t launch_select(const SelectArgs &a, cudaStream_t stream);
 int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, int32_t *seq_rows_unused,
                           cudaStream_t stream);

@@ -146,6 +146,40 @@ def test_missing_row_is_reported_not_guessed():
         sfs.sfs_session_destroy(session)
 
 
+@pytest.mark.parametrize("V,dtype", [(1000, torch.bfloat16), (1000, torch.float32), (70000, torch.bfloat16)])
+def test_prompt_rows_of_an_earlier_call_are_not_taken_for_this_ones(V, dtype):
+    """Extra rows are ignored: a call that brings the rows of its prompt leaves nothing that a later call of the session, with a shorter
+    prompt and fewer rows, could take for statistics of its own."""
+    S, P, B = 64, 40, 2
+    po, pg = params_pair()
+    gen = torch.Generator().manual_seed(3)
+    session = sfs.sfs_select_session_create(V, B, S)
+    out = dict(sel_count=torch.zeros(B, dtype=torch.int32, device=DEV))
+    kind = sfs.LOGITS_BF16 if dtype == torch.bfloat16 else sfs.LOGITS_F32
+
+    def call(P, rows):
+        tokens = torch.full((B, S), V - 1, dtype=torch.int32, device=DEV)
+        mask = torch.zeros((B, S), dtype=torch.uint8, device=DEV); mask[:, P:] = 1
+        state = torch.zeros((B, sfs.STATE_INTS), dtype=torch.int32, device=DEV)
+        sfs.sfs_state_init(state, B, S - P, pg)
+        logits = synthetic_step_logits(len(rows), V, gen, dtype).to(DEV)
+        sfs.sfs_select(session, logits, kind, V, torch.tensor(rows, dtype=torch.int32, device=DEV), None, len(rows), tokens, mask, B, S, P, state, pg,
+                       out["sel_count"])
+        sfs.sfs_check_device_status()
+        return [state_to_dict(state[b]) for b in range(B)], int(mask.sum())
+
+    try:
+        states, left = call(P, list(range(B * S)))                    # prompt rows too
+        assert [s["status"] for s in states] == [0, 0] and left < B * (S - P)
+        states, left = call(0, [b * S + i for b in range(B) for i in range(P, S)])      # rows of the positions below P are missing
+        assert [s["status"] for s in states] == [sfs.ERR_MISSING_ROW] * B
+        assert left == B * S and out["sel_count"].tolist() == [0, 0]
+        states, left = call(0, list(range(B * S)))                    # and a complete call still works
+        assert [s["status"] for s in states] == [0, 0] and left < B * S
+    finally:
+        sfs.sfs_session_destroy(session)
+
+
 def test_epilogue_microbenchmark_one_slow_one_fast_step():
     """bf16 logits [256, 126464] with planted winners; one exploratory and one accelerated step from a given
     span [lo, hi), compared with the oracle."""
