@@ -59,50 +59,54 @@ constexpr int kThreads = 256;
 constexpr uint32_t kNegInf2 = 0xFF80FF80u;
 
 // ---- a logits row as 16-byte chunks -----------------------------------------------------------------------------
-// A row may start anywhere (its stride need not be a multiple of 16 bytes): chunk c holds the elements c * PER - off ..
-// c * PER - off + PER - 1 of the row, off = elements between the 16-byte boundary at or before the row's start and the start.
-// Chunks that lie inside the row are one vector load; the first and last one are put together from the row's own elements,
-// with -inf in the places outside it (adds nothing, never is the maximum's first position).
+// A row may start anywhere (its stride need not be a multiple of 16 bytes).  The `whole` chunks between its first and last 16-byte
+// boundary come first, one vector load each; the elements before and after them, together, are the last one or two chunks, put
+// together from the row's own elements with -inf in the places beyond (adds nothing, never is the maximum's first position).
+// So an unaligned row has as many chunks as an aligned one: one more took another chunk of every thread's registers, or a
+// second sweep, at every length that fills them (fp32 65536, 2048 rows: 345 us instead of 178 under the same rule).
 template <typename T> struct RowChunks {
     static constexpr int PER = 16 / (int)sizeof(T);
-    const T *row;
-    const uint4 *base;
-    int off, vocab, n, in0, in1;                            // n chunks; [in0, in1) lie inside the row
+    const uint4 *first;
+    int head, whole, vocab;                                 // elements before the whole chunks, their number, elements in all
     __device__ __forceinline__ RowChunks(const T *logits, long long ld, int r, int V) {
-        row = logits + (long long)r * ld;
-        const unsigned long long a = (unsigned long long)row;
-        off = (int)(a & 15u) / (int)sizeof(T);
-        base = reinterpret_cast<const uint4 *>(a & ~15ull);
+        const T *row = logits + (long long)r * ld;
+        const int off = (int)((unsigned long long)row & 15u) / (int)sizeof(T);
         vocab = V;
-        n = (off + V + PER - 1) / PER; in0 = off ? 1 : 0; in1 = (off + V) / PER;
+        head = off ? min(V, PER - off) : 0;
+        first = reinterpret_cast<const uint4 *>(row + head);
+        whole = (V - head) / PER;
     }
+    __device__ __forceinline__ int chunks() const { return (vocab + PER - 1) / PER; }
     static __device__ __forceinline__ uint4 nothing();      // PER times -inf
-    __device__ __forceinline__ uint4 load(int c) const {
-        if (c >= in0 && c < in1) return ld_stream(base + c);
-        return c < n ? edge(c) : nothing();
+    __device__ __forceinline__ uint4 load(int c) const { return c < whole ? ld_stream(first + c) : nothing(); }      // a whole chunk
+    __device__ __forceinline__ uint4 load_edge(int c) const { return edge(first, head, whole, vocab, c); }          // whole <= c < chunks()
+    // The chunks made of the row's two ends.  By value: with an address taken, the chunks a thread keeps would not stay in registers.
+    static __device__ __forceinline__ int edge_index(int head, int whole, int vocab, int c, int e) {      // position of element e, -1: none
+        const int k = (c - whole) * PER + e, ends = vocab - whole * PER;
+        return k < head ? k : (k < ends ? k + whole * PER : -1);
     }
-    __device__ __noinline__ uint4 edge(int c) const;
-    __device__ __forceinline__ int index(int c, int e) const { return c * PER + e - off; }
+    static __device__ __noinline__ uint4 edge(const uint4 *first, int head, int whole, int vocab, int c);
+    static __device__ __noinline__ int first_edge(int head, int whole, int vocab, int c, uint4 q, float m);      // first position of m in one
 };
 template <> __device__ __forceinline__ uint4 RowChunks<__nv_bfloat16>::nothing() { return make_uint4(kNegInf2, kNegInf2, kNegInf2, kNegInf2); }
 template <> __device__ __forceinline__ uint4 RowChunks<float>::nothing() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
-template <> __device__ __noinline__ uint4 RowChunks<__nv_bfloat16>::edge(int c) const {
-    uint32_t w[4];
-    for (int k = 0; k < 4; ++k) {
-        uint32_t h[2];
-        for (int e = 0; e < 2; ++e) {
-            const int i = index(c, 2 * k + e);
-            h[e] = (i >= 0 && i < vocab) ? reinterpret_cast<const unsigned short *>(row)[i] : 0xFF80u;
-        }
-        w[k] = h[0] | (h[1] << 16);
+template <> __device__ __noinline__ uint4 RowChunks<__nv_bfloat16>::edge(const uint4 *first, int head, int whole, int vocab, int c) {
+    const unsigned short *row = reinterpret_cast<const unsigned short *>(first) - head;
+    uint32_t h[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        const int i = edge_index(head, whole, vocab, c, e);
+        h[e] = i >= 0 ? row[i] : 0xFF80u;
     }
-    return make_uint4(w[0], w[1], w[2], w[3]);
+    return make_uint4(h[0] | (h[1] << 16), h[2] | (h[3] << 16), h[4] | (h[5] << 16), h[6] | (h[7] << 16));
 }
-template <> __device__ __noinline__ uint4 RowChunks<float>::edge(int c) const {
+template <> __device__ __noinline__ uint4 RowChunks<float>::edge(const uint4 *first, int head, int whole, int vocab, int c) {
+    const float *row = reinterpret_cast<const float *>(first) - head;
     uint32_t w[4];
+#pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const int i = index(c, e);
-        w[e] = (i >= 0 && i < vocab) ? __float_as_uint(row[i]) : 0xFF800000u;
+        const int i = edge_index(head, whole, vocab, c, e);
+        w[e] = i >= 0 ? __float_as_uint(row[i]) : 0xFF800000u;
     }
     return make_uint4(w[0], w[1], w[2], w[3]);
 }
@@ -114,6 +118,15 @@ template <> __device__ __forceinline__ float chunk_elem<__nv_bfloat16>(const uin
 }
 template <> __device__ __forceinline__ float chunk_elem<float>(const uint4 &v, int e) {
     return __uint_as_float(e == 0 ? v.x : (e == 1 ? v.y : (e == 2 ? v.z : v.w)));
+}
+template <typename T> __device__ __noinline__ int RowChunks<T>::first_edge(int head, int whole, int vocab, int c, uint4 q, float m) {
+    int best = 0x7FFFFFFF;
+#pragma unroll
+    for (int e = 0; e < PER; ++e) {
+        const int i = edge_index(head, whole, vocab, c, e);
+        if (i >= 0 && chunk_elem<T>(q, e) == m) best = min(best, i);
+    }
+    return best;
 }
 template <typename T> __device__ __forceinline__ float chunk_max(const uint4 &v);
 template <> __device__ __forceinline__ float chunk_max<__nv_bfloat16>(const uint4 &v) {
@@ -131,10 +144,10 @@ template <> __device__ __forceinline__ uint32_t chunk_terms<float>(const uint4 &
     return canon2(pack2(__uint_as_float(v.x), __uint_as_float(v.y)), k) + canon2(pack2(__uint_as_float(v.z), __uint_as_float(v.w)), k);
 }
 
-// One cluster (1, 2, 4 or 8 CTAs) per logits row, any element type, length and alignment; a thread keeps NV 16-byte chunks of
-// the row in registers between the two passes (rows of more than C * 256 * NV chunks read the rest a second time, from L2).
-template <typename T, int NV>
-__global__ void __launch_bounds__(kThreads, NV > 8 ? 2 : 4)
+// One cluster (1, 2, 4 or 8 CTAs) of NT threads each per logits row, any element type, length and alignment; a thread keeps NV 16-byte
+// chunks of the row in registers between the two passes (rows of more than C * NT * NV chunks read the rest a second time, from L2).
+template <typename T, int NV, int NT>
+__global__ void __launch_bounds__(NT, NT < 256 ? 16 : (NV > 8 ? 2 : 4))
 rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
 {
     cg::cluster_group cluster = cg::this_cluster();
@@ -146,8 +159,8 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     const int n_rows = n_rows_ptr ? min(*n_rows_ptr, max_rows) : max_rows;
     if (row >= n_rows) return;                              // uniform over the cluster
 
-    __shared__ float s_wmax[kThreads / 32];
-    __shared__ unsigned long long s_wsum[kThreads / 32];
+    __shared__ float s_wmax[NT / 32];
+    __shared__ unsigned long long s_wsum[NT / 32];
     __shared__ float s_max_of[8];                           // slice maxima of all CTAs of the cluster, pushed by their owners
     __shared__ unsigned long long s_row_sum;                // rank 0 only: the peers add their sums here ...
     __shared__ int s_row_arg, s_arrived;                    // ... and their first-maximum candidates, then count themselves in
@@ -155,12 +168,21 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const RowChunks<T> rc(logits, ld, row, vocab);
-    const int stride = C * kThreads, c0 = rank * kThreads + tid;
+    const int stride = C * NT, c0 = rank * NT + tid, n = rc.chunks();
+
+    // this thread's chunks at the row's ends beyond those it keeps
+    auto rest_of_edges = [&](auto &&f) {
+        if (rc.whole < n)
+            for (int c = max(rc.whole, NV * stride); c < n; ++c) if ((c - c0) % stride == 0) f(c, rc.load_edge(c));
+    };
 
     // ---- the only pass over HBM: this thread's chunks of the row, kept in registers
     uint4 v[NV];
 #pragma unroll
     for (int j = 0; j < NV; ++j) v[j] = rc.load(c0 + j * stride);
+    if (rc.whole < n)
+#pragma unroll
+        for (int j = 0; j < NV; ++j) if (c0 + j * stride >= rc.whole && c0 + j * stride < n) v[j] = rc.load_edge(c0 + j * stride);
     if (tid == 0) { s_cta_arg = 0x7FFFFFFF; s_row_sum = 0; s_row_arg = 0x7FFFFFFF; s_arrived = 0; }
     // every CTA of the cluster announces that it runs (its shared memory exists) before anybody writes into a peer
     if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -169,13 +191,14 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     float lmax = -INFINITY;
 #pragma unroll
     for (int j = 0; j < NV; ++j) lmax = fmaxf(lmax, chunk_max<T>(v[j]));
-    for (int c = c0 + NV * stride; c < rc.n; c += 4 * stride) {                  // the rest of a longer row: four loads in flight
+    for (int c = c0 + NV * stride; c < rc.whole; c += 4 * stride) {                  // the rest of a longer row: four loads in flight
         uint4 q[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) q[u] = rc.load(c + u * stride);
 #pragma unroll
         for (int u = 0; u < 4; ++u) lmax = fmaxf(lmax, chunk_max<T>(q[u]));
     }
+    rest_of_edges([&](int, const uint4 &q) { lmax = fmaxf(lmax, chunk_max<T>(q)); });
     float m = warp_max(lmax);
     if (lane == 0) s_wmax[warp] = m;
     __syncthreads();
@@ -186,7 +209,7 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
         if (tid < C) {
             float t = s_wmax[0];
 #pragma unroll
-            for (int w = 1; w < kThreads / 32; ++w) t = fmaxf(t, s_wmax[w]);
+            for (int w = 1; w < NT / 32; ++w) t = fmaxf(t, s_wmax[w]);
             *cluster.map_shared_rank(&s_max_of[rank], tid) = t;
         }
         cluster.sync();
@@ -195,27 +218,24 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     } else {
         m = s_wmax[0];
 #pragma unroll
-        for (int w = 1; w < kThreads / 32; ++w) m = fmaxf(m, s_wmax[w]);
+        for (int w = 1; w < NT / 32; ++w) m = fmaxf(m, s_wmax[w]);
     }
 
     // ---- first position of the maximum (only threads that hold it look)
     if (lmax == m) {
         int best = 0x7FFFFFFF;
+        auto look = [&](int c, const uint4 &q) {
+            int at = -1;
 #pragma unroll
-        for (int j = NV - 1; j >= 0; --j) {
+            for (int e = RowChunks<T>::PER - 1; e >= 0; --e) if (chunk_elem<T>(q, e) == m) at = e;
+            if (at < 0 || c >= n) return;
+            if (c < rc.whole) best = min(best, rc.head + c * RowChunks<T>::PER + at);
+            else best = min(best, RowChunks<T>::first_edge(rc.head, rc.whole, rc.vocab, c, q, m));
+        };
 #pragma unroll
-            for (int e = RowChunks<T>::PER - 1; e >= 0; --e) {
-                const int idx = rc.index(c0 + j * stride, e);
-                if (chunk_elem<T>(v[j], e) == m && idx >= 0 && idx < vocab) best = idx;
-            }
-        }
-        for (int c = c0 + NV * stride; c < rc.n && best == 0x7FFFFFFF; c += stride) {
-            const uint4 q = rc.load(c);
-            for (int e = RowChunks<T>::PER - 1; e >= 0; --e) {
-                const int idx = rc.index(c, e);
-                if (chunk_elem<T>(q, e) == m && idx >= 0 && idx < vocab) best = idx;
-            }
-        }
+        for (int j = 0; j < NV; ++j) look(c0 + j * stride, v[j]);
+        for (int c = c0 + NV * stride; c < rc.whole && best == 0x7FFFFFFF; c += stride) look(c, rc.load(c));
+        rest_of_edges(look);                                                      // (they may hold the row's beginning)
         if (best != 0x7FFFFFFF) atomicMin(&s_cta_arg, best);
     }
 
@@ -224,20 +244,21 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
     unsigned long long acc = 0;
 #pragma unroll
     for (int j = 0; j < NV; ++j) acc += chunk_terms<T>(v[j], k);
-    for (int c = c0 + NV * stride; c < rc.n; c += 4 * stride) {
+    for (int c = c0 + NV * stride; c < rc.whole; c += 4 * stride) {
         uint4 q[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) q[u] = rc.load(c + u * stride);
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc += chunk_terms<T>(q[u], k);
     }
+    rest_of_edges([&](int, const uint4 &q) { acc += chunk_terms<T>(q, k); });
     acc = warp_sum_u64(acc);
     if (lane == 0) s_wsum[warp] = acc;
     __syncthreads();
     if (tid == 0) {
         unsigned long long t = 0;
 #pragma unroll
-        for (int w = 0; w < kThreads / 32; ++w) t += s_wsum[w];
+        for (int w = 0; w < NT / 32; ++w) t += s_wsum[w];
         const int arg = s_cta_arg;
         if (C > 1) {
             // report to rank 0 (integer adds and a minimum: any arrival order gives the same result), then leave
@@ -673,10 +694,10 @@ int32_t launch_bounds(const uint4 *logits, long long ld_chunks, int nchunks, int
     return SFS_OK;
 }
 
-template <typename T, int NV>
+template <typename T, int NV, int NT = kThreads>
 int32_t launch_cluster(const void *logits, long long ld, int vocab, const int32_t *d_n_rows, int max_rows, int C, const RowOut &out, cudaStream_t stream)
 {
-    SFS_CUDA(launch_pdl_cluster(rowstats_cluster<T, NV>, C, dim3((unsigned)(max_rows * C)), dim3(kThreads), 0, stream,
+    SFS_CUDA(launch_pdl_cluster(rowstats_cluster<T, NV, NT>, C, dim3((unsigned)(max_rows * C)), dim3(NT), 0, stream,
                                 reinterpret_cast<const T *>(logits), ld, vocab, d_n_rows, max_rows, out, out.err));
     return SFS_OK;
 }
@@ -684,26 +705,38 @@ int32_t launch_cluster(const void *logits, long long ld, int vocab, const int32_
 template <typename T>
 int32_t launch_rows(const void *logits, long long ld, int vocab, const int32_t *d_n_rows, int max_rows, const RowOut &out, cudaStream_t stream)
 {
-    // Cluster size and chunks kept per thread.  A CTA costs ~2 us besides its chunks, so the fewest CTAs that keep at least 65 %
-    // of the row in registers (8 chunks a thread; 16 for rows beyond 256 KB) are best while they fill the machine, and
-    // more of them, down to 4 chunks a thread, when the rows are few.  Measured, us at 4 / 64 / 512 rows, three buffers in turn:
-    // bf16 50257: C = 2 8.6 / 9.4 / 28.3, C = 4 5.6 / 7.2 / 30.9, C = 8 4.9 / 7.5 / 45.1; fp32 50257: C = 4 7.3 / 9.5 / 41.2,
-    // C = 8 4.5 / 7.5 / 43.5; bf16 32000: C = 2 4.6 / 4.8 / 16.0, C = 4 4.0 / 5.1 / 20.8; bf16 8000: C = 1 2.6 / 2.9 / 5.2,
-    // C = 2 3.7 / 4.0 / 10.8 (the one-CTA-per-row two-sweep kernel before: bf16 50257 14.4 / 14.4 / 41.0, fp32 12.3 / 14.4 / 55.2).
-    const bool aligned = (reinterpret_cast<uintptr_t>(logits) % 16) == 0 && (ld * (long long)sizeof(T)) % 16 == 0;
-    const int nchunks = (int)((vocab * (long long)sizeof(T) + 15) / 16) + (aligned ? 0 : 1);      // an unaligned row touches one more
+    // Cluster size and chunks kept per thread.  A cluster costs a barrier and each of its CTAs ~2 us besides its chunks, so the fewest
+    // CTAs are best that leave a thread no more chunks than the other rows' CTAs hide: the more rows, the more of a row may be read a
+    // second time (from L2).  Below one CTA per SM more of them, down to 4 chunks a thread.  16 chunks are kept while two CTAs per SM
+    // hold all rows, or where that saves the second reading without a cluster.  us at 64 / 256 / 512 / 2048 rows, in brackets with the rule
+    // before (65 % of every row in registers):
+    //   bf16 16384 3.9 / 5.0 / 7.8 / 25 [3.9 / 6.8 / 8.5 / 27], 32000 4.9 / 7.6 / 14.3 / 45 [4.9 / 9.8 / 17.2 / 58], 50257 7.3 / 17.2 / 27.8 / 83 [7.3 / 17.4 / 31 / 103];
+    //   fp32 16384 4.2 / 5.8 / 11.2 / 33 [4.2 / 7.6 / 13.6 / 44], 65536 7.1 / 24 / 43 / 133 [7.5 / 25 / 47 / 172], 100000 11.6 / 36 / 62 / 210 [12.3 / 42 / 80 / 307];
+    //   at odd addresses bf16 126464 8.9 / 33 / 58 / 184 [10.3 / 35 / 66 / 250], fp32 65536 7.1 / 26 / 46 / 139 [12.5 / 46 / 90 / 346].
+    // Rows of up to 2 KB take CTAs of 64 threads: 2048 rows of 64 bf16 values 5.8 [8.0].
+    const int nchunks = (int)((vocab * (long long)sizeof(T) + 15) / 16);
+    if (nchunks <= 128) return launch_cluster<T, 2, 64>(logits, ld, vocab, d_n_rows, max_rows, 1, out, stream);
+    const int most = max_rows >= 1024 ? 33 : (max_rows >= 384 ? 25 : 19);      // chunks per thread
     int C = 1;
-    while (C < 8 && (long long)C * 8 * kThreads * 20 < 13LL * nchunks) C *= 2;
-    while (C < 8 && (long long)max_rows * C < 2 * num_sms_rowstats() && nchunks > C * 4 * kThreads) C *= 2;
+    while (C < 8 && nchunks > C * kThreads * most) C *= 2;
+    while (C < 8 && (long long)max_rows * C < 128 && nchunks > C * 4 * kThreads) C *= 2;
     const int per_thread = (nchunks + C * kThreads - 1) / (C * kThreads);
     if (per_thread <= 1) return launch_cluster<T, 1>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
     if (per_thread <= 2) return launch_cluster<T, 2>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
     if (per_thread <= 4) return launch_cluster<T, 4>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
-    if (C < 8 || per_thread <= 8) return launch_cluster<T, 8>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
+    if (per_thread <= 8 || !((long long)max_rows * C <= 400 || (C == 1 && per_thread <= 16)))
+        return launch_cluster<T, 8>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
     return launch_cluster<T, 16>(logits, ld, vocab, d_n_rows, max_rows, C, out, stream);
 }
 
 }  // namespace
+
+static bool staged_shape(int32_t logits_dtype, int32_t vocab, int64_t ld, const void *d_logits)
+{
+    const bool fast = logits_dtype == SFS_LOGITS_BF16 && (vocab % 8) == 0 && (ld % 8) == 0 && aligned_to(d_logits, 16);
+    const int nchunks = vocab / 8;
+    return fast && nchunks >= 8192 && (nchunks + kStagedCluster - 1) / kStagedCluster <= 2560;
+}
 
 int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld,
                          const int32_t *d_n_rows, int32_t max_rows, const int32_t *d_rows,
@@ -713,24 +746,18 @@ int32_t launch_row_stats(const void *d_logits, int32_t logits_dtype, int32_t voc
 {
     if (max_rows <= 0) return SFS_OK;
     RowOut out{d_rows, d_argmax, d_sq, d_conf, d_pos_sq, d_pos_arg, grid, d_err};
-    const bool fast = logits_dtype == SFS_LOGITS_BF16 && (vocab % 8) == 0 && (ld % 8) == 0 && aligned_to(d_logits, 16);
-    if (fast) {
+    if (staged_shape(logits_dtype, vocab, ld, d_logits)) {
         const int nchunks = vocab / 8;
         // Long rows (128 KB and more, slices of at most 40 KB): staged through shared memory, seven CTAs to an SM, unless the rows
-        // are so few that the register form's four to an SM are resident at once: 126464 bf16 logits, 64 rows 10.1 us against
-        // 12.3, 122 rows 16.3 against 15.7, 512 rows 51.8 against 46.1.
-        if (nchunks >= 8192 && (nchunks + kStagedCluster - 1) / kStagedCluster <= 2560 && max_rows * kStagedCluster > 4 * num_sms_rowstats())
+        // are so few that the register form's CTAs are resident at once.  us, staged against registers: 126464 bf16 logits 64 rows 10.0 /
+        // 8.6, 128 rows 17.0 / 17.1, 512 rows 46 / 54; 151936, more than eight chunks a thread of eight CTAs, 4 rows 7.0 / 6.3, 16 rows 6.9 / 8.2,
+        // 64 rows 10.8 / 11.7.
+        const long long resident = nchunks > 8 * 8 * kThreads ? 32 : 4 * num_sms_rowstats();
+        if ((long long)max_rows * kStagedCluster > resident)
             return launch_staged(reinterpret_cast<const uint4 *>(d_logits), ld / 8, nchunks, vocab, d_n_rows, max_rows, out, stream);
     }
     return logits_dtype == SFS_LOGITS_BF16 ? launch_rows<__nv_bfloat16>(d_logits, ld, vocab, d_n_rows, max_rows, out, stream)
                                            : launch_rows<float>(d_logits, ld, vocab, d_n_rows, max_rows, out, stream);
-}
-
-static bool staged_shape(int32_t logits_dtype, int32_t vocab, int64_t ld, const void *d_logits)
-{
-    const bool fast = logits_dtype == SFS_LOGITS_BF16 && (vocab % 8) == 0 && (ld % 8) == 0 && aligned_to(d_logits, 16);
-    const int nchunks = vocab / 8;
-    return fast && nchunks >= 8192 && (nchunks + kStagedCluster - 1) / kStagedCluster <= 2560;
 }
 
 bool row_stats_two_pass_applies(const void *d_logits, int32_t logits_dtype, int32_t vocab, int64_t ld)

@@ -50,6 +50,28 @@ def test_generic_paths_match_oracle(V, ld):
     assert np.array_equal(arg, refb["argmax"]) and np.array_equal(sq, refb["sq"])
 
 
+# rows starting at every offset from a 16-byte boundary; lengths around a thread's chunks (64 and 256 threads; 4, 8 and 16 of them), around
+# what a cluster keeps, and beyond it; few rows, and so many that fewer CTAs take a row
+@pytest.mark.parametrize("V", [1, 3, 8, 13, 64, 513, 1017, 1024, 1030, 4096, 8192, 16384, 16399, 32768, 33000, 65536, 70001, 131072, 200003])
+@pytest.mark.parametrize("rows,pad", [(9, 0), (9, 1), (19, 3), (17, 5), (400, 3), (1100, 1)])
+def test_rows_at_any_address_match_oracle(V, rows, pad):
+    if rows * V > 4.5e7:
+        pytest.skip("as many rows of this length add nothing")
+    g = torch.Generator().manual_seed(V + rows)
+    flat = torch.randn(rows * (V + pad) + 3, generator=g)
+    x = flat[3:].view(rows, V + pad)                             # the first row off the boundary too
+    for r in range(rows):                                        # ties: first and last element, or one somewhere and the last, or the first alone
+        at = [(0, V - 1), (int(torch.randint(0, V, (1,), generator=g)), V - 1), (0,)][r % 3]
+        x[r, list(at)] = 7.0
+    for dtype, kind in ((torch.float32, sfs.LOGITS_F32), (torch.bfloat16, sfs.LOGITS_BF16)):
+        full = flat.to(dtype)
+        dev = full.to(DEV)
+        host = full[3:].view(rows, V + pad)[:, :V].contiguous()
+        ref = RS.row_stats(W.bf16_bits(host) if dtype == torch.bfloat16 else host.numpy())
+        arg, sq, _ = gpu_stats(dev[3:].view(rows, V + pad), V, V + pad, kind)
+        assert np.array_equal(arg, ref["argmax"]) and np.array_equal(sq, ref["sq"])
+
+
 def test_special_values_and_device_row_count():
     V = 4096
     x = torch.zeros((6, V), dtype=torch.float32)
