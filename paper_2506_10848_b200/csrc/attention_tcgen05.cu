@@ -94,8 +94,9 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
         if (lane == 0) {
             // ---------------- TMA producer: Q once, then K tiles and V^T tiles through their own rings (a K stage is free
             // again as soon as its last S = Q K^T has been computed, a V stage after its last P V)
-            tc::mbar_expect_tx(bar_q, NQ * Q_BYTES);
-            for (int t = 0; t < NQ; ++t)
+            const int n_q = PAIR ? n_streams : 1;          // (a second tile that holds no queries is not loaded: 1024 heads of 128 over 64 tokens 35.1 us instead of 36.3)
+            tc::mbar_expect_tx(bar_q, (uint32_t)(n_q * Q_BYTES));
+            for (int t = 0; t < n_q; ++t)
 #pragma unroll
                 for (int kb = 0; kb < KB; ++kb)
                     tc::tma_load_2d(tc::smem_u32(sQ) + t * Q_BYTES + kb * (QT * 128), &tmQ, h * DH + kb * 64, qrow0 + t * QT, bar_q);
