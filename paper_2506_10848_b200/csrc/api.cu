@@ -886,7 +886,7 @@ int32_t sfs_state_init(sfs_state *d_state, int32_t B, int32_t gen_len, const sfs
     SFS_REQUIRE(d_state != nullptr && B >= 1 && gen_len >= 0, SFS_ERR_INVALID_ARG, "state_init: bad arguments");
     int32_t rc = check_params(params, gen_len);
     if (rc != SFS_OK) return rc;
-    return launch_state_init(d_state, B, gen_len, *params, nullptr, (cudaStream_t)stream);
+    return launch_state_init(d_state, B, gen_len, *params, (cudaStream_t)stream);
 }
 
 int32_t sfs_select(sfs_session *s, const void *d_logits, int32_t logits_dtype, int64_t ld,

@@ -1,10 +1,10 @@
 // The transition rule S of one denoising step, on the device: the SlowFast rule (paper Section 3.3, Algorithm 1) or one of
 // the LLaDA strategies of Section 3.1 (low-confidence / random remasking, optionally block by block).
-// One CTA per sequence: it reads the row statistics the epilogue scattered by token position, applies the
-// exploratory (slow) or accelerated (fast) rule, unmasks the chosen positions in place, advances the
-// per-sequence state (k, s_cycle, e_cycle, H_W, phase) and lists the rows the next step needs.  The last CTA
-// to finish concatenates the per-sequence row lists (sequence-major, positions ascending) so that the
-// next forward pass gets one deterministic row list without a host round trip.
+// One CTA per sequence (with two-pass statistics a group of them, of which the last to finish goes on alone) reads the row
+// statistics scattered by token position, applies the exploratory (slow) or accelerated (fast) rule, unmasks the chosen
+// positions in place, advances the per-sequence state (k, s_cycle, e_cycle, H_W, phase) and lists the rows the next step needs.
+// The last CTA to finish concatenates the per-sequence row lists (sequence-major, positions ascending) so that the next forward
+// pass gets one deterministic row list without a host round trip.
 #include "sfs_common.cuh"
 #include "canonical.cuh"
 
@@ -461,7 +461,7 @@ int32_t launch_select(const SelectArgs &args, cudaStream_t stream)
     return SFS_OK;
 }
 
-int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, int32_t *, cudaStream_t stream)
+int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, cudaStream_t stream)
 {
     state_init_kernel<<<(B + 63) / 64, 64, 0, stream>>>(d_state, B, L, p);
     SFS_LAUNCH_CHECK();

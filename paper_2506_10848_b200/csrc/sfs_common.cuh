@@ -57,7 +57,8 @@ int32_t *device_status_word_if_any();
 // when about one launch latency of their own work is left: after their wait if they are short, before the last epilogue if they
 // are GEMMs.  Called first thing, a whole row of kernels becomes resident, and each reaches its wait so long before its input is
 // there that the code behind the wait has left the instruction cache by then (small projection after attention, 192 tokens: 4.9
-// us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).
+// us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).  The two-stream attention
+// alone calls it first thing: its CTAs leave the projection that follows no room on their SMs, so nothing becomes resident early.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -292,7 +293,6 @@ struct SelectArgs {
 };
 int32_t select_fits(int32_t L);                             // SFS_OK, or the error of a response too long (before any statistics are written)
 int32_t launch_select(const SelectArgs &a, cudaStream_t stream);
-int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, int32_t *seq_rows_unused,
-                          cudaStream_t stream);
+int32_t launch_state_init(sfs_state *d_state, int32_t B, int32_t L, const sfs_params &p, cudaStream_t stream);
 
 }  // namespace sfs

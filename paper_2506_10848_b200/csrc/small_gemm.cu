@@ -108,67 +108,64 @@ small_gemm_kernel(SmallGemmArgs g)
                 else *reinterpret_cast<uint4 *>(sA + r * ld + c * 8) = zero;
         if (!active || m0 >= M) { cp_async_wait(); return; }
     } else {
-        constexpr int PER = TILE / kWarps, ROWS = PER;      // rows of a warp, all in flight
+        constexpr int ROWS = TILE / kWarps;                 // rows of a warp, all in flight
         const int q4 = K / 4;
+        float4 v[ROWS][NCH];
+        int listed[ROWS] = {};                          // (all rows' entries at once: row by row, each would be a round trip)
+        if (EPI == SMALL_STORE) {                       // only the LM head takes a row list
 #pragma unroll
-        for (int r0 = 0; r0 < PER; r0 += ROWS) {
-            float4 v[ROWS][NCH];
-            int listed[ROWS] = {};                          // (all rows' entries at once: row by row, each would be a round trip)
-            if (EPI == SMALL_STORE) {                       // only the LM head takes a row list
+            for (int u = 0; u < ROWS; ++u) {
+                const int e = list_entry_early(g, m0 + warp * ROWS + u);
+                listed[u] = e >= 0 ? g.rows[e] : 0;
+            }
+            if (g.rows != nullptr && g.rows_known < M)
 #pragma unroll
                 for (int u = 0; u < ROWS; ++u) {
-                    const int e = list_entry_early(g, m0 + warp * PER + r0 + u);
-                    listed[u] = e >= 0 ? g.rows[e] : 0;
+                    const int e = list_entry_late(g, m0 + warp * ROWS + u, M);
+                    if (e >= 0) listed[u] = g.rows[e];
                 }
-                if (g.rows != nullptr && g.rows_known < M)
+        }
 #pragma unroll
-                    for (int u = 0; u < ROWS; ++u) {
-                        const int e = list_entry_late(g, m0 + warp * PER + r0 + u, M);
-                        if (e >= 0) listed[u] = g.rows[e];
-                    }
+        for (int u = 0; u < ROWS; ++u) {
+            const int m = m0 + warp * ROWS + u;
+            const long long src = EPI == SMALL_STORE && g.rows ? (m < M ? listed[u] : 0) : (m < g.M ? m : 0);
+            const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
+            const uint2 *er = nullptr;
+            if (SRC == SMALL_EMBED) {
+                int id = g.tokens[src];
+                id = id < 0 ? 0 : (id >= g.vocab ? g.vocab - 1 : id);     // out-of-range ids are clamped, never dereferenced
+                er = reinterpret_cast<const uint2 *>(g.emb + (long long)id * K);
             }
 #pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                const int m = m0 + warp * PER + r0 + u;
-                const long long src = EPI == SMALL_STORE && g.rows ? (m < M ? listed[u] : 0) : (m < g.M ? m : 0);
-                const float4 *xr = reinterpret_cast<const float4 *>(g.x + src * K);
-                const uint2 *er = nullptr;
-                if (SRC == SMALL_EMBED) {
-                    int id = g.tokens[src];
-                    id = id < 0 ? 0 : (id >= g.vocab ? g.vocab - 1 : id);     // out-of-range ids are clamped, never dereferenced
-                    er = reinterpret_cast<const uint2 *>(g.emb + (long long)id * K);
-                }
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    const int c = lane + 32 * k;
-                    v[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (m < g.M && c < q4) {
-                        if (SRC == SMALL_EMBED) {
-                            const uint2 e = er[c];
-                            v[u][k] = make_float4(bf16_bits_to_f32(e.x & 0xFFFFu), bf16_bits_to_f32(e.x >> 16), bf16_bits_to_f32(e.y & 0xFFFFu),
-                                                  bf16_bits_to_f32(e.y >> 16));
-                        } else v[u][k] = xr[c];
-                    }
+            for (int k = 0; k < NCH; ++k) {
+                const int c = lane + 32 * k;
+                v[u][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (m < g.M && c < q4) {
+                    if (SRC == SMALL_EMBED) {
+                        const uint2 e = er[c];
+                        v[u][k] = make_float4(bf16_bits_to_f32(e.x & 0xFFFFu), bf16_bits_to_f32(e.x >> 16), bf16_bits_to_f32(e.y & 0xFFFFu),
+                                              bf16_bits_to_f32(e.y >> 16));
+                    } else v[u][k] = xr[c];
                 }
             }
-            if (r0 == 0 && (!active || m0 >= M)) { cp_async_wait(); return; }
+        }
+        if (!active || m0 >= M) { cp_async_wait(); return; }
 #pragma unroll
-            for (int u = 0; u < ROWS; ++u) {
-                const int r = warp * PER + r0 + u, m = m0 + r;
-                float ss = 0.f;
+        for (int u = 0; u < ROWS; ++u) {
+            const int r = warp * ROWS + u, m = m0 + r;
+            float ss = 0.f;
 #pragma unroll
-                for (int k = 0; k < NCH; ++k) ss += v[u][k].x * v[u][k].x + v[u][k].y * v[u][k].y + v[u][k].z * v[u][k].z + v[u][k].w * v[u][k].w;
-                const float inv = rsqrtf(warp_sum(ss) / (float)K + g.eps);
+            for (int k = 0; k < NCH; ++k) ss += v[u][k].x * v[u][k].x + v[u][k].y * v[u][k].y + v[u][k].z * v[u][k].z + v[u][k].w * v[u][k].w;
+            const float inv = rsqrtf(warp_sum(ss) / (float)K + g.eps);
 #pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    const int c = lane + 32 * k;
-                    if (c >= q4) continue;
-                    if (SRC == SMALL_EMBED && nt == 0 && m < M) reinterpret_cast<float4 *>(g.x)[(long long)m * q4 + c] = v[u][k];      // the residual stream begins
-                    const uint2 gn = gain[k];
-                    *reinterpret_cast<uint2 *>(sA + r * ld + 4 * c) =
-                        make_uint2(pack2(v[u][k].x * inv * bf16_bits_to_f32(gn.x & 0xFFFFu), v[u][k].y * inv * bf16_bits_to_f32(gn.x >> 16)),
-                                   pack2(v[u][k].z * inv * bf16_bits_to_f32(gn.y & 0xFFFFu), v[u][k].w * inv * bf16_bits_to_f32(gn.y >> 16)));
-                }
+            for (int k = 0; k < NCH; ++k) {
+                const int c = lane + 32 * k;
+                if (c >= q4) continue;
+                if (SRC == SMALL_EMBED && nt == 0 && m < M) reinterpret_cast<float4 *>(g.x)[(long long)m * q4 + c] = v[u][k];      // the residual stream begins
+                const uint2 gn = gain[k];
+                *reinterpret_cast<uint2 *>(sA + r * ld + 4 * c) =
+                    make_uint2(pack2(v[u][k].x * inv * bf16_bits_to_f32(gn.x & 0xFFFFu), v[u][k].y * inv * bf16_bits_to_f32(gn.x >> 16)),
+                               pack2(v[u][k].z * inv * bf16_bits_to_f32(gn.y & 0xFFFFu), v[u][k].w * inv * bf16_bits_to_f32(gn.y >> 16)));
             }
         }
         if (K < Kp) for (int r = tid; r < TILE; r += kThreads) *reinterpret_cast<uint4 *>(sA + r * ld + K) = zero;      // K is a multiple of 8
