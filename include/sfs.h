@@ -168,8 +168,9 @@ int32_t sfs_row_stats(const void *d_logits, int32_t logits_dtype, int32_t vocab,
 /* The first of the two passes sfs_select runs over long bf16 rows (65536 to 163840 entries; other shapes return
  * SFS_ERR_UNSUPPORTED here and take the all-canonical kernels inside sfs_select): exact argmax, and an enclosure
  * d_lo[r] <= S_q <= d_hi[r] of the canonical denominator from a cheap pass (special-function exponentials, fp32 sums;
- * relative width 1.2e-4 plus vocab + 2).  sfs_select recomputes the canonical S_q only for rows whose enclosure leaves a
- * threshold comparison or the top-1 ranking of the step open, so its decisions are those of all-canonical values.
+ * relative width 1.2e-4, for rows with a maximum beyond 100 in magnitude 3.6e-7 more per unit, plus vocab + 2).  sfs_select
+ * recomputes the canonical S_q only for rows whose enclosure leaves a threshold comparison or the top-1 ranking of the step
+ * open, so its decisions are those of all-canonical values.
  * Exposed for tests and measurements. */
 int32_t sfs_row_stats_bounds(const void *d_logits, int32_t vocab, int64_t ld, const int32_t *d_n_rows, int32_t max_rows,
                              uint64_t *d_lo, uint64_t *d_hi, int32_t *d_argmax, void *stream);

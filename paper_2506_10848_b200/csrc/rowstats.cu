@@ -422,14 +422,17 @@ rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
 // that completes a row (a ticket per row) moves the slice sums to the row maximum and adds them in slice order:
 //     S~ = sum over slices, warps of ex2((c - m) log2 e) * sum_v ex2.approx(fma(x_v, log2 e, -c log2 e))       (fp32)
 // The canonical S_q = sum_v trunc(2^28 exp~(x_v - m)) lies in
-//     [ 2^28 S~ (1 - kEps) - V - 1 ,  2^28 S~ (1 + kEps) + 1 ]  intersected with [2^28, inf):
+//     [ 2^28 S~ (1 - eps) - V - 1 ,  2^28 S~ (1 + eps) + 1 ]  intersected with [2^28, inf):
 // the canonical exponential is within 1e-5 relative of exp (degree-4 fit 3.3e-6, its fp32 steps < 1e-6) and truncation loses
 // less than 1 per term (V terms); on this side an exponent (x - c) log2 e of magnitude up to 100 is rounded to 2^-24
 // relative (< 6e-6 absolute, i.e. < 4.2e-6 relative in the term), the same again for each of the two moves, ex2.approx is
 // within 2^-22 three times, and the fp32 sums (at most 32 sequential adds per thread, then pairwise levels) within 3e-6.
-// Worst case 2.8e-5; kEps = 6e-5.  A reference more than 100 (in log2 units) below the maximum it is moved to, and a sum
+// Worst case 2.8e-5.  Besides, -c log2 e, and the same of a slice's and of the row's maximum, are rounded to 2^-24 of their magnitude,
+// which shifts every term of a sum alike: relative 2^-24 |c| each, and a reference lies at most 100 log 2 below the maximum, so
+// 3 * 2^-24 (|m| + 70) in all.  The enclosure takes 6e-5, which holds both up to |m| = 100, and their sum beyond (with 6e-5 throughout rows
+// with logits of 600 and more lay outside theirs).  A reference more than 100 (in log2 units) below the maximum it is moved to, and a sum
 // that is not a finite number >= 1, yield an enclosure that contains everything, which sends the row to the canonical pass.
-constexpr double kEps = 6e-5;
+constexpr double kEps = 6e-5, kEpsTerms = 2.8e-5, kEpsPerUnit = 1.8e-7;
 constexpr int kSlices = 8;
 constexpr int kBoundsThreads = 128;
 
@@ -451,11 +454,12 @@ __device__ __forceinline__ void write_enclosure(const BoundsOut &out, int row, f
 {
     if (arg == 0x7FFFFFFF) arg = 0;
     const double Sd = (double)tot * (double)(1u << SFS_CONF_QBITS);
-    const double dlo = Sd * (1.0 - kEps) - (double)vocab - 1.0, dhi = Sd * (1.0 + kEps) + 1.0;
+    const double eps = fmax(kEps, kEpsTerms + kEpsPerUnit * (fabs((double)m) + 70.0));
+    const double dlo = Sd * (1.0 - eps) - (double)vocab - 1.0, dhi = Sd * (1.0 + eps) + 1.0;
     const unsigned long long floor_q = 1ull << SFS_CONF_QBITS;     // the maximum alone contributes 2^28
     unsigned long long lo = dlo > (double)floor_q ? (unsigned long long)dlo : floor_q;
     unsigned long long hi = (unsigned long long)dhi + 1ull;
-    if (open || !(tot >= 0.999f) || !(tot <= 3.0e38f)) { lo = 1ull; hi = ~0ull >> 1; }
+    if (open || !(eps <= 0.25) || !(tot >= 0.999f) || !(tot <= 3.0e38f)) { lo = 1ull; hi = ~0ull >> 1; }
     if (certain) lo = hi = floor_q;
     if (out.lo) out.lo[row] = lo;
     if (out.hi) out.hi[row] = hi;

@@ -177,6 +177,26 @@ def test_enclosures_of_the_cheap_pass_contain_the_canonical_denominator(V, ld):
     assert np.max(np.abs(mid[rows] - sq[rows].astype(np.float64)) / sq[rows].astype(np.float64)) <= 2e-5 + V / float(1 << 28)
 
 
+@pytest.mark.parametrize("far", [100, 400, 600, 1000, 3000, 20000, 1e6])
+def test_enclosures_hold_for_large_logits(far):
+    """The whole row far from zero: the products with log2 e that cancel are rounded to their own magnitude.  The enclosure must still hold,
+    and be no wider than that rounding asks for: 2 (2.8e-5 + 3 * 2^-24 (|m| + 70)), rounded up, unless it contains everything."""
+    V, R = 70000, 48
+    g = torch.Generator().manual_seed(int(far))
+    at = far * (1.0 + 0.013 * torch.arange(R // 2).repeat(2)) * torch.tensor([1.0] * (R // 2) + [-1.0] * (R // 2))
+    x = (torch.randn((R, V), generator=g) * torch.linspace(0.2, 6.0, R // 2).repeat(2)[:, None] + at[:, None]).to(torch.bfloat16)
+    ref = RS.row_stats(W.bf16_bits(x))
+    lo, hi, arg = gpu_bounds(x.to(DEV), V, V)
+    sq = ref["sq"].astype(np.uint64)
+    assert np.array_equal(arg, ref["argmax"])
+    assert np.all(lo <= sq) and np.all(sq <= hi), int((lo > sq).sum() + (hi < sq).sum())
+    m = np.abs(x.float().amax(dim=1).numpy().astype(np.float64))
+    eps = np.maximum(6e-5, 2.8e-5 + 1.8e-7 * (m + 70.0))
+    narrow = hi < (1 << 62)
+    assert np.all((hi - lo).astype(np.float64)[narrow] <= (2.05 * eps * (1.0 + eps) * sq.astype(np.float64) + V + 8)[narrow])
+    assert far > 3000 or narrow.all()
+
+
 @pytest.mark.parametrize("dtype", [sfs.LOGITS_BF16, sfs.LOGITS_F32])
 @pytest.mark.parametrize("R,V,ld", [(9, 2049, 2051), (9, 8197, 8199), (300, 8197, 8197), (9, 16391, 16391), (300, 33001, 33003), (9, 50257, 50257),
                                     (80, 50257, 50258), (3, 66003, 66005), (5, 140001, 140003), (300, 4099, 4100)])
