@@ -7,6 +7,7 @@
 #include "elementwise.cuh"
 #include "cache.cuh"
 #include "small_gemm.cuh"
+#include "small_layer.cuh"
 #include <math.h>
 
 #include <new>
@@ -330,10 +331,19 @@ static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active,
     const sfs_model *m = s->model;
     const sfs_config &c = m->cfg;
     const int T = B * S, d = c.d_model, ff = c.d_ff;
+    const bool fused = small_layer_fits(d, ff, c.n_heads, c.head_dim, B, S);
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
         if (l > 0 && (rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, l, B, S, nullptr, d_active, cache, st); })) != SFS_OK) return rc;
         if (cache && (rc = cache_values(s, l, T, d_active, st)) != SFS_OK) return rc;
+        if (fused) {
+            SmallLayerArgs a{};
+            a.qkv = s->attn_plan.direct; a.scale_log2 = s->attn_plan.args.scale_log2; a.B = B; a.S = S; a.n_heads = c.n_heads; a.d = d; a.ff = ff;
+            a.wo = bf(m->wo[l]); a.w_gate = bf(m->w_gate[l]); a.w_up = bf(m->w_up[l]); a.w_down = bf(m->w_down[l]); a.gain = bf(m->mlp_norm[l]); a.eps = c.rms_eps;
+            a.x = s->x; a.inc_attn = cache ? s->Ac[l] : nullptr; a.inc_mlp = cache ? s->Fc[l] : nullptr; a.d_active = d_active; a.err = device_status_word();
+            if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return launch_small_layer(a, st); })) != SFS_OK) return rc;
+            continue;
+        }
         if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, device_status_word(), st); })) != SFS_OK) return rc;
         rc = timed_launch(s, SFS_K_GEMM_O, st, [&] {
             SmallGemmArgs g = small_args(s, T, d, d, d_active);

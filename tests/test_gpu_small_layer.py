@@ -1,0 +1,47 @@
+"""GPU parity of the fused layer of small models (attention to down projection in one launch) against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import forward as F
+from paper_2506_10848_b200 import binding as sfs
+from paper_2506_10848_b200 import workloads as W
+
+from bf16_reference import forward_bf16_points
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+# tokens below, at and above a tile of 16 and of 32 rows; one tile of features per CTA or none for some (d_ff 8, 24), an odd number of them
+# (24, 344, 1032), an even one; both widths; several sequences with ragged last tiles; row tiles of 32 (2 x 224, 7 x 40)
+@pytest.mark.parametrize("d,ff,B,S", [(256, 688, 1, 8), (256, 688, 1, 40), (256, 688, 3, 24), (256, 8, 1, 16), (256, 24, 2, 72), (256, 344, 1, 200),
+                                      (128, 352, 1, 24), (128, 1032, 2, 40), (128, 64, 1, 136), (256, 688, 2, 224), (128, 1032, 7, 40),
+                                      (256, 344, 1, 408)])
+def test_logits_match_the_oracle(d, ff, B, S):
+    dct = W.TINY.asdict()
+    dct.update(d_model=d, d_ff=ff, n_heads=d // 64, vocab=512, mask_id=511, logit_scale=1.0)
+    shape = W.Shape(**dct)
+    # weights large enough that attention is not uniform and both branches move the residual stream
+    w = W.model_weights(shape, seed=d + ff, std=0.08, gain_std=0.2)
+    wd = {k: (v.to(DEV) if k != "layers" else [{kk: vv.to(DEV) for kk, vv in lw.items()} for lw in v]) for k, v in w.items()}
+    model = sfs.Model(shape, wd)
+    tok = W.prompt_ids(B, S, 510, seed=S)
+    session = sfs.sfs_session_create(model, B, S)
+    try:
+        got = torch.zeros((B * S, shape.vocab), dtype=torch.float32, device=DEV)
+        sfs.sfs_forward(session, tok.to(DEV), B, S, None, None, B * S, got, sfs.LOGITS_F32)
+        again = torch.zeros_like(got)
+        sfs.sfs_forward(session, tok.to(DEV), B, S, None, None, B * S, again, sfs.LOGITS_F32)
+        sfs.sfs_check_device_status()
+        assert torch.equal(got, again)
+        rows = [(b, t) for b in range(B) for t in range(S)]
+        ref = F.forward(F.ModelConfig(**shape.asdict()), W.weights_to_numpy(w, np.float64), tok.numpy(), rows=rows, dtype=np.float64)
+        err = got.cpu().double().numpy() - ref
+        # the bar is what rounding the operands to bf16 costs by itself at these weights, with a quarter more for other last bits
+        emu = np.concatenate([forward_bf16_points(F.ModelConfig(**shape.asdict()), w, tok[b].numpy(), range(S)) for b in range(B)]) - ref
+        assert np.linalg.norm(err) <= 1.25 * np.linalg.norm(emu)
+        assert np.linalg.norm(err, axis=1).max() <= 1.6 * np.linalg.norm(emu, axis=1).max()
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
