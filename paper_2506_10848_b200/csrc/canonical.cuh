@@ -69,27 +69,38 @@ __device__ __forceinline__ Consts2 canon_consts(float m) {
 }
 
 // Canonical S_q of the listed positions' logits rows (bf16, 16-byte aligned, a multiple of 8 entries), by `n_warps` warps of which
-// this one is `w`: a row is cut into items of kOpenChunks 16-byte chunks, four loads of a lane in flight, and every item's
-// integer sum is added to pos_sq of its position (which is zero before) — integer addition commutes, so the order of arrival
-// does not matter.  The rows come from L2: the first pass has just streamed them, or the LM head written them.
-constexpr int kOpenChunks = 128;
-__device__ __forceinline__ void recompute_rows(const LogitsRows &g, const int32_t *list, int n, const int32_t *pos_row, const float *pos_max,
+// this one is `w`: a row is cut into items, and every item's integer sum is added to pos_sq of its position (which is zero before) —
+// integer addition commutes, so the order of arrival does not matter.  The rows come from L2: the first pass has just streamed them,
+// or the LM head wrote them.  An item is a round trip, a warp's reduction and an atomic, so it is as long as spreads all rows over all
+// warps once (4 to 16 chunks a lane), with the loads of the next four chunks ahead of the terms of four: 53 rows of 126464 took 11000
+// clocks as items of four chunks whose row number was another round trip.
+constexpr int kOpenBatch = 4, kOpenMost = 4;                // chunks of a lane in a batch, batches in an item
+__device__ __forceinline__ void recompute_rows(const LogitsRows &g, const int32_t *list, const int32_t *row_of, int n, const float *pos_max,
                                                unsigned long long *pos_sq, int w, int n_warps)
 {
-    const int lane = threadIdx.x & 31, items = (g.chunks + kOpenChunks - 1) / kOpenChunks;
+    const int lane = threadIdx.x & 31, batch = 32 * kOpenBatch, row_batches = (g.chunks + batch - 1) / batch;
+    const int per = min(kOpenMost, max(1, (n * row_batches + n_warps - 1) / n_warps)), items = (row_batches + per - 1) / per;
     for (int it = w; it < n * items; it += n_warps) {
-        const int r = it / items, c0 = (it - r * items) * kOpenChunks + lane, c1 = min(g.chunks, (it - r * items + 1) * kOpenChunks);
+        const int r = it / items, first = (it - r * items) * per * batch + lane, end = min(g.chunks, first - lane + per * batch);
         const int pos = list[r];
-        const uint4 *rp = g.base + (long long)__ldcg(&pos_row[pos]) * g.ld;
-        const Consts2 k = canon_consts(__ldcg(&pos_max[pos]));
-        uint4 v[kOpenChunks / 32];
+        const uint4 *rp = g.base + (long long)row_of[r] * g.ld;
+        uint4 v[2][kOpenBatch];
+        auto fetch = [&](uint4 *q, int c) {
 #pragma unroll
-        for (int u = 0; u < kOpenChunks / 32; ++u)
-            v[u] = c0 + 32 * u < c1 ? __ldcg(rp + c0 + 32 * u) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+            for (int u = 0; u < kOpenBatch; ++u)
+                q[u] = c + 32 * u < end ? __ldcg(rp + c + 32 * u) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
+        };
+        fetch(v[0], first);
+        const Consts2 k = canon_consts(__ldcg(&pos_max[pos]));
         unsigned long long acc = 0;
 #pragma unroll
-        for (int u = 0; u < kOpenChunks / 32; ++u)          // 8 terms < 8 * 1.42 * 2^28 < 2^32
-            acc += canon_pair(v[u].x, k) + canon_pair(v[u].y, k) + canon_pair(v[u].z, k) + canon_pair(v[u].w, k);
+        for (int t = 0; t < kOpenMost; ++t) {
+            if (t >= per) break;
+            if (t + 1 < per) fetch(v[(t + 1) & 1], first + (t + 1) * batch);
+#pragma unroll
+            for (int u = 0; u < kOpenBatch; ++u)            // 8 terms < 8 * 1.42 * 2^28 < 2^32
+                acc += canon_pair(v[t & 1][u].x, k) + canon_pair(v[t & 1][u].y, k) + canon_pair(v[t & 1][u].z, k) + canon_pair(v[t & 1][u].w, k);
+        }
         acc = warp_sum_u64(acc);
         if (lane == 0) atomicAdd(&pos_sq[pos], acc);
     }

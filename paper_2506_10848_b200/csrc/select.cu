@@ -14,40 +14,43 @@ namespace {
 constexpr int kSelThreads = 256;
 constexpr unsigned long long kNoKey = ~0ull;
 constexpr int kGoesOn = 1 << 30;             // beside a sequence's row count: its next step will hardly be its last
+constexpr int kMostCluster = 8;               // sequences whose CTAs are one cluster at most
 constexpr int kPosBits = 17;                 // key = S_q << 17 | position  (S_q < 2^47, position < 2^17)
 
 struct BlockRed {
-    int n_cand, n_high, max_above, min_cand, n_masked, missing;
+    int n_cand, n_high, max_above, min_cand, n_masked, missing;      // (counts: at most 22755, see select_fits)
     unsigned long long kmin;                                // smallest key
 };
 
 __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+    const uint32_t hi = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32));
+    const uint32_t lo = __reduce_min_sync(0xffffffffu, (uint32_t)(v >> 32) == hi ? (uint32_t)v : ~0u);
+    return (unsigned long long)hi << 32 | lo;
 }
 
-__device__ BlockRed block_reduce(BlockRed v, int *s_tmp /* [6 * 8] */, unsigned long long *s_min /* [8] */) {
+// One barrier: each warp leaves its result, then every warp reduces the eight of them.  The chain of these block-wide steps is what
+// bounds a selection, so counts travel in pairs and minima of 64 bits as two instructions (ten shuffles before); the caller gives
+// each reduction tables of its own.
+constexpr int kSelWarps = kSelThreads / 32;
+__device__ BlockRed block_reduce(BlockRed v, int4 *s_int /* [8] */, unsigned long long *s_min /* [8] */) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    v.n_cand = warp_sum_i32(v.n_cand);   v.n_high = warp_sum_i32(v.n_high);
-    v.max_above = warp_max_i32(v.max_above); v.min_cand = warp_min_i32(v.min_cand);
-    v.n_masked = warp_sum_i32(v.n_masked);   v.missing = warp_sum_i32(v.missing);
+    int4 e = make_int4(warp_sum_i32(v.n_cand | v.n_high << 16), warp_sum_i32(v.n_masked | v.missing << 16), warp_max_i32(v.max_above), warp_min_i32(v.min_cand));
     v.kmin = warp_min_u64(v.kmin);
+    if (lane == 0) { s_int[warp] = e; s_min[warp] = v.kmin; }
     __syncthreads();
-    if (lane == 0) {
-        s_tmp[warp * 6 + 0] = v.n_cand; s_tmp[warp * 6 + 1] = v.n_high; s_tmp[warp * 6 + 2] = v.max_above;
-        s_tmp[warp * 6 + 3] = v.min_cand; s_tmp[warp * 6 + 4] = v.n_masked; s_tmp[warp * 6 + 5] = v.missing;
-        s_min[warp] = v.kmin;
-    }
+    e = s_int[lane & (kSelWarps - 1)];
+    const bool mine = lane < kSelWarps;                     // (maxima and minima do not mind the copies)
+    const int a = warp_sum_i32(mine ? e.x : 0), b = warp_sum_i32(mine ? e.y : 0);
+    return BlockRed{a & 0xFFFF, a >> 16, warp_max_i32(e.z), warp_min_i32(e.w), b & 0xFFFF, b >> 16, warp_min_u64(s_min[lane & (kSelWarps - 1)])};
+}
+// count (two of 16 bits at most) of all warps, and of those before this one; one barrier, the caller alternates between tables
+__device__ __forceinline__ int block_count(int warp_count, int *s_cnt /* [8] */, int *before) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) s_cnt[warp] = warp_count;
     __syncthreads();
-    BlockRed r{0, 0, -1, 0x7FFFFFFF, 0, 0, ~0ull};
-#pragma unroll
-    for (int w = 0; w < kSelThreads / 32; ++w) {
-        r.n_cand += s_tmp[w * 6 + 0]; r.n_high += s_tmp[w * 6 + 1];
-        r.max_above = max(r.max_above, s_tmp[w * 6 + 2]); r.min_cand = min(r.min_cand, s_tmp[w * 6 + 3]);
-        r.n_masked += s_tmp[w * 6 + 4]; r.missing += s_tmp[w * 6 + 5]; r.kmin = min(r.kmin, s_min[w]);
-    }
-    return r;
+    const int c = lane < kSelWarps ? s_cnt[lane] : 0;
+    if (before) *before = warp_sum_i32(lane < warp ? c : 0);
+    return warp_sum_i32(c);
 }
 
 enum { MODE_ALL = 0, MODE_TOPK = 1, MODE_HIGH = 2, MODE_RANDOM = 3 };
@@ -92,11 +95,12 @@ enum { F_MASKED = 1, F_HIGH = 2, F_SEL = 4, F_OPEN = 8 };
 //     U = the k-th smallest hi among the candidates: the k rows with the smallest hi all have S_q <= U, so a row with
 //     lo > U is not among the k most confident, and its lower bound (still > U) orders it behind them.  Only k = 1 is
 //     evaluated this way (U = the smallest hi); for k > 1 every candidate is recomputed.
-// m0 / lo0 / hi0: mask and enclosure of position threadIdx.x, loaded by the caller beside the state.
-__device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, uint8_t m0, unsigned long long lo0, unsigned long long hi0, uint8_t *s_fl,
-                              int32_t *s_list, int *s_tmp, unsigned long long *s_min)
+// Positions go to s_list, their logits rows to s_row.  m0 / lo0 / hi0 / row0: mask, enclosure and row of position threadIdx.x, loaded
+// by the caller beside the state.
+__device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, uint8_t m0, unsigned long long lo0, unsigned long long hi0, int32_t row0, uint8_t *s_fl,
+                              int32_t *s_list, int32_t *s_row, int4 *s_int, unsigned long long *s_min, int (*s_cnt)[kSelWarps])
 {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = a.L;
+    const int tid = threadIdx.x, lane = tid & 31, L = a.L;
     const StepAsk ask = step_ask(a.params, st, L);
     const long long base = (long long)b * a.S + a.P;
     const uint8_t *msk = a.mask + base;
@@ -111,7 +115,7 @@ __device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, u
             r.n_cand++;
             if ((first ? lo0 : plo[i]) != 0) r.kmin = min(r.kmin, first ? hi0 : phi[i]);
         }
-        r = block_reduce(r, s_tmp, s_min);
+        r = block_reduce(r, s_int, s_min);
         U = r.kmin;
         if (a.params.sampler == SFS_SAMPLER_LOW_CONFIDENCE) {
             const BlockStep blk = block_step(a.params, L, st.steps_done);
@@ -135,14 +139,13 @@ __device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, u
             }
         }
         const unsigned bal = __ballot_sync(0xffffffffu, open);
-        __syncthreads();
-        if (lane == 0) s_tmp[warp] = __popc(bal);
-        __syncthreads();
-        int before = n_open, total = 0;
-#pragma unroll
-        for (int w = 0; w < kSelThreads / 32; ++w) { const int c = s_tmp[w]; total += c; if (w < warp) before += c; }
+        int before;
+        const int total = block_count(__popc(bal), s_cnt[(i0 / kSelThreads) & 1], &before);
         if (i < L) s_fl[i] = open ? F_OPEN : 0;
-        if (open) s_list[before + __popc(bal & ((1u << lane) - 1u))] = i;
+        if (open) {
+            const int at = n_open + before + __popc(bal & ((1u << lane) - 1u));
+            s_list[at] = i; s_row[at] = i0 == 0 ? row0 : __ldcg(&a.pos_row[base + i]);
+        }
         n_open += total;
     }
     __syncthreads();
@@ -154,18 +157,23 @@ __device__ int list_open_rows(const SelectArgs &a, const sfs_state &st, int b, u
 // recomputation of those rows, warp by warp, adding integer partial sums to pos_sq, and the CTA that finishes last (a ticket)
 // goes on alone.  So the list, the recomputation and the choice are one launch: on 256 rows of 126464 logits the three kernels
 // they were took 6 + 9 + 11 us of a 45 us sfs_select call; DRAM has no part in it, the chain of block-wide steps bounds it.
-// Without two-pass statistics there is one CTA per sequence.
-// dynamic shared memory: keys u64[L] (before: the list of open rows) | flags u8[L]
+// Without two-pass statistics there is one CTA per sequence; those of up to eight sequences are a cluster (CLUSTER), whose CTAs tell
+// each other the lengths of their row lists instead of leaving them to the last one (2 sequences: 3500 of 9200 clocks).
+// State that follows from the step is worked out by every thread, from the same values: no thread waits for another's arithmetic.
+// dynamic shared memory: keys u64[L] (before: the list of open rows and their logits rows; after: the next step's rows) | flags u8[L]
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
 {
     extern __shared__ unsigned long long s_keys[];
-    const int L = a.L, S = a.S, P = a.P, b = blockIdx.x / a.groups, part = blockIdx.x - b * a.groups;
+    const int L = a.L, S = a.S, P = a.P, b = CLUSTER ? blockIdx.x : blockIdx.x / a.groups, part = CLUSTER ? 0 : blockIdx.x - b * a.groups;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint8_t *s_fl = reinterpret_cast<uint8_t *>(s_keys + L);
-    __shared__ int s_tmp[6 * (kSelThreads / 32)];
-    __shared__ unsigned long long s_min[kSelThreads / 32];
+    __shared__ int4 s_int[2][kSelWarps];
+    __shared__ unsigned long long s_min[2][kSelWarps];
+    __shared__ int s_cnt[4][kSelWarps];
     __shared__ sfs_state st;
     __shared__ int s_last;
+    __shared__ int2 s_seq[kMostCluster];                    // CLUSTER: (rows and flag, still decoding) of every sequence
 
     const long long base = (long long)b * S + P;
     int32_t *tok = a.tokens + base;
@@ -173,18 +181,19 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     unsigned long long *psq = a.pos_sq + base;
     const int32_t *parg = a.pos_arg + base;
     const sfs_params &p = a.params;
-    const bool two_pass = a.pos_lo != nullptr, vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
+    const bool two_pass = !CLUSTER && a.pos_lo != nullptr, vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
 
+    if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // this CTA runs
     pdl_wait();
     pdl_trigger();
     const int steps_before = tid == 0 && a.step_count ? *a.step_count : 0;      // (of the whole generation)
     // the state and everything about position tid (all of a sequence, usually) in one round trip
     uint8_t m0 = 0;
-    int32_t arg0 = 0;
+    int32_t arg0 = 0, row0 = 0;
     unsigned long long lo0 = 0, hi0 = 0;                    // two-pass: the enclosure; else lo0 = S_q
     if (tid < L) {
         m0 = msk[tid]; arg0 = parg[tid];
-        if (two_pass) { lo0 = __ldcg(&a.pos_lo[base + tid]); hi0 = a.pos_hi[base + tid]; }
+        if (two_pass) { lo0 = __ldcg(&a.pos_lo[base + tid]); hi0 = a.pos_hi[base + tid]; row0 = __ldcg(&a.pos_row[base + tid]); }
         else lo0 = psq[tid];
     }
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(&st)[tid] = reinterpret_cast<const int *>(a.state + b)[tid];
@@ -195,18 +204,19 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     const bool forced = !vanilla && (st.k_remaining == 1);
     if (a.groups > 1 && !active && part != 0) return;
     if (two_pass && active) {
-        int32_t *s_list = reinterpret_cast<int32_t *>(s_keys);
-        const int n_open = list_open_rows(a, st, b, m0, lo0, hi0, s_fl, s_list, s_tmp, s_min);
-        recompute_rows(a.lrows, s_list, n_open, a.pos_row + base, a.pos_max + base, psq, part * (kSelThreads / 32) + warp,
-                       a.groups * (kSelThreads / 32));
+        int32_t *s_list = reinterpret_cast<int32_t *>(s_keys), *s_row = s_list + L;
+        const int n_open = list_open_rows(a, st, b, m0, lo0, hi0, row0, s_fl, s_list, s_row, s_int[0], s_min[0], s_cnt);
+        recompute_rows(a.lrows, s_list, s_row, n_open, a.pos_max + base, psq, part * kSelWarps + warp, a.groups * kSelWarps);
         if (a.groups > 1) {
-            __threadfence();
             __syncthreads();
-            if (tid == 0) s_last = (atomicAdd(&a.seq_ticket[b], 1) == a.groups - 1) ? 1 : 0;
+            if (tid == 0) {                                 // (releases the whole CTA's sums, and acquires the others')
+                int before;
+                asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(before) : "l"(&a.seq_ticket[b]) : "memory");
+                s_last = before == a.groups - 1 ? 1 : 0;
+                if (s_last) a.seq_ticket[b] = 0;
+            }
             __syncthreads();
             if (!s_last) return;
-            __threadfence();
-            if (tid == 0) a.seq_ticket[b] = 0;
         } else {
             __threadfence();
             __syncthreads();
@@ -216,6 +226,10 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     int n_sel = 0, e_cand = -1, stable = 0, n_sure = 0;    // n_sure: candidates above the high threshold
     int rec_phase = phase0, rec_s = s0;
     int rec_hi = (phase0 == SFS_PHASE_SLOW) ? L : hi_fast;
+    // the state after this step (of the history only its length)
+    int phase1 = phase0, s1 = s0, hi1 = hi_fast, count1 = st.step_count, hist1 = st.hist_len, k1 = st.k_remaining, masked1 = st.n_masked, done1 = st.done, status1 = st.status;
+    const int hist0 = hist1;
+    bool stepped = false, slow_step = false, fell_back = false, new_cycle = false;
     BlockStep blk{};
     if (vanilla) { blk = block_step(p, L, steps0); rec_phase = blk.j; rec_s = blk.lo; rec_hi = blk.hi; e_cand = blk.k_b; }
 
@@ -250,12 +264,11 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             r.n_masked += m ? 1 : 0;
             s_keys[i] = key; s_fl[i] = fl;
         }
-        r = block_reduce(r, s_tmp, s_min);
+        r = block_reduce(r, s_int[1], s_min[1]);
         n_sure = r.n_high;
 
         if (r.missing > 0 || (r.n_cand == 0 && !vanilla)) {
-            // a needed row was not supplied (or the state is inconsistent): report, change nothing
-            if (tid == 0) st.status = SFS_ERR_MISSING_ROW;
+            status1 = SFS_ERR_MISSING_ROW;                  // a needed row was not supplied (or the state is inconsistent): report, change nothing
         } else {
             int mode, k_top = 0;
             if (p.sampler == SFS_SAMPLER_LOW_CONFIDENCE) {
@@ -269,38 +282,32 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             else if (r.n_high >= p.min_high_count) mode = MODE_HIGH;
             else { mode = MODE_TOPK; k_top = p.k_fast; }
 
-            // ---- scheduler state (Algorithm 1), one thread: what does not depend on the choice
-            if (tid == 0) {
-                st.steps_done++;
-                if (vanilla) {
-                    st.k_remaining--;
-                } else if (forced) {
-                    st.k_remaining = 0;
-                } else if (phase0 == SFS_PHASE_SLOW) {
-                    e_cand = (r.max_above >= 0) ? r.max_above : r.min_cand;
-                    if (st.hist_len < p.w_hist) st.hist[st.hist_len++] = e_cand;
-                    else { for (int h = 1; h < p.w_hist; ++h) st.hist[h - 1] = st.hist[h]; st.hist[p.w_hist - 1] = e_cand; }
-                    st.k_remaining--; st.step_count++; st.n_slow++;
-                    int sum = 0;                                          // (at most 8 positions below 2^17)
-                    long long sum2 = 0;
-                    for (int h = 0; h < st.hist_len; ++h) { sum += st.hist[h]; sum2 += (long long)st.hist[h] * st.hist[h]; }
-                    const int n = st.hist_len;
-                    const long long num = n * sum2 - (long long)sum * sum;               // n^2 * population variance, exact
-                    if (n >= p.w_hist && (double)num < (double)p.sigma2_stable * (double)((long long)n * n)) {
-                        stable = 1;
-                        st.phase = SFS_PHASE_FAST; st.hi = sum / n + 1;   // floor(mean(H_W)) + 1
-                    } else if (st.step_count >= p.k_max) {
-                        st.phase = SFS_PHASE_FAST; st.hi = e_cand + 1;
-                    }
-                } else {
-                    st.k_remaining--; st.n_fast++;
-                    if (mode == MODE_TOPK) st.n_fallback++;
+            // ---- scheduler state (Algorithm 1): what does not depend on the choice
+            stepped = true;
+            k1 = forced ? 0 : k1 - 1;
+            if (!vanilla && !forced && phase0 == SFS_PHASE_SLOW) {
+                slow_step = true;
+                e_cand = (r.max_above >= 0) ? r.max_above : r.min_cand;
+                const bool full = hist0 >= p.w_hist;        // the history with e_cand in it: appended, or the oldest dropped
+                hist1 = full ? hist0 : hist0 + 1;
+                int sum = 0;                                              // (at most 8 positions below 2^17)
+                long long sum2 = 0;
+                for (int h = 0; h < hist1; ++h) {
+                    const int e = full ? (h < p.w_hist - 1 ? st.hist[h + 1] : (h == p.w_hist - 1 ? e_cand : st.hist[h])) : (h < hist0 ? st.hist[h] : e_cand);
+                    sum += e; sum2 += (long long)e * e;
                 }
-            }
-            __syncthreads();
+                count1++;
+                const int n = hist1;
+                const long long num = n * sum2 - (long long)sum * sum;               // n^2 * population variance, exact
+                if (n >= p.w_hist && (double)num < (double)p.sigma2_stable * (double)((long long)n * n)) {
+                    stable = 1;
+                    phase1 = SFS_PHASE_FAST; hi1 = sum / n + 1;       // floor(mean(H_W)) + 1
+                } else if (count1 >= p.k_max) {
+                    phase1 = SFS_PHASE_FAST; hi1 = e_cand + 1;
+                }
+            } else if (!vanilla && !forced) fell_back = mode == MODE_TOPK;
             // is the span clean after this step?  (decides whether the next cycle starts)
-            const bool span = !vanilla && !forced && st.phase == SFS_PHASE_FAST;
-            const int span_hi = st.hi;
+            const bool span = !vanilla && !forced && phase1 == SFS_PHASE_FAST;
 
             // ---- choose
             const bool ranked = mode == MODE_TOPK && k_top > 1 && k_top < r.n_cand;      // (one or all: no ranking)
@@ -324,53 +331,39 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
                     }
                 }
                 if (sel) { fl = (uint8_t)((fl | F_SEL) & ~F_MASKED); s_fl[i] = fl; my_sel++; tok[i] = i == tid ? arg0 : parg[i]; msk[i] = 0; }
-                if ((fl & F_MASKED) && i >= s0 && i < span_hi) my_left++;
+                if ((fl & F_MASKED) && i >= s0 && i < hi1) my_left++;
             }
-            my_sel = warp_sum_i32(my_sel); my_left = warp_sum_i32(my_left);
-            if (lane == 0) { s_tmp[2 * warp] = my_sel; s_tmp[2 * warp + 1] = my_left; }
-            __syncthreads();
-            if (tid == 0) {
-                int left = 0;
-#pragma unroll
-                for (int w = 0; w < kSelThreads / 32; ++w) { n_sel += s_tmp[2 * w]; left += s_tmp[2 * w + 1]; }
-                st.n_masked = r.n_masked - n_sel;
-                if (span && left == 0 && st.n_masked > 0) {
-                    st.s_cycle = st.hi; st.phase = SFS_PHASE_SLOW; st.hist_len = 0; st.step_count = 0; st.n_cycles++;
-                }
-                if (st.n_masked == 0 || st.k_remaining == 0) {
-                    st.done = 1;
-                    if (st.n_masked > 0) st.status = SFS_ERR_STEP_LIMIT;
-                }
-            }
+            const int chosen = block_count(warp_sum_i32(my_sel | my_left << 16), s_cnt[2], nullptr), left = chosen >> 16;
+            n_sel = chosen & 0xFFFF;
+            masked1 = r.n_masked - n_sel;
+            if (span && left == 0 && masked1 > 0) { new_cycle = true; s1 = hi1; phase1 = SFS_PHASE_SLOW; hist1 = 0; count1 = 0; }
+            if (masked1 == 0 || k1 == 0) { done1 = 1; if (masked1 > 0) status1 = SFS_ERR_STEP_LIMIT; }
         }
     } else {
         // a finished (or stopped) sequence consumes the statistics supplied for it as well: nothing stale is left for a
         // later generation that reuses the scratch
         for (int i = tid; i < L; i += kSelThreads) { s_fl[i] = 0; psq[i] = 0; if (two_pass) a.pos_lo[base + i] = 0; }
     }
-    __syncthreads();
 
     // ---- ordered outputs (ballots and per-warp counts): selected positions, and the rows of the next step
+    const bool next_active = !done1 && status1 == SFS_OK;
+    // a single sequence's list is the whole list; a cluster's wait in shared memory for their place (the keys
+    // have been ranked: the counts' barrier lies between)
+    int32_t *const next = CLUSTER ? reinterpret_cast<int32_t *>(s_keys) : (a.B == 1 ? a.next_rows : a.seq_rows + (long long)b * L);
+    int n_out = 0, n_next = 0;
     {
-        const bool next_active = !st.done && st.status == SFS_OK;
-        const bool nforced = !vanilla && st.k_remaining == 1;
+        const bool nforced = !vanilla && k1 == 1;
         BlockStep nblk{};
-        if (vanilla) nblk = block_step(p, L, st.steps_done);
-        const int nlo = vanilla ? nblk.lo : (nforced ? 0 : st.s_cycle);
-        const int nhi = vanilla ? nblk.hi : (nforced ? L : ((st.phase == SFS_PHASE_SLOW) ? L : st.hi));
-        // a single sequence's list is the whole list
-        int32_t *const next = a.B == 1 ? a.next_rows : a.seq_rows + (long long)b * L;
-        int n_out = 0, n_next = 0;
+        if (vanilla) nblk = block_step(p, L, steps0 + (stepped ? 1 : 0));
+        const int nlo = vanilla ? nblk.lo : (nforced ? 0 : s1);
+        const int nhi = vanilla ? nblk.hi : (nforced ? L : ((phase1 == SFS_PHASE_SLOW) ? L : hi1));
         for (int i0 = 0; i0 < L; i0 += kSelThreads) {
             const int i = i0 + tid;
             const uint8_t fl = i < L ? s_fl[i] : 0;
             const bool sel = (fl & F_SEL) != 0, need = next_active && (fl & F_MASKED) && i >= nlo && i < nhi;
             const unsigned bs = __ballot_sync(0xffffffffu, sel), bn = __ballot_sync(0xffffffffu, need);
-            if (lane == 0) s_tmp[warp] = __popc(bs) | (__popc(bn) << 16);
-            __syncthreads();
-            int before = 0, total = 0;
-#pragma unroll
-            for (int w = 0; w < kSelThreads / 32; ++w) { const int c = s_tmp[w]; total += c; if (w < warp) before += c; }
+            int before;
+            const int total = block_count(__popc(bs) | (__popc(bn) << 16), s_cnt[(i0 / kSelThreads) & 1], &before);
             const unsigned lt = (1u << lane) - 1u;
             if (sel && a.sel_pos) {
                 const int o = n_out + (before & 0xFFFF) + __popc(bs & lt);
@@ -379,25 +372,50 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
             }
             if (need && next) next[n_next + (before >> 16) + __popc(bn & lt)] = b * S + P + i;
             n_out += total & 0xFFFF; n_next += total >> 16;
-            __syncthreads();
-        }
-        if (tid == 0) {
-            if (a.sel_count) a.sel_count[b] = n_out;
-            // May the next step finish the sequence?  It does when the budget ends.  Before that (SlowFast) its rows must be all that
-            // is masked, and no more than its ranking unmasks or, in the fast phase, twice what has just been unmasked or was sure.
-            const int reach = st.phase == SFS_PHASE_SLOW ? p.k_slow : max(p.k_fast, 2 * max(n_sel, n_sure));
-            const bool may_end = st.k_remaining <= 1 || (!vanilla && n_next == st.n_masked && reach >= st.n_masked);
-            const bool goes_on = next_active && !may_end;
-            a.seq_row_count[b] = n_next | (goes_on ? kGoesOn : 0);
-            if (a.trace) {
-                int32_t *t = a.trace + (long long)b * SFS_TRACE_INTS;
-                t[0] = rec_phase; t[1] = rec_s; t[2] = rec_hi; t[3] = e_cand; t[4] = stable; t[5] = n_sel;
-                t[6] = st.n_masked; t[7] = st.k_remaining;
-            }
-            if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0, steps_before, !goes_on);
         }
     }
+    // May the next step finish the sequence?  It does when the budget ends.  Before that (SlowFast) its rows must be all that
+    // is masked, and no more than its ranking unmasks or, in the fast phase, twice what has just been unmasked or was sure.
+    const int reach = phase1 == SFS_PHASE_SLOW ? p.k_slow : max(p.k_fast, 2 * max(n_sel, n_sure));
+    const bool may_end = k1 <= 1 || (!vanilla && n_next == masked1 && reach >= masked1);
+    const bool goes_on = next_active && !may_end;
+    const int2 seq = make_int2(n_next | (goes_on ? kGoesOn : 0), next_active ? 1 : 0);
+    if (tid == 0) {
+        if (a.sel_count) a.sel_count[b] = n_out;
+        if (!CLUSTER) a.seq_row_count[b] = seq.x;
+        if (a.trace) {
+            int32_t *t = a.trace + (long long)b * SFS_TRACE_INTS;
+            t[0] = rec_phase; t[1] = rec_s; t[2] = rec_hi; t[3] = e_cand; t[4] = stable; t[5] = n_sel;
+            t[6] = masked1; t[7] = k1;
+        }
+        if (a.B == 1) finish_step(a, n_next, next_active ? 1 : 0, steps_before, !goes_on);
+        if (slow_step) {                                    // (nobody reads the old history any more: a barrier lies behind the choice)
+            if (hist0 < p.w_hist) st.hist[hist0] = e_cand;
+            else { for (int h = 1; h < p.w_hist; ++h) st.hist[h - 1] = st.hist[h]; st.hist[p.w_hist - 1] = e_cand; }
+            st.n_slow++;
+        } else if (stepped && !vanilla && !forced) st.n_fast++;
+        st.phase = phase1; st.s_cycle = s1; st.hi = hi1; st.step_count = count1; st.hist_len = hist1; st.k_remaining = k1; st.n_masked = masked1;
+        st.steps_done = steps0 + (stepped ? 1 : 0); st.n_cycles += new_cycle ? 1 : 0; st.n_fallback += fell_back ? 1 : 0; st.done = done1; st.status = status1;
+    }
+    __syncwarp();
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(a.state + b)[tid] = reinterpret_cast<const int *>(&st)[tid];
+    if (CLUSTER) {
+        // every sequence its numbers to all, then its rows to their place (sequence-major)
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all run
+        if (tid < a.B) {
+            uint32_t at;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_seq[b])), "r"(tid));
+            asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(seq.x), "r"(seq.y) : "memory");
+        }
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        const int2 o = lane < a.B ? s_seq[lane] : make_int2(0, 0);
+        const int c = o.x & ~kGoesOn, off = warp_sum_i32(lane < b ? c : 0), all = warp_sum_i32(c), act = warp_sum_i32(o.y);
+        const bool on = __any_sync(0xffffffffu, (o.x & kGoesOn) != 0);
+        if (a.next_rows) for (int i = tid; i < n_next; i += kSelThreads) a.next_rows[off + i] = next[i];
+        if (b == 0 && tid == 0) finish_step(a, all, act, steps_before, !on);
+        return;
+    }
     if (a.B == 1) return;
 
     // ---- last sequence: concatenate the row lists, count the active sequences
@@ -416,7 +434,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
         int pre = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const int t = __shfl_up_sync(0xffffffffu, pre, o); if (lane >= o) pre += t; }
-        for (int k = warp; k < 32 && q0 + k < a.B; k += kSelThreads / 32) {
+        for (int k = warp; k < 32 && q0 + k < a.B; k += kSelWarps) {
             const int ck = __shfl_sync(0xffffffffu, c, k), ok = off + __shfl_sync(0xffffffffu, pre, k) - ck;
             if (a.next_rows)
                 for (int i = lane; i < ck; i += 32) a.next_rows[ok + i] = __ldcg(&a.seq_rows[(long long)(q0 + k) * L + i]);
@@ -453,11 +471,16 @@ int32_t launch_select(const SelectArgs &args, cudaStream_t stream)
     const size_t smem = select_shared(a.L);
     const int32_t rc = select_fits(a.L);
     if (rc != SFS_OK) return rc;
-    SFS_CUDA(allow_shared(select_kernel, smem));
     // two-pass statistics: two CTAs per SM over all sequences share the recomputation (k > 1 can ask for every row)
     a.groups = 1;
     if (a.pos_lo != nullptr) a.groups = a.B < 148 ? 296 / a.B : 1;
-    SFS_CUDA(launch_pdl(select_kernel, dim3((unsigned)(a.B * a.groups)), dim3((unsigned)(kSelThreads)), (size_t)(smem), stream, a));
+    else if (a.B > 1 && a.B <= kMostCluster) {
+        SFS_CUDA(allow_shared(select_kernel<true>, smem));
+        SFS_CUDA(launch_pdl_cluster(select_kernel<true>, a.B, dim3((unsigned)a.B), dim3(kSelThreads), smem, stream, a));
+        return SFS_OK;
+    }
+    SFS_CUDA(allow_shared(select_kernel<false>, smem));
+    SFS_CUDA(launch_pdl(select_kernel<false>, dim3((unsigned)(a.B * a.groups)), dim3((unsigned)(kSelThreads)), (size_t)(smem), stream, a));
     return SFS_OK;
 }
 
