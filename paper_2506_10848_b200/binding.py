@@ -72,27 +72,45 @@ def lib():
         L = ctypes.CDLL(LIB_PATH)
         L.sfs_last_error.restype = c_char_p
         L.sfs_status_string.restype = c_char_p
-        L.sfs_status_string.argtypes = [c_int32]
+        for name, kinds in _PROTOTYPES.items():
+            getattr(L, name).argtypes = [_KINDS[k] for k in kinds]
         _lib = L
     return _lib
 
 
+# Arguments in order: p pointer (a handle, a device or host address, None, byref), i int32, l int64, f float.  With them declared an
+# argument is converted on its way into the call instead of being wrapped first.
+_KINDS = {"p": c_void_p, "i": c_int32, "l": c_int64, "f": c_float}
+_PROTOTYPES = {
+    "sfs_status_string": "i", "sfs_row_stats": "piilpipppp", "sfs_row_stats_bounds": "pilpipppp", "sfs_state_init": "piipp",
+    "sfs_select_session_create": "iiip", "sfs_session_destroy": "p", "sfs_select": "ppilppippiiippppppppp", "sfs_linear": "plplpliiiifp",
+    "sfs_check_device_status": "p", "sfs_attention": "pppiiiip", "sfs_model_create": "ppp", "sfs_model_destroy": "p",
+    "sfs_session_create": "piip", "sfs_forward": "ppiippipip", "sfs_cache_enable": "pp", "sfs_cache_reset": "p", "sfs_cache_dump": "ppp",
+    "sfs_forward_cached": "ppiiipppipipppp", "sfs_generate": "ppiiippppip", "sfs_generate_begin": "ppiiipp", "sfs_generate_steps": "pipipppp",
+    "sfs_generate_end": "pppppp", "sfs_profile": "pippp", "sfs_select_static": "ipilppippiiippppppppp",
+}
+
+
 def _ptr(t):
-    """torch tensor / int / None -> c_void_p."""
-    if t is None:
-        return c_void_p(0)
-    if isinstance(t, int):
-        return c_void_p(t)
-    return c_void_p(t.data_ptr())
+    """torch tensor / int / None -> address."""
+    return t if t is None or isinstance(t, int) else t.data_ptr()
+
+
+_current = None          # once CUDA is up: (current device, its current stream's handle), without a stream object per call
 
 
 def _stream(stream):
+    global _current
     if stream is None:
+        if _current is not None:
+            return _current[1](_current[0]())
         import torch
-        return c_void_p(torch.cuda.current_stream().cuda_stream)
-    if isinstance(stream, int):
-        return c_void_p(stream)
-    return c_void_p(stream.cuda_stream)
+        handle = torch.cuda.current_stream().cuda_stream
+        get = getattr(torch._C, "_cuda_getDevice", None), getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if None not in get and get[1](get[0]()) == handle:
+            _current = get
+        return handle
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def _check(rc):
@@ -113,22 +131,22 @@ def sfs_version():
 
 
 def sfs_row_stats(logits, logits_dtype, vocab, ld, n_rows_dev, max_rows, argmax=None, sq=None, conf=None, stream=None):
-    _check(lib().sfs_row_stats(_ptr(logits), c_int32(logits_dtype), c_int32(vocab), c_int64(ld), _ptr(n_rows_dev),
-                               c_int32(max_rows), _ptr(argmax), _ptr(sq), _ptr(conf), _stream(stream)))
+    _check(lib().sfs_row_stats(_ptr(logits), logits_dtype, vocab, ld, _ptr(n_rows_dev),
+                               max_rows, _ptr(argmax), _ptr(sq), _ptr(conf), _stream(stream)))
 
 
 def sfs_row_stats_bounds(logits, vocab, ld, n_rows_dev, max_rows, lo, hi, argmax=None, stream=None):
-    _check(lib().sfs_row_stats_bounds(_ptr(logits), c_int32(vocab), c_int64(ld), _ptr(n_rows_dev), c_int32(max_rows), _ptr(lo), _ptr(hi),
+    _check(lib().sfs_row_stats_bounds(_ptr(logits), vocab, ld, _ptr(n_rows_dev), max_rows, _ptr(lo), _ptr(hi),
                                       _ptr(argmax), _stream(stream)))
 
 
 def sfs_state_init(state, B, gen_len, params, stream=None):
-    _check(lib().sfs_state_init(_ptr(state), c_int32(B), c_int32(gen_len), byref(params), _stream(stream)))
+    _check(lib().sfs_state_init(_ptr(state), B, gen_len, byref(params), _stream(stream)))
 
 
 def sfs_select_session_create(vocab, max_batch, max_seq):
     h = c_void_p()
-    _check(lib().sfs_select_session_create(c_int32(vocab), c_int32(max_batch), c_int32(max_seq), byref(h)))
+    _check(lib().sfs_select_session_create(vocab, max_batch, max_seq, byref(h)))
     return h
 
 
@@ -138,15 +156,15 @@ def sfs_session_destroy(session):
 
 def sfs_select(session, logits, logits_dtype, ld, rows, n_rows_dev, max_rows, tokens, mask, B, S, P, state, params,
                sel_count=None, sel_pos=None, sel_tok=None, next_rows=None, next_n_rows=None, trace=None, stream=None):
-    _check(lib().sfs_select(session, _ptr(logits), c_int32(logits_dtype), c_int64(ld), _ptr(rows), _ptr(n_rows_dev),
-                            c_int32(max_rows), _ptr(tokens), _ptr(mask), c_int32(B), c_int32(S), c_int32(P),
+    _check(lib().sfs_select(session, _ptr(logits), logits_dtype, ld, _ptr(rows), _ptr(n_rows_dev),
+                            max_rows, _ptr(tokens), _ptr(mask), B, S, P,
                             _ptr(state), byref(params), _ptr(sel_count), _ptr(sel_pos), _ptr(sel_tok),
                             _ptr(next_rows), _ptr(next_n_rows), _ptr(trace), _stream(stream)))
 
 
 def sfs_linear(A, lda, Bm, ldb, C, ldc, M, N, K, out_dtype=0, scale=1.0, stream=None):
-    _check(lib().sfs_linear(_ptr(A), c_int64(lda), _ptr(Bm), c_int64(ldb), _ptr(C), c_int64(ldc), c_int32(M), c_int32(N),
-                            c_int32(K), c_int32(out_dtype), c_float(scale), _stream(stream)))
+    _check(lib().sfs_linear(_ptr(A), lda, _ptr(Bm), ldb, _ptr(C), ldc, M, N,
+                            K, out_dtype, scale, _stream(stream)))
 
 
 def sfs_check_device_status(stream=None):
@@ -156,7 +174,7 @@ def sfs_check_device_status(stream=None):
 
 
 def sfs_attention(qk, vt, out, B, S, n_heads, head_dim, stream=None):
-    _check(lib().sfs_attention(_ptr(qk), _ptr(vt), _ptr(out), c_int32(B), c_int32(S), c_int32(n_heads), c_int32(head_dim),
+    _check(lib().sfs_attention(_ptr(qk), _ptr(vt), _ptr(out), B, S, n_heads, head_dim,
                                _stream(stream)))
 
 
@@ -188,13 +206,13 @@ class Model:
 
 def sfs_session_create(model, max_batch, max_seq):
     h = c_void_p()
-    _check(lib().sfs_session_create(model.handle if isinstance(model, Model) else model, c_int32(max_batch), c_int32(max_seq), byref(h)))
+    _check(lib().sfs_session_create(model.handle if isinstance(model, Model) else model, max_batch, max_seq, byref(h)))
     return h
 
 
 def sfs_forward(session, tokens, B, S, rows, n_rows_dev, max_rows, logits, logits_dtype, stream=None):
-    _check(lib().sfs_forward(session, _ptr(tokens), c_int32(B), c_int32(S), _ptr(rows), _ptr(n_rows_dev), c_int32(max_rows),
-                             _ptr(logits), c_int32(logits_dtype), _stream(stream)))
+    _check(lib().sfs_forward(session, _ptr(tokens), B, S, _ptr(rows), _ptr(n_rows_dev), max_rows,
+                             _ptr(logits), logits_dtype, _stream(stream)))
 
 
 def sfs_cache_enable(session, k_prompt=100, k_response=5, rho=0.25, off=False):
@@ -217,23 +235,23 @@ def sfs_forward_cached(session, tokens, B, S, P, state, rows, n_rows_dev, max_ro
                        stream=None):
     """Returns n_sel, the number of recomputed rows per sequence and layer in this step."""
     n = c_int32(0)
-    _check(lib().sfs_forward_cached(session, _ptr(tokens), c_int32(B), c_int32(S), c_int32(P), _ptr(state), _ptr(rows), _ptr(n_rows_dev),
-                                    c_int32(max_rows), _ptr(logits), c_int32(logits_dtype), _ptr(sets), _ptr(sims), byref(n),
+    _check(lib().sfs_forward_cached(session, _ptr(tokens), B, S, P, _ptr(state), _ptr(rows), _ptr(n_rows_dev),
+                                    max_rows, _ptr(logits), logits_dtype, _ptr(sets), _ptr(sims), byref(n),
                                     _stream(stream)))
     return n.value
 
 
 def sfs_generate(session, prompt, B, P, gen_len, params, out_tokens, state_out=None, trace=None, max_trace_steps=0, stream=None):
-    _check(lib().sfs_generate(session, _ptr(prompt), c_int32(B), c_int32(P), c_int32(gen_len), byref(params), _ptr(out_tokens),
-                              _ptr(state_out), _ptr(trace), c_int32(max_trace_steps), _stream(stream)))
+    _check(lib().sfs_generate(session, _ptr(prompt), B, P, gen_len, byref(params), _ptr(out_tokens),
+                              _ptr(state_out), _ptr(trace), max_trace_steps, _stream(stream)))
 
 
 def sfs_generate_begin(session, prompt, B, P, gen_len, params, stream=None):
-    _check(lib().sfs_generate_begin(session, _ptr(prompt), c_int32(B), c_int32(P), c_int32(gen_len), byref(params), _stream(stream)))
+    _check(lib().sfs_generate_begin(session, _ptr(prompt), B, P, gen_len, byref(params), _stream(stream)))
 
 
 def sfs_generate_steps(session, n_steps, trace=None, max_trace_steps=0, logits_dump=None, rows_dump=None, n_rows_dump=None, stream=None):
-    _check(lib().sfs_generate_steps(session, c_int32(n_steps), _ptr(trace), c_int32(max_trace_steps), _ptr(logits_dump),
+    _check(lib().sfs_generate_steps(session, n_steps, _ptr(trace), max_trace_steps, _ptr(logits_dump),
                                     _ptr(rows_dump), _ptr(n_rows_dump), _stream(stream)))
 
 
@@ -254,7 +272,7 @@ def sfs_profile(session, enable, read=True):
     ms = (c_float * n)()
     cnt = (c_int64 * n)()
     tot = c_int64(0)
-    _check(lib().sfs_profile(session, c_int32(1 if enable else 0), ms if read else None, cnt if read else None, byref(tot)))
+    _check(lib().sfs_profile(session, 1 if enable else 0, ms if read else None, cnt if read else None, byref(tot)))
     return dict(zip(K_CLASSES, list(ms))), dict(zip(K_CLASSES, list(cnt))), tot.value
 
 
@@ -264,7 +282,7 @@ STATIC_MAX_POSITIONS, STATIC_MAX_BATCH = 16384, 64
 def sfs_select_static(vocab, logits, logits_dtype, ld, rows, n_rows_dev, max_rows, tokens, mask, B, S, P, state, params,
                       sel_count=None, sel_pos=None, sel_tok=None, next_rows=None, next_n_rows=None, trace=None, stream=None):
     """sfs_select without a session: the scratch is a fixed array inside the library, so nothing is allocated."""
-    _check(lib().sfs_select_static(c_int32(vocab), _ptr(logits), c_int32(logits_dtype), c_int64(ld), _ptr(rows), _ptr(n_rows_dev),
-                                   c_int32(max_rows), _ptr(tokens), _ptr(mask), c_int32(B), c_int32(S), c_int32(P),
+    _check(lib().sfs_select_static(vocab, _ptr(logits), logits_dtype, ld, _ptr(rows), _ptr(n_rows_dev),
+                                   max_rows, _ptr(tokens), _ptr(mask), B, S, P,
                                    _ptr(state), byref(params), _ptr(sel_count), _ptr(sel_pos), _ptr(sel_tok),
                                    _ptr(next_rows), _ptr(next_n_rows), _ptr(trace), _stream(stream)))
