@@ -334,11 +334,20 @@ static int32_t small_body(sfs_session *s, int B, int S, const int32_t *d_active,
     const bool fused = small_layer_fits(d, ff, c.n_heads, c.head_dim, B, S);
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
-        if (l > 0 && (rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, l, B, S, nullptr, d_active, cache, st); })) != SFS_OK) return rc;
+        if (l > 0 && !fused && (rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return small_qkv(s, l, B, S, nullptr, d_active, cache, st); })) != SFS_OK) return rc;
         if (cache && (rc = cache_values(s, l, T, d_active, st)) != SFS_OK) return rc;
         if (fused) {
             SmallLayerArgs a{};
-            a.qkv = s->attn_plan.direct; a.scale_log2 = s->attn_plan.args.scale_log2; a.B = B; a.S = S; a.n_heads = c.n_heads; a.d = d; a.ff = ff;
+            // a layer's launch also projects the next one's q, k and v, into the buffers it does not read: the step's own, or (odd layers) the
+            // slabs, which these steps leave free
+            __nv_bfloat16 *const qk[2] = {s->qk, reinterpret_cast<__nv_bfloat16 *>(s->partial)}, *const vt[2] = {s->vt, qk[1] + (size_t)T * 2 * d};
+            const int in = l & 1, out = in ^ 1;
+            a.qkv = AttnShort{qk[in], qk[in] + d, vt[in], 2 * d, 2 * d, T};
+            if (l + 1 < c.n_layers) {
+                a.w_q = bf(m->wq[l + 1]); a.w_k = bf(m->wk[l + 1]); a.w_v = bf(m->wv[l + 1]); a.next_gain = bf(m->attn_norm[l + 1]);
+                a.qk_out = qk[out]; a.vt_out = vt[out]; a.k_dst = cache ? s->Kc[l + 1] : nullptr; a.table = s->rope_table;
+            }
+            a.scale_log2 = s->attn_plan.args.scale_log2; a.B = B; a.S = S; a.n_heads = c.n_heads; a.d = d; a.ff = ff;
             a.wo = bf(m->wo[l]); a.w_gate = bf(m->w_gate[l]); a.w_up = bf(m->w_up[l]); a.w_down = bf(m->w_down[l]); a.gain = bf(m->mlp_norm[l]); a.eps = c.rms_eps;
             a.x = s->x; a.inc_attn = cache ? s->Ac[l] : nullptr; a.inc_mlp = cache ? s->Fc[l] : nullptr; a.d_active = d_active; a.err = device_status_word();
             if ((rc = timed_launch(s, SFS_K_GEMM_GATE_UP, st, [&] { return launch_small_layer(a, st); })) != SFS_OK) return rc;

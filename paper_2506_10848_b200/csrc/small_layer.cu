@@ -1,5 +1,5 @@
 // A small model's layer behind its QKV projection in one launch: attention, output projection, residual add, RMSNorm, gate / up
-// with SwiGLU, down projection, residual add.
+// with SwiGLU, down projection, residual add, and the next layer's RMSNorm, QKV projection and rotary embedding.
 //
 // After the attention every token is on its own, so a cluster of eight CTAs takes 16 or 32 tokens through all of it.  The weights are
 // divided over the cluster (an eighth of each projection's output columns) and requested before the dependent-launch wait, one
@@ -9,9 +9,12 @@
 //   output      rows x d/8 columns, k divided over the warps, + residual                  -> sums of squares [CTA][rows]
 //   norm        of the same columns                                                       -> bf16 [CTA][rows][d/8]
 //   gate, up    rows x ff/8 features, both products of a feature in one thread             -> bf16 [CTA][rows][ff/8]
-//   down        rows x d/8 columns, k divided again, + residual                           -> x
+//   down        rows x d/8 columns, k divided again, + residual                           -> x, sums of squares [CTA][rows]
+//   norm        of the same columns                                                       -> bf16 [CTA][rows][d/8]
+//   q, k, v     rows x d/8 columns of each, weights where gate's and up's were; a thread has both halves of its rotary pairs
 // Bound: the chain of these exchanges: at 64 tokens, d 256, d_ff 688, 10600 clocks from the wait to the end, of which attention 3400, the
-// four messages 3400, products 3500; four launches took 12 us.  A 2-layer step 34.4 -> 26.0 us, one of 2 x 224 tokens 53.5 -> 38.9.  Between SMs of a cluster 20 bytes a clock leave a CTA, whatever carries them: 2 KB to each of
+// four messages 3400, products 3500; four launches took 12 us.  A 2-layer step 34.4 -> 26.0 us, one of 2 x 224 tokens 53.5 -> 38.9, and
+// 36.9 with the next QKV projection in it.  Between SMs of a cluster 20 bytes a clock leave a CTA, whatever carries them: 2 KB to each of
 // seven peers are there after 970 clocks by bulk copies, 1400 by remote stores and a cluster barrier (417 of them the empty barrier),
 // 1650 through L2 and 1830 by remote loads.  So the sums of squares go ahead and the rows follow normalised, as 16 bits (fp32 rows and a
 // norm in every CTA: 3600 clocks), and no copy carries what its receiver has.
@@ -43,12 +46,13 @@ struct Layout {
         rows = 16 * RT;
         ldk = d + 8; ldf = ((ff + 15) & ~15) + 8; ldh = 8 * (tiles | 1);      // an odd number of 16-byte chunks: conflict-free
         x_block = rows * nc * 2; h_block = rows * ldh * 2;
-        gu = 0;
-        down = gu + 2 * 8 * tiles * ldk * 2;
+        gu = 0;                              // (later: the next QKV projection's rows)
+        down = gu + (2 * 8 * tiles > 3 * nc ? 2 * 8 * tiles : 3 * nc) * ldk * 2;
         hid = down + nc * ldf * 2;
         wo = hid; red_o = wo + nc * ldk * 2;
         const int xs_bytes = CL * x_block, attn_bytes = d / kHead * rows * kHeadLd * 2;
-        int hid_bytes = CL * h_block;
+        int hid_bytes = CL * h_block;        // (later: two tables of partial sums)
+        if (hid_bytes < 2 * red) hid_bytes = 2 * red;
         if (hid_bytes < nc * ldk * 2 + red) hid_bytes = nc * ldk * 2 + red;
         if (hid_bytes < nc * ldk * 2 + scratch - xs_bytes) hid_bytes = nc * ldk * 2 + scratch - xs_bytes;
         xs = hid + hid_bytes;
@@ -93,7 +97,7 @@ __device__ __forceinline__ void await(uint32_t bar, int32_t *err) {
     if (!ok && err) atomicExch(err, SFS_ERR_TIMEOUT);
 }
 
-enum { BAR_WO = 0, BAR_GU = 1, BAR_WD = 2, BAR_ATTN = 3, BAR_SUMS = 4, BAR_X = 5, BAR_HID = 6, N_BARS = 7 };
+enum { BAR_WO = 0, BAR_GU = 1, BAR_WD = 2, BAR_ATTN = 3, BAR_SUMS = 4, BAR_X = 5, BAR_HID = 6, BAR_QKV = 7, BAR_SUMS2 = 8, BAR_X2 = 9, N_BARS = 10 };
 
 // NN: 8-column tiles of the output and down projections' columns in a CTA (d / 64); RT: tiles of 16 rows
 template <int NN, int RT>
@@ -124,6 +128,8 @@ small_layer_kernel(SmallLayerArgs g)
         expect_bytes(bar + 8 * BAR_ATTN, (units - my_units) * kUnitBytes);
         expect_bytes(bar + 8 * BAR_SUMS, (CL - 1) * ROWS * 4);
         expect_bytes(bar + 8 * BAR_X, (CL - 1) * L.x_block); expect_bytes(bar + 8 * BAR_HID, (CL - 1) * L.h_block);
+        expect_bytes(bar + 8 * BAR_QKV, 3 * NC * D * 2);
+        expect_bytes(bar + 8 * BAR_SUMS2, (CL - 1) * ROWS * 4); expect_bytes(bar + 8 * BAR_X2, (CL - 1) * L.x_block);
     }
     __syncthreads();
     cluster_arrive();                                       // this CTA runs: its shared memory may be written by its peers
@@ -152,12 +158,22 @@ small_layer_kernel(SmallLayerArgs g)
     constexpr int OWN = (ROWS * Q + kThreads - 1) / kThreads;
     const long long tok0 = (long long)b * g.S + row0;
     int own_row[OWN], own_col[OWN];
-    uint2 gain[OWN];
+    uint2 gain[OWN], next_gain[OWN];
+    float4 angle[OWN][2];                                   // (cos, sin) of this thread's four rotary pairs, if it has any
+    const bool next = g.w_q != nullptr;
+    constexpr int HALF = NC / 2;                            // rotary pairs of a CTA in each of q and k: pairs rank HALF .. of the d / 2
+    const int pair_head = rank * HALF / (kHead / 2), pair_j = rank * HALF % (kHead / 2);
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
         const int e = tid + i * kThreads;
         own_row[i] = e < ROWS * Q ? e / Q : ROWS; own_col[i] = 4 * (e % Q);
         gain[i] = *reinterpret_cast<const uint2 *>(g.gain + rank * NC + own_col[i]);
+        if (next) {
+            next_gain[i] = *reinterpret_cast<const uint2 *>(g.next_gain + rank * NC + own_col[i]);
+            if (own_row[i] < rows && own_col[i] < HALF)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) angle[i][h] = *reinterpret_cast<const float4 *>(g.table + (long long)(row0 + own_row[i]) * (kHead / 2) + pair_j + own_col[i] + 2 * h);
+        }
     }
 
     pdl_wait();
@@ -229,50 +245,58 @@ small_layer_kernel(SmallLayerArgs g)
     const uint32_t at_base = smem_addr(sAt + ra * kHeadLd) + 16 * hi;
     project([&](int s) { return at_base + (uint32_t)((s >> 2) * ROWS * kHeadLd * 2) + (s & 3) * 32; }, sO, L.ldk, D / 16);
     float *sums = reinterpret_cast<float *>(smem + L.sums);
-#pragma unroll
-    for (int i = 0; i < OWN; ++i) {
-        if (own_row[i] >= ROWS) continue;                   // (whole warps: Q divides 32, and ROWS * Q is a multiple of 32)
-        const float4 s = owned_sum(i);
-        if (g.inc_attn && own_row[i] < rows) *reinterpret_cast<float4 *>(g.inc_attn + (tok0 + own_row[i]) * D + rank * NC + own_col[i]) = s;
-        xr[i].x += s.x; xr[i].y += s.y; xr[i].z += s.z; xr[i].w += s.w;
-        float ss = xr[i].x * xr[i].x + xr[i].y * xr[i].y + xr[i].z * xr[i].z + xr[i].w * xr[i].w;
-#pragma unroll
-        for (int o = Q / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-        if (own_col[i] == 0) sums[rank * ROWS + own_row[i]] = ss;
-    }
-    send(smem_addr(sums + rank * ROWS), ROWS * 4, bar + 8 * BAR_SUMS, rank, tid);
-    await(bar + 8 * BAR_SUMS, g.err);
-    // ---- the normalised rows' message, its 16-byte chunks XOR-swizzled by row
     constexpr int CPR = NC / 8;                             // chunks of a message row; rows that share 128 bytes take other chunks
     auto chunk_at = [&](int r, int c) { return r * NC * 2 + ((c ^ ((r / (8 / CPR)) & (CPR - 1))) << 4); };
-    uint8_t *mine = smem + L.xs + rank * L.x_block;
+    // xr's norm: the sums of squares ahead, then the normalised rows' message, its 16-byte chunks XOR-swizzled by row
+    auto send_normalised = [&](const uint2 *gn, int bar_sums, int bar_x) {
+#pragma unroll
+        for (int i = 0; i < OWN; ++i) {
+            if (own_row[i] >= ROWS) continue;               // (whole warps: Q divides 32, and ROWS * Q is a multiple of 32)
+            float ss = xr[i].x * xr[i].x + xr[i].y * xr[i].y + xr[i].z * xr[i].z + xr[i].w * xr[i].w;
+#pragma unroll
+            for (int o = Q / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            if (own_col[i] == 0) sums[rank * ROWS + own_row[i]] = ss;
+        }
+        send(smem_addr(sums + rank * ROWS), ROWS * 4, bar + 8 * bar_sums, rank, tid);
+        await(bar + 8 * bar_sums, g.err);
+        uint8_t *mine = smem + L.xs + rank * L.x_block;
+#pragma unroll
+        for (int i = 0; i < OWN; ++i) {
+            if (own_row[i] >= ROWS) continue;
+            float ss = 0.f;
+#pragma unroll
+            for (int q = 0; q < CL; ++q) ss += sums[q * ROWS + own_row[i]];
+            const float inv = rsqrtf(ss / (float)D + g.eps);
+            *reinterpret_cast<uint2 *>(mine + chunk_at(own_row[i], own_col[i] >> 3) + 2 * (own_col[i] & 4)) =
+                make_uint2(pack2(xr[i].x * inv * bf16_bits_to_f32(gn[i].x & 0xFFFFu), xr[i].y * inv * bf16_bits_to_f32(gn[i].x >> 16)),
+                           pack2(xr[i].z * inv * bf16_bits_to_f32(gn[i].y & 0xFFFFu), xr[i].w * inv * bf16_bits_to_f32(gn[i].y >> 16)));
+        }
+        send(smem_addr(mine), (uint32_t)L.x_block, bar + 8 * bar_x, rank, tid);
+    };
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
         if (own_row[i] >= ROWS) continue;
-        float ss = 0.f;
-#pragma unroll
-        for (int q = 0; q < CL; ++q) ss += sums[q * ROWS + own_row[i]];
-        const float inv = rsqrtf(ss / (float)D + g.eps);
-        *reinterpret_cast<uint2 *>(mine + chunk_at(own_row[i], own_col[i] >> 3) + 2 * (own_col[i] & 4)) =
-            make_uint2(pack2(xr[i].x * inv * bf16_bits_to_f32(gain[i].x & 0xFFFFu), xr[i].y * inv * bf16_bits_to_f32(gain[i].x >> 16)),
-                       pack2(xr[i].z * inv * bf16_bits_to_f32(gain[i].y & 0xFFFFu), xr[i].w * inv * bf16_bits_to_f32(gain[i].y >> 16)));
+        const float4 s = owned_sum(i);
+        if (g.inc_attn && own_row[i] < rows) *reinterpret_cast<float4 *>(g.inc_attn + (tok0 + own_row[i]) * D + rank * NC + own_col[i]) = s;
+        xr[i].x += s.x; xr[i].y += s.y; xr[i].z += s.z; xr[i].w += s.w;
     }
-    send(smem_addr(mine), (uint32_t)L.x_block, bar + 8 * BAR_X, rank, tid);
+    send_normalised(gain, BAR_SUMS, BAR_X);
     await(bar + 8 * BAR_GU, g.err);
     await(bar + 8 * BAR_X, g.err);
-    pdl_trigger();                                          // (about a launch latency of work is left: see pdl_trigger)
+    pdl_trigger();                                          // (the next launch has its own weights to request)
 
+    const uint32_t x_base = smem_addr(smem + L.xs);
+    constexpr int SPB = NC / 16;                            // k-steps of a message
     // ---- gate and up: the warps take the 8-feature tiles in turn, two at a time
     __nv_bfloat16 *own_h = reinterpret_cast<__nv_bfloat16 *>(smem + L.hid + rank * L.h_block);
     {
-        const uint32_t x_base = smem_addr(smem + L.xs), b_addr = smem_addr(sG + ((lane >> 4) * 8 * tiles + (lane & 7)) * L.ldk + ((lane >> 3) & 1) * 8);      // lanes 0-15: gate, 16-31: up
+        const uint32_t b_addr = smem_addr(sG + ((lane >> 4) * 8 * tiles + (lane & 7)) * L.ldk + ((lane >> 3) & 1) * 8);      // lanes 0-15: gate, 16-31: up
         auto features = [&](auto many, int tb) {
             constexpr int T = decltype(many)::value;
             float ag[T][RT][4] = {}, au[T][RT][4] = {};
 #pragma unroll 4
             for (int s = 0; s < D / 16; ++s) {
                 uint32_t a[RT][4], w[T][4];
-                constexpr int SPB = NC / 16;                // k-steps of a message
 #pragma unroll
                 for (int r = 0; r < RT; ++r) ldmatrix4(a[r], x_base + (s / SPB) * L.x_block + chunk_at(r * 16 + (lane & 15), (s % SPB) * 2 + hi));
 #pragma unroll
@@ -297,9 +321,15 @@ small_layer_kernel(SmallLayerArgs g)
         if (tb < nt) features(std::integral_constant<int, 1>{}, tb);
     }
     send(smem_addr(own_h), (uint32_t)L.h_block, bar + 8 * BAR_HID, rank, tid);
+    if (next)                                               // (gate's and up's rows have been read)
+        for (int r = tid; r < 3 * NC; r += kThreads) {
+            const int map = r / NC, q = r - map * NC;       // q and k: first halves of the CTA's pairs, then second halves
+            const int row = map == 2 ? rank * NC + q : pair_head * kHead + pair_j + (q < HALF ? q : q - HALF + kHead / 2);
+            load_row(smem_addr(sG + r * L.ldk), (map == 0 ? g.w_q : (map == 1 ? g.w_k : g.w_v)) + (long long)row * D, D * 2, bar + 8 * BAR_QKV);
+        }
     await(bar + 8 * BAR_WD, g.err);
     await(bar + 8 * BAR_HID, g.err);
-    cluster_arrive_relaxed();                               // all messages have been received here: their senders may leave
+    if (!next) cluster_arrive_relaxed();                    // all messages have been received here: their senders may leave
 
     // ---- down projection and residual (an odd last tile is multiplied with zeros beside it)
     red = reinterpret_cast<float *>(smem + L.red_d);
@@ -307,11 +337,55 @@ small_layer_kernel(SmallLayerArgs g)
     project([&](int s) { return h_base + 16u * s_tile[2 * s + hi]; }, sD, L.ldf, (ff8 + 1) / 2);
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
-        if (own_row[i] >= rows) continue;
+        if (own_row[i] >= ROWS) continue;
         const float4 s = owned_sum(i);
+        xr[i].x += s.x; xr[i].y += s.y; xr[i].z += s.z; xr[i].w += s.w;
+        if (own_row[i] >= rows) continue;
         const long long at = (tok0 + own_row[i]) * D + rank * NC + own_col[i];
         if (g.inc_mlp) *reinterpret_cast<float4 *>(g.inc_mlp + at) = s;
-        *reinterpret_cast<float4 *>(g.x + at) = make_float4(xr[i].x + s.x, xr[i].y + s.y, xr[i].z + s.z, xr[i].w + s.w);
+        *reinterpret_cast<float4 *>(g.x + at) = xr[i];
+    }
+    if (next) {
+        // ---- the next layer's norm and QKV projection, one matrix after the other
+        send_normalised(next_gain, BAR_SUMS2, BAR_X2);
+        await(bar + 8 * BAR_QKV, g.err);
+        await(bar + 8 * BAR_X2, g.err);
+        cluster_arrive_relaxed();                           // (as above)
+        auto x_at = [&](int s) { return x_base + (uint32_t)((s / SPB) * L.x_block + chunk_at(ra, (s % SPB) * 2 + hi)); };
+#pragma unroll 1
+        for (int map = 0; map < 3; ++map) {
+            red = reinterpret_cast<float *>(smem + L.hid + (map & 1) * (kWarps * 16 * RLD * 4));      // (the other one may still be read)
+            project(x_at, sG + map * NC * L.ldk, L.ldk, D / 16);
+#pragma unroll
+            for (int i = 0; i < OWN; ++i) {
+                if (own_row[i] >= rows) continue;
+                const long long tok = tok0 + own_row[i];
+                const float4 lo = owned_sum(i);
+                if (map == 2) {
+                    const long long ld = (long long)g.B * g.S;
+                    __nv_bfloat16 *dst = g.vt_out + (rank * NC + own_col[i]) * ld + tok;       // values go out transposed
+                    dst[0] = __float2bfloat16_rn(lo.x); dst[ld] = __float2bfloat16_rn(lo.y);
+                    dst[2 * ld] = __float2bfloat16_rn(lo.z); dst[3 * ld] = __float2bfloat16_rn(lo.w);
+                } else if (own_col[i] < HALF) {
+                    own_col[i] += HALF;
+                    const float4 up = owned_sum(i);
+                    own_col[i] -= HALF;
+                    // the projection's result is rounded to bf16 and so is the rotated one, as when the two are kernels of their own
+                    const float a0 = round_bf16(lo.x), a1 = round_bf16(lo.y), a2 = round_bf16(lo.z), a3 = round_bf16(lo.w);
+                    const float b0 = round_bf16(up.x), b1 = round_bf16(up.y), b2 = round_bf16(up.z), b3 = round_bf16(up.w);
+                    const float4 c = angle[i][0], e = angle[i][1];
+                    const uint2 first = make_uint2(pack2(a0 * c.x - b0 * c.y, a1 * c.z - b1 * c.w), pack2(a2 * e.x - b2 * e.y, a3 * e.z - b3 * e.w));
+                    const uint2 second = make_uint2(pack2(b0 * c.x + a0 * c.y, b1 * c.z + a1 * c.w), pack2(b2 * e.x + a2 * e.y, b3 * e.z + a3 * e.w));
+                    const int col = pair_head * kHead + pair_j + own_col[i];
+                    __nv_bfloat16 *dst = g.qk_out + tok * (2 * D) + map * D + col;
+                    *reinterpret_cast<uint2 *>(dst) = first; *reinterpret_cast<uint2 *>(dst + kHead / 2) = second;
+                    if (map == 1 && g.k_dst) {
+                        dst = g.k_dst + tok * D + col;
+                        *reinterpret_cast<uint2 *>(dst) = first; *reinterpret_cast<uint2 *>(dst + kHead / 2) = second;
+                    }
+                }
+            }
+        }
     }
     cluster_wait();
 }
@@ -360,9 +434,9 @@ int row_tiles(int B, int S) { return tiles(B, S, 1) <= resident_clusters() ? 1 :
 }  // namespace
 
 // Widths whose weights and rows fit a cluster's shared memory, and one wave of clusters: the second costs as much as the separate kernels
-// save.  A step of two layers, us, those kernels / this one: d 256, d_ff 688: 8 tokens 30.8 / 24.6, 64 34.8 / 26.7, 192 41.0 / 30.8, 256 43.0 / 33.2,
-// 2 x 224 (14 clusters) 53.5 / 38.9, 512 (16 clusters, two waves) 59.4 / 57.4, 16 x 32 54.1 / 52.6; d_ff 256: 64 32.8 / 24.6, 512 49.2 / 49.3;
-// d 128, d_ff 352: 64 30.8 / 22.6, 448 40.7 / 30.7, 512 43.0 / 45.1; d_ff 1024: 64 32.8 / 26.0, 512 51.2 / 55.3.
+// save.  A step of two layers, us, those kernels / this one: d 256, d_ff 688: 8 tokens 30.8 / 24.6, 64 34.8 / 26.6, 192 41.0 / 30.8, 256 43.0 / 32.8,
+// 2 x 224 (14 clusters) 53.5 / 36.9, 512 (16 clusters, two waves) 59.4 / 57.4, 16 x 32 54.1 / 52.6; d_ff 256: 64 32.8 / 24.6, 512 49.2 / 49.3;
+// d 128, d_ff 352: 64 30.8 / 22.6, 448 40.7 / 28.7, 512 43.0 / 45.1; d_ff 1024: 64 32.8 / 26.0, 512 51.2 / 55.3.
 bool small_layer_fits(int d_model, int d_ff, int n_heads, int head_dim, int B, int S)
 {
     if (!(d_model == 128 || d_model == 256) || n_heads * head_dim != d_model || head_dim != kHead || d_ff / 8 > kMaxTiles || (long long)B * S > 1 << 16) return false;

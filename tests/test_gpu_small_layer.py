@@ -1,4 +1,4 @@
-"""GPU parity of the fused layer of small models (attention to down projection in one launch) against the oracle."""
+"""GPU parity of the fused layer of small models (attention to the next QKV projection in one launch) against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -20,7 +20,7 @@ DEV = "cuda:0"
                                       (256, 344, 1, 408)])
 def test_logits_match_the_oracle(d, ff, B, S):
     dct = W.TINY.asdict()
-    dct.update(d_model=d, d_ff=ff, n_heads=d // 64, vocab=512, mask_id=511, logit_scale=1.0)
+    dct.update(n_layers=3, d_model=d, d_ff=ff, n_heads=d // 64, vocab=512, mask_id=511, logit_scale=1.0)
     shape = W.Shape(**dct)
     # weights large enough that attention is not uniform and both branches move the residual stream
     w = W.model_weights(shape, seed=d + ff, std=0.08, gain_std=0.2)
