@@ -160,8 +160,9 @@ static int32_t session_plan(sfs_session *s, int32_t B, int32_t S)
     for (int l = 0; l < c.n_layers; ++l) {
         LayerPlans &lp = s->layer_plans[l];
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
-        // q | k go row-major into qk [T, 2d]; the v columns (>= 2d) go transposed into vt [d, T]
-        rc = weight_plan_create(&lp.qkv, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
+        // q | k go row-major into qk [T, 2d], rotated (or a rotary kernel follows); the v columns (>= 2d) go transposed into vt [d, T]
+        const GemmRope rope = {s->rope_table, S, c.head_dim, nullptr, nullptr};
+        rc = weight_plan_create(&lp.qkv, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr, gemm_rotates(T, d, d, c.head_dim) ? &rope : nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
         rc = weight_plan_create(&lp.o, s->attn, d, T, d, wo, 1, d, d, GEMM_RESIDUAL_F32, s->x, d, 1, 1.0f, nullptr, 0, 0, nullptr);
@@ -423,7 +424,7 @@ static int32_t run_uncached(sfs_session *s, const int32_t *d_tokens, int32_t B, 
             const LayerPlans &lp = s->layer_plans[l];
             if (l > 0 && (rc = timed_launch(s, SFS_K_RMSNORM, st, [&] { return launch_rmsnorm(s->x, s->partial, pending, pstride, m->attn_norm[l], s->h, nullptr, nullptr, T, d, c.rms_eps, st); })) != SFS_OK) return rc;
             if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(lp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-            if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
+            if (!lp.qkv.args.rope.table && (rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, nullptr, st); })) != SFS_OK) return rc;
             if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(s->attn_plan, d_active, err, st); })) != SFS_OK) return rc;
             if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(lp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
             pending = lp.o.args.splits > 1 ? lp.o.args.splits : 0;
@@ -457,9 +458,10 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
     int32_t rc;
     for (int l = 0; l < c.n_layers; ++l) {
         CacheLayerPlans &cp = s->cache_plans[l];
-        // a full refresh writes the values straight into the cache (and the rotary kernel the keys)
+        // a full refresh writes the values straight into the cache (and the rotated keys, or the rotary kernel does)
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
-        rc = weight_plan_create(&cp.qkv_store, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->Vtc[l], T, 2 * d, nullptr);
+        const GemmRope rope = {s->rope_table, S, c.head_dim, nullptr, s->Kc[l]};
+        rc = weight_plan_create(&cp.qkv_store, s->h, d, T, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->Vtc[l], T, 2 * d, nullptr, gemm_rotates(T, d, d, c.head_dim) ? &rope : nullptr);
         if (rc != SFS_OK) return rc;
         // Fresh values of the candidate rows, for the similarities only: V^T = W_v h^T, the weights taking the part of the rows, so that they
         // leave in the cached values' layout.  Not split over K: an unchanged row has to get its cached values again, bit for bit, which
@@ -487,7 +489,7 @@ static int32_t cache_plan(sfs_session *s, int32_t B, int32_t S, int32_t P)
 }
 
 // projections over the compact buffers of NR recomputed rows
-static int32_t gather_plan(sfs_session *s, int32_t NR, int32_t T, std::vector<GatherLayerPlans> **out)
+static int32_t gather_plan(sfs_session *s, int32_t NR, int32_t T, int32_t S, std::vector<GatherLayerPlans> **out)
 {
     auto it = s->gather_plans.find(NR);
     if (it != s->gather_plans.end()) { *out = &it->second; return SFS_OK; }
@@ -499,7 +501,10 @@ static int32_t gather_plan(sfs_session *s, int32_t NR, int32_t T, std::vector<Ga
     for (int l = 0; l < c.n_layers; ++l) {
         GatherLayerPlans &gp = v[l];
         const void *qkv[3] = {m->wq[l], m->wk[l], m->wv[l]};
-        rc = weight_plan_create(&gp.qkv, s->hg, d, NR, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, s->vt, T, 2 * d, nullptr);
+        // keys and values of the listed tokens go to their places in the cache, queries stay compact (or the rotary kernel moves them)
+        const GemmRope rope = {s->rope_table, S, c.head_dim, s->sel_rows, s->Kc[l]};
+        const bool rotates = gemm_rotates(NR, d, d, c.head_dim);
+        rc = weight_plan_create(&gp.qkv, s->hg, d, NR, d, qkv, 3, d, d, GEMM_STORE, s->qk, 2 * d, 0, 1.0f, rotates ? s->Vtc[l] : s->vt, T, 2 * d, nullptr, rotates ? &rope : nullptr);
         if (rc != SFS_OK) return rc;
         const void *wo[1] = {m->wo[l]};
         rc = weight_plan_create(&gp.o, s->attn, d, NR, d, wo, 1, d, d, GEMM_STORE, s->partial, d, 1, 1.0f, nullptr, 0, 0, nullptr);
@@ -561,7 +566,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
     }); };
     const sfs_state *state = d_state ? s->state_in : nullptr;
     std::vector<GatherLayerPlans> *gps = nullptr;
-    if (!(rp && rr) && NR > 0 && (rc = gather_plan(s, NR, T, &gps)) != SFS_OK) return rc;
+    if (!(rp && rr) && NR > 0 && (rc = gather_plan(s, NR, T, S, &gps)) != SFS_OK) return rc;
     const long long inc_stride = (rp && rr) ? 0 : (long long)s->max_batch * s->max_seq * d;     // A_l -> F_l
     int n_pend = 0;
     auto dump_all = [&](int l, cudaStream_t st) {          // a full refresh's dump lists every token
@@ -585,7 +590,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
                 const CacheLayerPlans &cl = s->cache_plans[l];
                 if (l > 0 && (rc = norm_all(m->attn_norm[l])) != SFS_OK) return rc;
                 if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(cl.qkv_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, s->Kc[l], st); })) != SFS_OK) return rc;
+                if (!cl.qkv_store.args.rope.table && (rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope(s->qk, 2 * d, T, S, c.n_heads, c.head_dim, s->rope_table, s->Kc[l], st); })) != SFS_OK) return rc;
                 if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch(cl.attn, d_active, err, st); })) != SFS_OK) return rc;
                 if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(cl.o_store, nullptr, d_active, err, st); })) != SFS_OK) return rc;
                 pend = s->Ac[l];
@@ -619,7 +624,7 @@ static int32_t run_cached(sfs_session *s, const int32_t *d_tokens, int32_t B, in
                     if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_cache_select(a, st); })) != SFS_OK) return rc;
                     if ((rc = timed_launch(s, SFS_K_CACHE, st, [&] { return launch_gather_rows_bf16(s->h, s->sel_rows, NR, d, s->hg, st); })) != SFS_OK) return rc;
                     if ((rc = timed_launch(s, SFS_K_GEMM_QKV, st, [&] { return gemm_launch(gp.qkv, nullptr, d_active, err, st); })) != SFS_OK) return rc;
-                    if ((rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope_scatter_kv(s->qk, 2 * d, NR, S, c.n_heads, c.head_dim, s->rope_table, s->sel_rows, s->Kc[l], s->vt, T, s->Vtc[l], T, st); })) != SFS_OK) return rc;
+                    if (!gp.qkv.args.rope.table && (rc = timed_launch(s, SFS_K_ROPE, st, [&] { return launch_rope_scatter_kv(s->qk, 2 * d, NR, S, c.n_heads, c.head_dim, s->rope_table, s->sel_rows, s->Kc[l], s->vt, T, s->Vtc[l], T, st); })) != SFS_OK) return rc;
                     if ((rc = timed_launch(s, SFS_K_ATTENTION, st, [&] { return attn_launch_queries(cl.attn, n_sel, d_active, err, st); })) != SFS_OK) return rc;
                     if ((rc = timed_launch(s, SFS_K_GEMM_O, st, [&] { return gemm_launch(gp.o, nullptr, d_active, err, st); })) != SFS_OK) return rc;
                 }

@@ -6,6 +6,15 @@
 
 namespace sfs {
 
+// The QKV projection with the rotary embedding in its epilogue: B matrices 0 and 1 (queries, keys) are rotated, 2 (values) goes to vt.
+// `rows` (optional) names the token of every output row: keys and values then go to the tokens' places, queries stay compact.
+struct GemmRope {
+    const float2 *table;                 // [positions, head_dim / 2] (cos, sin); a token's position is its index modulo S
+    int S, head_dim;
+    const int32_t *rows;
+    __nv_bfloat16 *k_dst;                // optional [tokens, n_per_map]: the keys go there instead of columns [n_per_map, 2 n_per_map) of C
+};
+
 enum GemmMode {
     GEMM_STORE = 0,          // C = scale * acc   (bf16 or fp32); optionally the trailing columns go transposed to `vt`
     GEMM_RESIDUAL_F32 = 1,   // C (fp32) += acc
@@ -30,6 +39,8 @@ struct GemmArgs {
     int splits, kb_per_split;        // split-K: the k-blocks are cut into `splits` ranges, range s writes slab s of C
     long long split_stride;          // elements between slabs
     int b_static;            // 1: B is a model weight, which no kernel in flight writes: it may be read before the dependent-launch wait
+    GemmRope rope;           // table == NULL: none
+    int rope_groups, rope_tiles;     // 16-pair groups of a head's halves, column tiles of each rotated matrix
     int acc_bufs;            // accumulator buffers in tensor memory (2 when they fit: epilogue overlaps the next tile)
     // Optional (GEMM_STORE, bf16 output, no split): row statistics of the stored values, taken in the epilogue.  Per output
     // row, column tile (few rows: N-block and column half of it) and epilogue-warp parity one record (maximum, reference, sum
@@ -56,7 +67,9 @@ struct GemmTune { int mb, bn, stages, splits, nb; };
 int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int32_t K,
                          const void *const *Bs, int32_t n_maps, int32_t n_per_map, int64_t ldb,
                          int32_t mode, void *C, int64_t ldc, int32_t out_f32, float scale,
-                         __nv_bfloat16 *vt, int64_t ldvt, int32_t vt_col0, const GemmTune *tune);
+                         __nv_bfloat16 *vt, int64_t ldvt, int32_t vt_col0, const GemmTune *tune, const GemmRope *rope = nullptr);
+// whether the QKV projection of M rows should rotate in its epilogue, or a rotary kernel follow a plain one
+bool gemm_rotates(int32_t M, int32_t K, int32_t n_per_map, int32_t head_dim);
 // Split-K for the residual projections (mode GEMM_RESIDUAL_F32): when `ws` is given and the planner finds that cutting
 // K fills the machine better, the plan writes `args.splits` fp32 partial products to the slabs ws + s * M * ldc (plain
 // stores, C itself is not touched) and the consumer of the residual stream adds them in slab order (launch_rmsnorm does),

@@ -54,6 +54,25 @@ int32_t make_tmap_bf16(CUtensorMap *out, const void *base, uint64_t rows, uint64
     return SFS_OK;
 }
 
+// A weight matrix for projections whose epilogue rotates pairs (j, j + half) of every head: the box's rows are, head by head, 16 rows of
+// the first half and the same 16 of the second, so that 32 consecutive accumulator columns hold 16 whole pairs.  Dimensions: k, row of a
+// half, half, head.  For a plain matrix half = 16.
+static int32_t make_tmap_pairs(CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols, uint64_t ld, uint32_t half, uint32_t box_heads)
+{
+    EncodeTiledFn enc = get_encode();
+    SFS_REQUIRE(enc != nullptr, SFS_ERR_CUDA, "cuTensorMapEncodeTiled is not available from the driver");
+    SFS_REQUIRE(aligned_to(base, 16) && (ld % 8) == 0 && (rows % (2 * half)) == 0 && box_heads >= 1 && 32 * box_heads <= 256, SFS_ERR_INVALID_ARG, "tensor map of rotary pairs");
+    cuuint64_t dims[4] = {cols, half, 2, rows / (2 * half)};
+    cuuint64_t strides[3] = {ld * 2, (cuuint64_t)half * ld * 2, (cuuint64_t)2 * half * ld * 2};
+    cuuint32_t box[4] = {64, 16, 2, box_heads};
+    cuuint32_t estr[4] = {1, 1, 1, 1};
+    CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void *>(base), dims, strides, box, estr,
+                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    SFS_REQUIRE(r == CUDA_SUCCESS, SFS_ERR_CUDA, "cuTensorMapEncodeTiled failed with %d", (int)r);
+    return SFS_OK;
+}
+
 namespace {
 
 constexpr int BM = 128, BK = 64;         // rows per CTA of one 256-row MMA block; K elements per stage
@@ -84,6 +103,7 @@ struct TileCoord {
     int n_local;     // first row of that B matrix (SwiGLU: first gate row = first up row)
     int ncol0;       // first output column
     int ncols;       // valid output columns of the tile (<= BN, SwiGLU: <= BN/2)
+    int j0;          // rotated tiles: the first of the 16 pairs the tile takes of each head (n_local: its first head), else -1
 };
 
 __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int m_groups)
@@ -94,7 +114,19 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int
     t.m0 = (tile - rest * m_groups) * g.tile_rows;
     const int n_tile = g.splits == 1 ? rest : rest / g.splits;
     t.split = rest - n_tile * g.splits;
-    if (g.mode == GEMM_SWIGLU) {
+    t.j0 = -1;
+    if (g.rope.table != nullptr) {
+        // queries and keys: tiles of 16 pairs of tile_cols / 32 heads, the groups of a head's pairs fastest; then the values, plain
+        if (n_tile < 2 * g.rope_tiles) {
+            t.map_idx = n_tile >= g.rope_tiles ? 1 : 0;
+            const int local = n_tile - t.map_idx * g.rope_tiles, hg = local / g.rope_groups;
+            t.j0 = 16 * (local - hg * g.rope_groups);
+            t.n_local = hg * (g.tile_cols / 32); t.ncol0 = t.map_idx * g.n_per_map; t.ncols = g.tile_cols;
+        } else {
+            t.map_idx = 2; t.n_local = (n_tile - 2 * g.rope_tiles) * g.tile_cols;
+            t.ncol0 = 2 * g.n_per_map + t.n_local; t.ncols = min(g.tile_cols, g.n_per_map - t.n_local);
+        }
+    } else if (g.mode == GEMM_SWIGLU) {
         t.map_idx = 0; t.n_local = n_tile * g.tile_cols; t.ncol0 = t.n_local; t.ncols = min(g.tile_cols, g.N - t.ncol0);
     } else {
         t.map_idx = (n_tile >= g.tiles_per_map ? 1 : 0) + (n_tile >= 2 * g.tiles_per_map ? 1 : 0);      // at most three matrices
@@ -103,6 +135,21 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int
         t.ncols = min(g.tile_cols, g.n_per_map - t.n_local);
     }
     return t;
+}
+
+// A k-block of a CTA's weight rows.  Projections that rotate: coordinates (k, row within a half, 0, head), plain rows as heads of 32.
+template <bool ROPE>
+__device__ __forceinline__ void load_weights(uint32_t dst, const CUtensorMap *map, int k, int row, int j0, uint32_t bar)
+{
+    if (ROPE) tc::tma_load_4d_2cta_elect(dst, map, k, j0, 0, row, bar);
+    else tc::tma_load_2d_2cta_elect(dst, map, k, row, bar);
+}
+// its first row (ROPE: head) for CTA `rank` of the pair, whose share is `half` rows
+template <bool ROPE>
+__device__ __forceinline__ int weight_row0(const TileCoord &t, int rank, int half, bool shared_rows)
+{
+    if (ROPE) return (t.j0 >= 0 ? t.n_local : t.n_local / 32) + rank * (half / 32);
+    return shared_rows ? t.n_local : t.n_local + rank * half;
 }
 
 // k-blocks of the pair's first tile whose weights are requested before the dependent-launch wait
@@ -176,8 +223,112 @@ struct EpiShare {
     int blocks, seg;             // number of blocks (1 or 2), accumulator columns of each that may be valid
     int col_end;                 // columns at or beyond this belong to another tile or matrix
     int rec, rec_block;          // fused row statistics: record of block 0, records between blocks
+    int head0, j0;               // rotated tiles: head of the first 32 accumulator columns, first of the 16 pairs
     __device__ __forceinline__ int lim(int b) const { return min(col_end, col0 + b * col_block + seg); }
 };
+
+// V columns of the QKV projection go out transposed: the 32 lanes hold 32 consecutive tokens of a feature (LISTED: of the row list's)
+template <bool LISTED>
+__device__ __forceinline__ void epilogue_values(const GemmArgs &g, const EpiShare &e, int par, int lane, int M)
+{
+    const int upb = (e.seg + 31) / 32;
+    const int n_pieces = (e.blocks * upb - par + 1) / 2;
+    auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u >= upb ? 1 : 0; return 32 * (u - *b * upb); };
+    uint32_t v[32];
+    int b0;
+    if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(e.tmem + (uint32_t)b0 * e.tmem_block + (uint32_t)c, v); }
+    for (int pc = 0; pc < n_pieces; ++pc) {
+        int b;
+        const int c = piece_col(pc, &b);
+        uint16_t h[32];
+        tc::tmem_ld_wait32(v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) { __nv_bfloat16 r = __float2bfloat16_rn(__uint_as_float(v[j]) * g.scale); h[j] = *reinterpret_cast<uint16_t *>(&r); }
+        if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(e.tmem + (uint32_t)bn2 * e.tmem_block + (uint32_t)c2, v); }
+        const int grow = e.row0 + b * e.row_block + lane, col0 = e.col0 + b * e.col_block + c;
+        if (grow < M) {
+            uint16_t *dst = reinterpret_cast<uint16_t *>(g.vt) + (long long)(col0 - g.vt_col0) * g.ldvt + (LISTED && g.rope.rows ? g.rope.rows[grow] : grow);
+            const int nv = e.lim(b) - col0;                            // valid features of this piece
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (j < nv) dst[(long long)j * g.ldvt] = h[j];
+        }
+    }
+}
+
+// The parked unit of a rotated tile: 16-byte chunks 4 p .. 4 p + 3 are pairs j0 .. j0 + 15 of head `head` + p, first halves then second
+// halves; `heads` of them are this share's.  `tok`: this lane's row's token (a row of the list: keys go to their token's row).
+__device__ __forceinline__ void flush_pairs(const GemmArgs &g, uint32_t stage, int lane, int grow0, int M, int ncol0, int head, int heads, int j0, int tok)
+{
+    const int c = lane & 7, dh = g.rope.head_dim, h = head + (c >> 2), col = h * dh + ((c >> 1) & 1) * (dh / 2) + j0 + 8 * (c & 1);
+    const bool key = ncol0 != 0 && g.rope.k_dst != nullptr;
+    __nv_bfloat16 *base = key ? g.rope.k_dst : reinterpret_cast<__nv_bfloat16 *>(g.C) + ncol0;
+    const long long ld = key ? g.n_per_map : g.ldc;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int r = 4 * i + (lane >> 3), grow = grow0 + r, t = __shfl_sync(0xffffffffu, tok, r);
+        if (grow >= M || (c >> 2) >= heads || col >= g.n_per_map) continue;
+        *reinterpret_cast<uint4 *>(base + (long long)(key ? t : grow) * ld + col) = ld_shared_v4(stage + r * 128 + ((c ^ (r & 7)) << 4));
+    }
+}
+
+// A rotated tile: of every 32 accumulator columns (a head's), j and 16 + j are a pair.  The projection is rounded to bf16 and so is
+// its rotation, as two kernels would.  A function of its own: beside the other epilogues its angles spilled (664 bytes), and the
+// epilogue of 512 x 192 took 32 us instead of 11.
+__device__ __forceinline__ void epilogue_pairs(const GemmArgs &g, const EpiShare &e, uint32_t stage, int par, int lane, int M)
+{
+    const int upb = (e.seg + 63) / 64;                       // units of 64 columns per block: those of all blocks, numbered on, alternate between the parities
+    for (int b = 0; b < e.blocks; ++b) {
+        int u = (par + b * upb) & 1;
+        if (u >= upb) continue;
+        // every row's 128 bytes of the table by eight lanes, through the stage; they serve every head of the tile
+        const int grow = e.row0 + b * e.row_block + lane;
+        const int tok = grow < M ? (g.rope.rows ? g.rope.rows[grow] : grow) : 0, pos = tok % g.rope.S;
+        float2 cs[16];
+        {
+            uint4 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                v[i] = reinterpret_cast<const uint4 *>(g.rope.table + (long long)__shfl_sync(0xffffffffu, pos, 4 * i + (lane >> 3)) * (g.rope.head_dim / 2) + e.j0)[lane & 7];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int r = 4 * i + (lane >> 3);
+                st_shared_v4(stage + r * 128 + (((lane & 7) ^ (r & 7)) << 4), v[i].x, v[i].y, v[i].z, v[i].w);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const uint4 w = ld_shared_v4(stage + lane * 128 + ((j ^ (lane & 7)) << 4));
+                cs[2 * j] = make_float2(__uint_as_float(w.x), __uint_as_float(w.y)); cs[2 * j + 1] = make_float2(__uint_as_float(w.z), __uint_as_float(w.w));
+            }
+            __syncwarp();
+        }
+        const uint32_t t0 = e.tmem + (uint32_t)b * e.tmem_block;
+        uint32_t x[32];
+        tc::tmem_ld32(t0 + 64u * u, x);
+        for (; u < upb; u += 2) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {                    // two heads to a parked unit
+                uint32_t o[16];
+                tc::tmem_ld_wait32(x);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t p = pack_bf16(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1])), q = pack_bf16(__uint_as_float(x[16 + 2 * j]), __uint_as_float(x[17 + 2 * j]));
+                    const float p0 = __uint_as_float(p << 16), p1 = __uint_as_float(p & 0xFFFF0000u), q0 = __uint_as_float(q << 16), q1 = __uint_as_float(q & 0xFFFF0000u);
+                    const float2 a = cs[2 * j], c = cs[2 * j + 1];
+                    o[j] = pack_bf16(p0 * a.x - q0 * a.y, p1 * c.x - q1 * c.y);
+                    o[8 + j] = pack_bf16(q0 * a.x + p0 * a.y, q1 * c.x + p1 * c.y);
+                }
+                if (h == 0) tc::tmem_ld32(t0 + 64u * u + 32u, x);
+                else if (u + 2 < upb) tc::tmem_ld32(t0 + 64u * (u + 2), x);
+                park16(stage, lane, 4 * h, o);
+            }
+            __syncwarp();
+            flush_pairs(g, stage, lane, e.row0 + b * e.row_block, M, e.col0, e.head0 + 2 * u, e.seg / 32 - 2 * u, e.j0, tok);
+            __syncwarp();
+        }
+    }
+}
 
 // One warp's share of a tile's epilogue: 32 rows of every block, the 64-column (fp32: 32-column) units of parity `par`.
 // A unit may reach past the block's valid columns: those accumulator columns exist (inside the 256-column buffer) and
@@ -273,30 +424,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
         }
         if (stats_on) stats_flush();
     } else if (g.vt != nullptr && e.col0 >= g.vt_col0) {
-        // ---- V columns of the QKV projection go out transposed: the 32 lanes hold 32 consecutive tokens of a feature
-        const int upb = (e.seg + 31) / 32;
-        const int n_pieces = (e.blocks * upb - par + 1) / 2;
-        auto piece_col = [&](int pc, int *b) { const int u = par + 2 * pc; *b = u >= upb ? 1 : 0; return 32 * (u - *b * upb); };
-        uint32_t v[32];
-        int b0;
-        if (n_pieces > 0) { const int c = piece_col(0, &b0); tc::tmem_ld32(e.tmem + (uint32_t)b0 * e.tmem_block + (uint32_t)c, v); }
-        for (int pc = 0; pc < n_pieces; ++pc) {
-            int b;
-            const int c = piece_col(pc, &b);
-            uint16_t h[32];
-            tc::tmem_ld_wait32(v);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) { __nv_bfloat16 r = __float2bfloat16_rn(__uint_as_float(v[j]) * g.scale); h[j] = *reinterpret_cast<uint16_t *>(&r); }
-            if (pc + 1 < n_pieces) { int bn2; const int c2 = piece_col(pc + 1, &bn2); tc::tmem_ld32(e.tmem + (uint32_t)bn2 * e.tmem_block + (uint32_t)c2, v); }
-            const int grow = e.row0 + b * e.row_block + lane, col0 = e.col0 + b * e.col_block + c;
-            if (grow < M) {
-                uint16_t *dst = reinterpret_cast<uint16_t *>(g.vt) + (long long)(col0 - g.vt_col0) * g.ldvt + grow;
-                const int nv = e.lim(b) - col0;                            // valid features of this piece
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    if (j < nv) dst[(long long)j * g.ldvt] = h[j];
-            }
-        }
+        epilogue_values<false>(g, e, par, lane, M);
     } else {
         // ---- fp32 output (residual add, split-K slab, or fp32 logits): units of 32 columns
         const int upb = (e.seg + 31) / 32;
@@ -325,7 +453,7 @@ __device__ __forceinline__ void epilogue_tile(const GemmArgs &g, const EpiShare 
     }
 }
 
-template <bool STATS>
+template <bool STATS, bool ROPE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
             const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, GemmArgs g)
@@ -385,10 +513,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (warp == 0 && pre > 0) {
         const TileCoord t = tile_coord(g, pair, (g.M + MB * 2 * BM - 1) / (MB * 2 * BM));
         const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1) : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
-        const int brow = swiglu ? t.n_local : t.n_local + (int)rank * HALF, kb0 = t.split * g.kb_per_split;
+        const int brow = weight_row0<ROPE>(t, (int)rank, HALF, swiglu), j0 = max(t.j0, 0), kb0 = t.split * g.kb_per_split;
         for (int j = 0; j < pre; ++j) {
             if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)(STAGE_BYTES - (MB - blocks_of(t, g.M)) * A_BYTES));
-            tc::tma_load_2d_2cta_elect(smem_base + j * STAGE_BYTES + MB * A_BYTES, mb, (kb0 + j) * BK, brow, lead_full + 8 * j);
+            load_weights<ROPE>(smem_base + j * STAGE_BYTES + MB * A_BYTES, mb, (kb0 + j) * BK, brow, j0, lead_full + 8 * j);
         }
     }
     pdl_wait();                                             // the kernel before this one has completed: global memory from here on
@@ -419,7 +547,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             // leader: first half of the weight rows (SwiGLU: the gate rows); peer: second half (the up rows)
             const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1)
                                            : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
-            const int brow = swiglu ? t.n_local : t.n_local + (int)rank * HALF;
+            const int brow = weight_row0<ROPE>(t, (int)rank, HALF, swiglu), j0 = max(t.j0, 0);
             const int arow = t.m0 + (int)rank * BM, mbt = blocks_of(t, M);
             const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
@@ -433,7 +561,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 if (rank == 0 && !early) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)(STAGE_BYTES - (MBS - mbt) * A_BYTES));
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 if (mbt == 2) tc::tma_load_2d_2cta_elect(sa + A_BYTES, &tmA, kb * BK, arow + 2 * BM, lead_full + 8 * s);
-                if (!early) tc::tma_load_2d_2cta_elect(sa + MBS * A_BYTES, mb, kb * BK, brow, lead_full + 8 * s);
+                if (!early) load_weights<ROPE>(sa + MBS * A_BYTES, mb, kb * BK, brow, j0, lead_full + 8 * s);
                 s = ns; ph = nph;
             }
         }
@@ -519,7 +647,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             e.col0 = t.ncol0; e.col_block = 0; e.blocks = blocks_of(t, M); e.seg = STATS ? BN : t.ncols;      // (every record is written)
             e.col_end = min(t.ncol0 + t.ncols, g.N);
             e.rec = 2 * (t.ncol0 / BN); e.rec_block = 0;
-            epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
+            e.head0 = t.n_local; e.j0 = t.j0;
+            if constexpr (ROPE) {
+                if (t.j0 >= 0) epilogue_pairs(g, e, stage, par, lane, M);
+                else epilogue_values<true>(g, e, par, lane, M);
+            } else epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0 && tile + (int)n_bufs * num_pairs < num_tiles) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);     // (if it is used again)
@@ -548,7 +680,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 // holds gate rows, N-block 1 the up rows of the same features.  Of an N-block's accumulators every CTA holds its 64 rows:
 // tensor-memory lanes 0-63 the columns [0, BN/2), lanes 64-127 the columns [BN/2, BN), in BN/2 tensor-memory columns.
 // Warp roles, ring, hand-over and bounded waits are those of the pair kernel above.
-template <bool STATS>
+template <bool STATS, bool ROPE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
 gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB0,
                 const __grid_constant__ CUtensorMap tmB1, const __grid_constant__ CUtensorMap tmB2, GemmArgs g)
@@ -596,12 +728,12 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         const TileCoord t = tile_coord(g, pair, (g.M + 2 * FM - 1) / (2 * FM));
         const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
         const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
-        const int brow0 = t.n_local + (int)rank * HALF, brow1 = swiglu ? brow0 : brow0 + BN, kb0 = t.split * g.kb_per_split;
+        const int brow0 = weight_row0<ROPE>(t, (int)rank, HALF, false), brow1 = swiglu ? brow0 : brow0 + BN, j0 = max(t.j0, 0), kb0 = t.split * g.kb_per_split;
         for (int j = 0; j < pre; ++j) {
             const uint32_t sa = smem_base + j * STAGE_BYTES;
             if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * j, 2u * (uint32_t)STAGE_BYTES);
-            tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, (kb0 + j) * BK, brow0, lead_full + 8 * j);
-            if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, (kb0 + j) * BK, brow1, lead_full + 8 * j);
+            load_weights<ROPE>(sa + FM * BK * 2, m0, (kb0 + j) * BK, brow0, j0, lead_full + 8 * j);
+            if (!ROPE && NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, (kb0 + j) * BK, brow1, lead_full + 8 * j);
         }
     }
     pdl_wait();                                             // the kernel before this one has completed: global memory from here on
@@ -619,7 +751,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             const TileCoord t = tile_coord(g, tile, m_groups);
             const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
             const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
-            const int brow0 = t.n_local + (int)rank * HALF, brow1 = swiglu ? brow0 : brow0 + BN;
+            const int brow0 = weight_row0<ROPE>(t, (int)rank, HALF, false), brow1 = swiglu ? brow0 : brow0 + BN, j0 = max(t.j0, 0);
             const int arow = t.m0 + (int)rank * FM;
             const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
             for (int kb = kb0; kb < kb1; ++kb, ++it) {
@@ -631,8 +763,8 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 const uint32_t sa = smem_base + s * STAGE_BYTES;
                 if (it >= (uint32_t)pre) {
                     if (rank == 0) tc::mbar_expect_tx_elect(bar_full + 8 * s, 2u * (uint32_t)STAGE_BYTES);
-                    tc::tma_load_2d_2cta_elect(sa + FM * BK * 2, m0, kb * BK, brow0, lead_full + 8 * s);
-                    if (NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, kb * BK, brow1, lead_full + 8 * s);
+                    load_weights<ROPE>(sa + FM * BK * 2, m0, kb * BK, brow0, j0, lead_full + 8 * s);
+                    if (!ROPE && NB == 2) tc::tma_load_2d_2cta_elect(sa + FM * BK * 2 + B_BYTES, m1, kb * BK, brow1, lead_full + 8 * s);
                 }
                 tc::tma_load_2d_2cta_elect(sa, &tmA, kb * BK, arow, lead_full + 8 * s);
                 s = ns; ph = nph;
@@ -713,7 +845,12 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
             e.col0 = t.ncol0 + hq * HALF; e.col_block = BN; e.blocks = swiglu ? 1 : NB; e.seg = HALF;
             e.col_end = min(t.ncol0 + t.ncols, g.N);
             e.rec = 4 * NB * (t.ncol0 / (NB * BN)) + 2 * hq; e.rec_block = 4;
-            epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
+            e.head0 = t.n_local + hq * (HALF / 32); e.j0 = t.j0;
+            if (ROPE && t.j0 >= 0) e.col0 = t.ncol0;        // (which matrix: the columns follow from the heads)
+            if constexpr (ROPE) {
+                if (t.j0 >= 0) epilogue_pairs(g, e, stage, par, lane, M);
+                else epilogue_values<true>(g, e, par, lane, M);
+            } else epilogue_tile<STATS>(g, e, t.split, stage, par, lane, M);
             tc::tc_fence_before();
             __syncwarp();
             if (lane == 0 && tile + 2 * num_pairs < num_tiles) tc::mbar_arrive_cluster(lead_acc_empty + 8 * buf);
@@ -740,8 +877,12 @@ int num_sms()
 }
 
 // column tiles of a problem at `tile_cols` output columns per tile
-int col_tiles(int mode, int n_maps, int n_per_map, int tile_cols)
+int col_tiles(int mode, int n_maps, int n_per_map, int tile_cols, int rope_dim = 0)
 {
+    if (rope_dim) {                                          // two rotated matrices (16 pairs of tile_cols / 32 heads a tile) and a plain one
+        const int heads = n_per_map / rope_dim, per_tile = tile_cols / 32;
+        return 2 * (rope_dim / 32) * ((heads + per_tile - 1) / per_tile) + (n_per_map + tile_cols - 1) / tile_cols;
+    }
     const int per_map = (n_per_map + tile_cols - 1) / tile_cols;
     return mode == GEMM_SWIGLU ? per_map : n_maps * per_map;
 }
@@ -761,11 +902,11 @@ int stages_for(int mb, int bn)
 // (240 x 2 ranges instead of 512 x 240 x 4), QKV 1000 rows 70.4 -> 61.9, 1536 rows 90.8 -> 82.9, gate / up 1536 rows 168 -> 153.
 // The epilogue hides behind the next tile when two accumulators fit tensor memory, except for a pair's last tile.
 // Splitting K pays for few rows only: the slabs grow with M, the idle pairs they avoid do not.
-long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int mb, int bn, int splits)
+long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int rope_dim, int pairs, int mb, int bn, int splits)
 {
     const long long num_kb = (K + BK - 1) / BK, kbps = (num_kb + splits - 1) / splits;
     const int m_groups = (M + mb * 2 * BM - 1) / (mb * 2 * BM);
-    const long long tiles = (long long)m_groups * col_tiles(mode, n_maps, n_per_map, mode == GEMM_SWIGLU ? bn / 2 : bn) * ((num_kb + kbps - 1) / kbps);
+    const long long tiles = (long long)m_groups * col_tiles(mode, n_maps, n_per_map, mode == GEMM_SWIGLU ? bn / 2 : bn, rope_dim) * ((num_kb + kbps - 1) / kbps);
     const long long waves = (tiles + pairs - 1) / pairs;
     const long long mma = (long long)mb * bn * 2 + 80, load = (long long)(mb * BM + bn / 2) * 128 / 54, least = mb == 1 ? 540 : 980;
     long long kb_clk = mma > load ? mma : load;
@@ -780,14 +921,15 @@ long long model_clocks(int M, int K, int mode, int n_maps, int n_per_map, int pa
 
 // Tile shape (MB blocks of 256 rows, width bn) and number of K ranges with the smallest modelled time.  Wide, tall tiles
 // win when there are many tiles; narrower or shorter ones, or a split K, when a big tile would leave most pairs idle.
-void pick_tile(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int max_splits, int *mb_out, int *bn_out, int *splits_out)
+void pick_tile(int M, int K, int mode, int n_maps, int n_per_map, int rope_dim, int pairs, int max_splits, int *mb_out, int *bn_out, int *splits_out)
 {
-    const int step = (mode == GEMM_SWIGLU) ? 32 : 16;
+    const int step = rope_dim ? 64 : (mode == GEMM_SWIGLU ? 32 : 16);      // (a CTA's half of a rotating tile: whole groups of 16 pairs)
     long long best_cost = -1;
     for (int mb = (M > 2 * BM ? 2 : 1); mb >= 1; --mb)
         for (int bn = 256; bn >= 32; bn -= step)
             for (int sp = 1; sp <= max_splits; ++sp) {
-                const long long cost = model_clocks(M, K, mode, n_maps, n_per_map, pairs, mb, bn, sp);
+                if (rope_dim && (n_per_map / rope_dim) % (bn / 32) != 0 && bn > 64) continue;      // (see gemm_rotates)
+                const long long cost = model_clocks(M, K, mode, n_maps, n_per_map, rope_dim, pairs, mb, bn, sp);
                 if (best_cost < 0 || cost < best_cost) { best_cost = cost; *mb_out = mb; *bn_out = bn; *splits_out = sp; }
             }
 }
@@ -797,11 +939,11 @@ void pick_tile(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int
 // of a split K costs its reader ~600 clocks and 1.2e-3 per element.  At 128 rows, 8B widths this picks QKV 192 x 1 (24.8 us; the
 // next best 224: 25.4, nb = 2: 28.1), O 192 x 1 in 3 ranges of K (12.0; 2 ranges of 128: 13.0), gate / up 192 (40.2; 224: 40.8),
 // down 256 x 1 in 4 ranges (24.0; 192 in 3: 24.8).
-long long model_clocks_few(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int bn, int nb, int splits)
+long long model_clocks_few(int M, int K, int mode, int n_maps, int n_per_map, int rope_dim, int pairs, int bn, int nb, int splits)
 {
     const long long num_kb = (K + BK - 1) / BK, kbps = (num_kb + splits - 1) / splits;
     const int tile_cols = mode == GEMM_SWIGLU ? bn : nb * bn;
-    const long long tiles = (long long)col_tiles(mode, n_maps, n_per_map, tile_cols) * ((num_kb + kbps - 1) / kbps);
+    const long long tiles = (long long)col_tiles(mode, n_maps, n_per_map, tile_cols, rope_dim) * ((num_kb + kbps - 1) / kbps);
     const long long waves = (tiles + pairs - 1) / pairs;
     const long long issue = 255 + 165 * nb, port = (long long)(FM + nb * bn / 2) * 128 / 40;
     const long long hbm = (tiles < pairs ? tiles : pairs) * (long long)nb * bn * 128 / 3370;
@@ -813,16 +955,19 @@ long long model_clocks_few(int M, int K, int mode, int n_maps, int n_per_map, in
     return waves * kbps * kb_clk + epi + (splits > 1 ? slab * splits : 0);
 }
 
-void pick_tile_few(int M, int K, int mode, int n_maps, int n_per_map, int pairs, int max_splits, int *bn_out, int *nb_out, int *splits_out)
+void pick_tile_few(int M, int K, int mode, int n_maps, int n_per_map, int rope_dim, int pairs, int max_splits, int *bn_out, int *nb_out, int *splits_out)
 {
     long long best_cost = -1;
-    for (int nb = (mode == GEMM_SWIGLU ? 2 : 1); nb <= 2; ++nb)
-        for (int bn = 256; bn >= 32; bn -= 32)
+    for (int nb = (mode == GEMM_SWIGLU ? 2 : 1); nb <= (rope_dim ? 1 : 2); ++nb)
+        for (int bn = 256; bn >= 32; bn -= rope_dim ? 64 : 32)
             for (int sp = 1; sp <= max_splits; ++sp) {
-                const long long cost = model_clocks_few(M, K, mode, n_maps, n_per_map, pairs, bn, nb, sp);
+                const long long cost = model_clocks_few(M, K, mode, n_maps, n_per_map, rope_dim, pairs, bn, nb, sp);
                 if (best_cost < 0 || cost < best_cost) { best_cost = cost; *bn_out = bn; *nb_out = nb; *splits_out = sp; }
             }
 }
+
+// Clocks of the rotary kernel that a rotating epilogue saves: 104 rows of 2 x 4096 4.0 us with its hand-over, 512 6.3, 1536 12, 2048 17.
+long long rope_kernel_clocks(int M, int n_per_map) { return 6600 + (long long)((double)M * n_per_map * 3e-3); }
 
 int stages_for_few(int bn, int nb)
 {
@@ -835,10 +980,24 @@ int stages_for_few(int bn, int nb)
 
 int gemm_num_sms() { return num_sms(); }
 
+// A rotating tile takes 16 pairs of each of bn / 32 heads.  Where tiles stream weights (128 rows) a last one of fewer heads costs nothing;
+// otherwise whole tiles only (512 rows of 32 heads: 192 columns, a tenth of them padding, 58 us where 176 plain ones take 52), and a
+// projection that is faster by more than the model's error than a plain one and the rotary kernel.
+bool gemm_rotates(int32_t M, int32_t K, int32_t n_per_map, int32_t head_dim)
+{
+    if (M <= 2 * FM) return true;
+    const int pairs = num_sms() / 2;
+    int mb = 1, bn = 256, sp = 1;
+    pick_tile(M, K, GEMM_STORE, 3, n_per_map, 0, pairs, 1, &mb, &bn, &sp);
+    const long long plain = model_clocks(M, K, GEMM_STORE, 3, n_per_map, 0, pairs, mb, bn, 1) + rope_kernel_clocks(M, n_per_map);
+    pick_tile(M, K, GEMM_STORE, 3, n_per_map, head_dim, pairs, 1, &mb, &bn, &sp);
+    return (n_per_map / head_dim) % (bn / 32) == 0 && model_clocks(M, K, GEMM_STORE, 3, n_per_map, head_dim, pairs, mb, bn, 1) * 100 < plain * 97;
+}
+
 int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int32_t K,
                          const void *const *Bs, int32_t n_maps, int32_t n_per_map, int64_t ldb,
                          int32_t mode, void *C, int64_t ldc, int32_t out_f32, float scale,
-                         __nv_bfloat16 *vt, int64_t ldvt, int32_t vt_col0, const GemmTune *tune)
+                         __nv_bfloat16 *vt, int64_t ldvt, int32_t vt_col0, const GemmTune *tune, const GemmRope *rope)
 {
     SFS_REQUIRE(M >= 1 && K >= 1 && n_per_map >= 1 && n_maps >= 1 && n_maps <= 3, SFS_ERR_INVALID_ARG, "gemm: bad sizes");
     SFS_REQUIRE((K % 8) == 0 && (lda % 8) == 0 && (ldb % 8) == 0, SFS_ERR_INVALID_ARG, "gemm: K, lda, ldb must be multiples of 8");
@@ -850,20 +1009,24 @@ int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int
     int sp_unused = 1;
     // at most 128 rows: few-row tiles (a pair's 256-row MMA would be half padding); tune->mb = 1 or 2 forces the pair kernel
     const bool few = (M <= 2 * FM) && !(tune && (tune->mb == 1 || tune->mb == 2));
-    const int step = few ? 32 : ((mode == GEMM_SWIGLU) ? 32 : 16);
-    if (few) pick_tile_few(M, K, mode, n_maps, n_per_map, num_sms() / 2, 1, &bn, &nb, &sp_unused);
-    else pick_tile(M, K, mode, n_maps, n_per_map, num_sms() / 2, 1, &mb, &bn, &sp_unused);
+    const int rope_dim = rope ? rope->head_dim : 0;
+    SFS_REQUIRE(!rope || (mode == GEMM_STORE && !out_f32 && n_maps == 3 && vt != nullptr && vt_col0 == 2 * n_per_map && scale == 1.0f && (rope_dim % 32) == 0 &&
+                          (n_per_map % rope_dim) == 0 && (n_per_map % 32) == 0), SFS_ERR_INVALID_ARG, "gemm: rotary epilogue takes the QKV projection of whole heads");
+    const int step = rope ? 64 : (few ? 32 : ((mode == GEMM_SWIGLU) ? 32 : 16));
+    if (few) pick_tile_few(M, K, mode, n_maps, n_per_map, rope_dim, num_sms() / 2, 1, &bn, &nb, &sp_unused);
+    else pick_tile(M, K, mode, n_maps, n_per_map, rope_dim, num_sms() / 2, 1, &mb, &bn, &sp_unused);
     if (tune) {                                              // measurement overrides; invalid values are ignored
         if (tune->mb == 1 || tune->mb == 2) mb = tune->mb;
         if (tune->bn >= 32 && tune->bn <= 256 && (tune->bn % step) == 0) bn = tune->bn;
-        if (few && (tune->nb == 1 || tune->nb == 2) && mode != GEMM_SWIGLU) nb = tune->nb;
+        if (few && (tune->nb == 1 || tune->nb == 2) && mode != GEMM_SWIGLU && !rope) nb = tune->nb;
     }
     p->bn = bn; p->n_maps = n_maps; p->n_per_map = n_per_map;
     int32_t rc = make_tmap_bf16(&p->tmA, A, (uint64_t)M, (uint64_t)K, (uint64_t)lda, few ? FM : BM);
     if (rc != SFS_OK) return rc;
     for (int i = 0; i < 3; ++i) {
         const void *b = Bs[i < n_maps ? i : 0];
-        rc = make_tmap_bf16(&p->tmB[i], b, (uint64_t)n_per_map, (uint64_t)K, (uint64_t)ldb, (uint32_t)(bn / 2));
+        if (rope) rc = make_tmap_pairs(&p->tmB[i], b, (uint64_t)n_per_map, (uint64_t)K, (uint64_t)ldb, i < 2 ? (uint32_t)rope_dim / 2 : 16, (uint32_t)bn / 64);
+        else rc = make_tmap_bf16(&p->tmB[i], b, (uint64_t)n_per_map, (uint64_t)K, (uint64_t)ldb, (uint32_t)(bn / 2));
         if (rc != SFS_OK) return rc;
     }
     GemmArgs &g = p->args;
@@ -873,7 +1036,8 @@ int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int
     g.few = few ? 1 : 0; g.tile_rows = few ? 2 * FM : mb * 2 * BM;
     g.tile_cols = (mode == GEMM_SWIGLU) ? (few ? bn : bn / 2) : (few ? nb * bn : bn);
     g.tiles_per_map = (mode == GEMM_SWIGLU) ? 0x3FFFFFFF : (n_per_map + g.tile_cols - 1) / g.tile_cols;
-    g.n_col_tiles = col_tiles(mode, n_maps, n_per_map, g.tile_cols);
+    g.n_col_tiles = col_tiles(mode, n_maps, n_per_map, g.tile_cols, rope_dim);
+    if (rope) { g.rope = *rope; g.rope_groups = rope_dim / 32; g.rope_tiles = (g.n_col_tiles - (n_per_map + g.tile_cols - 1) / g.tile_cols) / 2; }
     g.stages = few ? stages_for_few(bn, nb) : stages_for(mb, bn);
     if (tune && tune->stages >= 1 && tune->stages <= g.stages) g.stages = tune->stages;
     g.acc_bufs = few || (g.mb * ((bn + 31) & ~31) <= 256) ? 2 : 1;
@@ -892,8 +1056,8 @@ int32_t gemm_plan_enable_split(GemmPlan *p, float *ws, int32_t max_splits, const
     if (!f32_out || ws == nullptr || max_splits < 2) return SFS_OK;
     int mb = g.mb, bn = g.bn, nb = g.nb, sp = 1;
     const bool few = g.few != 0;
-    if (few) pick_tile_few(g.M, g.K, g.mode, p->n_maps, p->n_per_map, num_sms() / 2, max_splits, &bn, &nb, &sp);
-    else pick_tile(g.M, g.K, g.mode, p->n_maps, p->n_per_map, num_sms() / 2, max_splits, &mb, &bn, &sp);
+    if (few) pick_tile_few(g.M, g.K, g.mode, p->n_maps, p->n_per_map, 0, num_sms() / 2, max_splits, &bn, &nb, &sp);
+    else pick_tile(g.M, g.K, g.mode, p->n_maps, p->n_per_map, 0, num_sms() / 2, max_splits, &mb, &bn, &sp);
     if (tune) {
         if (tune->mb == 1 || tune->mb == 2) mb = tune->mb;
         if (tune->bn >= 32 && tune->bn <= 256 && (tune->bn % 16) == 0) bn = tune->bn;
@@ -923,42 +1087,32 @@ int32_t gemm_plan_enable_split(GemmPlan *p, float *ws, int32_t max_splits, const
 
 int32_t gemm_launch(const GemmPlan &p, const int32_t *d_m, const int32_t *d_active, int32_t *err, cudaStream_t stream)
 {
-    // always ask for more than half of an SM's shared memory: one CTA per SM, so the allocation of all 512
-    // tensor-memory columns can never wait for a co-resident CTA
-    static bool configured[kMaxDevices] = {};
-    bool &done = configured[current_device_slot()];
-    if (!done) {
-        SFS_CUDA(cudaFuncSetAttribute(gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-        SFS_CUDA(cudaFuncSetAttribute(gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-        done = true;
-    }
     GemmArgs g = p.args;
     g.d_m = d_m; g.err = err; g.d_active = d_active;
-    if (g.few) {
-        static bool configured1[kMaxDevices] = {};
-        bool &done1 = configured1[current_device_slot()];
-        if (!done1) {
-            SFS_CUDA(cudaFuncSetAttribute(gemm_few_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-            SFS_CUDA(cudaFuncSetAttribute(gemm_few_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
-            done1 = true;
-        }
-        size_t smem1 = (size_t)g.stages * (FM * BK * 2 + g.nb * (g.bn / 2) * BK * 2) + kBarBytes + kEpiStageBytes + 1024;
-        if (smem1 < 120 * 1024) smem1 = 120 * 1024;            // one CTA per SM: all 512 tensor-memory columns are its own
-        const long long tiles1 = (long long)((g.M + 2 * FM - 1) / (2 * FM)) * g.n_col_tiles * g.splits;
-        const int pairs1 = num_sms() / 2;
-        const dim3 grid1((unsigned)(2 * (tiles1 < pairs1 ? tiles1 : pairs1)));
-        if (g.stats) SFS_CUDA(launch_pdl(gemm_few_kernel<true>, grid1, dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
-        else SFS_CUDA(launch_pdl(gemm_few_kernel<false>, grid1, dim3(kGemmThreads), smem1, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
-        return SFS_OK;
-    }
-    size_t smem = (size_t)g.stages * (g.mb * A_BYTES + (g.bn / 2) * BK * 2) + kBarBytes + kEpiStageBytes + 1024;
-    if (smem < 120 * 1024) smem = 120 * 1024;
-    const long long tiles = (long long)((g.M + g.mb * 2 * BM - 1) / (g.mb * 2 * BM)) * g.n_col_tiles * g.splits;
     const int pairs = num_sms() / 2;
-    dim3 grid((unsigned)(2 * (tiles < pairs ? tiles : pairs)), 1, 1);
-    if (g.stats) SFS_CUDA(launch_pdl(gemm_kernel<true>, grid, dim3(kGemmThreads), smem, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
-    else SFS_CUDA(launch_pdl(gemm_kernel<false>, grid, dim3(kGemmThreads), smem, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
-    return SFS_OK;
+    auto launch = [&](auto kernel, bool *configured, size_t smem, long long tiles) -> int32_t {
+        bool &done = configured[current_device_slot()];
+        if (!done) {
+            SFS_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget));
+            done = true;
+        }
+        // always ask for more than half of an SM's shared memory: one CTA per SM, so the allocation of all 512
+        // tensor-memory columns can never wait for a co-resident CTA
+        if (smem < 120 * 1024) smem = 120 * 1024;
+        SFS_CUDA(launch_pdl(kernel, dim3((unsigned)(2 * (tiles < pairs ? tiles : pairs))), dim3(kGemmThreads), smem, stream, p.tmA, p.tmB[0], p.tmB[1], p.tmB[2], g));
+        return SFS_OK;
+    };
+    static bool configured[6][kMaxDevices] = {};
+    const size_t fixed = kBarBytes + kEpiStageBytes + 1024, b_bytes = (size_t)(g.bn / 2) * BK * 2;
+    const long long tiles = (long long)((g.M + g.tile_rows - 1) / g.tile_rows) * g.n_col_tiles * g.splits;
+    if (g.few) {
+        const size_t smem = (size_t)g.stages * (FM * BK * 2 + g.nb * b_bytes) + fixed;
+        if (g.rope.table) return launch(gemm_few_kernel<false, true>, configured[0], smem, tiles);
+        return g.stats ? launch(gemm_few_kernel<true, false>, configured[1], smem, tiles) : launch(gemm_few_kernel<false, false>, configured[2], smem, tiles);
+    }
+    const size_t smem = (size_t)g.stages * (g.mb * A_BYTES + b_bytes) + fixed;
+    if (g.rope.table) return launch(gemm_kernel<false, true>, configured[3], smem, tiles);
+    return g.stats ? launch(gemm_kernel<true, false>, configured[4], smem, tiles) : launch(gemm_kernel<false, false>, configured[5], smem, tiles);
 }
 
 }  // namespace sfs
