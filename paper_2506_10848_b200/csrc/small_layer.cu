@@ -145,13 +145,13 @@ small_layer_kernel(SmallLayerArgs g)
         }
     }
     // where the down projection finds a tile of features: CTA q's begin at tile q ff8 / CL
-    __shared__ uint16_t s_tile[kMaxTiles + 1];              // in 16 bytes from the first message
-    for (int q = tid; q <= ff8; q += kThreads) {
-        int c = q * CL / max(ff8, 1);
-        c = min(c, CL - 1);
+    __shared__ uint16_t s_tile[kMaxTiles + 1];              // in 16 bytes from the first message; beyond the last tile, the last one again
+    for (int i = tid; i <= ff8; i += kThreads) {
+        const int q = min(i, ff8 - 1);
+        int c = q * CL / ff8;
         while (c + 1 < CL && q >= (c + 1) * ff8 / CL) ++c;
         while (c > 0 && q < c * ff8 / CL) --c;
-        s_tile[q] = (uint16_t)(q < ff8 ? (c * L.h_block >> 4) + q - c * ff8 / CL : 0);
+        s_tile[i] = (uint16_t)((c * L.h_block >> 4) + q - c * ff8 / CL);
     }
     if (g.ff & 15) for (int r = tid; r < NC; r += kThreads) *reinterpret_cast<uint4 *>(sD + r * L.ldf + g.ff) = make_uint4(0, 0, 0, 0);
     // the (row, four columns) of x this thread owns
@@ -205,8 +205,10 @@ small_layer_kernel(SmallLayerArgs g)
 
     const int rt = warp % RT, kp = warp / RT, ra = rt * 16 + (lane & 15), hi = lane >> 4;      // ldmatrix of A: row, second half of a k-step
     float *red = reinterpret_cast<float *>(smem + L.red_o);
-    // rows x this CTA's columns: k-steps [kp, kp + 1) / KP of `steps`, A's 16 bytes of (step, half, row) where a_at says
-    auto project = [&](auto &&a_at, const __nv_bfloat16 *sb, int ldb, int steps) {
+    // rows x this CTA's columns: k-steps [kp, kp + 1) / KP of `halves` / 2, A's 16 bytes of (step, half, row) where a_at says.  The second half
+    // of a last step that has none is zeroed: a zero weight alone would make NaN of an infinity, and of anything that is not a feature
+    auto project = [&](auto &&a_at, const __nv_bfloat16 *sb, int ldb, int halves) {
+        const int steps = (halves + 1) / 2;
         float acc[NN][4] = {};
         const uint32_t b_addr = smem_addr(sb + ((lane >> 4) * 8 + (lane & 7)) * ldb + ((lane >> 3) & 1) * 8);
         const int s1 = (kp + 1) * steps / KP;
@@ -214,6 +216,7 @@ small_layer_kernel(SmallLayerArgs g)
         for (int s = kp * steps / KP; s < s1; ++s) {
             uint32_t a[4];
             ldmatrix4(a, a_at(s));
+            if (2 * s + 1 == halves) a[2] = a[3] = 0;
 #pragma unroll
             for (int t = 0; t < NN; t += 2) {
                 uint32_t w[4];
@@ -243,7 +246,7 @@ small_layer_kernel(SmallLayerArgs g)
 
     // ---- output projection and residual, the norm's sums
     const uint32_t at_base = smem_addr(sAt + ra * kHeadLd) + 16 * hi;
-    project([&](int s) { return at_base + (uint32_t)((s >> 2) * ROWS * kHeadLd * 2) + (s & 3) * 32; }, sO, L.ldk, D / 16);
+    project([&](int s) { return at_base + (uint32_t)((s >> 2) * ROWS * kHeadLd * 2) + (s & 3) * 32; }, sO, L.ldk, D / 8);
     float *sums = reinterpret_cast<float *>(smem + L.sums);
     constexpr int CPR = NC / 8;                             // chunks of a message row; rows that share 128 bytes take other chunks
     auto chunk_at = [&](int r, int c) { return r * NC * 2 + ((c ^ ((r / (8 / CPR)) & (CPR - 1))) << 4); };
@@ -331,10 +334,10 @@ small_layer_kernel(SmallLayerArgs g)
     await(bar + 8 * BAR_HID, g.err);
     if (!next) cluster_arrive_relaxed();                    // all messages have been received here: their senders may leave
 
-    // ---- down projection and residual (an odd last tile is multiplied with zeros beside it)
+    // ---- down projection and residual
     red = reinterpret_cast<float *>(smem + L.red_d);
     const uint32_t h_base = smem_addr(smem + L.hid) + ra * L.ldh * 2;
-    project([&](int s) { return h_base + 16u * s_tile[2 * s + hi]; }, sD, L.ldf, (ff8 + 1) / 2);
+    project([&](int s) { return h_base + 16u * s_tile[2 * s + hi]; }, sD, L.ldf, ff8);
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
         if (own_row[i] >= ROWS) continue;
@@ -355,7 +358,7 @@ small_layer_kernel(SmallLayerArgs g)
 #pragma unroll 1
         for (int map = 0; map < 3; ++map) {
             red = reinterpret_cast<float *>(smem + L.hid + (map & 1) * (kWarps * 16 * RLD * 4));      // (the other one may still be read)
-            project(x_at, sG + map * NC * L.ldk, L.ldk, D / 16);
+            project(x_at, sG + map * NC * L.ldk, L.ldk, D / 8);
 #pragma unroll
             for (int i = 0; i < OWN; ++i) {
                 if (own_row[i] >= rows) continue;

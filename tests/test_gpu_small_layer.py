@@ -14,10 +14,10 @@ DEV = "cuda:0"
 
 
 # tokens below, at and above a tile of 16 and of 32 rows; one tile of features per CTA or none for some (d_ff 8, 24), an odd number of them
-# (24, 344, 1032), an even one; both widths; several sequences with ragged last tiles; row tiles of 32 (2 x 224, 7 x 40)
+# (24, 56, 344, 1032), an even one; both widths; several sequences with ragged last tiles; row tiles of 32 (2 x 224, 7 x 40, 240)
 @pytest.mark.parametrize("d,ff,B,S", [(256, 688, 1, 8), (256, 688, 1, 40), (256, 688, 3, 24), (256, 8, 1, 16), (256, 24, 2, 72), (256, 344, 1, 200),
                                       (128, 352, 1, 24), (128, 1032, 2, 40), (128, 64, 1, 136), (256, 688, 2, 224), (128, 1032, 7, 40),
-                                      (256, 344, 1, 408)])
+                                      (256, 344, 1, 408), (128, 24, 7, 40), (128, 56, 1, 240)])
 def test_logits_match_the_oracle(d, ff, B, S):
     dct = W.TINY.asdict()
     dct.update(n_layers=3, d_model=d, d_ff=ff, n_heads=d // 64, vocab=512, mask_id=511, logit_scale=1.0)
@@ -42,6 +42,55 @@ def test_logits_match_the_oracle(d, ff, B, S):
         emu = np.concatenate([forward_bf16_points(F.ModelConfig(**shape.asdict()), w, tok[b].numpy(), range(S)) for b in range(B)]) - ref
         assert np.linalg.norm(err) <= 1.25 * np.linalg.norm(emu)
         assert np.linalg.norm(err, axis=1).max() <= 1.6 * np.linalg.norm(emu, axis=1).max()
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
+
+
+def leave_nan_in_shared_memory():
+    """A forward pass whose weights are NaN throughout: what its kernels leave in shared memory is NaN almost everywhere."""
+    dct = W.TINY.asdict()
+    dct.update(n_layers=2, d_model=128, d_ff=1024, n_heads=2, vocab=4096, mask_id=4095, logit_scale=1.0)
+    shape = W.Shape(**dct)
+    w = W.model_weights(shape, seed=0)
+    for t in [v for k, v in w.items() if k != "layers"] + [v for lw in w["layers"] for v in lw.values()]:
+        t.fill_(float("nan"))
+    wd = {k: (v.to(DEV) if k != "layers" else [{kk: vv.to(DEV) for kk, vv in lw.items()} for lw in v]) for k, v in w.items()}
+    model = sfs.Model(shape, wd)
+    session = sfs.sfs_session_create(model, 1, 448)
+    try:
+        logits = torch.zeros((448, shape.vocab), dtype=torch.float32, device=DEV)
+        sfs.sfs_forward(session, W.prompt_ids(1, 448, 4094, seed=0).to(DEV), 1, 448, None, None, 448, logits, sfs.LOGITS_F32)
+        sfs.sfs_check_device_status()
+        assert torch.isnan(logits).all()
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
+
+
+# fewer tiles of features than CTAs: the first CTA has none, and the half k-step beside an odd last tile has no features to read.  Row tiles of
+# 32 (15 and more tiles of 16), whose row 16 would then read the padding between two weight rows, which nobody writes
+@pytest.mark.parametrize("ff", [8, 24, 40, 56])
+@pytest.mark.parametrize("B,S", [(1, 240), (7, 40)])
+def test_what_other_kernels_left_in_shared_memory_is_not_read(ff, B, S):
+    dct = W.TINY.asdict()
+    dct.update(n_layers=3, d_model=128, d_ff=ff, n_heads=2, vocab=512, mask_id=511, logit_scale=1.0)
+    shape = W.Shape(**dct)
+    w = W.model_weights(shape, seed=ff, std=0.08, gain_std=0.2)
+    wd = {k: (v.to(DEV) if k != "layers" else [{kk: vv.to(DEV) for kk, vv in lw.items()} for lw in v]) for k, v in w.items()}
+    model = sfs.Model(shape, wd)
+    tok = W.prompt_ids(B, S, 510, seed=S).to(DEV)
+    session = sfs.sfs_session_create(model, B, S)
+    try:
+        first = None
+        for _ in range(4):
+            leave_nan_in_shared_memory()
+            got = torch.zeros((B * S, shape.vocab), dtype=torch.float32, device=DEV)
+            sfs.sfs_forward(session, tok, B, S, None, None, B * S, got, sfs.LOGITS_F32)
+            sfs.sfs_check_device_status()
+            assert torch.isfinite(got).all(), torch.unique((~torch.isfinite(got)).any(dim=1).nonzero()[:, 0] % S).tolist()
+            first = got if first is None else first
+            assert torch.equal(got, first)
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
