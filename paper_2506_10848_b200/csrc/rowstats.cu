@@ -9,16 +9,12 @@
 // in flight, seven CTAs per SM).
 #include "sfs_common.cuh"
 #include "canonical.cuh"
+#include "tc05.cuh"
 
 #include <math_constants.h>
 
 namespace sfs {
 namespace {
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ int cluster_size() { int r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ int cluster_rank() { int r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
-__device__ __forceinline__ uint32_t in_cta(uint32_t addr, int rank) { uint32_t r; asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank)); return r; }
 
 // ---- what the CTAs of a row's cluster tell each other -------------------------------------------------------------
 // Every CTA its slice maximum to every CTA, then its sum and its candidate for the argmax to rank 0.  Each value is a remote store
@@ -33,33 +29,26 @@ struct Exchange {
 };
 __device__ __forceinline__ void exchange_init(Exchange &x, int C)      // one thread; then the cluster's start barrier
 {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n\tmbarrier.init.shared::cta.b64 [%1], 1;" ::"r"(smem_addr(&x.bar_max)), "r"(smem_addr(&x.bar_part)) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&x.bar_max)), "r"(4 * C) : "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(&x.bar_part)), "r"(16 * C) : "memory");
-}
-__device__ __forceinline__ void exchange_await(unsigned long long &bar, int32_t *err)      // bounded: the row's result is meaningless on expiry
-{
-    uint32_t ok = 0;
-    for (int i = 0; i < (1 << 20) && !ok; ++i)
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(smem_addr(&bar)) : "memory");
-    if (!ok && err) atomicExch(err, SFS_ERR_TIMEOUT);       // a peer never reported
+    const uint32_t bar_max = tc::smem_u32(&x.bar_max), bar_part = tc::smem_u32(&x.bar_part);
+    tc::mbar_init(bar_max, 1); tc::mbar_init(bar_part, 1);
+    tc::mbar_init_fence();
+    tc::mbar_expect_tx(bar_max, 4 * C); tc::mbar_expect_tx(bar_part, 16 * C);
 }
 __device__ __forceinline__ void send_max(Exchange &x, int rank, int to, float v)
 {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                 ::"r"(in_cta(smem_addr(&x.max_of[rank]), to)), "r"(__float_as_uint(v)), "r"(in_cta(smem_addr(&x.bar_max), to)) : "memory");
+                 ::"r"(tc::mapa(tc::smem_u32(&x.max_of[rank]), to)), "r"(__float_as_uint(v)), "r"(tc::mapa(tc::smem_u32(&x.bar_max), to)) : "memory");
 }
 __device__ __forceinline__ void send_part(Exchange &x, int rank, unsigned long long sum, int arg)
 {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(in_cta(smem_addr(&x.part_of[rank]), 0)), "r"((uint32_t)sum), "r"((uint32_t)(sum >> 32)), "r"(arg), "r"(0), "r"(in_cta(smem_addr(&x.bar_part), 0)) : "memory");
+                 ::"r"(tc::mapa(tc::smem_u32(&x.part_of[rank]), 0)), "r"((uint32_t)sum), "r"((uint32_t)(sum >> 32)), "r"(arg), "r"(0), "r"(tc::mapa(tc::smem_u32(&x.bar_part), 0)) : "memory");
 }
 // the whole row's maximum: `mine` is this CTA's, the same in threads 0 .. C - 1 (called by all threads, after the start barrier)
 __device__ __forceinline__ float exchange_max(Exchange &x, int C, int rank, float mine, int32_t *err)
 {
     if ((int)threadIdx.x < C) send_max(x, rank, threadIdx.x, mine);
-    exchange_await(x.bar_max, err);
+    tc::mbar_await(tc::smem_u32(&x.bar_max), err);
     float m = x.max_of[0];
     for (int r = 1; r < C; ++r) m = fmaxf(m, x.max_of[r]);
     return m;
@@ -69,7 +58,7 @@ __device__ __forceinline__ bool exchange_parts(Exchange &x, int C, int rank, uns
 {
     send_part(x, rank, sum, arg);
     if (rank != 0) return false;
-    exchange_await(x.bar_part, err);
+    tc::mbar_await(tc::smem_u32(&x.bar_part), err);
     sum = 0; arg = 0x7FFFFFFF;
     for (int r = 0; r < C; ++r) { const uint4 p = x.part_of[r]; sum += (unsigned long long)p.y << 32 | p.x; arg = min(arg, (int)p.z); }
     return true;
@@ -204,7 +193,7 @@ template <typename T, int NV, int NT>
 __global__ void __launch_bounds__(NT, NT < 256 ? 16 : (NV > 8 ? 2 : 4))
 rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
 {
-    const int C = cluster_size(), rank = cluster_rank();
+    const int C = (int)tc::cluster_nctarank(), rank = (int)tc::cluster_ctarank();
     const int row  = blockIdx.x / C;
     pdl_wait();
     pdl_trigger();
@@ -234,9 +223,9 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
 #pragma unroll
         for (int j = 0; j < NV; ++j) if (c0 + j * stride >= rc.whole && c0 + j * stride < n) v[j] = rc.load_edge(c0 + j * stride);
     if (tid == 0) { s_cta_arg = 0x7FFFFFFF; if (C > 1) exchange_init(s_x, C); }
-    __syncwarp();
+    __syncwarp();                                           // (here and not only below: the compiler then has registers for all of v)
     // every CTA of the cluster announces that it runs (its shared memory exists) before anybody writes into a peer
-    if (C > 1) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    if (C > 1) tc::cluster_arrive();
 
     // ---- pass 1: exact maximum
     float lmax = -INFINITY;
@@ -257,7 +246,7 @@ rowstats_cluster(const T *__restrict__ logits, long long ld, int vocab, const in
 #pragma unroll
     for (int w = 1; w < NT / 32; ++w) m = fmaxf(m, s_wmax[w]);
     if (C > 1) {
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all peers run
+        tc::cluster_wait();                                 // all peers run
         m = exchange_max(s_x, C, rank, m, err);
     }
 
@@ -315,7 +304,7 @@ __global__ void __launch_bounds__(kStagedThreads)
 rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int nchunks, int per_cta, int vocab,
                      const int32_t *__restrict__ n_rows_ptr, int max_rows, RowOut out, int32_t *err)
 {
-    const int C = cluster_size(), rank = cluster_rank();
+    const int C = (int)tc::cluster_nctarank(), rank = (int)tc::cluster_ctarank();
     const int row  = blockIdx.x / C;
     pdl_wait();
     pdl_trigger();
@@ -332,31 +321,25 @@ rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int c0 = rank * per_cta;                          // first 16-byte chunk of this CTA's slice
     const int n = max(0, min(per_cta, nchunks - c0));
-    const uint32_t bar = smem_addr(&s_bar);
+    const uint32_t bar = tc::smem_u32(&s_bar);
     if (tid == 0) {
         s_cta_arg = 0x7FFFFFFF;
         exchange_init(s_x, C);
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        tc::mbar_init(bar, 1);
+        tc::mbar_init_fence();
         if (n > 0) {
             const uint32_t bytes = (uint32_t)n * 16u;
-            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+            tc::mbar_expect_tx(bar, bytes);
             asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                         ::"r"(smem_addr(s_slice)), "l"(logits + (long long)row * ld_chunks + c0), "r"(bytes), "r"(bar) : "memory");
+                         ::"r"(tc::smem_u32(s_slice)), "l"(logits + (long long)row * ld_chunks + c0), "r"(bytes), "r"(bar) : "memory");
         } else {
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+            tc::mbar_arrive(bar);
         }
     }
     __syncthreads();
     // every CTA of the cluster announces that it runs (its shared memory exists) before anybody writes into a peer
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    {   // bounded wait for the slice; on expiry the status word is set and the row's result is meaningless
-        uint32_t ok = 0;
-        for (int i = 0; i < (1 << 20) && !ok; ++i)
-            asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                         : "=r"(ok) : "r"(bar) : "memory");
-        if (!ok && err) atomicExch(err, SFS_ERR_TIMEOUT);
-    }
+    tc::cluster_arrive();
+    tc::mbar_await(bar, err);                               // the slice
 
     // ---- pass 1: exact maximum
     __nv_bfloat162 mx = as_bf162(kNegInf2);
@@ -368,7 +351,7 @@ rowstats_staged_bf16(const uint4 *__restrict__ logits, long long ld_chunks, int 
     float m = warp_max(lmax);
     if (lane == 0) s_wmax[warp] = m;
     __syncthreads();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all peers run
+    tc::cluster_wait();                                     // all peers run
     m = s_wmax[0];
 #pragma unroll
     for (int w = 1; w < kStagedThreads / 32; ++w) m = fmaxf(m, s_wmax[w]);

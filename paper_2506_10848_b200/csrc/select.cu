@@ -7,6 +7,7 @@
 // pass gets one deterministic row list without a host round trip.
 #include "sfs_common.cuh"
 #include "canonical.cuh"
+#include "tc05.cuh"
 
 namespace sfs {
 namespace {
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     const sfs_params &p = a.params;
     const bool two_pass = !CLUSTER && a.pos_lo != nullptr, vanilla = p.sampler != SFS_SAMPLER_SLOWFAST;
 
-    if (CLUSTER) asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");      // this CTA runs
+    if (CLUSTER) tc::cluster_arrive();      // this CTA runs
     pdl_wait();
     pdl_trigger();
     const int steps_before = tid == 0 && a.step_count ? *a.step_count : 0;      // (of the whole generation)
@@ -401,14 +402,12 @@ __global__ void __launch_bounds__(kSelThreads) select_kernel(SelectArgs a)
     if (tid < (int)(sizeof(sfs_state) / 4)) reinterpret_cast<int *>(a.state + b)[tid] = reinterpret_cast<const int *>(&st)[tid];
     if (CLUSTER) {
         // every sequence its numbers to all, then its rows to their place (sequence-major)
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");      // all run
+        tc::cluster_wait();                                 // all run
         if (tid < a.B) {
-            uint32_t at;
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(&s_seq[b])), "r"(tid));
+            const uint32_t at = tc::mapa(tc::smem_u32(&s_seq[b]), (uint32_t)tid);
             asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(at), "r"(seq.x), "r"(seq.y) : "memory");
         }
-        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+        tc::cluster_sync();
         const int2 o = lane < a.B ? s_seq[lane] : make_int2(0, 0);
         const int c = o.x & ~kGoesOn, off = warp_sum_i32(lane < b ? c : 0), all = warp_sum_i32(c), act = warp_sum_i32(o.y);
         const bool on = __any_sync(0xffffffffu, (o.x & kGoesOn) != 0);

@@ -24,7 +24,7 @@ using namespace small;
 constexpr int TILE = 32, kThreads = 256, kWarps = kThreads / 32;
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -163,8 +163,8 @@ small_gemm_kernel(SmallGemmArgs g)
     __syncthreads();
 
     // ---- 16 rows x (8 + 8) columns and half of k per warp; even and odd k-steps accumulate apart, which halves the chain again
-    const uint32_t a_addr = smem_addr(sA + (wm * 16 + (lane & 15)) * ld + (lane >> 4) * 8);
-    const uint32_t b_addr = smem_addr(sB + ((lane >> 4) * 16 + wn * 8 + (lane & 7)) * ld + ((lane >> 3) & 1) * 8);
+    const uint32_t a_addr = smem_u32(sA + (wm * 16 + (lane & 15)) * ld + (lane >> 4) * 8);
+    const uint32_t b_addr = smem_u32(sB + ((lane >> 4) * 16 + wn * 8 + (lane & 7)) * ld + ((lane >> 3) & 1) * 8);
     float acc[2][2][4] = {};
     const int steps = Kp / 16, mid = (steps + 1) / 2, end = wk ? steps : mid;
     int k = wk ? mid : 0;

@@ -65,19 +65,8 @@ struct Layout {
     }
 };
 
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }      // (orders no memory)
 __device__ __forceinline__ void load_row(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-__device__ __forceinline__ void expect_bytes(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
 // This CTA's `bytes` at `at` into the same place of its peers (called by all threads; what the CTA has written there is visible to the copy)
 __device__ __forceinline__ void send(uint32_t at, uint32_t bytes, uint32_t bar, int rank, int tid) {
@@ -86,16 +75,11 @@ __device__ __forceinline__ void send(uint32_t at, uint32_t bytes, uint32_t bar, 
     if (tid < CL - 1) {
         const int p = (rank + 1 + tid) % CL;
         asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(peer_addr(at, p)), "r"(at), "r"(bytes), "r"(peer_addr(bar, p)) : "memory");
+                     ::"r"(tc::mapa(at, p)), "r"(at), "r"(bytes), "r"(tc::mapa(bar, p)) : "memory");
     }
 }
-// bounded: on expiry the status word is set and the step's result is meaningless
-__device__ __forceinline__ void await(uint32_t bar, int32_t *err) {
-    uint32_t ok = 0;
-    for (int i = 0; i < (1 << 20) && !ok; ++i)
-        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(ok) : "r"(bar) : "memory");
-    if (!ok && err) atomicExch(err, SFS_ERR_TIMEOUT);
-}
+// (the lanes together again: ldmatrix and mma.sync follow)
+__device__ __forceinline__ void await(uint32_t bar, int32_t *err) { tc::mbar_await(bar, err); __syncwarp(); }
 
 enum { BAR_WO = 0, BAR_GU = 1, BAR_WD = 2, BAR_ATTN = 3, BAR_SUMS = 4, BAR_X = 5, BAR_HID = 6, BAR_QKV = 7, BAR_SUMS2 = 8, BAR_X2 = 9, N_BARS = 10 };
 
@@ -116,32 +100,32 @@ small_layer_kernel(SmallLayerArgs g)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = blockIdx.x % CL, tile = blockIdx.x / CL;
     const int per_seq = (g.S + ROWS - 1) / ROWS, b = tile / per_seq, row0 = (tile - b * per_seq) * ROWS, rows = min(ROWS, g.S - row0);
     const int ff8 = g.ff / 8, t0 = rank * ff8 / CL, nt = (rank + 1) * ff8 / CL - t0, tiles = (ff8 + CL - 1) / CL;      // 8-feature tiles: this CTA's, at most
-    const uint32_t bar = smem_addr(s_bar);
+    const uint32_t bar = smem_u32(s_bar);
     // attention: unit u = (head, tile of 16 rows) is CTA u % CL's
     const int units = g.n_heads * RT, my_units = units > rank ? (units - rank + CL - 1) / CL : 0;
     constexpr uint32_t kUnitBytes = 16 * kHeadLd * 2;
 
     if (tid == 0) {
-        for (int i = 0; i < N_BARS; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8 * i) : "memory");
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        expect_bytes(bar + 8 * BAR_WO, NC * D * 2); expect_bytes(bar + 8 * BAR_GU, 2 * nt * 8 * D * 2); expect_bytes(bar + 8 * BAR_WD, NC * g.ff * 2);
-        expect_bytes(bar + 8 * BAR_ATTN, (units - my_units) * kUnitBytes);
-        expect_bytes(bar + 8 * BAR_SUMS, (CL - 1) * ROWS * 4);
-        expect_bytes(bar + 8 * BAR_X, (CL - 1) * L.x_block); expect_bytes(bar + 8 * BAR_HID, (CL - 1) * L.h_block);
-        expect_bytes(bar + 8 * BAR_QKV, 3 * NC * D * 2);
-        expect_bytes(bar + 8 * BAR_SUMS2, (CL - 1) * ROWS * 4); expect_bytes(bar + 8 * BAR_X2, (CL - 1) * L.x_block);
+        for (int i = 0; i < N_BARS; ++i) tc::mbar_init(bar + 8 * i, 1);
+        tc::mbar_init_fence();
+        tc::mbar_expect_tx(bar + 8 * BAR_WO, NC * D * 2); tc::mbar_expect_tx(bar + 8 * BAR_GU, 2 * nt * 8 * D * 2); tc::mbar_expect_tx(bar + 8 * BAR_WD, NC * g.ff * 2);
+        tc::mbar_expect_tx(bar + 8 * BAR_ATTN, (units - my_units) * kUnitBytes);
+        tc::mbar_expect_tx(bar + 8 * BAR_SUMS, (CL - 1) * ROWS * 4);
+        tc::mbar_expect_tx(bar + 8 * BAR_X, (CL - 1) * L.x_block); tc::mbar_expect_tx(bar + 8 * BAR_HID, (CL - 1) * L.h_block);
+        tc::mbar_expect_tx(bar + 8 * BAR_QKV, 3 * NC * D * 2);
+        tc::mbar_expect_tx(bar + 8 * BAR_SUMS2, (CL - 1) * ROWS * 4); tc::mbar_expect_tx(bar + 8 * BAR_X2, (CL - 1) * L.x_block);
     }
     __syncthreads();
-    cluster_arrive();                                       // this CTA runs: its shared memory may be written by its peers
+    tc::cluster_arrive();                                   // this CTA runs: its shared memory may be written by its peers
     // ---- weights: constant, so before the wait (rows of this CTA's columns, in the order they are needed)
     for (int r = tid; r < 2 * NC + 2 * nt * 8; r += kThreads) {
-        if (r < NC) load_row(smem_addr(sO + r * L.ldk), g.wo + (long long)(rank * NC + r) * D, D * 2, bar + 8 * BAR_WO);
+        if (r < NC) load_row(smem_u32(sO + r * L.ldk), g.wo + (long long)(rank * NC + r) * D, D * 2, bar + 8 * BAR_WO);
         else if (r < NC + 2 * nt * 8) {
             const int q = r - NC, up = q >= nt * 8 ? 1 : 0, f = q - up * nt * 8;
-            load_row(smem_addr(sG + (up * 8 * tiles + f) * L.ldk), (up ? g.w_up : g.w_gate) + (long long)(t0 * 8 + f) * D, D * 2, bar + 8 * BAR_GU);
+            load_row(smem_u32(sG + (up * 8 * tiles + f) * L.ldk), (up ? g.w_up : g.w_gate) + (long long)(t0 * 8 + f) * D, D * 2, bar + 8 * BAR_GU);
         } else {
             const int q = r - NC - 2 * nt * 8;
-            load_row(smem_addr(sD + q * L.ldf), g.w_down + (long long)(rank * NC + q) * g.ff, (uint32_t)g.ff * 2, bar + 8 * BAR_WD);
+            load_row(smem_u32(sD + q * L.ldf), g.w_down + (long long)(rank * NC + q) * g.ff, (uint32_t)g.ff * 2, bar + 8 * BAR_WD);
         }
     }
     // where the down projection finds a tile of features: CTA q's begin at tile q ff8 / CL
@@ -191,10 +175,10 @@ small_layer_kernel(SmallLayerArgs g)
         __nv_bfloat16 *dst = sAt + (head * ROWS + r0) * kHeadLd;
         attn_merge<kWarps>(sP, sP + kWarps * 16 * kPartLd, min(kWarps, (g.S + 31) / 32), g.scale_log2, warp, lane,
                            [&](int r, int col, uint2 v) { *reinterpret_cast<uint2 *>(dst + r * kHeadLd + col) = v; });
-        if (u == rank) cluster_wait();                      // (the peers run)
-        send(smem_addr(dst), kUnitBytes, bar + 8 * BAR_ATTN, rank, tid);
+        if (u == rank) tc::cluster_wait();                  // (the peers run)
+        send(smem_u32(dst), kUnitBytes, bar + 8 * BAR_ATTN, rank, tid);
     }
-    if (my_units == 0 || !active) cluster_wait();
+    if (my_units == 0 || !active) tc::cluster_wait();
     if (!active) {
         // nothing left to decode: the copies requested above are awaited, nobody reads them
         for (int i = BAR_WO; i <= BAR_WD; ++i) await(bar + 8 * i, g.err);
@@ -210,7 +194,7 @@ small_layer_kernel(SmallLayerArgs g)
     auto project = [&](auto &&a_at, const __nv_bfloat16 *sb, int ldb, int halves) {
         const int steps = (halves + 1) / 2;
         float acc[NN][4] = {};
-        const uint32_t b_addr = smem_addr(sb + ((lane >> 4) * 8 + (lane & 7)) * ldb + ((lane >> 3) & 1) * 8);
+        const uint32_t b_addr = smem_u32(sb + ((lane >> 4) * 8 + (lane & 7)) * ldb + ((lane >> 3) & 1) * 8);
         const int s1 = (kp + 1) * steps / KP;
 #pragma unroll 4
         for (int s = kp * steps / KP; s < s1; ++s) {
@@ -245,7 +229,7 @@ small_layer_kernel(SmallLayerArgs g)
     };
 
     // ---- output projection and residual, the norm's sums
-    const uint32_t at_base = smem_addr(sAt + ra * kHeadLd) + 16 * hi;
+    const uint32_t at_base = smem_u32(sAt + ra * kHeadLd) + 16 * hi;
     project([&](int s) { return at_base + (uint32_t)((s >> 2) * ROWS * kHeadLd * 2) + (s & 3) * 32; }, sO, L.ldk, D / 8);
     float *sums = reinterpret_cast<float *>(smem + L.sums);
     constexpr int CPR = NC / 8;                             // chunks of a message row; rows that share 128 bytes take other chunks
@@ -260,7 +244,7 @@ small_layer_kernel(SmallLayerArgs g)
             for (int o = Q / 2; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
             if (own_col[i] == 0) sums[rank * ROWS + own_row[i]] = ss;
         }
-        send(smem_addr(sums + rank * ROWS), ROWS * 4, bar + 8 * bar_sums, rank, tid);
+        send(smem_u32(sums + rank * ROWS), ROWS * 4, bar + 8 * bar_sums, rank, tid);
         await(bar + 8 * bar_sums, g.err);
         uint8_t *mine = smem + L.xs + rank * L.x_block;
 #pragma unroll
@@ -274,7 +258,7 @@ small_layer_kernel(SmallLayerArgs g)
                 make_uint2(pack2(xr[i].x * inv * bf16_bits_to_f32(gn[i].x & 0xFFFFu), xr[i].y * inv * bf16_bits_to_f32(gn[i].x >> 16)),
                            pack2(xr[i].z * inv * bf16_bits_to_f32(gn[i].y & 0xFFFFu), xr[i].w * inv * bf16_bits_to_f32(gn[i].y >> 16)));
         }
-        send(smem_addr(mine), (uint32_t)L.x_block, bar + 8 * bar_x, rank, tid);
+        send(smem_u32(mine), (uint32_t)L.x_block, bar + 8 * bar_x, rank, tid);
     };
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
@@ -288,12 +272,12 @@ small_layer_kernel(SmallLayerArgs g)
     await(bar + 8 * BAR_X, g.err);
     pdl_trigger();                                          // (the next launch has its own weights to request)
 
-    const uint32_t x_base = smem_addr(smem + L.xs);
+    const uint32_t x_base = smem_u32(smem + L.xs);
     constexpr int SPB = NC / 16;                            // k-steps of a message
     // ---- gate and up: the warps take the 8-feature tiles in turn, two at a time
     __nv_bfloat16 *own_h = reinterpret_cast<__nv_bfloat16 *>(smem + L.hid + rank * L.h_block);
     {
-        const uint32_t b_addr = smem_addr(sG + ((lane >> 4) * 8 * tiles + (lane & 7)) * L.ldk + ((lane >> 3) & 1) * 8);      // lanes 0-15: gate, 16-31: up
+        const uint32_t b_addr = smem_u32(sG + ((lane >> 4) * 8 * tiles + (lane & 7)) * L.ldk + ((lane >> 3) & 1) * 8);      // lanes 0-15: gate, 16-31: up
         auto features = [&](auto many, int tb) {
             constexpr int T = decltype(many)::value;
             float ag[T][RT][4] = {}, au[T][RT][4] = {};
@@ -323,20 +307,20 @@ small_layer_kernel(SmallLayerArgs g)
         for (; tb + kWarps < nt; tb += 2 * kWarps) features(std::integral_constant<int, 2>{}, tb);
         if (tb < nt) features(std::integral_constant<int, 1>{}, tb);
     }
-    send(smem_addr(own_h), (uint32_t)L.h_block, bar + 8 * BAR_HID, rank, tid);
+    send(smem_u32(own_h), (uint32_t)L.h_block, bar + 8 * BAR_HID, rank, tid);
     if (next)                                               // (gate's and up's rows have been read)
         for (int r = tid; r < 3 * NC; r += kThreads) {
             const int map = r / NC, q = r - map * NC;       // q and k: first halves of the CTA's pairs, then second halves
             const int row = map == 2 ? rank * NC + q : pair_head * kHead + pair_j + (q < HALF ? q : q - HALF + kHead / 2);
-            load_row(smem_addr(sG + r * L.ldk), (map == 0 ? g.w_q : (map == 1 ? g.w_k : g.w_v)) + (long long)row * D, D * 2, bar + 8 * BAR_QKV);
+            load_row(smem_u32(sG + r * L.ldk), (map == 0 ? g.w_q : (map == 1 ? g.w_k : g.w_v)) + (long long)row * D, D * 2, bar + 8 * BAR_QKV);
         }
     await(bar + 8 * BAR_WD, g.err);
     await(bar + 8 * BAR_HID, g.err);
-    if (!next) cluster_arrive_relaxed();                    // all messages have been received here: their senders may leave
+    if (!next) tc::cluster_arrive_relaxed();                // all messages have been received here: their senders may leave
 
     // ---- down projection and residual
     red = reinterpret_cast<float *>(smem + L.red_d);
-    const uint32_t h_base = smem_addr(smem + L.hid) + ra * L.ldh * 2;
+    const uint32_t h_base = smem_u32(smem + L.hid) + ra * L.ldh * 2;
     project([&](int s) { return h_base + 16u * s_tile[2 * s + hi]; }, sD, L.ldf, ff8);
 #pragma unroll
     for (int i = 0; i < OWN; ++i) {
@@ -353,7 +337,7 @@ small_layer_kernel(SmallLayerArgs g)
         send_normalised(next_gain, BAR_SUMS2, BAR_X2);
         await(bar + 8 * BAR_QKV, g.err);
         await(bar + 8 * BAR_X2, g.err);
-        cluster_arrive_relaxed();                           // (as above)
+        tc::cluster_arrive_relaxed();                       // (as above)
         auto x_at = [&](int s) { return x_base + (uint32_t)((s / SPB) * L.x_block + chunk_at(ra, (s % SPB) * 2 + hi)); };
 #pragma unroll 1
         for (int map = 0; map < 3; ++map) {
@@ -390,7 +374,7 @@ small_layer_kernel(SmallLayerArgs g)
             }
         }
     }
-    cluster_wait();
+    tc::cluster_wait();
 }
 
 constexpr int kSharedMost = 226 * 1024;                      // a CTA's most, minus the static arrays

@@ -2,11 +2,12 @@
 #pragma once
 #include "sfs_common.cuh"
 #include "attention.cuh"
+#include "tc05.cuh"
 
 namespace sfs {
 namespace small {
 
-__device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+using tc::smem_u32;
 __device__ __forceinline__ void ldmatrix4(uint32_t *r, uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
 }

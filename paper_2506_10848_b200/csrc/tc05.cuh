@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "../../include/sfs.h"
+
 namespace sfs {
 namespace tc {
 
@@ -45,6 +47,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
     *abort_flag = 1;
     return false;
+}
+// Bounded wait for the first phase, by kernels that go on when it gives up: the status word says that the result is meaningless.  Every
+// lane polls and leaves the loop for itself.
+constexpr uint32_t kAwaitPolls = 1u << 20;
+__device__ __forceinline__ void mbar_await(uint32_t bar, int32_t *err) {
+    bool ok = false;
+    for (uint32_t i = 0; i < kAwaitPolls && !ok; ++i) ok = mbar_try(bar, 0);
+    if (!ok && err) atomicExch(err, SFS_ERR_TIMEOUT);
 }
 
 // ---- TMA -------------------------------------------------------------------------------------------
@@ -131,21 +141,25 @@ __device__ __forceinline__ void mma_commit_elect(uint32_t bar) {
                  "@P tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
 
-// ---- CTA pairs (cluster of two, tcgen05 cta_group::2) --------------------------------------------------
-__device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+// ---- clusters ------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_ctarank() { uint32_t r; asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r)); return r; }
+__device__ __forceinline__ uint32_t cluster_nctarank() { uint32_t r; asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r)); return r; }
 // shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t mapa(uint32_t smem_addr, uint32_t rank) {
     uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// the same without ordering memory: nothing is handed over through it
-__device__ __forceinline__ void cluster_sync_relaxed() {
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
-}
+// The cluster's barrier.  The aligned form is one instruction of a whole warp, so the lanes are gathered before it: a polling loop, or rows
+// that some lanes skip, may have left them apart.
+__device__ __forceinline__ void cluster_arrive() { __syncwarp(); asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { __syncwarp(); asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync() { cluster_arrive(); cluster_wait(); }
+// without ordering memory: nothing is handed over through it
+__device__ __forceinline__ void cluster_arrive_relaxed() { __syncwarp(); asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_relaxed() { cluster_arrive_relaxed(); asm volatile("barrier.cluster.wait.aligned;" ::: "memory"); }
+
+// ---- CTA pairs (cluster of two, tcgen05 cta_group::2) --------------------------------------------------
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {     // the barrier may live in the peer CTA
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
 }
