@@ -45,7 +45,6 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     constexpr int V_BYTES = DH * KT * 2;
     constexpr uint32_t TMEM_COLS = 512;                  // S / P and O of each stream: 2 x (128 + DH) columns
 
-    pdl_trigger();                                       // (may run beside the end of the kernel before it: see pdl_wait below)
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sQ = smem, *sK = smem + NQ * Q_BYTES, *sV = sK + KV_STAGES * K_BYTES;
@@ -88,6 +87,7 @@ attention_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant_
     const uint32_t tmem_S = tmem_base, tmem_O = tmem_base + 2 * KT;      // stream w: + w * KT, + w * DH
 
     pdl_wait();                                          // the kernel before this one has completed: global memory from here on
+    pdl_trigger();                                       // (not before the wait: see pdl_trigger)
     const bool live = !(a.d_active && *a.d_active == 0); // nothing left to decode: straight to the teardown (uniform)
     if (live) {
     if (warp == 0) {

@@ -57,8 +57,10 @@ int32_t *device_status_word_if_any();
 // when about one launch latency of their own work is left: after their wait if they are short, before the last epilogue if they
 // are GEMMs.  Called first thing, a whole row of kernels becomes resident, and each reaches its wait so long before its input is
 // there that the code behind the wait has left the instruction cache by then (small projection after attention, 192 tokens: 4.9
-// us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).  The two-stream attention
-// alone calls it first thing: its CTAs leave the projection that follows no room on their SMs, so nothing becomes resident early.
+// us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).  Never before the wait: where a
+// QKV projection leaves SMs idle, all CTAs of an attention of few queries fit beside it, and if those release the output projection at
+// once its CTAs fill the rest, long before their input (us a layer of 128 rows, 16 / 20 / 28 / 32 heads of 128: 67.9 / 77.4 / 102.4 / 121.7,
+// released behind the wait 63.9 / 73.4 / 99.0 / 120.5).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
