@@ -106,6 +106,18 @@ def test_lockstep_long_responses(L):
     run_lockstep(B=1, P=8, L=L, V=64, pkw=dict(max_steps=3), seed=L)
 
 
+# without enclosures the sequences of a small batch are a cluster of as many CTAs (up to eight), more of them leave their lists to the last CTA
+@pytest.mark.parametrize("B", [5, 6, 7, 8, 9, 33])
+def test_lockstep_batches_around_a_cluster(B):
+    run_lockstep(B=B, P=5, L=40, V=64, pkw=dict(k_slow=2), seed=B)
+
+
+# a cluster whose CTAs take more shared memory than a launch has unasked
+@pytest.mark.parametrize("B", [3, 8])
+def test_lockstep_cluster_of_long_responses(B):
+    run_lockstep(B=B, P=8, L=5000, V=64, pkw=dict(max_steps=3), seed=B)
+
+
 @pytest.mark.parametrize("seed,pkw", [
     (10, dict(k_max=3, w_hist=3, sigma2_stable=30.0, k_slow=2, k_fast=3)),
     (11, dict(k_max=1, w_hist=1, k_slow=4, min_high_count=3)),

@@ -94,3 +94,32 @@ def test_what_other_kernels_left_in_shared_memory_is_not_read(ff, B, S):
     finally:
         sfs.sfs_session_destroy(session)
         model.close()
+
+
+# two heads: attention units for two, four, and (a single sequence of 440 tokens, 32-row tiles) four of a cluster's eight CTAs
+@pytest.mark.parametrize("B,P,L", [(1, 40, 32), (3, 88, 32), (1, 392, 48)])
+def test_steps_after_the_last_sequence_is_done_change_nothing(B, P, L):
+    """All steps enqueued at once: those after the end find no active sequence and leave the kernel early, and the next generation is as
+    the first."""
+    dct = W.TINY.asdict()
+    dct.update(n_layers=3, d_model=128, d_ff=352, n_heads=2, vocab=512, mask_id=511, logit_scale=60.0)
+    shape = W.Shape(**dct)
+    model = sfs.Model(shape, W.model_weights(shape, seed=3, std=0.08, gain_std=0.2, device=DEV))
+    session = sfs.sfs_session_create(model, B, P + L)
+    prompt = W.prompt_ids(B, P, 510, seed=L).to(DEV)
+    try:
+        want = torch.zeros((B, P + L), dtype=torch.int32, device=DEV)
+        state = torch.zeros((B, sfs.STATE_INTS), dtype=torch.int32, device=DEV)
+        sfs.sfs_generate(session, prompt, B, P, L, sfs.Params.default(), want, state)
+        done_after = int(state[:, sfs.STATE_FIELDS.index("steps_done")].max())
+        assert done_after < L
+        for _ in range(3):
+            got, end = torch.zeros_like(want), torch.zeros_like(state)
+            sfs.sfs_generate_begin(session, prompt, B, P, L, sfs.Params.default())
+            sfs.sfs_generate_steps(session, L)
+            sfs.sfs_generate_end(session, got, end)
+            sfs.sfs_check_device_status()
+            assert torch.equal(got, want) and torch.equal(end, state)
+    finally:
+        sfs.sfs_session_destroy(session)
+        model.close()
