@@ -966,7 +966,8 @@ void pick_tile_few(int M, int K, int mode, int n_maps, int n_per_map, int rope_d
             }
 }
 
-// Clocks of the rotary kernel that a rotating epilogue saves: 104 rows of 2 x 4096 4.0 us with its hand-over, 512 6.3, 1536 12, 2048 17.
+// Clocks of the rotary kernel that a rotating epilogue does without: 104 rows of 2 x 4096 4.0 us with its hand-over, 512 6.3, 1536 12, 2048 17
+// (of the 4.0, 2 are left when the epilogue has done the work: see gemm_rotates).
 long long rope_kernel_clocks(int M, int n_per_map) { return 6600 + (long long)((double)M * n_per_map * 3e-3); }
 
 int stages_for_few(int bn, int nb)
@@ -981,17 +982,26 @@ int stages_for_few(int bn, int nb)
 int gemm_num_sms() { return num_sms(); }
 
 // A rotating tile takes 16 pairs of each of bn / 32 heads.  Where tiles stream weights (128 rows) a last one of fewer heads costs nothing;
-// otherwise whole tiles only (512 rows of 32 heads: 192 columns, a tenth of them padding, 58 us where 176 plain ones take 52), and a
-// projection that is faster by more than the model's error than a plain one and the rotary kernel.
+// otherwise whole tiles only (512 rows of 32 heads: 192 columns, a tenth of them padding, 58 us where 176 plain ones take 52).  And only where
+// the projection is faster by more than the model's error than a plain one and the rotary kernel: beyond 48 heads of 128 it is not at up to
+// 128 rows, whose plain tiles then take two weight blocks each, in one wave instead of two.
+// us a layer in the chain (d_ff 3 d), with the rotary kernel / rotating; forward passes of 8, 64, 128 tokens, then 128 rows of a cached 1024 + 512 (where a
+// scatter of keys and values goes too): 8 heads of 128 42.9 / 42.1, 44.2 / 43.7, 46.7 / 45.3, 85.6 / 83.6; 16 59.8 / 60.0, 62.9 / 61.1, 65.7 / 63.9,
+// 112.7 / 109.2; 24 85.7 / 83.9, 83.7 / 81.1, 88.8 / 85.6, 145.1 / 140.1; 32 109.1 / 107.2, 113.6 / 111.4, 122.0 / 120.5, 180.7 / 175.9 (spreads 0.02 to 0.2, at 32
+// heads 1); 49 219.9 / 229.5, 230.7 / 237.5, 249.2 / 253.9, 329 / 334; 64 351 / 358, 371 / 379, 394 / 400, 499 / 505 (spreads 1 to 12).
+// 384 and 1536 rows: 8 heads 60.3 / 56.8 and 89.4 / 85.8, 16 92.8 / 91.0 and 196 / 191 (18), 32 heads of 64 91.0 / 90.2 and 209 / 204 (11).
 bool gemm_rotates(int32_t M, int32_t K, int32_t n_per_map, int32_t head_dim)
 {
-    if (M <= 2 * FM) return true;
+    const bool few = M <= 2 * FM;
     const int pairs = num_sms() / 2;
-    int mb = 1, bn = 256, sp = 1;
-    pick_tile(M, K, GEMM_STORE, 3, n_per_map, 0, pairs, 1, &mb, &bn, &sp);
-    const long long plain = model_clocks(M, K, GEMM_STORE, 3, n_per_map, 0, pairs, mb, bn, 1) + rope_kernel_clocks(M, n_per_map);
-    pick_tile(M, K, GEMM_STORE, 3, n_per_map, head_dim, pairs, 1, &mb, &bn, &sp);
-    return (n_per_map / head_dim) % (bn / 32) == 0 && model_clocks(M, K, GEMM_STORE, 3, n_per_map, head_dim, pairs, mb, bn, 1) * 100 < plain * 97;
+    int mb = 1, bn = 256, nb = 1, sp = 1;
+    auto clocks = [&](int rope_dim) {
+        if (few) pick_tile_few(M, K, GEMM_STORE, 3, n_per_map, rope_dim, pairs, 1, &bn, &nb, &sp);
+        else pick_tile(M, K, GEMM_STORE, 3, n_per_map, rope_dim, pairs, 1, &mb, &bn, &sp);
+        return few ? model_clocks_few(M, K, GEMM_STORE, 3, n_per_map, rope_dim, pairs, bn, nb, 1) : model_clocks(M, K, GEMM_STORE, 3, n_per_map, rope_dim, pairs, mb, bn, 1);
+    };
+    const long long plain = clocks(0) + rope_kernel_clocks(M, n_per_map), rotating = clocks(head_dim);
+    return (few || (n_per_map / head_dim) % (bn / 32) == 0) && rotating * 100 < plain * 97;
 }
 
 int32_t gemm_plan_create(GemmPlan *p, const void *A, int64_t lda, int32_t M, int32_t K,

@@ -130,3 +130,10 @@ def test_a_rotary_kernel_runs_where_the_projection_does_not_rotate(forms, heads,
 # at the 8B width 512 rows want tiles that whole heads do not fill
 def test_forms_at_the_8b_width(forms):
     assert [forms.qkv_rotates(M, 4096, 32, 128) for M in (128, 512, 1000, 1536, 2048, 6144)] == [1, 0, 1, 1, 1, 1]
+
+
+# up to 128 rows: beyond 48 heads of 128 one wave takes two weight blocks a tile, which only the plain form has
+def test_forms_of_few_rows(forms):
+    for M in (8, 64, 128):
+        assert [forms.qkv_rotates(M, 128 * heads, heads, 128) for heads in (6, 9, 16, 20, 32, 48, 49, 56, 64)] == [1, 1, 1, 1, 1, 1, 0, 0, 0]
+        assert [forms.qkv_rotates(M, 64 * heads, heads, 64) for heads in (10, 16, 32, 64)] == [1, 1, 1, 1]
