@@ -21,6 +21,8 @@
  *     0-based: i = pos - P.
  *   * bf16 matrices are row-major with the contraction dimension contiguous: a weight of a layer that
  *     maps in -> out is stored [out, in].
+ *   * The same call on the same inputs gives the same bits.  A sequence's logits may differ in their last bits with what runs
+ *     beside it: kernels, tiles and with them the order of sums are chosen by B, S and the number of rows.
  *   * Confidence comparisons are taken on the canonical fixed-point softmax denominator S_q (Q28, see
  *     sfs_row_stats), never on a floating-point probability, so results do not depend on reduction order.
  */
@@ -283,7 +285,10 @@ int32_t sfs_generate_end(sfs_session *session, int32_t *d_out_tokens, sfs_state 
 
 /* ---- instrumentation ------------------------------------------------------------------------------------ */
 
-/* Kernel classes of one denoising step, in launch order. */
+/* Kernel classes of one denoising step, in launch order.  A launch that does the work of several is counted once, under the class of its
+ * main product: QKV projections may rotate queries and keys (no ROPE launch then) or, in small models, start from the embedding
+ * or the norm; GATE_UP may be a small model's whole layer, from its attention to the next layer's queries, keys and values; LM_HEAD
+ * may include the final norm and the first pass of the row statistics; SELECT recomputes rows whose statistics were left open. */
 #define SFS_K_EMBED        0
 #define SFS_K_RMSNORM      1
 #define SFS_K_GEMM_QKV     2
