@@ -13,7 +13,7 @@
 //   norm        of the same columns                                                       -> bf16 [CTA][rows][d/8]
 //   q, k, v     rows x d/8 columns of each, weights where gate's and up's were; a thread has both halves of its rotary pairs
 // Bound: the chain of these exchanges: at 64 tokens, d 256, d_ff 688, 10600 clocks from the wait to the end, of which attention 3400, the
-// four messages 3400, products 3500; four launches took 12 us.  A 2-layer step 34.4 -> 26.0 us, one of 2 x 224 tokens 53.5 -> 38.9, and
+// four messages 3400, products 3500; four launches took 12 us.  A 2-layer step 33.3 -> 26.6 us, one of 2 x 224 tokens 53.5 -> 38.9, and
 // 36.9 with the next QKV projection in it.  Between SMs of a cluster 20 bytes a clock leave a CTA, whatever carries them: 2 KB to each of
 // seven peers are there after 970 clocks by bulk copies, 1400 by remote stores and a cluster barrier (417 of them the empty barrier),
 // 1650 through L2 and 1830 by remote loads.  So the sums of squares go ahead and the rows follow normalised, as 16 bits (fp32 rows and a
