@@ -137,7 +137,6 @@ small_layer_kernel(SmallLayerArgs g)
         while (c > 0 && q < c * ff8 / CL) --c;
         s_tile[i] = (uint16_t)((c * L.h_block >> 4) + q - c * ff8 / CL);
     }
-    if (g.ff & 15) for (int r = tid; r < NC; r += kThreads) *reinterpret_cast<uint4 *>(sD + r * L.ldf + g.ff) = make_uint4(0, 0, 0, 0);
     // the (row, four columns) of x this thread owns
     constexpr int OWN = (ROWS * Q + kThreads - 1) / kThreads;
     const long long tok0 = (long long)b * g.S + row0;
@@ -189,26 +188,26 @@ small_layer_kernel(SmallLayerArgs g)
 
     const int rt = warp % RT, kp = warp / RT, ra = rt * 16 + (lane & 15), hi = lane >> 4;      // ldmatrix of A: row, second half of a k-step
     float *red = reinterpret_cast<float *>(smem + L.red_o);
-    // rows x this CTA's columns: k-steps [kp, kp + 1) / KP of `halves` / 2, A's 16 bytes of (step, half, row) where a_at says.  The second half
-    // of a last step that has none is zeroed: a zero weight alone would make NaN of an infinity, and of anything that is not a feature
+    // rows x this CTA's columns: k-steps [kp, kp + 1) / KP of `halves` / 2, A's 16 bytes of (step, half, row) where a_at says.  A last step
+    // without a second half is an MMA of half its depth: there are no features to multiply, and what lies there may be NaN
     auto project = [&](auto &&a_at, const __nv_bfloat16 *sb, int ldb, int halves) {
-        const int steps = (halves + 1) / 2;
         float acc[NN][4] = {};
         const uint32_t b_addr = smem_u32(sb + ((lane >> 4) * 8 + (lane & 7)) * ldb + ((lane >> 3) & 1) * 8);
-        const int s1 = (kp + 1) * steps / KP;
-#pragma unroll 4
-        for (int s = kp * steps / KP; s < s1; ++s) {
+        const int steps = (halves + 1) / 2, odd = kp == KP - 1 ? halves & 1 : 0, s1 = (kp + 1) * steps / KP - odd;
+        auto step = [&](int s, auto whole) {
             uint32_t a[4];
             ldmatrix4(a, a_at(s));
-            if (2 * s + 1 == halves) a[2] = a[3] = 0;
 #pragma unroll
             for (int t = 0; t < NN; t += 2) {
                 uint32_t w[4];
                 ldmatrix4(w, b_addr + (uint32_t)(t * 8 * ldb * 2) + s * 32);
-                mma_16816(acc[t], a, w[0], w[1]);
-                mma_16816(acc[t + 1], a, w[2], w[3]);
+                if constexpr (decltype(whole)::value) { mma_16816(acc[t], a, w[0], w[1]); mma_16816(acc[t + 1], a, w[2], w[3]); }
+                else { mma_1688(acc[t], a, w[0]); mma_1688(acc[t + 1], a, w[2]); }
             }
-        }
+        };
+#pragma unroll 4
+        for (int s = kp * steps / KP; s < s1; ++s) step(s, std::true_type{});
+        if (odd) step(s1, std::false_type{});
         float *p = red + (kp * ROWS + rt * 16 + (lane >> 2)) * RLD + 2 * (lane & 3);
 #pragma unroll
         for (int t = 0; t < NN; ++t) {
@@ -415,7 +414,8 @@ int resident_clusters()
 }
 
 int tiles(int B, int S, int RT) { return B * ((S + 16 * RT - 1) / (16 * RT)); }
-// Tiles of 16 rows while their clusters are resident at once (a message is half as long, a product half as many MMAs), else of 32
+// Tiles of 16 rows while their clusters are resident at once (a message is half as long, a product half as many MMAs), else of 32 (whose
+// products divide k over four warps instead of eight: a sequence's last bits are not those it has in a smaller batch)
 int row_tiles(int B, int S) { return tiles(B, S, 1) <= resident_clusters() ? 1 : 2; }
 
 }  // namespace

@@ -73,6 +73,7 @@ def forms(tmp_path_factory):
 @pytest.mark.parametrize("M,heads,dh,S,T,listed,mb,bn", [
     (40, 10, 64, 40, 40, False, 0, 0), (120, 9, 128, 40, 120, False, 0, 0), (128, 6, 128, 64, 128, False, 0, 256), (8, 16, 128, 8, 8, False, 0, 64),
     (128, 32, 128, 1536, 1536, True, 0, 0), (52, 9, 128, 264, 264, True, 0, 192), (77, 10, 64, 120, 240, True, 0, 128), (1, 6, 128, 72, 72, True, 0, 0),
+    (40, 1, 128, 40, 40, False, 0, 0), (24, 1, 64, 48, 48, True, 0, 0), (16, 3, 64, 16, 16, False, 0, 128),
     (136, 8, 128, 136, 136, False, 1, 256), (528, 8, 128, 264, 528, False, 2, 256), (520, 16, 64, 520, 520, False, 2, 128), (1032, 32, 128, 344, 1032, False, 0, 0),
     (200, 8, 128, 512, 1024, True, 1, 64), (384, 8, 128, 768, 1536, True, 2, 128), (400, 9, 128, 200, 400, False, 1, 256)])
 def test_both_forms_give_the_same_bits(forms, M, heads, dh, S, T, listed, mb, bn):

@@ -112,10 +112,10 @@ def test_lockstep_batches_around_a_cluster(B):
     run_lockstep(B=B, P=5, L=40, V=64, pkw=dict(k_slow=2), seed=B)
 
 
-# a cluster whose CTAs take more shared memory than a launch has unasked
-@pytest.mark.parametrize("B", [3, 8])
-def test_lockstep_cluster_of_long_responses(B):
-    run_lockstep(B=B, P=8, L=5000, V=64, pkw=dict(max_steps=3), seed=B)
+# a cluster whose CTAs take more shared memory than a launch has unasked, and the most that a response may take
+@pytest.mark.parametrize("B,L", [(3, 5000), (8, 5000), (8, 22752)])
+def test_lockstep_cluster_of_long_responses(B, L):
+    run_lockstep(B=B, P=8, L=L, V=64, pkw=dict(max_steps=2 if L > 5000 else 3), seed=B)
 
 
 @pytest.mark.parametrize("seed,pkw", [
