@@ -106,6 +106,9 @@ struct TileCoord {
     int j0;          // rotated tiles: the first of the 16 pairs the tile takes of each head (n_local: its first head), else -1
 };
 
+// (ROPE: the kernels of projections that rotate.  Asked of the arguments, the question and its divisions cost the other projections 0.2 us each: a
+// layer of 10 heads of 64 at 8 rows, with a rotary kernel 36.4 us, without the question 35.7)
+template <bool ROPE>
 __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int m_groups)
 {
     TileCoord t;
@@ -115,7 +118,7 @@ __device__ __forceinline__ TileCoord tile_coord(const GemmArgs &g, int tile, int
     const int n_tile = g.splits == 1 ? rest : rest / g.splits;
     t.split = rest - n_tile * g.splits;
     t.j0 = -1;
-    if (g.rope.table != nullptr) {
+    if (ROPE) {
         // queries and keys: tiles of 16 pairs of tile_cols / 32 heads, the groups of a head's pairs fastest; then the values, plain
         if (n_tile < 2 * g.rope_tiles) {
             t.map_idx = n_tile >= g.rope_tiles ? 1 : 0;
@@ -157,7 +160,7 @@ __device__ __forceinline__ int early_weights(const GemmArgs &g, int pair, int st
 {
     const int num_kb = (g.K + BK - 1) / BK;
     if (g.splits == 1) return min(stages, num_kb);
-    const int kb0 = tile_coord(g, pair, (g.M + g.tile_rows - 1) / g.tile_rows).split * g.kb_per_split;
+    const int kb0 = tile_coord<false>(g, pair, (g.M + g.tile_rows - 1) / g.tile_rows).split * g.kb_per_split;
     return min(stages, min(num_kb, kb0 + g.kb_per_split) - kb0);
 }
 
@@ -511,7 +514,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // row count is below the planned one, is half as high (an LM head planned for 512 rows and given 256 took 370 us, 1.9x)
     auto blocks_of = [&](const TileCoord &t, int rows) { return MB == 2 && t.m0 + 2 * BM < rows ? 2 : 1; };
     if (warp == 0 && pre > 0) {
-        const TileCoord t = tile_coord(g, pair, (g.M + MB * 2 * BM - 1) / (MB * 2 * BM));
+        const TileCoord t = tile_coord<ROPE>(g, pair, (g.M + MB * 2 * BM - 1) / (MB * 2 * BM));
         const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1) : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
         const int brow = weight_row0<ROPE>(t, (int)rank, HALF, swiglu), j0 = max(t.j0, 0), kb0 = t.split * g.kb_per_split;
         for (int j = 0; j < pre; ++j) {
@@ -543,7 +546,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-            const TileCoord t = tile_coord(g, tile, m_groups);
+            const TileCoord t = tile_coord<ROPE>(g, tile, m_groups);
             // leader: first half of the weight rows (SwiGLU: the gate rows); peer: second half (the up rows)
             const CUtensorMap *mb = swiglu ? (rank == 0 ? &tmB0 : &tmB1)
                                            : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
@@ -567,7 +570,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
         if (!live && pre > 0) {
             // nothing left to decode: the stages requested above are completed and awaited, nobody reads them
-            const int mbt = blocks_of(tile_coord(g, pair, m_groups), g.M);
+            const int mbt = blocks_of(tile_coord<ROPE>(g, pair, m_groups), g.M);
             for (int j = 0; j < pre; ++j) {
                 const uint32_t sa = smem_base + j * STAGE_BYTES;
                 tc::tma_load_2d_2cta_elect(sa, &tmA, 0, 0, lead_full + 8 * j);
@@ -600,7 +603,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * buf_stride;
-                const TileCoord t = tile_coord(g, tile, m_groups);
+                const TileCoord t = tile_coord<ROPE>(g, tile, m_groups);
                 const bool second = blocks_of(t, M) == 2;
                 const int kb0 = t.split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
                 for (int kb = kb0; kb < kb1; ++kb) {
@@ -635,7 +638,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         uint32_t lt = 0;
         bool ok = true;
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {
-            const TileCoord t = tile_coord(g, tile, m_groups);
+            const TileCoord t = tile_coord<ROPE>(g, tile, m_groups);
             const uint32_t buf = lt % n_bufs, use = lt / n_bufs;
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
@@ -725,7 +728,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     // the first tile's weight rows are requested before the wait (see the pair kernel)
     const int pre = (g.b_static && g.d_m == nullptr) ? early_weights(g, pair, STAGES) : 0;
     if (warp == 0 && pre > 0) {
-        const TileCoord t = tile_coord(g, pair, (g.M + 2 * FM - 1) / (2 * FM));
+        const TileCoord t = tile_coord<ROPE>(g, pair, (g.M + 2 * FM - 1) / (2 * FM));
         const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
         const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
         const int brow0 = weight_row0<ROPE>(t, (int)rank, HALF, false), brow1 = swiglu ? brow0 : brow0 + BN, j0 = max(t.j0, 0), kb0 = t.split * g.kb_per_split;
@@ -748,7 +751,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         bool ok = true;
         bool ready = tc::mbar_test(bar_empty, 1u);
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs) {
-            const TileCoord t = tile_coord(g, tile, m_groups);
+            const TileCoord t = tile_coord<ROPE>(g, tile, m_groups);
             const CUtensorMap *m0 = swiglu ? &tmB0 : (t.map_idx == 0 ? &tmB0 : (t.map_idx == 1 ? &tmB1 : &tmB2));
             const CUtensorMap *m1 = swiglu ? &tmB1 : m0;
             const int brow0 = weight_row0<ROPE>(t, (int)rank, HALF, false), brow1 = swiglu ? brow0 : brow0 + BN, j0 = max(t.j0, 0);
@@ -800,7 +803,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
                 if (!ok) break;
                 tc::tc_fence_after();
                 const uint32_t d_tmem = tmem_base + buf * 256u;
-                const int kb0 = tile_coord(g, tile, m_groups).split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
+                const int kb0 = tile_coord<ROPE>(g, tile, m_groups).split * g.kb_per_split, kb1 = min(num_kb, kb0 + g.kb_per_split);
                 for (int kb = kb0; kb < kb1; ++kb) {
                     if (!ready) ready = tc::mbar_wait(bar_full + 8 * s, ph, &s_abort);
                     ok = __all_sync(0xffffffffu, ready);
@@ -833,7 +836,7 @@ gemm_few_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
         uint32_t lt = 0;
         bool ok = true;
         for (int tile = pair; tile < num_tiles && ok; tile += num_pairs, ++lt) {
-            const TileCoord t = tile_coord(g, tile, m_groups);
+            const TileCoord t = tile_coord<ROPE>(g, tile, m_groups);
             const uint32_t buf = lt & 1u, use = lt >> 1;
             ok = tc::mbar_wait(bar_acc_full + 8 * buf, use & 1u, &s_abort) && !s_abort;
             if (!ok) break;
@@ -986,10 +989,10 @@ int gemm_num_sms() { return num_sms(); }
 // the projection is faster by more than the model's error than a plain one and the rotary kernel: beyond 48 heads of 128 it is not at up to
 // 128 rows, whose plain tiles then take two weight blocks each, in one wave instead of two.
 // us a layer in the chain (d_ff 3 d), with the rotary kernel / rotating; forward passes of 8, 64, 128 tokens, then 128 rows of a cached 1024 + 512 (where a
-// scatter of keys and values goes too): 8 heads of 128 42.9 / 42.1, 44.2 / 43.7, 46.7 / 45.3, 85.6 / 83.6; 16 59.8 / 60.0, 62.9 / 61.1, 65.7 / 63.9,
-// 112.7 / 109.2; 24 85.7 / 83.9, 83.7 / 81.1, 88.8 / 85.6, 145.1 / 140.1; 32 109.1 / 107.2, 113.6 / 111.4, 122.0 / 120.5, 180.7 / 175.9 (spreads 0.02 to 0.2, at 32
-// heads 1); 49 219.9 / 229.5, 230.7 / 237.5, 249.2 / 253.9, 329 / 334; 64 351 / 358, 371 / 379, 394 / 400, 499 / 505 (spreads 1 to 12).
-// 384 and 1536 rows: 8 heads 60.3 / 56.8 and 89.4 / 85.8, 16 92.8 / 91.0 and 196 / 191 (18), 32 heads of 64 91.0 / 90.2 and 209 / 204 (11).
+// scatter of keys and values goes too): 8 heads of 128 44.2 / 43.3, 44.6 / 44.7, 47.6 / 46.3, 86.3 / 84.6; 16 59.8 / 59.8, 62.6 / 61.3, 65.8 / 64.1,
+// 111.8 / 108.9; 24 81.6 / 79.3, 84.0 / 82.3, 89.0 / 85.9, 143.9 / 139.4; 32 110.0 / 109.2, 114.1 / 112.0, 119.6 / 117.9, 180.2 / 175.5 (spreads 0.02 to 0.2, at 32
+// heads up to 1.6); 49 219.9 / 229.5, 230.7 / 237.5, 249.2 / 253.9, 329 / 334; 64 351 / 358, 371 / 379, 394 / 400, 499 / 505 (spreads 1 to 12).
+// 384 and 1536 rows: 8 heads 59.4 / 56.1 and 88.3 / 84.6, 16 92.1 / 89.8 and 192 / 187 (5).
 bool gemm_rotates(int32_t M, int32_t K, int32_t n_per_map, int32_t head_dim)
 {
     const bool few = M <= 2 * FM;

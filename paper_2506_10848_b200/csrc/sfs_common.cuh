@@ -59,8 +59,8 @@ int32_t *device_status_word_if_any();
 // there that the code behind the wait has left the instruction cache by then (small projection after attention, 192 tokens: 4.9
 // us from wait to end, 2.8 when released late; tiny step 55 -> 49 us, 8B forward at 104 rows 3990 -> 3946).  Never before the wait: where a
 // QKV projection leaves SMs idle, all CTAs of an attention of few queries fit beside it, and if those release the output projection at
-// once its CTAs fill the rest, long before their input (us a layer of 128 rows, 16 / 20 / 28 / 32 heads of 128: 67.9 / 77.4 / 102.4 / 121.7,
-// released behind the wait 63.9 / 73.4 / 99.0 / 120.5).
+// once its CTAs fill the rest, long before their input (us a layer of 128 rows, 16 / 20 / 28 / 32 heads of 128: 67.7 / 76.9 / 102.4 / 118.6,
+// released behind the wait 64.1 / 73.7 / 99.7 / 117.9).
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
